@@ -4,6 +4,8 @@
 #pragma once
 
 #include "thc_internal.cuh"
+#include "chol.cuh"
+#include "oz_gemm.cuh"
 
 #include <math.h>
 
@@ -40,29 +42,6 @@ __global__ void gather_cols(const double* __restrict__ R, long ng, const int* __
   if (i >= (long)np * np) return;
   const int P = (int)(i / np), Q = (int)(i % np);
   S[i] = R[(long)P * ng + pts[Q]];
-}
-
-// Column j of the Cholesky factor L (row-major, lower), left-looking: every
-// thread recomputes the pivot d_j = S_jj - sum_t L_jt^2 and forms its L_ij.
-// A pivot below 1e-12 S_jj marks the metric numerically singular.
-__global__ void chol_column(const double* __restrict__ S, double* __restrict__ L, int n, int j, int* bad) {
-  const int i = j + (int)((long)blockIdx.x * TB + threadIdx.x);
-  if (i >= n) return;
-  double d = S[(long)j * n + j];
-  const double sjj = d;
-  for (int t = 0; t < j; t++) d -= L[(long)j * n + t] * L[(long)j * n + t];
-  if (!(d > 1e-12 * sjj)) {
-    if (i == j) atomicOr(bad, 1);
-    return;
-  }
-  const double ljj = sqrt(d);
-  if (i == j) {
-    L[(long)j * n + j] = ljj;
-    return;
-  }
-  double a = S[(long)i * n + j];
-  for (int t = 0; t < j; t++) a -= L[(long)i * n + t] * L[(long)j * n + t];
-  L[(long)i * n + j] = a / ljj;
 }
 
 // X = L^-T L^-1 X for every column r of X[n][ng], in place.
@@ -202,6 +181,27 @@ inline bool fit_geometry(const int* grid_host, const double* lattice_host, const
       geo.tw[geo.off[ax] + t] = make_double2(cos(ang), sin(ang));
     }
   return true;
+}
+
+// gemm_z's product in the faster of its two forms.
+inline cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA,
+                               const double2* B, int ldb, long sB, double2* C, int ldc, long sC, int batch,
+                               const OzWork& w, cudaStream_t s) {
+  if (w.buf && oz_wins(M, N, K, batch) && w.bytes >= oz_work_min(K))
+    return oz_gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, w, s);
+  return gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, s);
+}
+
+// Scratch of the digit products of a fit and of its adjoint: the whole
+// operands of the metric, the solve and the products of depth kdeep (over the
+// grid or its G set, npts x ndeep; 0: none), up to 1.25 GB (larger slabs
+// measured no faster for the metric).  At least what the solve's least slab
+// needs: without room for more the other products run on the FP64 pipe.
+inline cudaError_t fit_scratch(OzWork& w, int npts, long ng, int nfunc, int ndeep, int kdeep, cudaStream_t s) {
+  const size_t least = oz_work_min(npts);
+  size_t want = std::max(oz_work_bytes(npts, (int)ng, nfunc, 1), oz_work_bytes(npts, (int)ng, npts, 1));
+  if (ndeep > 0) want = std::max(want, std::max(oz_work_min(kdeep), oz_work_bytes(npts, ndeep, kdeep, 1)));
+  return oz_alloc(w, std::max(least, std::min(want, (size_t)5 << 28)), least, s);
 }
 
 }  // namespace

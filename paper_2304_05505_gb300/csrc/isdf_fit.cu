@@ -119,6 +119,12 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
   const int* off = geo.off;
 
   cudaStream_t s = (cudaStream_t)stream;
+  // The all-FP64 form takes its products from exact digits on the tensor cores
+  // (metric 397 -> 15 ms, solve 75 -> 4 ms at 3x3x3 k, N_P = 600, 40^3 grid).
+  // THC_MIXED keeps the FP64 pipe's sums: the solve passes a change of 1e-15 in
+  // the metric on as 1e-12 (cond(S) 1e4), which changes FP32 roundings of the
+  // contraction's operands, so that V would move by 1e-10 to 1e-7 per element.
+  const bool dig = precision == THC_FP64;
   const int nk = n1 * n2 * n3;
   const long npq = (long)npts * npts;
   // step boundaries: 0 start, 1 after B R S, 2 after Cholesky, 3 after the
@@ -136,7 +142,8 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
   int *eX = nullptr, *ps0 = nullptr, *tcerr = nullptr;
   float* pbc = nullptr;
   double2 *Ugc = nullptr, *Bm = nullptr, *F = nullptr, *Xq = nullptr, *W = nullptr, *twd = nullptr;
-  double *R = nullptr, *S = nullptr, *L = nullptr, *rPd = nullptr;
+  double *R = nullptr, *S = nullptr, *L = nullptr, *Linv = nullptr, *rPd = nullptr;
+  OzWork oz;
   int *ptsd = nullptr, *gmd = nullptr, *flatd = nullptr, *bad = nullptr;
   cudaError_t e = cudaSuccess;
   thc_status st = THC_OK;
@@ -148,6 +155,8 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     if ((e = cudaMalloc(&R, sizeof(double) * (size_t)npts * ng)) != cudaSuccess) break;
     if ((e = cudaMalloc(&S, sizeof(double) * npq)) != cudaSuccess) break;
     if ((e = cudaMalloc(&L, sizeof(double) * npq)) != cudaSuccess) break;
+    if (dig && (e = cudaMalloc(&Linv, sizeof(double) * npq)) != cudaSuccess) break;
+    if (dig && (e = fit_scratch(oz, npts, ng, nfunc, npts, nG, s)) != cudaSuccess) break;
     if ((e = cudaMalloc(&bad, sizeof(int))) != cudaSuccess) break;
     if ((e = cudaMalloc(&twd, sizeof(double2) * tw.size())) != cudaSuccess) break;
     if ((e = cudaMalloc(&gmd, sizeof(int) * gm.size())) != cudaSuccess) break;
@@ -164,19 +173,17 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     if ((e = cudaMemcpyAsync(rPd, rP.data(), sizeof(double) * rP.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess)
       break;
     if ((e = cudaMemsetAsync(bad, 0, sizeof(int), s)) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(L, 0, sizeof(double) * npq, s)) != cudaSuccess) break;
     // 1. B = conj(U[:, points])^T U, R = |B|^2, S = R[:, points]
     mark(0);
     gather_conj<<<blocks((long)npts * nfunc), TB, 0, s>>>((const double2*)U, nfunc, ng, ptsd, npts, Ugc);
-    if ((e = gemm_z(A_MK, B_KN, npts, (int)ng, nfunc, Ugc, nfunc, 0, (const double2*)U, (int)ng, 0, Bm, (int)ng,
-                    0, 1, s)) != cudaSuccess)
+    if ((e = gemm_z_best(A_MK, B_KN, npts, (int)ng, nfunc, Ugc, nfunc, 0, (const double2*)U, (int)ng, 0, Bm, (int)ng,
+                         0, 1, oz, s)) != cudaSuccess)
       break;
     abs2_kernel<<<blocks((long)npts * ng), TB, 0, s>>>(Bm, (long)npts * ng, R);
     gather_cols<<<blocks(npq), TB, 0, s>>>(R, ng, ptsd, npts, S);
     // 2. xi = S^-1 R
     mark(1);
-    for (int j = 0; j < npts; j++) chol_column<<<blocks(npts - j), TB, 0, s>>>(S, L, npts, j, bad);
-    if ((e = cudaGetLastError()) != cudaSuccess) break;
+    if ((e = chol_factor(S, L, npts, bad, s)) != cudaSuccess) break;
     if ((e = cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
     if (hbad) {
@@ -185,7 +192,13 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
       break;
     }
     mark(2);
-    chol_solve<<<blocks(ng), TB, 0, s>>>(L, R, npts, ng);
+    if (dig) {
+      // (Bm is free once R and S are taken from it: scratch of the inverse and of the products)
+      if ((e = chol_inverse(L, Linv, (double*)Bm, npts, oz, s)) != cudaSuccess) break;
+      if ((e = chol_apply(Linv, R, (double*)Bm, npts, (int)ng, oz, s)) != cudaSuccess) break;
+    } else {
+      chol_solve<<<blocks(ng), TB, 0, s>>>(L, R, npts, ng);
+    }
     mark(3);
     if (xi_out &&
         (e = cudaMemcpyAsync(xi_out, R, sizeof(double) * npts * ng, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
@@ -240,7 +253,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
             if (!tc) {
               scale_xi<<<blocks((long)npts * nG), TB, 0, s>>>(F, ng, flatd, gmd, nG, rPd, npts, B, x0, x1, x2, w,
                                                               Xq);
-              if ((e = gemm_z(A_MK, B_NK_CONJ, npts, npts, nG, Xq, nG, 0, Xq, nG, 0, W, npts, 0, 1, s)) !=
+              if ((e = gemm_z_best(A_MK, B_NK_CONJ, npts, npts, nG, Xq, nG, 0, Xq, nG, 0, W, npts, 0, 1, oz, s)) !=
                   cudaSuccess)
                 break;
               add_kernel<<<blocks(npq), TB, 0, s>>>(V + (long)q * npq, W, npq);
@@ -273,12 +286,13 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     mark(5);
     if ((e = cudaGetLastError()) != cudaSuccess) break;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
-    if (tcerr) {
-      int h = 0;
-      if ((e = cudaMemcpy(&h, tcerr, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
-      if (h) {
+    {
+      int h = 0, ho = 0;
+      if (tcerr && (e = cudaMemcpy(&h, tcerr, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
+      if (dig && (e = cudaMemcpy(&ho, oz.err(), sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
+      if (h || ho) {
         st = THC_ERR_TIMEOUT;
-        set_global_error("thc_rebuild_kernel: a device wait of the tensor-core contraction timed out");
+        set_global_error("thc_rebuild_kernel: a device wait of a tensor-core product timed out");
         break;
       }
     }
@@ -292,9 +306,10 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     set_global_error(std::string("thc_fit_kernel: ") + cudaGetErrorString(e));
     st = e == cudaErrorMemoryAllocation ? THC_ERR_OOM : THC_ERR_CUDA;
   }
-  void* ptrs[] = {Ugc, Bm, F, Xq, W, twd, R, S, L, rPd, ptsd, gmd, flatd, bad, Xq32, Bpl, eX, ps0, pbc, tcerr};
+  void* ptrs[] = {Ugc, Bm, F, Xq, W, twd, R, S, L, Linv, rPd, ptsd, gmd, flatd, bad, Xq32, Bpl, eX, ps0, pbc, tcerr};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  oz_free(oz);
   for (auto& x : ev)
     if (x) cudaEventDestroy(x);
   return st;

@@ -1,0 +1,40 @@
+// FP64 matrix products on the tensor cores from exact bf16 digits (oz_gemm.cu).
+#pragma once
+
+#include "thc_internal.cuh"
+
+// Scratch of the products: digit planes, row exponents and the error word of
+// the kernels' bounded waits, one device allocation of `bytes` bytes.  A
+// product that does not fit is taken in slabs (of the batch, or of the rows of
+// the larger operand).  Owned by one caller on one stream at a time.
+struct OzWork {
+  unsigned char* buf = nullptr;
+  size_t bytes = 0;
+  int* err() const { return (int*)buf; }
+};
+
+// Deepest real K of a product (its int64 sums stay below 2^62).
+constexpr long OZ_MAX_K = 1L << 19;
+
+// Scratch bytes for a product of this shape taken whole (complex), and the
+// least a product of depth K (complex) can run with.
+size_t oz_work_bytes(int M, int N, int K, int batch);
+size_t oz_work_min(int K);
+
+// Allocates scratch: `want` bytes, or halves of it down to `least` where the
+// device has no room for more (cudaErrorMemoryAllocation when it has not even
+// that), and clears its error word on `s`.  oz_free gives it back.
+cudaError_t oz_alloc(OzWork& w, size_t want, size_t least, cudaStream_t s);
+void oz_free(OzWork& w);
+
+// Whether the digit form is the faster one for this complex product.
+bool oz_wins(int M, int N, int K, int batch);
+
+// gemm_z's product (operand layouts of GemmA, GemmB) from digits.
+cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
+                      int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s);
+
+// Real C[m][n] = alpha sum_k A(m, k) B(n, k) (+ C when acc): A(m, k) = A[m lda + k]
+// or, a_km, A[k lda + m]; B(n, k) = B[n ldb + k] or, b_kn, B[k ldb + n].  alpha is 1 or -1.
+cudaError_t oz_gemm_d(bool a_km, bool b_kn, int M, int N, int K, const double* A, long lda, const double* B, long ldb,
+                      double* C, long ldc, double alpha, bool acc, const OzWork& w, cudaStream_t s);

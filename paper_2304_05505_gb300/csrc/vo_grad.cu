@@ -358,6 +358,10 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     }
 
   cudaStream_t s = (cudaStream_t)stream;
+  // THC_FP64 takes its products from exact digits on the tensor cores; THC_MIXED
+  // keeps the FP64 pipe's sums wherever a solve with the metric follows (as in
+  // isdf_fit.cu: their last bits decide FP32 roundings of the later products).
+  const bool dig = precision == THC_FP64;
   // step boundaries: 0 start, 1 after the fixed-kernel part (D, W, M, Y, g_e),
   // 2 after the fit, 3 after the (q, G) contraction, 4 after the DFT adjoint,
   // the solve and S-bar, 5 after the orbital adjoint and the sum
@@ -372,7 +376,8 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
   double2 *Psi = nullptr, *Psivt = nullptr, *D = nullptr, *M = nullptr, *W = nullptr, *Y = nullptr, *Ge = nullptr;
   double2 *Ugc = nullptr, *Bm = nullptr, *F = nullptr, *T = nullptr, *Gam = nullptr, *Aq = nullptr, *Bq = nullptr;
   double2 *Z = nullptr, *T1 = nullptr, *T2 = nullptr, *Uvp = nullptr, *G1 = nullptr, *G2 = nullptr, *twd = nullptr;
-  double *R = nullptr, *S = nullptr, *L = nullptr, *Lam = nullptr, *Sbar = nullptr, *rPd = nullptr, *part = nullptr;
+  OzWork oz;
+  double *R = nullptr, *S = nullptr, *L = nullptr, *Linv = nullptr, *Lam = nullptr, *Sbar = nullptr, *rPd = nullptr, *part = nullptr;
   int *ptsd = nullptr, *gmd = nullptr, *flatd = nullptr, *bad = nullptr, *kqd = nullptr, *qkd = nullptr;
   // tensor-core state of the (q, G) contraction (THC_MIXED)
   float2* Aq32 = nullptr;
@@ -426,6 +431,8 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
       break;
     if ((e = cudaMemsetAsync(bad, 0, sizeof(int), s)) != cudaSuccess) break;
 
+    if ((e = fit_scratch(oz, np, ng, nf, precision == THC_FP64 ? std::max(nf, nvir) : np, (int)ng, s)) != cudaSuccess) break;
+
     // 1. the kernel held fixed: Psi, Psi_v at the points, D, W, M, Y, E_x, g_e
     mark(0);
     const double2* U2 = (const double2*)U;
@@ -434,19 +441,19 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
                                                              true, false, Psi);
     point_values<<<blocks((long)nk * nvir * np), TB, 0, s>>>(Uv2, nk, nvir, ng, ptsd, np, g1, g2, g3, n1, n2, n3,
                                                              true, true, Psivt);
-    if ((e = gemm_z(A_MK, B_NK_CONJ, np, np, nocc, Psi, nocc, (long)np * nocc, Psi, nocc, (long)np * nocc, D, np,
-                    npq, nk, s)) != cudaSuccess)
+    if ((e = gemm_z_best(A_MK, B_NK_CONJ, np, np, nocc, Psi, nocc, (long)np * nocc, Psi, nocc, (long)np * nocc, D, np,
+                    npq, nk, oz, s)) != cudaSuccess)
       break;
     kcorr_kernel<<<blocks(npq), TB, 0, s>>>(D, (const double2*)V, kqd, qkd, nk, npq, W, M);
     wv_partial<<<NPART, TB, 0, s>>>(W, (const double2*)V, nk * npq, part);
     if (ex_host &&
         (e = cudaMemcpyAsync(hpart.data(), part, sizeof(double) * NPART, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
       break;
-    if ((e = gemm_z(A_MK, B_KN, np, nocc, np, M, np, npq, Psi, nocc, (long)np * nocc, Y, nocc, (long)np * nocc, nk,
-                    s)) != cudaSuccess)
+    if ((e = gemm_z_best(A_MK, B_KN, np, nocc, np, M, np, npq, Psi, nocc, (long)np * nocc, Y, nocc, (long)np * nocc,
+                         nk, oz, s)) != cudaSuccess)
       break;
-    if ((e = gemm_z(A_MK_CONJ, B_KN, nvir, nocc, np, Psivt, np, (long)nvir * np, Y, nocc, (long)np * nocc, Ge, nocc,
-                    (long)nvir * nocc, nk, s)) != cudaSuccess)
+    if ((e = gemm_z_best(A_MK_CONJ, B_KN, nvir, nocc, np, Psivt, np, (long)nvir * np, Y, nocc, (long)np * nocc, Ge, nocc,
+                    (long)nvir * nocc, nk, oz, s)) != cudaSuccess)
       break;
     cudaFree(D);
     cudaFree(M);
@@ -462,14 +469,17 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     if ((e = cudaMalloc(&R, sizeof(double) * (size_t)np * ng)) != cudaSuccess) break;
     if ((e = cudaMalloc(&S, sizeof(double) * npq)) != cudaSuccess) break;
     if ((e = cudaMalloc(&L, sizeof(double) * npq)) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(L, 0, sizeof(double) * npq, s)) != cudaSuccess) break;
+    if (dig && (e = cudaMalloc(&Linv, sizeof(double) * npq)) != cudaSuccess) break;
+    if ((e = cudaMalloc(&F, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
+    if ((e = cudaMalloc(&T, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
     gather_conj<<<blocks((long)np * nf), TB, 0, s>>>(U2, nf, ng, ptsd, np, Ugc);
-    if ((e = gemm_z(A_MK, B_KN, np, (int)ng, nf, Ugc, nf, 0, U2, (int)ng, 0, Bm, (int)ng, 0, 1, s)) != cudaSuccess)
+    if ((e = dig ? gemm_z_best(A_MK, B_KN, np, (int)ng, nf, Ugc, nf, 0, U2, (int)ng, 0, Bm, (int)ng, 0, 1, oz, s)
+                 : gemm_z(A_MK, B_KN, np, (int)ng, nf, Ugc, nf, 0, U2, (int)ng, 0, Bm, (int)ng, 0, 1, s)) !=
+        cudaSuccess)
       break;
     abs2_kernel<<<blocks((long)np * ng), TB, 0, s>>>(Bm, (long)np * ng, R);
     gather_cols<<<blocks(npq), TB, 0, s>>>(R, ng, ptsd, np, S);
-    for (int j = 0; j < np; j++) chol_column<<<blocks(np - j), TB, 0, s>>>(S, L, np, j, bad);
-    if ((e = cudaGetLastError()) != cudaSuccess) break;
+    if ((e = chol_factor(S, L, np, bad, s)) != cudaSuccess) break;
     if ((e = cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
     if (hbad) {
@@ -477,9 +487,13 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
       set_global_error("thc_vo_gradient: the Gram matrix of the points is not positive definite");
       break;
     }
-    chol_solve<<<blocks(ng), TB, 0, s>>>(L, R, np, ng);   // R now holds xi
-    if ((e = cudaMalloc(&F, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&T, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
+    if (dig) {
+      if ((e = chol_inverse(L, Linv, (double*)F, np, oz, s)) != cudaSuccess) break;
+      if ((e = chol_apply(Linv, R, (double*)F, np, (int)ng, oz, s)) != cudaSuccess) break;
+    } else {
+      chol_solve<<<blocks(ng), TB, 0, s>>>(L, R, np, ng);
+    }
+    // R now holds xi
     const long tot = (long)np * ng;
     dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(R, true, F, tot, g3, 1, twd + geo.off[2]);
     dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(F, false, T, tot, g2, g3, twd + geo.off[1]);
@@ -538,7 +552,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
             coulomb_conj<<<blocks((long)np * nG), TB, 0, s>>>(F, ng, flatd, gmd, nG, np, B, x0, x1, x2, Bq);
             if (!tc) {
               phase_w<<<blocks(npq), TB, 0, s>>>(W + (long)q * npq, np, rPd, qx, qy, qz, c, Aq);
-              if ((e = gemm_z(A_MK, B_KN, np, nG, np, Aq, np, 0, Bq, nG, 0, Z, nG, 0, 1, s)) != cudaSuccess) break;
+              if ((e = gemm_z_best(A_MK, B_KN, np, nG, np, Aq, np, 0, Bq, nG, 0, Z, nG, 0, 1, oz, s)) != cudaSuccess) break;
             } else {
               phase_w32<<<blocks(npq), TB, 0, s>>>(W + (long)q * npq, np, rPd, qx, qy, qz, c, Aq32, lda);
               if ((e = row_exponents_c(Aq32, 0, lda, 1, np, np, eA, s)) != cudaSuccess) break;
@@ -572,9 +586,17 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(F, false, T, tot, g1, (long)g2 * g3, twd + geo.off[0]);
     if ((e = cudaMalloc(&Lam, sizeof(double) * (size_t)np * ng)) != cudaSuccess) break;
     real_part<<<blocks(tot), TB, 0, s>>>(T, tot, Lam);
-    chol_solve<<<blocks(ng), TB, 0, s>>>(L, Lam, np, ng);
+    if (dig) {
+      if ((e = chol_apply(Linv, Lam, (double*)F, np, (int)ng, oz, s)) != cudaSuccess) break;
+    } else {
+      chol_solve<<<blocks(ng), TB, 0, s>>>(L, Lam, np, ng);
+    }
     if ((e = cudaMalloc(&Sbar, sizeof(double) * npq)) != cudaSuccess) break;
-    {
+    // S-bar = -Lam xi^T
+    if (dig && ng <= OZ_MAX_K && oz.bytes >= oz_work_min((int)((ng + 1) / 2))) {
+      if ((e = oz_gemm_d(false, false, np, np, (int)ng, Lam, ng, R, ng, Sbar, np, -1.0, false, oz, s)) != cudaSuccess)
+        break;
+    } else {
       dim3 grid((np + DT - 1) / DT, (np + DT - 1) / DT);
       gemm_d_nt<<<grid, TB, 0, s>>>(np, np, ng, Lam, ng, R, ng, Sbar, np, -1.0);
     }
@@ -599,13 +621,13 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     // 126 chunks of 1024); else, and in THC_FP64, FP64 GEMMs
     const bool tc_orb = tc && 2L * ng <= 126L * 1024;
     if (!tc_orb) {
-      if ((e = gemm_z(A_MK, B_NK, np, nf, (int)ng, Bm, (int)ng, 0, U2, (int)ng, 0, T1, nf, 0, 1, s)) != cudaSuccess)
+      if ((e = gemm_z_best(A_MK, B_NK, np, nf, (int)ng, Bm, (int)ng, 0, U2, (int)ng, 0, T1, nf, 0, 1, oz, s)) != cudaSuccess)
         break;
-      if ((e = gemm_z(A_KM, B_KN, nf, (int)ng, np, Ugc, nf, 0, Bm, (int)ng, 0, T2, (int)ng, 0, 1, s)) !=
+      if ((e = gemm_z_best(A_KM, B_KN, nf, (int)ng, np, Ugc, nf, 0, Bm, (int)ng, 0, T2, (int)ng, 0, 1, oz, s)) !=
           cudaSuccess)
         break;
-      if ((e = gemm_z(A_MK, B_NK, nvir, nocc, (int)ng, Uv2, (int)ng, (long)nvir * ng, T2, (int)ng, (long)nocc * ng,
-                      G1, nocc, (long)nvir * nocc, nk, s)) != cudaSuccess)
+      if ((e = gemm_z_best(A_MK, B_NK, nvir, nocc, (int)ng, Uv2, (int)ng, (long)nvir * ng, T2, (int)ng, (long)nocc * ng,
+                      G1, nocc, (long)nvir * nocc, nk, oz, s)) != cudaSuccess)
         break;
     } else {
       const int ldy = (int)(ng + (ng & 1));           // FP32 grid rows 16-byte strided
@@ -644,19 +666,20 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     }
     point_values<<<blocks((long)nk * nvir * np), TB, 0, s>>>(Uv2, nk, nvir, ng, ptsd, np, g1, g2, g3, n1, n2, n3,
                                                              false, true, Uvp);
-    if ((e = gemm_z(A_MK_CONJ, B_KN, nvir, nocc, np, Uvp, np, (long)nvir * np, T1, nf, nocc, G2, nocc,
-                    (long)nvir * nocc, nk, s)) != cudaSuccess)
+    if ((e = gemm_z_best(A_MK_CONJ, B_KN, nvir, nocc, np, Uvp, np, (long)nvir * np, T1, nf, nocc, G2, nocc,
+                    (long)nvir * nocc, nk, oz, s)) != cudaSuccess)
       break;
     combine_g<<<blocks(ngo), TB, 0, s>>>(Ge, G1, G2, ngo, -4.0 / nk, (double2*)g_out, (double2*)g_explicit_out);
     mark(5);
     if ((e = cudaGetLastError()) != cudaSuccess) break;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
-    if (tcerr) {
-      int h = 0;
-      if ((e = cudaMemcpy(&h, tcerr, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
-      if (h) {
+    {
+      int h = 0, ho = 0;
+      if (tcerr && (e = cudaMemcpy(&h, tcerr, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
+      if ((e = cudaMemcpy(&ho, oz.err(), sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
+      if (h || ho) {
         st = THC_ERR_TIMEOUT;
-        set_global_error("thc_vo_gradient: a device wait of the tensor-core contraction timed out");
+        set_global_error("thc_vo_gradient: a device wait of a tensor-core product timed out");
         break;
       }
     }
@@ -676,10 +699,11 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     st = e == cudaErrorMemoryAllocation ? THC_ERR_OOM : THC_ERR_CUDA;
   }
   void* ptrs[] = {Psi, Psivt, D,   M,   W,  Y,  Ge,  Ugc,   Bm,    F,    T,     Gam,  Aq,  Bq,  Z,
-                  T1,  T2,    Uvp, G1,  G2, twd, R,  S,     L,     Lam,  Sbar,  rPd,  part, ptsd, gmd,
+                  T1,  T2,    Uvp, G1,  G2, twd, R,  S,     L,     Linv,  Lam,  Sbar,  rPd,  part, ptsd, gmd,
                   flatd, bad, kqd, qkd, Aq32, Bpl, eA,  eB,  ps0, pbc, tcerr, Y32, A2, Uv32, eOrb};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  oz_free(oz);
   for (auto& x : ev)
     if (x) cudaEventDestroy(x);
   return st;
