@@ -183,15 +183,6 @@ inline bool fit_geometry(const int* grid_host, const double* lattice_host, const
   return true;
 }
 
-// gemm_z's product in the faster of its two forms.
-inline cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA,
-                               const double2* B, int ldb, long sB, double2* C, int ldc, long sC, int batch,
-                               const OzWork& w, cudaStream_t s) {
-  if (w.buf && oz_wins(M, N, K, batch) && w.bytes >= oz_work_min(K))
-    return oz_gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, w, s);
-  return gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, s);
-}
-
 // Scratch of the digit products of a fit and of its adjoint: the whole
 // operands of the metric, the solve and the products of depth kdeep (over the
 // grid or its G set, npts x ndeep; 0: none), up to 1.25 GB (larger slabs

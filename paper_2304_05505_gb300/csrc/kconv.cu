@@ -25,6 +25,7 @@
 //                      lanes per element, first axis by shuffles)
 //   kconv_kernel       any mesh: one thread per element, its N_k values in
 //                      shared memory ([k][thread], conflict-free)
+//   (FP64, axes of 1 to 4 points: kconv_fix.cu)
 // All run the separable 3-D DFT axis by axis with radix-2/3/4 butterflies or
 // a direct DFT for other lengths, multiply by Vh and transform back.
 //
@@ -1283,6 +1284,7 @@ cudaError_t mlo_combine_c2z(const float2* M, const uint32_t* Mlo, double2* out, 
 
 cudaError_t kconv_z(const double2* D, const double2* Vh, double2* M, long npq, int n1, int n2,
                     int n3, cudaStream_t s) {
+  if (kconv_fix_applies(n1, n2, n3)) return kconv_fix_z(D, Vh, M, npq, n1, n2, n3, s);
   return kconv_launch<double>(D, Vh, M, npq, n1, n2, n3, s);
 }
 

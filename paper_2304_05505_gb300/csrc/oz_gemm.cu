@@ -9,12 +9,14 @@
 // of a double).  A digit has at most 8 significant bits, so the planes
 // 2^(-9 s) d_s are exact bf16 numbers, products of two digits are exact in
 // FP32, and with C_c = sum over s + t = c of A_s B_t
-//   A B = 2^(e_a + e_b - 16) (C_0 + C_1 + ... + C_6)   (C_7 and on dropped, 2^-63).
+//   A B = 2^(e_a + e_b - 16) (C_0 + C_1 + ... + C_7)   (C_8 and on dropped, 2^-72:
+// C_7 costs 6 of the 34 digit products; without it rows with a few dominant
+// entries, as those of the collocation, lose 1e-15 of their products).
 // Over a chunk of 64 K the classes C_0 .. C_3 are sums of at most 4 x 64
 // integers of at most 2^16 in units of 2^(-9 c): below 2^24, where the tensor
 // core's FP32 accumulator is exact whatever its rounding.  After every chunk
 // they are added into one int64 per output (units of C_3; |sum| < K 2^43), with
-// the whole units of C_4; what is left of C_4 and C_5 + C_6 go into one FP32
+// the whole units of C_4; what is left of C_4 and C_5 + C_6 + C_7 go into one FP32
 // number.  The double is rounded once, from integers.  So the result carries
 // the error of rounding the operands at 2^-63 of their row scale, the dropped
 // classes and one final rounding: 5e-17 of the result on random operands of
@@ -27,15 +29,16 @@
 // One CTA per SM loops over 128 x 80 output tiles, all of K each:
 //   warp 0    TMA: one box of [7 planes][128 rows][32 K] and one of
 //             [7][80][32] per stage (91 KB, two stages, 64B swizzle)
-//   warp 1    28 digit products per 16 K, one MMA (128 x 80 x 16) each, into
-//             six accumulators of 80 TMEM columns: C_0 .. C_4, and C_5 + C_6.
+//   warp 1    34 digit products per 16 K, one MMA (128 x 80 x 16) each, into
+//             six accumulators of 80 TMEM columns: C_0 .. C_4, and C_5 + C_6 + C_7.
 //             A wider tile would read less shared memory per product (6.5 KB
 //             here, 52 cycles of 40 MMA cycles), but six accumulators fill
-//             TMEM: C_4 shares none, since rounding it with C_5 and C_6 on
+//             TMEM: C_4 shares none, since rounding it with C_5 .. C_7 on
 //             the way would leave 2^-51 of the result.
-//   warps 4-19  drain C_0 .. C_3 while C_4 .. C_6 are still being multiplied,
-//             and C_4 .. C_6 under the next chunk's C_0 .. C_3: the
-//             accumulators need no second set.
+//   warps 4-19  drain one accumulator after the other, each as soon as the
+//             chunk's last product into it is done and while the later classes
+//             are still being multiplied; the next chunk starts on C_0 when C_0
+//             is drained.  So the accumulators need no second set.
 // The integer epilogue keeps the FP64 pipe (2 results per SM and clock) out of
 // the kernel: conversion and rounding of an output are about 30 integer
 // instructions.
@@ -53,6 +56,7 @@ constexpr int ND = 7;                                  // digits
 constexpr int TL = 128, TN = 80, TK = 32;              // lane rows, column rows, K of a stage
 constexpr uint32_t LPL = TL * TK * 2, CPL = TN * TK * 2;    // bytes of a plane tile: 8 KB, 5 KB
 constexpr uint32_t STAGE = ND * (LPL + CPL);           // 91 KB
+constexpr int NACC = 6;                                // accumulators: C_0 .. C_4, and C_5 + C_6 + C_7
 constexpr int STAGES = 2;
 constexpr int CHUNK_ST = 2;                            // stages of an exact chunk (64 K)
 constexpr size_t SMEM = STAGES * STAGE + 1024 + 128;
@@ -121,21 +125,17 @@ __device__ __forceinline__ void tmem_ld10(uint32_t t, float* v) {
   for (int i = 0; i < 10; i++) v[i] = __uint_as_float(r[i]);
 }
 
-// acc[j] += the integers v 2^up of class columns t .. t + 9, times `unit` (in units of C_3).
-__device__ __forceinline__ void add_class(uint32_t t, float up, int unit, long long* acc) {
-  float v[EH];
-  tmem_ld10(t, v);
-#pragma unroll
-  for (int j = 0; j < EH; j++) acc[j] += (long long)__float2int_rn(v[j] * up) * unit;
-}
+// v 2^s outside the normal range (out of line: it is as long as the rest).
+__device__ __noinline__ double scale_slow(double v, int s) { return ldexp(v, s); }
 
-// The double nearest (a + f) 2^sexp (a an integer, |a| < 2^62, f a small FP32 part), by integer operations.
+// The double nearest (a + f) 2^sexp (a an integer, |a| < 2^62, f a small FP32 part), by integer operations
+// (a negation, too, would go through the FP64 pipe).
 __device__ __forceinline__ double round_sum(long long a, float f, int sexp) {
   const int fi = __float2int_rn(f);          // |f| < 2^22: at most 2^8 per chunk of 64 K
   a += fi;
   f -= (float)fi;                            // |f| <= 1/2
   unsigned long long m = a < 0 ? -(unsigned long long)a : (unsigned long long)a;
-  if (m == 0) return ldexp((double)f, sexp);
+  if (m == 0) return f == 0.f ? 0.0 : scale_slow((double)f, sexp);
   if (a < 0) f = -f;
   int s = __clzll((long long)m) - 1;
   m <<= s;                                   // leading bit 62 (s >= 0)
@@ -147,10 +147,15 @@ __device__ __forceinline__ double round_sum(long long a, float f, int sexp) {
   }
   m = (m + 511 + ((m >> 10) & 1)) >> 10;     // 53 bits, to nearest, ties to even
   const int E = 1085 + sexp - s;             // value = m 2^(sexp - s + 10), 2^52 <= m <= 2^53
-  double r;
-  if (E >= 1 && E <= 2045) r = __longlong_as_double((long long)(((unsigned long long)(E - 1) << 52) + m));
-  else r = ldexp((double)m, sexp - s + 10);
-  return a < 0 ? -r : r;
+  if (E < 1 || E > 2045) {
+    const double r = scale_slow((double)m, sexp - s + 10);
+    return a < 0 ? -r : r;
+  }
+  return __longlong_as_double((long long)(((unsigned long long)(E - 1) << 52) + m | (unsigned long long)a & 1ull << 63));
+}
+
+__device__ __forceinline__ double flip(double x) {
+  return __longlong_as_double(__double_as_longlong(x) ^ (long long)(1ull << 63));
 }
 
 __global__ void __launch_bounds__(NT, 1)
@@ -159,14 +164,14 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE);
-  uint32_t* tmem_slot = (uint32_t*)(bars + 12);
+  uint32_t* tmem_slot = (uint32_t*)(bars + 17);
   const uint32_t sbase = smem_u32(smem), bar0 = smem_u32(bars);
   auto FULL = [&](int s) { return bar0 + 8u * s; };
   auto EMPTY = [&](int s) { return bar0 + 8u * (2 + s); };
-  // accumulators of C_0 .. C_3 (h = 0) and C_4 .. C_6 (h = 1): complete, drained
-  auto AFULL = [&](int h) { return bar0 + 8u * (4 + h); };
-  auto AEMPTY = [&](int h) { return bar0 + 8u * (6 + h); };
-  const uint32_t DONE = bar0 + 8u * 8;
+  // accumulator c (C_0 .. C_4, and 5: C_5 + C_6 + C_7): complete, drained
+  auto AFULL = [&](int c) { return bar0 + 8u * (4 + c); };
+  auto AEMPTY = [&](int c) { return bar0 + 8u * (10 + c); };
+  const uint32_t DONE = bar0 + 8u * 16;
 
   __shared__ int abort_flag;
   if (threadIdx.x == 0) abort_flag = *(volatile int*)err;
@@ -177,8 +182,10 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
     for (int s = 0; s < 2; s++) {
       mbar_init(FULL(s), 1);
       mbar_init(EMPTY(s), 1);
-      mbar_init(AFULL(s), 1);
-      mbar_init(AEMPTY(s), EPI_W);
+    }
+    for (int c = 0; c < NACC; c++) {
+      mbar_init(AFULL(c), 1);
+      mbar_init(AEMPTY(c), EPI_W);
     }
     mbar_init(DONE, 1);
     mbar_fence_init();
@@ -234,34 +241,26 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
             const uint32_t sl = it & 1;
             const bool first = st == c * CHUNK_ST, last = st == st1 - 1;
             if (!mbar_wait(FULL(sl), (it >> 1) & 1, err, 8)) { ok = false; break; }
-            if (first && !mbar_wait(AEMPTY(0), (ch & 1) ^ 1, err, 4)) { ok = false; break; }
             tc_fence_after();
             const uint64_t al = d0 + ((sl * STAGE) >> 4), bn = al + ((ND * LPL) >> 4);
-            // C_0 .. C_3
 #pragma unroll
-            for (int cl = 0; cl < 4; cl++)
+            for (int c6 = 0; c6 < NACC; c6++) {
+              if (first) {
+                if (!mbar_wait(AEMPTY(c6), (ch & 1) ^ 1, err, 4)) { ok = false; break; }
+                tc_fence_after();
+              }
 #pragma unroll
-              for (int s = 0; s <= cl; s++)
+              for (int cl = c6 == 5 ? 7 : c6; cl >= c6; cl--)      // C_7, C_6, C_5
 #pragma unroll
-                for (int kk = 0; kk < 2; kk++)
-                  mma_bf16(tmem + cl * TN, al + s * PL + 2 * kk, bn + (cl - s) * PC + 2 * kk,
-                           !(first && s == 0 && kk == 0));
-            if (last) commit(AFULL(0));
-            if (first) {
-              if (!mbar_wait(AEMPTY(1), (ch & 1) ^ 1, err, 4)) { ok = false; break; }
-              tc_fence_after();
+                for (int s = cl == 7; s <= min(cl, ND - 1); s++)
+#pragma unroll
+                  for (int kk = 0; kk < 2; kk++)
+                    mma_bf16(tmem + c6 * TN, al + s * PL + 2 * kk, bn + (cl - s) * PC + 2 * kk,
+                             !(first && (cl < 5 || cl == 7) && s == (cl == 7) && kk == 0));
+              if (last) commit(AFULL(c6));
             }
-            // C_4, and C_6 + C_5
-#pragma unroll
-            for (int cl = 6; cl >= 4; cl--)
-#pragma unroll
-              for (int s = 0; s <= cl; s++)
-#pragma unroll
-                for (int kk = 0; kk < 2; kk++)
-                  mma_bf16(tmem + min(cl, 5) * TN, al + s * PL + 2 * kk, bn + (cl - s) * PC + 2 * kk,
-                           !(first && cl != 5 && s == 0 && kk == 0));
+            if (!ok) break;
             commit(EMPTY(sl));
-            if (last) commit(AFULL(1));
           }
         }
       }
@@ -285,39 +284,37 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
         rest[j] = 0.f;
       }
       for (int c = 0; c < nchunk; c++, ch++) {
-        if (!mbar_wait_warp(AFULL(0), ch & 1, err, 16)) { ok = false; break; }
-        tc_fence_after();
         // class c holds integers in units of 2^(-9 c); in units of C_3 they count 2^(27 - 9 c)
 #pragma unroll
-        for (int f = 0; f < EC; f += EH) {
-          add_class(tl + f, 1.f, 1 << 27, acc + f);
-          add_class(tl + TN + f, 0x1p9f, 1 << 18, acc + f);
-          add_class(tl + 2 * TN + f, 0x1p18f, 1 << 9, acc + f);
-          add_class(tl + 3 * TN + f, 0x1p27f, 1, acc + f);
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(AEMPTY(0));
-        if (!mbar_wait_warp(AFULL(1), ch & 1, err, 16)) { ok = false; break; }
-        tc_fence_after();
+        for (int c6 = 0; c6 < NACC; c6++) {
+          // (every lane polls: the sleeping wait of one lane woke up to 250 ns late, six times a chunk)
+          if (!__all_sync(0xffffffffu, mbar_wait(AFULL(c6), ch & 1, err, 16))) { ok = false; break; }
+          tc_fence_after();
 #pragma unroll
-        for (int f = 0; f < EC; f += EH) {
-          float v[EH];
-          tmem_ld10(tl + 4 * TN + f, v);
+          for (int f = 0; f < EC; f += EH) {
+            float v[EH];
+            tmem_ld10(tl + c6 * TN + f, v);
+            if (f + EH == EC) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(AEMPTY(c6));
+            }
 #pragma unroll
-          for (int j = 0; j < EH; j++) {
-            const float x4 = v[j] * 0x1p27f;       // C_4 in units of C_3, a multiple of 2^-9
-            const int n4 = __float2int_rn(x4);
-            acc[f + j] += n4;
-            rest[f + j] += x4 - (float)n4;
+            for (int j = 0; j < EH; j++) {
+              if (c6 < 4) {
+                acc[f + j] += (long long)__float2int_rn(v[j] * (float)(1 << (9 * (c6 & 3)))) * (1 << (27 - 9 * (c6 & 3)));
+              } else if (c6 == 4) {
+                const float x4 = v[j] * 0x1p27f;   // C_4 in units of C_3, a multiple of 2^-9
+                const int n4 = __float2int_rn(x4);
+                acc[f + j] += n4;
+                rest[f + j] += x4 - (float)n4;
+              } else {
+                rest[f + j] = fmaf(v[j], 0x1p27f, rest[f + j]);
+              }
+            }
           }
-          tmem_ld10(tl + 5 * TN + f, v);
-#pragma unroll
-          for (int j = 0; j < EH; j++) rest[f + j] = fmaf(v[j], 0x1p27f, rest[f + j]);
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(AEMPTY(1));
+        if (!ok) break;
       }
       if (!ok) break;
       const int i = li * TL + 32 * q + lane, j0 = ni * TN + EC * h;
@@ -335,11 +332,14 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
             double x = round_sum(acc[j], rest[j], es + e0), y = two ? round_sum(acc[j + 1], rest[j + 1], es + e1) : 0.0;
             if (ei == NB_ROW || e0 == NB_ROW) x = __longlong_as_double(0x7ff8000000000000ll);
             if (ei == NB_ROW || e1 == NB_ROW) y = __longlong_as_double(0x7ff8000000000000ll);
+            if (g.alpha < 0) {
+              x = flip(x);
+              y = flip(y);
+            }
             if (g.pairs) {
               reinterpret_cast<double2*>(out)[(long)b * g.sbo + (long)(col >> 1) * g.ldo + i] = make_double2(x, y);
             } else {
               double* o = out + (long)b * g.sbo + (long)col * g.ldo + i;
-              if (g.alpha < 0) x = -x, y = -y;
               if (g.acc) {
                 o[0] += x;
                 if (two) o[g.ldo] += y;
@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ 
     if (CX == 2) {
       const double2 v = in ? *reinterpret_cast<const double2*>(p + 2 * j) : make_double2(0.0, 0.0);
       x[2 * j] = v.x;
-      x[2 * j + 1] = conj ? -v.y : v.y;
+      x[2 * j + 1] = conj ? flip(v.y) : v.y;
     } else {
       x[j] = in ? p[j] : 0.0;
     }
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ 
     if (CX == 2) {
       const double2 v = in ? *reinterpret_cast<const double2*>(p) : make_double2(0.0, 0.0);
       t[k][2 * r] = v.x;
-      t[k][2 * r + 1] = conj ? -v.y : v.y;
+      t[k][2 * r + 1] = conj ? flip(v.y) : v.y;
     } else {
       t[k][r] = in ? p[0] : 0.0;
     }
@@ -599,6 +599,7 @@ cudaError_t launch(const OzMaps& maps, const OzShape& g, const int* eL, const in
   if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
   if (e != cudaSuccess) return e;
   oz_kernel<<<(unsigned)std::min<long>(g.units, nsm), NT, SMEM, s>>>(maps, g, eL, eN, out, w.err());
+  if (w.launches) ++*w.launches;
   return cudaGetLastError();
 }
 
@@ -638,6 +639,7 @@ cudaError_t product(Side L, Side N, int K, int batch, double* out, long ldo, lon
       uint16_t* pN = (uint16_t*)((unsigned char*)eN + align256(sizeof(int) * (size_t)n.rows * nb));
       cudaError_t e = prepare<CX>(n, K, nb, eN, pN, s);
       if (e != cudaSuccess) return e;
+      if (w.launches) *w.launches += 2;
       unsigned char* lbuf = (unsigned char*)eN + side_bytes(n.rows, plane_rows(n), Kr, nb);
       OzMaps maps;
       if ((e = plane_map(&maps.n, pN, nb, plane_rows(n), Kr, ldp, TN)) != cudaSuccess) return e;
@@ -648,6 +650,7 @@ cudaError_t product(Side L, Side N, int K, int batch, double* out, long ldo, lon
         int* eL = (int*)lbuf;
         uint16_t* pL = (uint16_t*)(lbuf + align256(sizeof(int) * (size_t)l.rows * nb));
         if ((e = prepare<CX>(l, K, nb, eL, pL, s)) != cudaSuccess) return e;
+        if (w.launches) *w.launches += 2;
         if ((e = plane_map(&maps.l, pL, nb, plane_rows(l), Kr, ldp, TL)) != cudaSuccess) return e;
         OzShape g;
         g.nl = (int)plane_rows(l);
@@ -712,7 +715,13 @@ cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int
                       int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s) {
   Side a{(const double*)A, M, la == A_KM ? 1L : (long)lda, la == A_KM ? (long)lda : 1L, sA, la == A_MK_CONJ, false};
   Side b{(const double*)B, N, lb == B_KN ? 1L : (long)ldb, lb == B_KN ? (long)ldb : 1L, sB, lb == B_NK_CONJ, false};
-  if (M <= N) {
+  // The embedded operand may be either one.  The time of the two choices, in
+  // units of 1 / 152 of a tile's 114 cycles per real K: the tiles, and the
+  // planes of both operands (22 bytes read and written per real at 6.5 TB/s).
+  auto cost = [](long lanes, long cols) {
+    return (double)((lanes + TL - 1) / TL) * ((cols + TN - 1) / TN) + 0.009 * (lanes + cols);
+  };
+  if (cost(N, 2L * M) <= cost(2L * N, M)) {
     // embedded A as the columns, lanes along N: out[m][n] one double2 per lane
     a.emb = true;
     return product<2>(b, a, K, batch, (double*)C, ldc, sC, true, 1.0, false, w, s);
@@ -720,6 +729,14 @@ cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int
   // embedded B as the lanes (real columns of the interleaved C), plain A rows as the columns
   b.emb = true;
   return product<2>(b, a, K, batch, (double*)C, 2L * ldc, 2 * sC, false, 1.0, false, w, s);
+}
+
+cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
+                        int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s) {
+  if (w.buf && oz_wins(M, N, K, batch) && w.bytes >= oz_work_min(K))
+    return oz_gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, w, s);
+  if (w.launches) ++*w.launches;
+  return gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, s);
 }
 
 cudaError_t oz_gemm_d(bool a_km, bool b_kn, int M, int N, int K, const double* A, long lda, const double* B, long ldb,

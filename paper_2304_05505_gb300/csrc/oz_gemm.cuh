@@ -3,16 +3,6 @@
 
 #include "thc_internal.cuh"
 
-// Scratch of the products: digit planes, row exponents and the error word of
-// the kernels' bounded waits, one device allocation of `bytes` bytes.  A
-// product that does not fit is taken in slabs (of the batch, or of the rows of
-// the larger operand).  Owned by one caller on one stream at a time.
-struct OzWork {
-  unsigned char* buf = nullptr;
-  size_t bytes = 0;
-  int* err() const { return (int*)buf; }
-};
-
 // Deepest real K of a product (its int64 sums stay below 2^62).
 constexpr long OZ_MAX_K = 1L << 19;
 
@@ -29,6 +19,10 @@ void oz_free(OzWork& w);
 
 // Whether the digit form is the faster one for this complex product.
 bool oz_wins(int M, int N, int K, int batch);
+
+// gemm_z's product in the faster of its two forms (w.buf may be null).
+cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
+                        int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s);
 
 // gemm_z's product (operand layouts of GemmA, GemmB) from digits.
 cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,

@@ -10,6 +10,7 @@
 //   S4b KC  = conj(X) Y        gemm   (A = X conjugated)
 //   S5  E_x = -(1/N_k) <Psi, Y> ex_reduce
 #include "thc_internal.cuh"
+#include "oz_gemm.cuh"
 
 #include <stdlib.h>
 #include <string.h>
@@ -137,6 +138,7 @@ void free_all(thc_ctx* c) {
     if (c->ev[i]) cudaEventDestroy(c->ev[i]);
   for (cudaEvent_t e : c->prof) cudaEventDestroy(e);
   c->prof.clear();
+  oz_free(c->oz);
   if (c->tc_err_host) cudaFreeHost(c->tc_err_host);
   c->tc_err_host = nullptr;
   for (cudaEvent_t& e : c->cev)
@@ -348,6 +350,28 @@ thc_status thc_destroy(thc_ctx* c) {
   return THC_OK;
 }
 
+// Scratch of an FP64 context's digit products: its largest product whole, up
+// to 2 GB, less where the device has no room (the products then go in smaller
+// slabs, and without any on the FP64 pipe).
+static void oz_prepare(thc_ctx* c) {
+  if (c->precision != THC_FP64 || c->oz_asked) return;
+  c->oz_asked = true;
+  const int nk = c->nk, N = c->nbas, n = c->nocc, P = c->nisdf;
+  if (!oz_wins(P, P, n, nk) && !oz_wins(P, n, P, nk) && !oz_wins(P, n, N, nk)) return;
+  const size_t want = std::max({oz_work_bytes(P, n, N, nk), oz_work_bytes(P, P, n, nk), oz_work_bytes(P, n, P, nk),
+                                oz_work_bytes(N, n, P, nk)});
+  if (oz_alloc(c->oz, std::min(want, (size_t)2 << 30), oz_work_min(std::min(N, P)), c->stream) != cudaSuccess) {
+    cudaGetLastError();
+    oz_free(c->oz);
+    return;
+  }
+  if (cudaMallocHost(&c->tc_err_host, sizeof(int)) != cudaSuccess) {
+    cudaGetLastError();
+    c->tc_err_host = nullptr;
+    oz_free(c->oz);
+  }
+}
+
 static thc_status finite_check(thc_ctx* c, const double2* p, long n) {
   CKC(c, cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
   CKC(c, check_finite_z(p, n, c->flag, c->stream));
@@ -364,6 +388,7 @@ thc_status thc_set_collocation(thc_ctx* c, const double* X) {
   thc_status st = finite_check(c, x, n);
   if (st != THC_OK) return st;
   drop_graph(c);
+  oz_prepare(c);
   if (c->precision == THC_FP64) {
     CKC(c, cudaMemcpyAsync(c->X64, x, n * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
   } else if (c->precision == THC_MIXED_SIMT) {
@@ -452,28 +477,30 @@ static thc_status build_fp64(thc_ctx* c, const double2* C, double2* KC, double* 
   double2* M = (double2*)c->M;
   double2* Y = (double2*)c->Y;
   cudaStream_t s = c->stream;
+  c->n_launch = 3;   // the convolution and the two kernels of the energy; the products add theirs
+  c->oz.launches = &c->n_launch;
   CKC(c, mark(c, 0, s, true));
-  CKC(c, gemm_z(A_KM, B_KN, P, n, N, c->X64, P, (long)N * P, C, n, (long)N * n, Psi, n,
-                (long)P * n, nk, s));
+  CKC(c, gemm_z_best(A_KM, B_KN, P, n, N, c->X64, P, (long)N * P, C, n, (long)N * n, Psi, n,
+                (long)P * n, nk, c->oz, s));
   CKC(c, mark(c, 1, s, true));
-  CKC(c, gemm_z(A_MK, B_NK_CONJ, P, P, n, Psi, n, (long)P * n, Psi, n, (long)P * n, D, P, PP,
-                nk, s));
+  CKC(c, gemm_z_best(A_MK, B_NK_CONJ, P, P, n, Psi, n, (long)P * n, Psi, n, (long)P * n, D, P, PP,
+                nk, c->oz, s));
   CKC(c, mark(c, 2, s, true));
   CKC(c, kconv_z(D, c->Vh64, M, PP, c->n1, c->n2, c->n3, s));
   CKC(c, mark(c, 3, s, true));
   if (Kao) {
-    CKC(c, gemm_z(A_MK_CONJ, B_KN, N, P, P, c->X64, P, (long)N * P, M, P, PP, c->Wao, P, (long)N * P, nk, s));
+    CKC(c, gemm_z_best(A_MK_CONJ, B_KN, N, P, P, c->X64, P, (long)N * P, M, P, PP, c->Wao, P, (long)N * P, nk, c->oz, s));
     CKC(c, mark(c, 4, s, true));
-    CKC(c, gemm_z(A_MK, B_NK, N, N, P, c->Wao, P, (long)N * P, c->X64, P, (long)N * P, Kao, N, (long)N * N, nk, s));
+    CKC(c, gemm_z_best(A_MK, B_NK, N, N, P, c->Wao, P, (long)N * P, c->X64, P, (long)N * P, Kao, N, (long)N * N, nk, c->oz, s));
     CKC(c, mark(c, 5, s, true));
     CKC(c, ex_reduce_z(D, M, (long)nk * PP, nk, c->partial, c->n_partial, ex, s));
     CKC(c, mark(c, 6, s, true));
     return THC_OK;
   }
-  CKC(c, gemm_z(A_MK, B_KN, P, n, P, M, P, PP, Psi, n, (long)P * n, Y, n, (long)P * n, nk, s));
+  CKC(c, gemm_z_best(A_MK, B_KN, P, n, P, M, P, PP, Psi, n, (long)P * n, Y, n, (long)P * n, nk, c->oz, s));
   CKC(c, mark(c, 4, s, true));
-  CKC(c, gemm_z(A_MK_CONJ, B_KN, N, n, P, c->X64, P, (long)N * P, Y, n, (long)P * n, KC, n,
-                (long)N * n, nk, s));
+  CKC(c, gemm_z_best(A_MK_CONJ, B_KN, N, n, P, c->X64, P, (long)N * P, Y, n, (long)P * n, KC, n,
+                (long)N * n, nk, c->oz, s));
   CKC(c, mark(c, 5, s, true));
   CKC(c, ex_reduce_z(Psi, Y, (long)nk * P * n, nk, c->partial, c->n_partial, ex, s));
   CKC(c, mark(c, 6, s, true));
@@ -871,12 +898,13 @@ thc_status thc_debug_fail_alloc(int nth) {
 thc_status thc_sync(thc_ctx* c) {
   if (!c) return THC_ERR_ARG;
   // the error word comes back with the stream's last work: one wait
-  if (c->tc_err) CKC(c, cudaMemcpyAsync(c->tc_err_host, c->tc_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  int* err = c->tc_err ? c->tc_err : c->oz.buf ? c->oz.err() : nullptr;
+  if (err) CKC(c, cudaMemcpyAsync(c->tc_err_host, err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CKC(c, cudaStreamSynchronize(c->stream));
-  if (!c->tc_err) return THC_OK;
+  if (!err) return THC_OK;
   const int h = *c->tc_err_host;
   if (h) {
-    CKC(c, cudaMemset(c->tc_err, 0, sizeof(int)));
+    CKC(c, cudaMemset(err, 0, sizeof(int)));
     c->last_error = "device wait timed out, code " + std::to_string(h);
     return THC_ERR_TIMEOUT;
   }
@@ -981,7 +1009,9 @@ thc_status thc_hermitian_kernel(const thc_ctx* c, int* hermitian) {
 
 thc_status thc_launches_per_build(const thc_ctx* c, int* launches) {
   if (!c || !launches) return THC_ERR_ARG;
-  // FP64 and CUDA-core forms: S1, S2, S3, S4a, S4b, E_x partial, E_x final.
+  // FP64 and CUDA-core forms: S1, S2, S3, S4a, S4b, E_x partial, E_x final
+  // (FP64 after a build: that build's count; a product from digits is five
+  // kernels, per slab).
   // Tensor-core form: S1 3 (exponents, embed, GEMM), S2 2 (slices with their
   // row exponents and the embedded Psi^H, GEMM), S3 + S4a 5 (the convolution, the row
   // exponents of M: in the convolution plus a conversion kernel on the
@@ -995,7 +1025,7 @@ thc_status thc_launches_per_build(const thc_ctx* c, int* launches) {
     const int s4b = tc_partial_elems(c->nbas, 2 * c->nocc, 2 * c->nisdf, c->nk) > 0 ? 1 : 0;
     *launches = 3 + s1 + 2 + 1 + 4 + s4a + 3 + s4b + (s4a && c->nocc % 2 == 0 ? 1 : 2);
   } else {
-    *launches = 7;
+    *launches = c->precision == THC_FP64 && c->n_launch ? c->n_launch : 7;
   }
   return THC_OK;
 }

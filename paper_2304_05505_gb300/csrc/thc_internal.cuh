@@ -9,6 +9,18 @@
 #include "../../include/thc.h"
 #include "tc_gemm.cuh"
 
+// Scratch of the digit products (oz_gemm.cuh): digit planes, row exponents and
+// the error word of the kernels' bounded waits, one device allocation of
+// `bytes` bytes.  A product that does not fit is taken in slabs (of the batch,
+// or of the rows of the larger operand).  Owned by one caller on one stream at
+// a time.
+struct OzWork {
+  unsigned char* buf = nullptr;
+  size_t bytes = 0;
+  int* launches = nullptr;   // counts the kernels launched, when set
+  int* err() const { return (int*)buf; }
+};
+
 // ---------------------------------------------------------------------------
 // complex helpers (interleaved re, im)
 // ---------------------------------------------------------------------------
@@ -46,6 +58,11 @@ struct thc_ctx {
   int device;
   cudaStream_t stream;
   bool have_x, have_v, built;
+  // THC_FP64: scratch of the digit products of S1, S2, S4a and S4b, taken when
+  // the inputs are first set; without it they run on the FP64 pipe
+  OzWork oz;
+  bool oz_asked;
+  int n_launch;     // kernels of the last FP64 build (0: none yet)
   // the tensor-core build replayed as a CUDA graph while not profiled: its
   // executable graph and the caller buffers it was captured with
   cudaGraphExec_t gexec;
@@ -189,6 +206,10 @@ cudaError_t kconv_c_rowexp(const float2* D, const float2* Vh, float2* M, int np,
                            cudaStream_t s);
 // out = M plus its fp16 remainders (kconv_c_herm's Mlo), complex128.
 cudaError_t mlo_combine_c2z(const float2* M, const uint32_t* Mlo, double2* out, long n, cudaStream_t s);
+// The FP64 convolution with fixed-point DFTs (meshes with axes of 1 to 4 points).
+bool kconv_fix_applies(int n1, int n2, int n3);
+cudaError_t kconv_fix_z(const double2* D, const double2* Vh, double2* M, long npq, int n1, int n2, int n3,
+                        cudaStream_t s);
 // Vh[a] = (1/N_k) sum_q V[q] w^{+a.q} in FP64; writes FP64 or FP32 output.
 cudaError_t prepare_kernel_z(const double2* V, double2* Vh64, float2* Vh32, long npq, int n1,
                              int n2, int n3, cudaStream_t s);

@@ -58,3 +58,55 @@ def test_fit_of_nonfinite_orbitals_is_rejected(thc):
     U[3, 5] = complex("nan")
     with pytest.raises(thc.ThcError):
         thc.thc_fit_kernel(U, (13, 14, 15), np.diag([5.0, 5.0, 5.0]), (1, 1, 1), np.arange(40))
+
+
+@pytest.mark.parametrize("mesh,nbas,nocc,nisdf", [
+    ((4, 4, 4), 33, 20, 79),     # radix-4 lanes; N_P one short of a tile's columns
+    ((3, 3, 3), 40, 33, 129),    # radix-3 lanes
+    ((2, 4, 3), 65, 16, 81),     # mixed axes
+    ((1, 3, 2), 96, 64, 256),    # one lane an element, whole tiles
+    ((4, 1, 1), 130, 41, 333),
+])
+def test_fp64_build_from_digits(thc, mesh, nbas, nocc, nisdf):
+    """The FP64 build whose products and k-convolution run from digits and in
+    fixed point, against the FP64 oracle: each step rounds once at 2^-53 of
+    its result (the sums are exact to 2^-60), so the bound is 1e-13 of the
+    largest entry, of E_x and of the Hermitian deviation."""
+    from oracle import thc_oracle as O
+    from paper_2304_05505_gb300 import cells
+    r = cells.random_problem(mesh, nbas=nbas, nocc=nocc, nisdf=nisdf, seed=nisdf)
+    ref = O.build(r["X"], r["C"], r["V"], r["mesh"], route="direct", keep=True)
+    eb = thc.ExchangeBuild(dict(n1=mesh[0], n2=mesh[1], n3=mesh[2], nbas=nbas, nocc=nocc, nisdf=nisdf), "fp64")
+    eb.set_collocation(r["X"])
+    eb.set_kernel(r["V"])
+    KC, ex = eb.build(r["C"])
+    eb.sync()
+    assert np.abs(KC.cpu().numpy() - ref["KC"]).max() <= 1e-13 * np.abs(ref["KC"]).max()
+    assert abs(float(ex[0]) - ref["Ex"]) <= 1e-13 * abs(ref["Ex"])
+    K, ex2 = eb.build_K(r["C"])
+    eb.sync()
+    Kr = np.einsum("kmp,kpq,knq->kmn", r["X"].conj(), ref["M"], r["X"])
+    assert np.abs(K.cpu().numpy() - Kr).max() <= 1e-13 * np.abs(Kr).max()
+    eb.close()
+
+
+@pytest.mark.parametrize("mesh", [(4, 4, 4), (3, 2, 1)])
+def test_fixed_point_convolution_range(thc, mesh):
+    """The k-convolution of values spread over 40 orders of magnitude between
+    the elements (each has its own scale), and of a NaN, which reaches every
+    k of its own element and no other."""
+    nk, npq = int(np.prod(mesh)), 50
+    rng = np.random.default_rng(3)
+    s = 10.0 ** rng.uniform(-20, 20, size=npq)
+    D = (rng.normal(size=(nk, npq)) + 1j * rng.normal(size=(nk, npq))) * s
+    V = (rng.normal(size=(nk, npq)) + 1j * rng.normal(size=(nk, npq))) / s ** 2
+    d = np.fft.fftn(D.reshape(mesh + (npq,)), axes=(0, 1, 2))
+    v = np.fft.ifftn(V.reshape(mesh + (npq,)), axes=(0, 1, 2)) * nk
+    ref = np.fft.ifftn(d * v, axes=(0, 1, 2)).reshape(nk, npq)
+    D[nk - 1, 7] = complex(0.0, float("nan"))
+    M = torch.empty((nk, npq), dtype=torch.complex128, device="cuda")
+    thc.thc_kconv_noalloc(torch.from_numpy(D).cuda(), torch.from_numpy(V).cuda(), M, mesh, npq)
+    got = M.cpu().numpy()
+    assert np.isnan(got[:, 7]).all()
+    keep = np.arange(npq) != 7
+    assert (np.abs(got - ref)[:, keep] <= 1e-14 * np.abs(ref).max(0)[keep]).all()
