@@ -93,6 +93,27 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, in
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
+// The same wait taken by a converged warp, with one answer for every lane: one
+// test and a vote when the phase is already complete.
+__device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity, int* err, int code) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  if (__all_sync(0xffffffffu, done)) return true;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code));
+}
+
+// One lane of a converged warp (the same one each time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e != 0;
+}
+
 // Bounded wait that ignores the error word: used after a failed wait, so that
 // a copy still in flight lands before the block exits.
 __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {

@@ -177,7 +177,7 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
   if (threadIdx.x == 0) abort_flag = *(volatile int*)err;
   __syncthreads();
   if (abort_flag) return;   // an earlier CTA gave up a wait: skip the work
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; s++) {
       mbar_init(FULL(s), 1);
@@ -199,7 +199,7 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const int nchunk = (g.nst + CHUNK_ST - 1) / CHUNK_ST;
   // unit -> (batch entry, lane tile, column tile), column tiles fastest: CTAs side by side share the lane tile
   auto decode = [&](long u, int& b, int& li, int& ni) {
@@ -209,8 +209,10 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
     b = (int)(r / g.tl);
   };
 
+  // (warps 0 and 1 keep all lanes in their loops and elect one per batch of
+  // copies or MMAs: see tc_gemm.cu)
   if (warp == 0) {
-    if (lane == 0) {
+    {
       uint32_t it = 0;
       bool ok = true;
       for (long u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
@@ -218,10 +220,13 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
         decode(u, b, li, ni);
         for (int st = 0; st < g.nst; st++, it++) {
           const uint32_t sl = it & 1;
-          if (!mbar_wait(EMPTY(sl), ((it >> 1) & 1) ^ 1, err, 2)) { ok = false; break; }
-          mbar_expect_tx(FULL(sl), STAGE);
-          tma_load_3d(sbase + sl * STAGE, &maps.l, FULL(sl), st * TK, li * TL, b * ND);
-          tma_load_3d(sbase + sl * STAGE + ND * LPL, &maps.n, FULL(sl), st * TK, ni * TN, b * ND);
+          if (!mbar_wait_uniform(EMPTY(sl), ((it >> 1) & 1) ^ 1, err, 2)) { ok = false; break; }
+          if (elect_one()) {
+            mbar_expect_tx(FULL(sl), STAGE);
+            tma_load_3d(sbase + sl * STAGE, &maps.l, FULL(sl), st * TK, li * TL, b * ND);
+            tma_load_3d(sbase + sl * STAGE + ND * LPL, &maps.n, FULL(sl), st * TK, ni * TN, b * ND);
+          }
+          __syncwarp();
         }
       }
       // the copies still in flight land before the CTA exits (on the normal path they have)
@@ -229,7 +234,7 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
       for (uint32_t j = it - n; j < it; j++) mbar_drain(FULL(j & 1), (j >> 1) & 1);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       const uint64_t d0 = desc64(sbase);
       constexpr uint64_t PL = LPL >> 4, PC = CPL >> 4;
       uint32_t it = 0, ch = 0;
@@ -240,32 +245,36 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
           for (int st = c * CHUNK_ST; st < st1; st++, it++) {
             const uint32_t sl = it & 1;
             const bool first = st == c * CHUNK_ST, last = st == st1 - 1;
-            if (!mbar_wait(FULL(sl), (it >> 1) & 1, err, 8)) { ok = false; break; }
+            if (!mbar_wait_uniform(FULL(sl), (it >> 1) & 1, err, 8)) { ok = false; break; }
             tc_fence_after();
             const uint64_t al = d0 + ((sl * STAGE) >> 4), bn = al + ((ND * LPL) >> 4);
 #pragma unroll
             for (int c6 = 0; c6 < NACC; c6++) {
               if (first) {
-                if (!mbar_wait(AEMPTY(c6), (ch & 1) ^ 1, err, 4)) { ok = false; break; }
+                if (!mbar_wait_uniform(AEMPTY(c6), (ch & 1) ^ 1, err, 4)) { ok = false; break; }
                 tc_fence_after();
               }
+              if (elect_one()) {
 #pragma unroll
-              for (int cl = c6 == 5 ? 7 : c6; cl >= c6; cl--)      // C_7, C_6, C_5
+                for (int cl = c6 == 5 ? 7 : c6; cl >= c6; cl--)      // C_7, C_6, C_5
 #pragma unroll
-                for (int s = cl == 7; s <= min(cl, ND - 1); s++)
+                  for (int s = cl == 7; s <= min(cl, ND - 1); s++)
 #pragma unroll
-                  for (int kk = 0; kk < 2; kk++)
-                    mma_bf16(tmem + c6 * TN, al + s * PL + 2 * kk, bn + (cl - s) * PC + 2 * kk,
-                             !(first && (cl < 5 || cl == 7) && s == (cl == 7) && kk == 0));
-              if (last) commit(AFULL(c6));
+                    for (int kk = 0; kk < 2; kk++)
+                      mma_bf16(tmem + c6 * TN, al + s * PL + 2 * kk, bn + (cl - s) * PC + 2 * kk,
+                               !(first && (cl < 5 || cl == 7) && s == (cl == 7) && kk == 0));
+                if (last) commit(AFULL(c6));
+                if (c6 == NACC - 1) commit(EMPTY(sl));
+              }
+              __syncwarp();
             }
             if (!ok) break;
-            commit(EMPTY(sl));
           }
         }
       }
       // every MMA issued complete before TMEM is released
-      commit(DONE);
+      if (elect_one()) commit(DONE);
+      __syncwarp();
       mbar_drain(DONE, 0);
     }
   } else if (warp >= EPI0) {

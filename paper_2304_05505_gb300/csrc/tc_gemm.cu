@@ -48,13 +48,21 @@
 //   warp 0      TMA producer: A planes (or the FP32 A tile) and B planes per
 //               32-wide real-K block into a ring in shared memory, 64B
 //               swizzle, running ahead across units
-//   warp 1      allocates 512 TMEM columns = two accumulator sets (leading
-//               class, the other classes; 128 columns each) so that the
-//               epilogue of one unit overlaps the MMAs of the next; lane 0
-//               issues tcgen05.mma (M = 128, N = 128, K = 16, f16 x f16 -> f32),
-//               6 or 8 per K step
-//   CV:  warps 2-9 converters, warps 10-17 epilogue (8 warps, 64 columns each)
-//   else warps 2-3 idle, warps 4-19 epilogue (16 warps, 32 columns each)
+//   warp 1      allocates 512 TMEM columns and issues tcgen05.mma (M = 128,
+//               N = 128, K = 16, f16 x f16 -> f32), 6 or 8 per K step.
+//               Plane-fed forms: two accumulator sets (leading class, the
+//               other classes; 128 columns each), so that the epilogue of one
+//               unit overlaps the MMAs of the next.  Converted forms: one set,
+//               whose two accumulators are handed over one by one, and four
+//               stages of converted A planes (48 columns each)
+//   CV:  warps 2-9 converters (FP32 tile -> slices -> TMEM), warps 10-25 epilogue
+//   else warps 2-3 idle, warps 4-19 epilogue (32 columns each)
+// What binds: reading operands from shared memory (128 B per cycle: an MMA
+// with both operands there takes its full 64 cycles for them), which is why
+// the converted forms keep A in TMEM, and the issue of the MMAs (see warps 0
+// and 1 below).  At 4 x 4 x 4 k, N_P = 1200, N = 432, n = 60 the two together
+// took S4a's kernel from 0.354 to 0.268 ms, S4b's from 0.154 to 0.119 and
+// S1's from 0.138 to 0.096 (A in TMEM by itself: no gain).
 // The epilogue warps (4 per TMEM lane quadrant) read both accumulators with
 // tcgen05.ld, scale by exact powers of two and store (or write the partial
 // sums), then release the accumulator set.  Each warp turns its 32-row x
@@ -85,21 +93,18 @@ constexpr int MAX_CHUNK_KB = 32;                             // K blocks per exa
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t STAGE_BYTES = 2 * NPL * TILE_BYTES;       // A and B planes of one K block: 48 KB
 constexpr uint32_t EPI_TILE = 32 * 16;                       // floats per epilogue warp (32 rows x 16)
-// Shared memory: the operand rings, 256 B of barriers, then the epilogue
-// warps' staging tiles.  Plane-fed forms: a 192 KB ring and 16 epilogue
-// warps; converted forms: 208 KB of rings (see the kernel) and 8 epilogue
-// warps.  Both come to the same total.
+// Shared memory: the operand rings (192 KB), 512 B of barriers, then the 16
+// epilogue warps' staging tiles.
 template <int CV> struct Smem {
-  static constexpr uint32_t RING = CV ? 208 * 1024 : 192 * 1024;
-  static constexpr size_t BYTES = RING + 1024 + 256 + (CV ? 8 : 16) * EPI_TILE * 4;
+  static constexpr uint32_t RING = 192 * 1024;
+  static constexpr size_t BYTES = RING + 1024 + 512 + 16 * EPI_TILE * 4;
 };
-static_assert(Smem<1>::BYTES <= 232448 && Smem<0>::BYTES <= 232448, "227 KB of shared memory per block");
+static_assert(Smem<0>::BYTES <= 232448, "227 KB of shared memory per block");
 
-// Warp roles: 0 TMA, 1 MMA, then (CV) 8 converter warps, then the epilogue.
-// The converted-A forms take 8 epilogue warps, the others 16.
+// Warp roles: 0 TMA, 1 MMA, then (CV) 8 converter warps, then 16 epilogue warps.
 template <int CV> struct Roles {
   static constexpr int CONV_WARPS = CV ? 8 : 0;                 // warps 2 .. 2 + CONV_WARPS - 1
-  static constexpr int EPI = CV ? 8 : 16;                       // epilogue warps
+  static constexpr int EPI = 16;                                // epilogue warps
   static constexpr int EPI0 = CV ? 2 + CONV_WARPS : 4;          // first epilogue warp
   static constexpr int NT = (EPI0 + EPI) * 32;                  // threads
   static constexpr int COLS = 4 * BN / EPI;                     // columns of a unit per epilogue warp
@@ -129,6 +134,23 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b,
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+
+// The same with A in tensor memory (16 K: 8 columns of two fp16 each, row = lane).
+__device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc,
+                                           uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// Eight 32-bit columns of this thread's TMEM lane from w.
+__device__ __forceinline__ void tmem_st8(uint32_t t, const uint32_t* w) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(t), "r"(w[0]),
+               "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
@@ -165,6 +187,24 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, float* va,
     vb[i] = __uint_as_float(r[16 + i]);
   }
 }
+
+// 16 consecutive fp32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld16(uint32_t t, float* v) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+      "%13, %14, %15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(t)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
+}
+
+// 32 consecutive fp32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld32(uint32_t t, float* v) { tmem_ld16x2(t, t + 16, v, v + 16); }
 
 // Float offset of 16-byte chunk c (0..3) of row r in a 32 x 16 staging tile;
 // the chunk index is XORed with bits 1-2 of the row so that 8 lanes writing
@@ -243,6 +283,28 @@ __device__ __forceinline__ void slice8_f16x(const float* x, const float* lo, flo
   }
 }
 
+// A warp's 32-row x 16-column staging tile into a partial-sum buffer: lane ->
+// (row, 4 columns), 8 rows x 64 B per instruction.
+__device__ __forceinline__ void put_block(float* __restrict__ part, const float* stg, const Geometry& g, int b, int kc,
+                                          int row0, int col0) {
+  const int lane = threadIdx.x & 31, f = lane >> 3, col = col0 + 4 * f;
+#pragma unroll
+  for (int it = 0; it < 4; it++) {
+    const int rr = (lane & 7) + 8 * it, row = row0 + rr;
+    if (row >= g.M || col >= g.Nr) continue;
+    const float4 v = *reinterpret_cast<const float4*>(stg + stage_off(rr, f));
+    float* o = part + (((long)kc * g.batch + b) * g.M + row) * g.Nr + col;
+    if (g.Nr % 4 == 0) {
+      *reinterpret_cast<float4*>(o) = v;
+    } else {
+      const float w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+        if (col + i < g.Nr) o[i] = w4[i];
+    }
+  }
+}
+
 // OUT: 0 = FP32 result, 1 = FP64 result, 2 = partial sums (split K)
 // NP: 6 or 8 slice products per real product (see the header).
 // AR (A resident, short K in one chunk): the A tile of all K (4 blocks x 3
@@ -251,11 +313,10 @@ __device__ __forceinline__ void slice8_f16x(const float* x, const float* lo, flo
 // 24 KB.  Each CTA takes a contiguous range of units so that consecutive units
 // share their A tile.
 // CV (A converted in shared memory, 1, 2 or 3): A is an FP32 (interleaved
-// complex) matrix; CV = 3 adds its fp16 remainders (map a[1], 64B swizzle).  TMA brings 16 KB FP32 tiles into a 3-stage staging ring;
+// complex) matrix; CV = 3 adds its fp16 remainders (map a[1], 64B swizzle).  TMA brings 16 KB FP32 tiles into a staging ring;
 // converter warps cut each tile into the three fp16 slices with the rows'
-// exponents and write them in the 64B-swizzled K-major layout the MMA reads,
-// then fence the generic-proxy writes for the async proxy and arrive on the
-// stage's full barrier beside the TMA bytes of the B planes.
+// exponents and store them in TMEM (row = lane, two K values a column), where
+// the MMA reads A from.
 template <int OUT, int NP, bool AR, int CV>
 __global__ void __launch_bounds__(Roles<CV>::NT, 1)
 tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restrict__ eA, long seA,
@@ -270,19 +331,20 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
   constexpr int EPI_W = Roles<CV>::EPI, EPI_W0 = Roles<CV>::EPI0, EPI_COLS = Roles<CV>::COLS;
   constexpr uint32_t RING_BYTES = Smem<CV>::RING;
   // Converted forms: three decoupled rings so that the DRAM stream of A runs
-  // well ahead of the MMAs: FP32 A tiles (SA_STAGES x 16 KB, from DRAM), B
-  // planes (B_STAGES x 24 KB, TMA only) and the converted A planes (STAGES x
-  // 24 KB, written by the converter warps).
+  // well ahead of the MMAs: FP32 A tiles (SA_STAGES x 16 KB, from DRAM) and B
+  // planes (B_STAGES x 24 KB) in shared memory, the converted A planes in TMEM.
   // CV = 3: each FP32 stage also holds the fp16 tile of the remainders (8 KB)
-  constexpr int SA_STAGES = CV == 3 ? 3 : 4, B_STAGES = CV == 3 ? 3 : 4;
+  constexpr int SA_STAGES = CV == 3 ? 4 : 6, B_STAGES = 4;
   constexpr uint32_t SA_HI = BM * BKR * 4;                         // 16 KB: FP32 tile
   constexpr uint32_t SA_BYTES = CV == 3 ? SA_HI + BM * BKR * 2 : SA_HI;
   constexpr uint32_t PL_BYTES = NPL * TILE_BYTES;                  // 24 KB: three planes of one operand
-  constexpr uint32_t B_OFF = SA_STAGES * SA_BYTES + 2 * PL_BYTES;  // CV: the B ring after the A plane ring
+  constexpr uint32_t B_OFF = SA_STAGES * SA_BYTES;                 // CV: the B ring
+  constexpr uint32_t TA_COL = 256, TA_STAGE = NPL * BKR / 2;       // CV: converted A stages in TMEM (48 columns each)
   // what precedes the plane ring: the resident A tile, or the FP32 staging ring
   constexpr uint32_t A_BYTES = AR ? AKB * NPL * TILE_BYTES : CV ? SA_STAGES * SA_BYTES : 0;
   constexpr uint32_t SBYTES = (AR || CV) ? PL_BYTES : STAGE_BYTES;  // bytes of one plane-ring stage
-  constexpr int STAGES = CV ? 2 : (RING_BYTES - A_BYTES) / SBYTES;
+  constexpr int STAGES = CV ? 4 : (RING_BYTES - A_BYTES) / SBYTES;
+  static_assert(!CV || TA_COL + STAGES * TA_STAGE <= TMEM_COLS, "TMEM columns");
   static_assert(STAGES >= 2 && STAGES <= 4, "ring stages");
   static_assert(!CV || B_OFF + B_STAGES * PL_BYTES <= RING_BYTES, "ring size");
   uint64_t* bars = (uint64_t*)(smem + RING_BYTES);
@@ -290,8 +352,8 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
   // loaded / released, FP32 tile landed / converted [SA_STAGES each], B planes
   // landed / consumed [B_STAGES each], MMAs drained.  CV: full / empty are the
   // converted A planes.
-  uint32_t* tmem_slot = (uint32_t*)(bars + 31);
-  float* epi_stage = (float*)(smem + RING_BYTES + 256);   // EPI_W tiles of EPI_TILE floats
+  uint32_t* tmem_slot = (uint32_t*)(bars + 63);
+  float* epi_stage = (float*)(smem + RING_BYTES + 512);   // EPI_W tiles of EPI_TILE floats
   const uint32_t sbase = smem_u32(smem);
   const uint32_t bar0 = smem_u32(bars);
   auto FULL = [&](int s) { return bar0 + 8u * s; };
@@ -304,15 +366,15 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
   auto SEMPTY = [&](int s) { return bar0 + 8u * (14 + SA_STAGES + s); };               // CV: FP32 tile converted
   auto BFULL = [&](int s) { return bar0 + 8u * (14 + 2 * SA_STAGES + s); };            // CV: B planes landed
   auto BEMPTY = [&](int s) { return bar0 + 8u * (14 + 2 * SA_STAGES + B_STAGES + s); };  // CV: B planes consumed
-  const uint32_t MMA_DONE = bar0 + 8u * 30;    // every MMA of the CTA complete
-  static_assert(2 * SA_STAGES + 2 * B_STAGES <= 16, "barrier slots 14 .. 29");
+  const uint32_t MMA_DONE = bar0 + 8u * 62;    // every MMA of the CTA complete
+  static_assert(2 * SA_STAGES + 2 * B_STAGES <= 48, "barrier slots 14 .. 61");
 
   __shared__ int abort_flag;
   if (threadIdx.x == 0) abort_flag = *(volatile int*)err;
   __syncthreads();
   if (abort_flag) return;   // an earlier CTA gave up a wait: skip the work
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; s++) {
@@ -350,7 +412,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   // units of this CTA: strided (CTAs running side by side share the A tile
   // through L2) or, A resident, one contiguous range
@@ -381,12 +443,18 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
     b = (int)(r / g.mt);
   };
 
+  // Warps 0 and 1 run their loops with all lanes (the loop state is uniform)
+  // and elect one lane for each batch of instructions.  In a branch of one
+  // lane the operands of a tcgen05.mma or a TMA copy are moved to the uniform
+  // registers one by one by a loop over the lanes: 50 cycles an MMA with the
+  // SM to itself and 150 to 400 beside the converters, against 18 and 33 to 87.
   if (warp == 0) {
-    if (lane == 0) {
-      for (int s = 0; s < NPL; s++) {
-        asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&maps.a[s]) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&maps.b[s]) : "memory");
-      }
+    {
+      if (elect_one())
+        for (int s = 0; s < NPL; s++) {
+          asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&maps.a[s]) : "memory");
+          asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&maps.b[s]) : "memory");
+        }
       uint32_t it = 0, agen = 0, nfull = 0, nsa = 0;   // K blocks; B (or A and B) and FP32 A copies issued
       long gprev = -1;
       bool ok = true;
@@ -398,11 +466,14 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
           const long grp = (long)b * g.mt + mi;
           if (grp != gprev) {
             // reload the resident A tile once the MMAs on the previous one are done
-            if (agen > 0 && !mbar_wait(AOP_EMPTY, (agen - 1) & 1, err, 32)) { ok = false; break; }
-            mbar_expect_tx(AOP_FULL, g.nkb * NPL * TILE_BYTES);
-            for (int kb = 0; kb < g.nkb; kb++)
-              for (int p = 0; p < NPL; p++)
-                tma_load_3d(sbase + (kb * NPL + p) * TILE_BYTES, &maps.a[p], AOP_FULL, kb * BKR, mi * BM, bz);
+            if (agen > 0 && !mbar_wait_uniform(AOP_EMPTY, (agen - 1) & 1, err, 32)) { ok = false; break; }
+            if (elect_one()) {
+              mbar_expect_tx(AOP_FULL, g.nkb * NPL * TILE_BYTES);
+              for (int kb = 0; kb < g.nkb; kb++)
+                for (int p = 0; p < NPL; p++)
+                  tma_load_3d(sbase + (kb * NPL + p) * TILE_BYTES, &maps.a[p], AOP_FULL, kb * BKR, mi * BM, bz);
+            }
+            __syncwarp();
             gprev = grp;
             agen++;
           }
@@ -414,36 +485,45 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
           if constexpr (CV != 0) {
             // the FP32 A tile into the staging ring, the B planes into the plane ring
             const int sa = it % SA_STAGES;
-            if (!mbar_wait(SEMPTY(sa), ((it / SA_STAGES) & 1) ^ 1, err, 2)) { ok = false; break; }
-            mbar_expect_tx(SFULL(sa), SA_BYTES);
-            if constexpr (CV == 1 || CV == 3)
-              tma_load_3d(sbase + sa * SA_BYTES, &maps.a[0], SFULL(sa), kb * BKR, mi * BM, bz);
-            else   // [K][rows] source: 16 complex K values (rows of the box) x 128 complex rows
-              tma_load_3d(sbase + sa * SA_BYTES, &maps.a[0], SFULL(sa), mi * 2 * BM, kb * (BKR / 2), bz);
-            if constexpr (CV == 3)   // the remainders' fp16 tile beside it
-              tma_load_3d(sbase + sa * SA_BYTES + SA_HI, &maps.a[1], SFULL(sa), kb * BKR, mi * BM, bz);
+            if (!mbar_wait_uniform(SEMPTY(sa), ((it / SA_STAGES) & 1) ^ 1, err, 2)) { ok = false; break; }
+            if (elect_one()) {
+              mbar_expect_tx(SFULL(sa), SA_BYTES);
+              if constexpr (CV == 1 || CV == 3)
+                tma_load_3d(sbase + sa * SA_BYTES, &maps.a[0], SFULL(sa), kb * BKR, mi * BM, bz);
+              else   // [K][rows] source: 16 complex K values (rows of the box) x 128 complex rows
+                tma_load_3d(sbase + sa * SA_BYTES, &maps.a[0], SFULL(sa), mi * 2 * BM, kb * (BKR / 2), bz);
+              if constexpr (CV == 3)   // the remainders' fp16 tile beside it
+                tma_load_3d(sbase + sa * SA_BYTES + SA_HI, &maps.a[1], SFULL(sa), kb * BKR, mi * BM, bz);
+            }
+            __syncwarp();
             nsa++;
             const int sb = it % B_STAGES;
-            if (!mbar_wait(BEMPTY(sb), ((it / B_STAGES) & 1) ^ 1, err, 2)) { ok = false; break; }
-            mbar_expect_tx(BFULL(sb), PL_BYTES);
-            for (int p = 0; p < NPL; p++)
-              tma_load_3d(sbase + B_OFF + sb * PL_BYTES + p * TILE_BYTES, &maps.b[p], BFULL(sb), kb * BKR,
-                          ni * BN, bz);
+            if (!mbar_wait_uniform(BEMPTY(sb), ((it / B_STAGES) & 1) ^ 1, err, 2)) { ok = false; break; }
+            if (elect_one()) {
+              mbar_expect_tx(BFULL(sb), PL_BYTES);
+              for (int p = 0; p < NPL; p++)
+                tma_load_3d(sbase + B_OFF + sb * PL_BYTES + p * TILE_BYTES, &maps.b[p], BFULL(sb), kb * BKR,
+                            ni * BN, bz);
+            }
+            __syncwarp();
             nfull++;
             continue;
           }
-          if (!mbar_wait(EMPTY(st), ph ^ 1, err, 2)) { ok = false; break; }
-          mbar_expect_tx(FULL(st), SBYTES);
-          const uint32_t dst = sbase + A_BYTES + st * SBYTES;
-          if constexpr (AR) {
-            for (int p = 0; p < NPL; p++)
-              tma_load_3d(dst + p * TILE_BYTES, &maps.b[p], FULL(st), kb * BKR, ni * BN, bz);
-          } else {
-            for (int p = 0; p < NPL; p++)
-              tma_load_3d(dst + p * TILE_BYTES, &maps.a[p], FULL(st), kb * BKR, mi * BM, bz);
-            for (int p = 0; p < NPL; p++)
-              tma_load_3d(dst + (NPL + p) * TILE_BYTES, &maps.b[p], FULL(st), kb * BKR, ni * BN, bz);
+          if (!mbar_wait_uniform(EMPTY(st), ph ^ 1, err, 2)) { ok = false; break; }
+          if (elect_one()) {
+            mbar_expect_tx(FULL(st), SBYTES);
+            const uint32_t dst = sbase + A_BYTES + st * SBYTES;
+            if constexpr (AR) {
+              for (int p = 0; p < NPL; p++)
+                tma_load_3d(dst + p * TILE_BYTES, &maps.b[p], FULL(st), kb * BKR, ni * BN, bz);
+            } else {
+              for (int p = 0; p < NPL; p++)
+                tma_load_3d(dst + p * TILE_BYTES, &maps.a[p], FULL(st), kb * BKR, mi * BM, bz);
+              for (int p = 0; p < NPL; p++)
+                tma_load_3d(dst + (NPL + p) * TILE_BYTES, &maps.b[p], FULL(st), kb * BKR, ni * BN, bz);
+            }
           }
+          __syncwarp();
           nfull++;
         }
       }
@@ -467,7 +547,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_f16(BM, BN);
       const uint64_t dbase = smem_desc(sbase);
       uint32_t it = 0, local = 0, agen = 0;
@@ -479,15 +559,18 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
         if constexpr (AR) {
           const long grp = (long)b * g.mt + mi;
           if (grp != gprev) {
-            if (agen > 0) mma_commit(AOP_EMPTY);      // arrives when the MMAs issued so far are done
-            if (!mbar_wait(AOP_FULL, agen & 1, err, 64)) break;
+            // arrives when the MMAs issued so far are done
+            if (agen > 0 && elect_one()) mma_commit(AOP_EMPTY);
+            __syncwarp();
+            if (!mbar_wait_uniform(AOP_FULL, agen & 1, err, 64)) break;
             fence_after();
             gprev = grp;
             agen++;
           }
         }
-        const int set = local & 1;
-        if (!mbar_wait(AEMPTY(set), ((local >> 1) & 1) ^ 1, err, 4)) break;
+        // CV: one accumulator set; its two halves are handed over one by one
+        const int set = CV ? 0 : local & 1;
+        if (!mbar_wait_uniform(AEMPTY(set), (CV ? local & 1 : (local >> 1) & 1) ^ 1, err, 4)) break;
         fence_after();
         const uint32_t accA = tmem + 256 * set, accBC = accA + 128;
         const int kb0 = kc * g.ckb, kb1 = min(g.nkb, (kc + 1) * g.ckb);
@@ -495,8 +578,8 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
           const int st = it % STAGES;
           const uint32_t ph = (it / STAGES) & 1;
           const int sb = it % B_STAGES;
-          if (!mbar_wait(FULL(st), ph, err, 8)) { ok = false; break; }
-          if (CV && !mbar_wait(BFULL(sb), (it / B_STAGES) & 1, err, 8)) { ok = false; break; }
+          if (!mbar_wait_uniform(FULL(st), ph, err, 8)) { ok = false; break; }
+          if (CV && !mbar_wait_uniform(BFULL(sb), (it / B_STAGES) & 1, err, 8)) { ok = false; break; }
           fence_after();
           // descriptors: one base per stage, planes and K steps are offsets of
           // (bytes >> 4) in the start-address field (no carry: smem < 256 KB)
@@ -506,39 +589,86 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
                                  : CV ? dbase + ((B_OFF + sb * PL_BYTES) >> 4)
                                       : aBase + ((NPL * TILE_BYTES) >> 4);
           constexpr uint64_t PL = TILE_BYTES >> 4;
+          if constexpr (CV != 0) {
+            // A from TMEM.  Each accumulator sees its products in the order of
+            // the other forms; the leading class goes first for both K steps,
+            // so that at a unit's end its accumulator is drained under the
+            // last products of the other, and at its start the first products
+            // only wait for the leading accumulator.
+            const uint32_t ta = tmem + TA_COL + TA_STAGE * st;
+            if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < BKR / 16; kk++) {
-            const uint64_t a = aBase + 2 * kk, b2 = bBase + 2 * kk;   // 32 B per K step
-            const uint32_t acc = (kb == kb0 && kk == 0) ? 0u : 1u;
-            mma_f16(accA, a, b2, idesc, acc);                           // exact leading class (0,0)
-            // the other classes, smallest first, into the second accumulator
-            if constexpr (NP == 8) {
-              mma_f16(accBC, a + PL, b2 + 2 * PL, idesc, acc);          // (1,2)
-              mma_f16(accBC, a + 2 * PL, b2 + PL, idesc, 1u);           // (2,1)
-              mma_f16(accBC, a, b2 + 2 * PL, idesc, 1u);                // (0,2)
-            } else {
-              mma_f16(accBC, a, b2 + 2 * PL, idesc, acc);               // (0,2)
+              for (int kk = 0; kk < BKR / 16; kk++)
+                mma_f16_ts(accA, ta + 8 * kk, bBase + 2 * kk, idesc, (kb == kb0 && kk == 0) ? 0u : 1u);
+              if (kb == kb1 - 1) mma_commit(AFULL(0));
             }
-            mma_f16(accBC, a + 2 * PL, b2, idesc, 1u);                  // (2,0)
-            mma_f16(accBC, a + PL, b2 + PL, idesc, 1u);                 // (1,1)
-            mma_f16(accBC, a, b2 + PL, idesc, 1u);                      // (0,1)
-            mma_f16(accBC, a + PL, b2, idesc, 1u);                      // (1,0)
+            __syncwarp();
+            if (kb == kb0) {
+              if (!mbar_wait_uniform(AEMPTY(1), (local & 1) ^ 1, err, 4)) { ok = false; break; }
+              fence_after();
+            }
+            if (elect_one()) {
+#pragma unroll
+              for (int kk = 0; kk < BKR / 16; kk++) {
+                const uint32_t a = ta + 8 * kk;
+                const uint64_t b2 = bBase + 2 * kk;
+                const uint32_t acc = (kb == kb0 && kk == 0) ? 0u : 1u;
+                constexpr uint32_t TP = BKR / 2;                            // columns of a plane
+                if constexpr (NP == 8) {
+                  mma_f16_ts(accBC, a + TP, b2 + 2 * PL, idesc, acc);       // (1,2)
+                  mma_f16_ts(accBC, a + 2 * TP, b2 + PL, idesc, 1u);        // (2,1)
+                  mma_f16_ts(accBC, a, b2 + 2 * PL, idesc, 1u);             // (0,2)
+                } else {
+                  mma_f16_ts(accBC, a, b2 + 2 * PL, idesc, acc);            // (0,2)
+                }
+                mma_f16_ts(accBC, a + 2 * TP, b2, idesc, 1u);               // (2,0)
+                mma_f16_ts(accBC, a + TP, b2 + PL, idesc, 1u);              // (1,1)
+                mma_f16_ts(accBC, a, b2 + PL, idesc, 1u);                   // (0,1)
+                mma_f16_ts(accBC, a + TP, b2, idesc, 1u);                   // (1,0)
+              }
+              mma_commit(EMPTY(st));
+              mma_commit(BEMPTY(sb));
+            }
+            __syncwarp();
+            continue;
           }
-          mma_commit(EMPTY(st));
-          if (CV) mma_commit(BEMPTY(sb));
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < BKR / 16; kk++) {
+              const uint64_t a = aBase + 2 * kk, b2 = bBase + 2 * kk;   // 32 B per K step
+              const uint32_t acc = (kb == kb0 && kk == 0) ? 0u : 1u;
+              mma_f16(accA, a, b2, idesc, acc);                           // exact leading class (0,0)
+              // the other classes, smallest first, into the second accumulator
+              if constexpr (NP == 8) {
+                mma_f16(accBC, a + PL, b2 + 2 * PL, idesc, acc);          // (1,2)
+                mma_f16(accBC, a + 2 * PL, b2 + PL, idesc, 1u);           // (2,1)
+                mma_f16(accBC, a, b2 + 2 * PL, idesc, 1u);                // (0,2)
+              } else {
+                mma_f16(accBC, a, b2 + 2 * PL, idesc, acc);               // (0,2)
+              }
+              mma_f16(accBC, a + 2 * PL, b2, idesc, 1u);                  // (2,0)
+              mma_f16(accBC, a + PL, b2 + PL, idesc, 1u);                 // (1,1)
+              mma_f16(accBC, a, b2 + PL, idesc, 1u);                      // (0,1)
+              mma_f16(accBC, a + PL, b2, idesc, 1u);                      // (1,0)
+            }
+            mma_commit(EMPTY(st));
+          }
+          __syncwarp();
         }
         if (!ok) break;
-        mma_commit(AFULL(set));
+        if (elect_one()) mma_commit(AFULL(CV ? 1 : set));
+        __syncwarp();
       }
       // every MMA issued by this thread complete before TMEM is released
-      mma_commit(MMA_DONE);
+      if (elect_one()) mma_commit(MMA_DONE);
+      __syncwarp();
       mbar_drain(MMA_DONE, 0);
     }
   } else if (CV != 0 && warp >= 2 && warp < 2 + CONV_WARPS) {
-    // converter warps: warp w handles rows 32 (w & 3) .. + 31 (one per lane)
-    // and K half w >> 2 (16 reals = two 8-real chunks of each plane)
-    const int w = warp - 2;
-    const int r = 32 * (w & 3) + lane, hf = w >> 2;
+    // converter warps: a warp handles the 32 rows of its TMEM lane quadrant
+    // (one per lane) and one K half (16 reals = 8 columns of each plane)
+    const int r = 32 * (warp & 3) + lane, hf = (warp - 2) >> 2;
+    const uint32_t tdst = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + TA_COL + 8 * hf;
     uint32_t it = 0;
     bool ok = true;
     for (long u = u_begin; u < u_end && ok; u += u_step) {
@@ -551,10 +681,11 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
       const int kb1 = min(g.nkb, (kc + 1) * g.ckb);
       for (int kb = kc * g.ckb; kb < kb1; kb++, it++) {
         const int sa = it % SA_STAGES, st = it % STAGES;
-        if (!mbar_wait(SFULL(sa), (it / SA_STAGES) & 1, err, 128)) { ok = false; break; }
-        if (!mbar_wait(EMPTY(st), ((it / STAGES) & 1) ^ 1, err, 256)) { ok = false; break; }
+        if (!mbar_wait_uniform(SFULL(sa), (it / SA_STAGES) & 1, err, 128)) { ok = false; break; }
+        if (!mbar_wait_uniform(EMPTY(st), ((it / STAGES) & 1) ^ 1, err, 256)) { ok = false; break; }
+        fence_after();   // the MMAs that read this TMEM stage are complete
         const unsigned char* src = smem + sa * SA_BYTES;
-        unsigned char* dstp = smem + A_BYTES + st * SBYTES;
+        uint32_t wp[NPL][8];
 #pragma unroll
         for (int k2 = 0; k2 < 2; k2++) {
           const int pc = 2 * hf + k2;               // 8 reals = one 16-byte chunk of each plane
@@ -592,14 +723,15 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
           } else {
             slice8_f16(x, sc, wd);
           }
-          // plane row r, 64B swizzle: chunk pc at r * 64 + 16 (pc ^ ((r >> 1) & 3))
-          const uint32_t off = r * 64 + 16 * (pc ^ ((r >> 1) & 3));
 #pragma unroll
           for (int p = 0; p < NPL; p++)
-            *reinterpret_cast<uint4*>(dstp + p * TILE_BYTES + off) = make_uint4(wd[p][0], wd[p][1], wd[p][2], wd[p][3]);
+#pragma unroll
+            for (int j = 0; j < 4; j++) wp[p][4 * k2 + j] = wd[p][j];
         }
-        // the planes were written by the generic proxy; the MMA reads them through the async proxy
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+#pragma unroll
+        for (int p = 0; p < NPL; p++) tmem_st8(tdst + TA_STAGE * st + (BKR / 2) * p, wp[p]);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        fence_before();
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(SEMPTY(sa));
@@ -626,14 +758,94 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
         if (row0 + lane < g.M) ea = row_exp(eA, (long)b * seA + row0 + lane);
         if (lane < EPI_COLS / 2 && cbase + 2 * lane < g.Nr) ebl = eB[(long)b * seB + (cbase >> 1) + lane];
       }
-      const int set = local & 1;
-      if (!mbar_wait_warp(AFULL(set), (local >> 1) & 1, err, 16)) break;
-      fence_after();
+      const int set = CV ? 0 : local & 1;
       const uint32_t accA = tmem + lane_off + 256 * set, accBC = accA + 128;
-#pragma unroll 1
+      // CV: both halves of the warp's columns into registers as soon as each
+      // accumulator is complete, so that the next unit's products can start;
+      // with split K the leading sums are written while the others are summed
+      float ca[CV ? 32 : 1];
+      if constexpr (CV != 0) {
+        static_assert(EPI_COLS == 32, "columns of an epilogue warp");
+        if (!__all_sync(0xffffffffu, mbar_wait(AFULL(0), local & 1, err, 16))) break;
+        fence_after();
+        tmem_ld32(accA + EPI_COLS * h, ca);
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(AEMPTY(0));
+        if constexpr (OUT == 2) {
+#pragma unroll
+          for (int qq = 0; qq < 2; qq++) {
+            if (cbase + 16 * qq < g.Nr) {
+              // the exact leading sum as an int32 (ca / 2^16 is an integer below 2^24)
+#pragma unroll
+              for (int j = 0; j < 16; j += 4)
+                *reinterpret_cast<float4*>(stg + stage_off(lane, j >> 2)) =
+                    make_float4(__int_as_float(__float2int_rn(ca[16 * qq + j] * 0x1p-16f)),
+                                __int_as_float(__float2int_rn(ca[16 * qq + j + 1] * 0x1p-16f)),
+                                __int_as_float(__float2int_rn(ca[16 * qq + j + 2] * 0x1p-16f)),
+                                __int_as_float(__float2int_rn(ca[16 * qq + j + 3] * 0x1p-16f)));
+              __syncwarp();
+              put_block(reinterpret_cast<float*>(ps0), stg, g, b, kc, row0, cbase + 16 * qq);
+              __syncwarp();
+            }
+          }
+        }
+        if (!__all_sync(0xffffffffu, mbar_wait(AFULL(1), local & 1, err, 16))) break;
+        fence_after();
+        if constexpr (OUT == 2) {
+          tmem_ld32(accBC + EPI_COLS * h, ca);
+        } else if constexpr (OUT == 0) {   // ca is exact: one rounding in the add
+#pragma unroll
+          for (int qq = 0; qq < 2; qq++) {
+            float vb[16];
+            tmem_ld16(accBC + EPI_COLS * h + 16 * qq, vb);
+#pragma unroll
+            for (int j = 0; j < 16; j++) ca[16 * qq + j] += vb[j];
+          }
+        }
+        if constexpr (OUT != 1) {          // (OUT = 1 reads them as it goes)
+          fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(AEMPTY(1));
+        }
+        if constexpr (OUT == 2) {
+#pragma unroll
+          for (int qq = 0; qq < 2; qq++) {
+            if (cbase + 16 * qq < g.Nr) {
+#pragma unroll
+              for (int j = 0; j < 16; j += 4)
+                *reinterpret_cast<float4*>(stg + stage_off(lane, j >> 2)) =
+                    make_float4(ca[16 * qq + j] * 0x1p-16f, ca[16 * qq + j + 1] * 0x1p-16f,
+                                ca[16 * qq + j + 2] * 0x1p-16f, ca[16 * qq + j + 3] * 0x1p-16f);
+              __syncwarp();
+              put_block(pbc, stg, g, b, kc, row0, cbase + 16 * qq);
+              __syncwarp();
+            }
+          }
+          continue;
+        }
+      } else {
+        if (!mbar_wait_warp(AFULL(set), (local >> 1) & 1, err, 16)) break;
+        fence_after();
+      }
+#pragma unroll
       for (int qq = 0; qq < EPI_COLS / 16; qq++) {
+        __syncwarp();
         float va[16], vb[16];
-        tmem_ld16x2(accA + EPI_COLS * h + 16 * qq, accBC + EPI_COLS * h + 16 * qq, va, vb);
+        if constexpr (CV != 0) {
+#pragma unroll
+          for (int j = 0; j < 16; j++) va[j] = ca[16 * qq + j];
+          if constexpr (OUT == 1) {
+            tmem_ld16(accBC + EPI_COLS * h + 16 * qq, vb);
+            if (qq == 1) {
+              fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(AEMPTY(1));
+            }
+          }
+        } else {
+          tmem_ld16x2(accA + EPI_COLS * h + 16 * qq, accBC + EPI_COLS * h + 16 * qq, va, vb);
+        }
         const int col0 = cbase + 16 * qq;             // even: complex pairs stay together
         if (col0 >= g.Nr) continue;                   // the whole block is padding (warp-uniform)
         if constexpr (OUT == 1) {
@@ -675,11 +887,11 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
             for (int j = 0; j < 16; j += 4) {
               const float s0 = pow2f(ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1)) - 30);
               const float s1 = pow2f(ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1) + 1) - 30);
-              // va is exact: one rounding in the add
-              y[j] = (va[j] + vb[j]) * s0;
-              y[j + 1] = (va[j + 1] + vb[j + 1]) * s0;
-              y[j + 2] = (va[j + 2] + vb[j + 2]) * s1;
-              y[j + 3] = (va[j + 3] + vb[j + 3]) * s1;
+              // va is exact: one rounding in the add (CV: added when vb was read)
+              y[j] = (CV ? va[j] : va[j] + vb[j]) * s0;
+              y[j + 1] = (CV ? va[j + 1] : va[j + 1] + vb[j + 1]) * s0;
+              y[j + 2] = (CV ? va[j + 2] : va[j + 2] + vb[j + 2]) * s1;
+              y[j + 3] = (CV ? va[j + 3] : va[j + 3] + vb[j + 3]) * s1;
               *reinterpret_cast<float4*>(stg + stage_off(lane, j >> 2)) = make_float4(y[j], y[j + 1], y[j + 2], y[j + 3]);
             }
             if (g.herm == 1) {
@@ -742,9 +954,11 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
           __syncwarp();   // the tile is rewritten by the next block
         }
       }
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(AEMPTY(set));
+      if constexpr (CV == 0) {
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(AEMPTY(set));
+      }
     }
   }
   fence_before();
