@@ -612,6 +612,35 @@ cudaError_t launch(const OzMaps& maps, const OzShape& g, const int* eL, const in
   return cudaGetLastError();
 }
 
+// One slab: lane planes pL with exponents eL against column planes pN, eN.
+template <int CX>
+cudaError_t slab(const Side& l, const Side& n, int K, int nb, const int* eL, const uint16_t* pL, const int* eN,
+                 const uint16_t* pN, double* out, long ldo, long sbo, bool pairs, double alpha, bool acc, const OzWork& w,
+                 cudaStream_t s) {
+  const int Kr = K * CX, ldp = pad8i(Kr);
+  OzMaps maps;
+  cudaError_t e = plane_map(&maps.n, pN, nb, plane_rows(n), Kr, ldp, TN);
+  if (e == cudaSuccess) e = plane_map(&maps.l, pL, nb, plane_rows(l), Kr, ldp, TL);
+  if (e != cudaSuccess) return e;
+  OzShape g;
+  g.nl = (int)plane_rows(l);
+  g.nn = (int)plane_rows(n);
+  g.nst = (Kr + TK - 1) / TK;
+  g.tl = (g.nl + TL - 1) / TL;
+  g.tn = (g.nn + TN - 1) / TN;
+  g.lsh = l.emb;
+  g.nsh = n.emb;
+  g.el = l.rows;
+  g.en = n.rows;
+  g.units = (long)nb * g.tl * g.tn;
+  g.pairs = pairs;
+  g.acc = acc;
+  g.alpha = alpha;
+  g.ldo = ldo;
+  g.sbo = sbo;
+  return launch<CX>(maps, g, eL, eN, out, w, s);
+}
+
 // out(lane i, column j) over batch entries, in slabs that fit the scratch.
 // pairs: the N side is embedded and out is complex [j / 2][i].
 template <int CX>
@@ -650,8 +679,6 @@ cudaError_t product(Side L, Side N, int K, int batch, double* out, long ldo, lon
       if (e != cudaSuccess) return e;
       if (w.launches) *w.launches += 2;
       unsigned char* lbuf = (unsigned char*)eN + side_bytes(n.rows, plane_rows(n), Kr, nb);
-      OzMaps maps;
-      if ((e = plane_map(&maps.n, pN, nb, plane_rows(n), Kr, ldp, TN)) != cudaSuccess) return e;
       for (int l0 = 0; l0 < L.rows; l0 += lrows) {
         Side l = L;
         l.src += ((long)b0 * L.sb + (long)l0 * L.lr) * CX;
@@ -660,27 +687,10 @@ cudaError_t product(Side L, Side N, int K, int batch, double* out, long ldo, lon
         uint16_t* pL = (uint16_t*)(lbuf + align256(sizeof(int) * (size_t)l.rows * nb));
         if ((e = prepare<CX>(l, K, nb, eL, pL, s)) != cudaSuccess) return e;
         if (w.launches) *w.launches += 2;
-        if ((e = plane_map(&maps.l, pL, nb, plane_rows(l), Kr, ldp, TL)) != cudaSuccess) return e;
-        OzShape g;
-        g.nl = (int)plane_rows(l);
-        g.nn = (int)plane_rows(n);
-        g.nst = (Kr + TK - 1) / TK;
-        g.tl = (g.nl + TL - 1) / TL;
-        g.tn = (g.nn + TN - 1) / TN;
-        g.lsh = l.emb;
-        g.nsh = n.emb;
-        g.el = l.rows;
-        g.en = n.rows;
-        g.units = (long)nb * g.tl * g.tn;
-        g.pairs = pairs;
-        g.acc = acc;
-        g.alpha = alpha;
-        g.ldo = ldo;
-        g.sbo = sbo;
         // pairs: double2 units along rows; embedded lanes: two doubles per complex column
         double* o = out + (pairs ? 2 * ((long)b0 * sbo + (long)n0 * ldo + l0)
                                  : (long)b0 * sbo + (long)n0 * ldo + (L.emb ? 2L : 1L) * l0);
-        if ((e = launch<CX>(maps, g, eL, eN, o, w, s)) != cudaSuccess) return e;
+        if ((e = slab<CX>(l, n, K, nb, eL, pL, eN, pN, o, ldo, sbo, pairs, alpha, acc, w, s)) != cudaSuccess) return e;
       }
     }
   }
@@ -746,6 +756,28 @@ cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, i
     return oz_gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, w, s);
   if (w.launches) ++*w.launches;
   return gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, s);
+}
+
+size_t oz_lane_bytes(int N, int K) { return side_bytes(N, N, 2 * K, 1); }
+
+cudaError_t oz_lane_prepare(const double2* B, int ldb, int N, int K, void* lanes, cudaStream_t s) {
+  if (2L * K > OZ_MAX_K) return cudaErrorInvalidValue;
+  const Side b{(const double*)B, N, 1L, (long)ldb, 0, false, false};
+  return prepare<2>(b, K, 1, (int*)lanes, (uint16_t*)((unsigned char*)lanes + align256(sizeof(int) * (size_t)N)), s);
+}
+
+cudaError_t oz_gemm_z_lanes(int la, int M, int N, int K, const double2* A, int lda, const void* lanes, double2* C,
+                            int ldc, const OzWork& w, cudaStream_t s) {
+  if (w.bytes < HEAD + side_bytes(M, 2L * M, 2 * K, 1)) return cudaErrorMemoryAllocation;
+  const Side a{(const double*)A, M, la == A_KM ? 1L : (long)lda, la == A_KM ? (long)lda : 1L, 0, la == A_MK_CONJ, true};
+  const Side b{nullptr, N, 1L, 1L, 0, false, false};
+  int* eA = (int*)(w.buf + HEAD);
+  uint16_t* pA = (uint16_t*)((unsigned char*)eA + align256(sizeof(int) * (size_t)M));
+  const cudaError_t e = prepare<2>(a, K, 1, eA, pA, s);
+  if (e != cudaSuccess) return e;
+  return slab<2>(b, a, K, 1, (const int*)lanes,
+                 (const uint16_t*)((const unsigned char*)lanes + align256(sizeof(int) * (size_t)N)), eA, pA, (double*)C,
+                 ldc, 0, true, 1.0, false, w, s);
 }
 
 cudaError_t oz_gemm_d(bool a_km, bool b_kn, int M, int N, int K, const double* A, long lda, const double* B, long ldb,

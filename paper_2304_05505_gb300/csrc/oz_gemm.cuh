@@ -28,6 +28,13 @@ cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, i
 cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
                       int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s);
 
+// The same product of A (any layout) with a B of N columns stored [k][n] whose
+// digits were prepared once: oz_lane_bytes of device memory at `lanes`.
+size_t oz_lane_bytes(int N, int K);
+cudaError_t oz_lane_prepare(const double2* B, int ldb, int N, int K, void* lanes, cudaStream_t s);
+cudaError_t oz_gemm_z_lanes(int la, int M, int N, int K, const double2* A, int lda, const void* lanes, double2* C,
+                            int ldc, const OzWork& w, cudaStream_t s);
+
 // Real C[m][n] = alpha sum_k A(m, k) B(n, k) (+ C when acc): A(m, k) = A[m lda + k]
 // or, a_km, A[k lda + m]; B(n, k) = B[n ldb + k] or, b_kn, B[k ldb + n].  alpha is 1 or -1.
 cudaError_t oz_gemm_d(bool a_km, bool b_kn, int M, int N, int K, const double* A, long lda, const double* B, long ldb,

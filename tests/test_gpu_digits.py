@@ -110,3 +110,34 @@ def test_fixed_point_convolution_range(thc, mesh):
     assert np.isnan(got[:, 7]).all()
     keep = np.arange(npq) != 7
     assert (np.abs(got - ref)[:, keep] <= 1e-14 * np.abs(ref).max(0)[keep]).all()
+
+
+def _pair_orbitals(kind, nf, nr, seed):
+    rng = np.random.default_rng(seed)
+    U = rng.normal(size=(nf, nr)) + 1j * rng.normal(size=(nf, nr))
+    if kind == "spread":         # residuals over several orders: few candidates per bin
+        U *= np.exp(0.5 * rng.normal(size=(1, nr)))
+    elif kind == "rank":         # pair Gram of rank 25: the trace ends the selection inside a block
+        U = rng.normal(size=(nf, 5)) @ (U[:5] * np.exp(0.3 * rng.normal(size=(1, nr))))
+    elif kind == "flat":         # more than 800 candidates within a bin of the largest: single pivots
+        U *= (1 + 1e-4 * rng.uniform(size=nr)) / np.sqrt((np.abs(U) ** 2).sum(0))
+    return U
+
+
+@pytest.mark.parametrize("kind,nf,nr,npts", [
+    ("spread", 700, 1600, 20),      # the smallest selection that goes in blocks
+    ("spread", 450, 2305, 41),      # a block and one pivot
+    ("spread", 410, 2500, 130),     # earlier rows' products in the later blocks
+    ("rank", 420, 2400, 64),
+    ("flat", 420, 2400, 24),
+])
+def test_pivots_in_blocks_match_oracle(thc, kind, nf, nr, npts):
+    """Selections large enough to go in blocks of pivots take the oracle's
+    points in its order, and leave its residuals to 1e-12 of the largest
+    diagonal entry (sums of at most 130 rows, each rounded once)."""
+    U = _pair_orbitals(kind, nf, nr, npts)
+    ref = S.pivoted_cholesky(U, npts)
+    pts, resid = thc.thc_select_points(torch.from_numpy(U).cuda(), npts)
+    assert np.array_equal(pts, ref["points"])
+    scale = float((np.sum(np.abs(U) ** 2, axis=0) ** 2).max())
+    assert np.abs(resid.cpu().numpy() - ref["resid"]).max() <= 1e-12 * scale
