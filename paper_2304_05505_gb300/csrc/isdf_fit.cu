@@ -25,52 +25,74 @@
 // at most 1024 reals; chunks are combined in FP64.
 #include "isdf_common.cuh"
 #include "tc_gemm.cuh"
+#include "slices.cuh"
 
 namespace {
 
-// Xq[P][G] = F[P][flat[G]] * sqrt(w v(G + q)) * exp(-i q.r_P), with
-// K = (gm[G] + qf) B (Cartesian) and v(K) = 4 pi / |K|^2 (0 for K = 0).
-__global__ void scale_xi(const double2* __restrict__ F, long ng, const int* __restrict__ flat,
-                         const int* __restrict__ gm, int nG, const double* __restrict__ rP, int np, Recip B,
-                         double q0, double q1, double q2, double w, double2* __restrict__ Xq) {
-  const long i = (long)blockIdx.x * TB + threadIdx.x;
-  if (i >= (long)np * nG) return;
-  const int P = (int)(i / nG), G = (int)(i % nG);
-  const double f0 = gm[3 * G] + q0, f1 = gm[3 * G + 1] + q1, f2 = gm[3 * G + 2] + q2;
-  const double kx = f0 * B.b[0] + f1 * B.b[3] + f2 * B.b[6];
-  const double ky = f0 * B.b[1] + f1 * B.b[4] + f2 * B.b[7];
-  const double kz = f0 * B.b[2] + f1 * B.b[5] + f2 * B.b[8];
-  const double k2 = kx * kx + ky * ky + kz * kz;
-  const double sv = k2 > 1e-12 ? sqrt(w * 4.0 * M_PI / k2) : 0.0;
-  const double qx = q0 * B.b[0] + q1 * B.b[3] + q2 * B.b[6];
-  const double qy = q0 * B.b[1] + q1 * B.b[4] + q2 * B.b[7];
-  const double qz = q0 * B.b[2] + q1 * B.b[5] + q2 * B.b[8];
-  double s, c;
-  sincos(-(qx * rP[3 * P] + qy * rP[3 * P + 1] + qz * rP[3 * P + 2]), &s, &c);
-  const double2 x = F[(long)P * ng + flat[G]];
-  Xq[i] = make_double2(sv * (x.x * c - x.y * s), sv * (x.x * s + x.y * c));
+// What one representative of q needs beside F: sv[G] = sqrt(w v(G + q)), with
+// K = (gm[G] + qf) B (Cartesian) and v(K) = 4 pi / |K|^2 (0 for K = 0), and
+// ph[P] = exp(-i q.r_P) as (cos, sin).  (A sincos and a square root per (P, G)
+// made scale_xi 5.3 ms at N_P = 600, N_G = 59319, five times its product.)
+__global__ void q_tables(const int* __restrict__ gm, int nG, const double* __restrict__ rP, int np, Recip B, double q0,
+                         double q1, double q2, double w, double* __restrict__ sv, double2* __restrict__ ph,
+                         unsigned* __restrict__ rowmax) {
+  const int i = (int)(blockIdx.x * TB + threadIdx.x);
+  if (i < nG) {
+    const double f0 = gm[3 * i] + q0, f1 = gm[3 * i + 1] + q1, f2 = gm[3 * i + 2] + q2;
+    const double kx = f0 * B.b[0] + f1 * B.b[3] + f2 * B.b[6];
+    const double ky = f0 * B.b[1] + f1 * B.b[4] + f2 * B.b[7];
+    const double kz = f0 * B.b[2] + f1 * B.b[5] + f2 * B.b[8];
+    const double k2 = kx * kx + ky * ky + kz * kz;
+    sv[i] = k2 > 1e-12 ? sqrt(w * 4.0 * M_PI / k2) : 0.0;
+  }
+  if (i < np) {
+    const double qx = q0 * B.b[0] + q1 * B.b[3] + q2 * B.b[6];
+    const double qy = q0 * B.b[1] + q1 * B.b[4] + q2 * B.b[7];
+    const double qz = q0 * B.b[2] + q1 * B.b[5] + q2 * B.b[8];
+    double s, c;
+    sincos(-(qx * rP[3 * i] + qy * rP[3 * i + 1] + qz * rP[3 * i + 2]), &s, &c);
+    ph[i] = make_double2(c, s);
+    rowmax[i] = 0u;
+  }
 }
 
-// The same, rounded to FP32, rows ldq complex apart.
-__global__ void scale_xi_f32(const double2* __restrict__ F, long ng, const int* __restrict__ flat,
-                             const int* __restrict__ gm, int nG, const double* __restrict__ rP, int np, Recip B,
-                             double q0, double q1, double q2, double w, float2* __restrict__ Xq, int ldq) {
-  const long i = (long)blockIdx.x * TB + threadIdx.x;
-  if (i >= (long)np * nG) return;
-  const int P = (int)(i / nG), G = (int)(i % nG);
-  const double f0 = gm[3 * G] + q0, f1 = gm[3 * G + 1] + q1, f2 = gm[3 * G + 2] + q2;
-  const double kx = f0 * B.b[0] + f1 * B.b[3] + f2 * B.b[6];
-  const double ky = f0 * B.b[1] + f1 * B.b[4] + f2 * B.b[7];
-  const double kz = f0 * B.b[2] + f1 * B.b[5] + f2 * B.b[8];
-  const double k2 = kx * kx + ky * ky + kz * kz;
-  const double sv = k2 > 1e-12 ? sqrt(w * 4.0 * M_PI / k2) : 0.0;
-  const double qx = q0 * B.b[0] + q1 * B.b[3] + q2 * B.b[6];
-  const double qy = q0 * B.b[1] + q1 * B.b[4] + q2 * B.b[7];
-  const double qz = q0 * B.b[2] + q1 * B.b[5] + q2 * B.b[8];
-  double s, c;
-  sincos(-(qx * rP[3 * P] + qy * rP[3 * P + 1] + qz * rP[3 * P + 2]), &s, &c);
-  const double2 x = F[(long)P * ng + flat[G]];
-  Xq[(long)P * ldq + G] = make_float2((float)(sv * (x.x * c - x.y * s)), (float)(sv * (x.x * s + x.y * c)));
+constexpr int SG = 4;   // G vectors per thread of scale_xi (one row P per block)
+
+// Xq[P][G] = F[P][flat[G]] sv[G] ph[P], in FP64 or rounded to FP32, rows ldq complex apart; FP32: also each row's
+// largest |re|, |im| (its bits, by atomicMax).
+template <typename CT>
+__global__ void __launch_bounds__(TB) scale_xi(const double2* __restrict__ F, long ng, const int* __restrict__ flat,
+                                               int nG, const double* __restrict__ sv, const double2* __restrict__ ph,
+                                               CT* __restrict__ Xq, long ldq, unsigned* __restrict__ rowmax) {
+  const int P = blockIdx.y, g0 = blockIdx.x * (TB * SG) + threadIdx.x;
+  const double c = ph[P].x, s = ph[P].y;
+  unsigned m = 0;
+#pragma unroll
+  for (int i = 0; i < SG; i++) {
+    const int G = g0 + i * TB;
+    if (G < nG) {
+      const double v = sv[G];
+      const double2 x = F[(long)P * ng + flat[G]];
+      const double re = v * (x.x * c - x.y * s), im = v * (x.x * s + x.y * c);
+      if constexpr (sizeof(CT) == sizeof(float2)) {
+        const float2 o = make_float2((float)re, (float)im);
+        m = max(m, max(__float_as_uint(o.x) & 0x7fffffffu, __float_as_uint(o.y) & 0x7fffffffu));
+        Xq[P * ldq + G] = o;
+      } else {
+        Xq[P * ldq + G] = make_double2(re, im);
+      }
+    }
+  }
+  if constexpr (sizeof(CT) == sizeof(float2)) {
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(rowmax + P, m);
+  }
+}
+
+// e[P] = the smallest e with the row's largest value below 2^e (0 for a zero row).
+__global__ void row_exps(const unsigned* __restrict__ rowmax, int np, int* __restrict__ e) {
+  const int i = (int)(blockIdx.x * TB + threadIdx.x);
+  if (i < np) e[i] = row_exponent((double)__uint_as_float(rowmax[i]));
 }
 
 // V += W (complex)
@@ -141,7 +163,9 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
   uint16_t* Bpl = nullptr;
   int *eX = nullptr, *ps0 = nullptr, *tcerr = nullptr;
   float* pbc = nullptr;
-  double2 *Ugc = nullptr, *Bm = nullptr, *F = nullptr, *Xq = nullptr, *W = nullptr, *twd = nullptr;
+  double2 *Ugc = nullptr, *Bm = nullptr, *F = nullptr, *Xq = nullptr, *W = nullptr, *twd = nullptr, *phd = nullptr;
+  double* svd = nullptr;
+  unsigned* rmax = nullptr;
   double *R = nullptr, *S = nullptr, *L = nullptr, *Linv = nullptr, *rPd = nullptr;
   OzWork oz;
   int *ptsd = nullptr, *gmd = nullptr, *flatd = nullptr, *bad = nullptr;
@@ -208,10 +232,9 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     Ugc = nullptr;
     if ((e = cudaMalloc(&F, sizeof(double2) * (size_t)npts * ng)) != cudaSuccess) break;
     const long tot = (long)npts * ng;
-    dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(R, true, F, tot, g3, 1, twd + off[2]);
-    dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(F, false, Bm, tot, g2, g3, twd + off[1]);
-    dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(Bm, false, F, tot, g1, (long)g2 * g3, twd + off[0]);
-    if ((e = cudaGetLastError()) != cudaSuccess) break;
+    if ((e = dft_axis(R, true, F, tot, g3, 1, twd + off[2], s)) != cudaSuccess) break;
+    if ((e = dft_axis(F, false, Bm, tot, g2, g3, twd + off[1], s)) != cudaSuccess) break;
+    if ((e = dft_axis(Bm, false, F, tot, g1, (long)g2 * g3, twd + off[0], s)) != cudaSuccess) break;
     mark(4);
     // 4. V^q, one Hermitian product per representative of q
     cudaFree(Bm);
@@ -239,6 +262,10 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
       break;
     }
     if ((e = cudaMalloc(&W, sizeof(double2) * npq)) != cudaSuccess) break;
+    if ((e = cudaMalloc(&svd, sizeof(double) * nG)) != cudaSuccess) break;
+    if ((e = cudaMalloc(&phd, sizeof(double2) * npts)) != cudaSuccess) break;
+    if ((e = cudaMalloc(&rmax, sizeof(unsigned) * npts)) != cudaSuccess) break;
+    const dim3 sgrid((nG + TB * SG - 1) / (TB * SG), npts);
     double2* V = (double2*)V_out;
     if ((e = cudaMemsetAsync(V, 0, sizeof(double2) * nk * npq, s)) != cudaSuccess) break;
     const double sc = vol / ng;   // xh = (Omega / N_g) DFT(xi)
@@ -250,9 +277,9 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
       for (double x0 : r0)
         for (double x1 : r1)
           for (double x2 : r2) {
+            q_tables<<<blocks(std::max(nG, npts)), TB, 0, s>>>(gmd, nG, rPd, npts, B, x0, x1, x2, w, svd, phd, rmax);
             if (!tc) {
-              scale_xi<<<blocks((long)npts * nG), TB, 0, s>>>(F, ng, flatd, gmd, nG, rPd, npts, B, x0, x1, x2, w,
-                                                              Xq);
+              scale_xi<double2><<<sgrid, TB, 0, s>>>(F, ng, flatd, nG, svd, phd, Xq, nG, nullptr);
               if ((e = gemm_z_best(A_MK, B_NK_CONJ, npts, npts, nG, Xq, nG, 0, Xq, nG, 0, W, npts, 0, 1, oz, s)) !=
                   cudaSuccess)
                 break;
@@ -261,9 +288,8 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
             }
             // Xq Xq^H on tensor cores: A = Xq (FP32, sliced in the GEMM), B =
             // the embedded conj(Xq)^T, both with the exact row exponents of Xq
-            scale_xi_f32<<<blocks((long)npts * nG), TB, 0, s>>>(F, ng, flatd, gmd, nG, rPd, npts, B, x0, x1, x2, w,
-                                                                Xq32, ldq);
-            if ((e = row_exponents_c(Xq32, 0, ldq, 1, npts, nG, eX, s)) != cudaSuccess) break;
+            scale_xi<float2><<<sgrid, TB, 0, s>>>(F, ng, flatd, nG, svd, phd, Xq32, ldq, rmax);
+            row_exps<<<blocks(npts), TB, 0, s>>>(rmax, npts, eX);
             for (int g0 = 0; g0 < nG && e == cudaSuccess; g0 += slab) {
               const int gn = std::min(slab, nG - g0);
               TcOperand opA, opB;
@@ -306,7 +332,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     set_global_error(std::string("thc_fit_kernel: ") + cudaGetErrorString(e));
     st = e == cudaErrorMemoryAllocation ? THC_ERR_OOM : THC_ERR_CUDA;
   }
-  void* ptrs[] = {Ugc, Bm, F, Xq, W, twd, R, S, L, Linv, rPd, ptsd, gmd, flatd, bad, Xq32, Bpl, eX, ps0, pbc, tcerr};
+  void* ptrs[] = {Ugc, Bm, F, Xq, W, twd, R, S, L, Linv, rPd, phd, svd, rmax, ptsd, gmd, flatd, bad, Xq32, Bpl, eX, ps0, pbc, tcerr};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   oz_free(oz);
