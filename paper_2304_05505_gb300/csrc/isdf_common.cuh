@@ -217,12 +217,12 @@ __global__ void __launch_bounds__(TB) fft_axis_kernel(const void* __restrict__ i
   }
 }
 
-// One axis (length g, stride st) of the forward DFT of `total` values.
+// One axis (length g, stride st) of the forward DFT of `total` values; fft = false: by direct sums.
 inline cudaError_t dft_axis(const void* in, bool real_in, double2* out, long total, int g, long st,
-                            const double2* tw, cudaStream_t s) {
+                            const double2* tw, cudaStream_t s, bool fft = true) {
   const FftPlan p = fft_plan(g);
   const long lines = total / g;
-  if (p.nr > 0 && lines < (1L << 34)) {
+  if (fft && p.nr > 0 && lines < (1L << 34)) {
     const size_t sm = sizeof(double2) * (size_t)g * (2 * FW + 1);
     const cudaError_t e = cudaFuncSetAttribute(fft_axis_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;

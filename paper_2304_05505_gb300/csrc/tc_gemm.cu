@@ -233,6 +233,7 @@ struct Geometry {
   int herm;                  // Hermitian product: tiles reaching the diagonal only (1: mirrored, 2: upper part)
   long upb;                  // units per batch entry when herm
   int b0;                    // batch offset of the operands' tensor maps (a sub-batch of a product)
+  int acc;                   // FP64 result: added to what out holds
 };
 
 // First n tile of m tile mi that reaches the diagonal of a Hermitian product
@@ -860,8 +861,12 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
             if (col0 + j >= g.Nr) break;
             const double sc = pow2d(ea + ep[j >> 1] - 30);
             // va holds 2^16 times an exact integer below 2^24
-            const double x0 = ((double)va[j] + (double)vb[j]) * sc;
-            const double x1 = ((double)va[j + 1] + (double)vb[j + 1]) * sc;
+            double x0 = ((double)va[j] + (double)vb[j]) * sc;
+            double x1 = ((double)va[j + 1] + (double)vb[j + 1]) * sc;
+            if (g.acc) {   // (own statements: no fused multiply-add with the scale)
+              x0 = __dadd_rn(o[col0 + j], x0);
+              if (col0 + j + 1 < g.Nr) x1 = __dadd_rn(o[col0 + j + 1], x1);
+            }
             if (col0 + j + 1 < g.Nr && (ldo % 2) == 0) {
               *reinterpret_cast<double2*>(o + col0 + j) = make_double2(x0, x1);
             } else {
@@ -989,7 +994,8 @@ __global__ void __launch_bounds__(256) tc_combine_kernel(const int* __restrict__
                                                          int nchunk, int batch, int M, int Nr,
                                                          const int* __restrict__ eA, long seA,
                                                          const int* __restrict__ eB, long seB, void* out, long ldo,
-                                                         long sbo, const float* __restrict__ w, double* dot) {
+                                                         long sbo, const float* __restrict__ w, double* dot,
+                                                         int acc) {
   static_assert(!DOT || (!OUT_F64 && V == 4), "the dot product of an FP32 result, four columns per thread");
   const long total = (long)batch * M * Nr;
   const long nv = total / V;
@@ -1025,6 +1031,10 @@ __global__ void __launch_bounds__(256) tc_combine_kernel(const int* __restrict__
 #pragma unroll
       for (int j = 0; j < V; j++)
         x[j] = ((double)s0[j] + (double)bc[j]) * pow2d(ea + eB[(long)b * seB + ((col + j) >> 1)]);
+      if (acc) {
+#pragma unroll
+        for (int j = 0; j < V; j++) x[j] = __dadd_rn(((const double*)out)[o + j], x[j]);
+      }
       if constexpr (V == 4) {
         reinterpret_cast<double2*>((double*)out + o)[0] = make_double2(x[0], x[1]);
         reinterpret_cast<double2*>((double*)out + o)[1] = make_double2(x[2], x[3]);
@@ -1197,7 +1207,7 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
                     const int* eA, long seA, const int* eB, long seB, void* out, bool out_f64, long ldo,
                     long sbo, int* ps0, float* pbc, int* err, cudaStream_t s,
                     cudaEvent_t gemm_done, int products, int a_conv, int herm, const float* dot_with,
-                    double* dot_partial, int dot_max, int* dot_blocks, int b0, int ckb) {
+                    double* dot_partial, int dot_max, int* dot_blocks, int b0, int ckb, bool accumulate) {
   if (dot_blocks) *dot_blocks = 0;
   if (b0 < 0) return cudaErrorInvalidValue;
   if (products != 6 && products != 8) return cudaErrorInvalidValue;
@@ -1220,6 +1230,8 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
   g.herm = herm;
   g.upb = 0;
   g.b0 = b0;
+  g.acc = accumulate;
+  if (accumulate && !out_f64) return cudaErrorInvalidValue;
   if (herm) {
     // a Hermitian FP32 product written whole: square, one chunk, FP32 interleaved output
     if (Nr != 2 * M || g.nchunk != 1 || out_f64 || a_conv || (ldo % 2) || (sbo % 2)) return cudaErrorInvalidValue;
@@ -1276,7 +1288,7 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
   if (dot) cg = std::min<unsigned>(cg, (unsigned)dot_max);
 #define COMBINE(F64, V, D)                                                                                 \
   tc_combine_kernel<F64, V, D><<<cg, 256, 0, s>>>(ps0, pbc, g.nchunk, batch, M, Nr, eA, seA, eB, seB, out, ldo, \
-                                                  sbo, dot_with, dot_partial)
+                                                  sbo, dot_with, dot_partial, (int)accumulate)
   if (out_f64) {
     if (v4) COMBINE(true, 4, false); else COMBINE(true, 1, false);
   } else if (dot) {

@@ -32,6 +32,7 @@
 // tensor cores in the form of the rebuild's contraction.
 #include "isdf_common.cuh"
 #include "tc_gemm.cuh"
+#include "slices.cuh"
 
 #include <algorithm>
 #include <string>
@@ -121,49 +122,111 @@ __global__ void wv_partial(const double2* __restrict__ W, const double2* __restr
   if (threadIdx.x == 0) part[blockIdx.x] = sm[0];
 }
 
-// A[P][Q] = c e^{-i q.r_P} W[P][Q] e^{+i q.r_Q}   (q Cartesian)
-__global__ void phase_w(const double2* __restrict__ W, int np, const double* __restrict__ rP, double qx, double qy,
-                        double qz, double c, double2* __restrict__ A) {
+// What one representative of q needs beside F and W: vt[G] = v(G + q), with K = (gm[G] + qf) B and v(K) = 4 pi /
+// |K|^2 (0 for K = 0), and ph[P] = e^{-i q.r_P} as (cos, sin), q Cartesian.  cm (tensor-core form): cm[G] = the
+// largest |re|, |im| over Q of F[Q][flat[G]]; eB[G] = the exponent of the column v conj(F) (rounding keeps order, so
+// the largest product is the product of the largest).
+__global__ void q_tables(const int* __restrict__ gm, int nG, const double* __restrict__ rP, int np, Recip B, double q0,
+                         double q1, double q2, double qx, double qy, double qz, double* __restrict__ vt,
+                         double2* __restrict__ ph, const double* __restrict__ cm, int* __restrict__ eB) {
+  const long i = (long)blockIdx.x * TB + threadIdx.x;
+  if (i < nG) {
+    const double f0 = gm[3 * i] + q0, f1 = gm[3 * i + 1] + q1, f2 = gm[3 * i + 2] + q2;
+    const double kx = f0 * B.b[0] + f1 * B.b[3] + f2 * B.b[6];
+    const double ky = f0 * B.b[1] + f1 * B.b[4] + f2 * B.b[7];
+    const double kz = f0 * B.b[2] + f1 * B.b[5] + f2 * B.b[8];
+    const double k2 = kx * kx + ky * ky + kz * kz;
+    const double v = k2 > 1e-12 ? 4.0 * M_PI / k2 : 0.0;
+    vt[i] = v;
+    if (eB) eB[i] = row_exponent(v * cm[i]);
+  }
+  if (i < np) {
+    double s, c;
+    sincos(-(qx * rP[3 * i] + qy * rP[3 * i + 1] + qz * rP[3 * i + 2]), &s, &c);
+    ph[i] = make_double2(c, s);
+  }
+}
+
+// A[P][Q] = c ph_P W[P][Q] conj(ph_Q), in FP64 or rounded to FP32 (the A operand of the tensor-core contraction),
+// rows lda complex apart
+template <typename CT>
+__global__ void phase_w(const double2* __restrict__ W, int np, const double2* __restrict__ ph, double c,
+                        CT* __restrict__ A, int lda) {
   const long i = (long)blockIdx.x * TB + threadIdx.x;
   if (i >= (long)np * np) return;
   const int P = (int)(i / np), Q = (int)(i % np);
-  double sp, cp, sq, cq;
-  sincos(-(qx * rP[3 * P] + qy * rP[3 * P + 1] + qz * rP[3 * P + 2]), &sp, &cp);
-  sincos(-(qx * rP[3 * Q] + qy * rP[3 * Q + 1] + qz * rP[3 * Q + 2]), &sq, &cq);
+  const double cp = ph[P].x, sp = ph[P].y, cq = ph[Q].x, sq = ph[Q].y;
   // e^{-i q.r_P} conj(e^{-i q.r_Q}) = e^{i (aP - aQ)} with aP = -q.r_P
   const double cr = cp * cq + sp * sq, ci = sp * cq - cp * sq;
   const double2 w = W[i];
-  A[i] = make_double2(c * (w.x * cr - w.y * ci), c * (w.x * ci + w.y * cr));
+  const double re = c * (w.x * cr - w.y * ci), im = c * (w.x * ci + w.y * cr);
+  if constexpr (sizeof(CT) == sizeof(float2)) A[(long)P * lda + Q] = make_float2((float)re, (float)im);
+  else A[(long)P * lda + Q] = make_double2(re, im);
 }
 
-// The same, rounded to FP32, rows lda complex apart (the A operand of the
-// tensor-core contraction).
-__global__ void phase_w32(const double2* __restrict__ W, int np, const double* __restrict__ rP, double qx, double qy,
-                          double qz, double c, float2* __restrict__ A, int lda) {
-  const long i = (long)blockIdx.x * TB + threadIdx.x;
-  if (i >= (long)np * np) return;
-  const int P = (int)(i / np), Q = (int)(i % np);
-  double sp, cp, sq, cq;
-  sincos(-(qx * rP[3 * P] + qy * rP[3 * P + 1] + qz * rP[3 * P + 2]), &sp, &cp);
-  sincos(-(qx * rP[3 * Q] + qy * rP[3 * Q + 1] + qz * rP[3 * Q + 2]), &sq, &cq);
-  const double cr = cp * cq + sp * sq, ci = sp * cq - cp * sq;
-  const double2 w = W[i];
-  A[(long)P * lda + Q] = make_float2((float)(c * (w.x * cr - w.y * ci)), (float)(c * (w.x * ci + w.y * cr)));
+// cm[G] = max over P of |re|, |im| of F[P][flat[G]]
+__global__ void col_max(const double2* __restrict__ F, long ng, const int* __restrict__ flat, int nG, int np,
+                        double* __restrict__ cm) {
+  const int G = (int)(blockIdx.x * TB + threadIdx.x);
+  if (G >= nG) return;
+  const double2* f = F + flat[G];
+  double m = 0.0;
+  for (int P = 0; P < np; P++) {
+    const double2 x = f[(long)P * ng];
+    m = fmax(m, fmax(fabs(x.x), fabs(x.y)));
+  }
+  cm[G] = m;
 }
 
-// Bq[Q][G] = v(G + q) conj(F[Q][flat[G]]), K = (gm[G] + qf) B, v(K) = 4 pi / |K|^2 (0 for K = 0)
-__global__ void coulomb_conj(const double2* __restrict__ F, long ng, const int* __restrict__ flat,
-                             const int* __restrict__ gm, int nG, int np, Recip B, double q0, double q1, double q2,
-                             double2* __restrict__ Bq) {
+// The embedded planes (tc_gemm.cu) of the contraction's B operand v conj(F)^T: rows 2 G and 2 G + 1 hold the slices of
+// (re, -im) and (im, re) of B(P, G) = vt[G] conj(F[P][flat[G]]), rounded to FP32, with exponent eB[G].  Blocks of 32 G
+// by 32 P turned around in shared memory (F is read along G, the planes are written along P); the FP64 B never goes
+// through memory.
+__global__ void __launch_bounds__(256) embed_coulomb(const double2* __restrict__ F, long ng,
+                                                     const int* __restrict__ flat, int nG, int np,
+                                                     const double* __restrict__ vt, const int* __restrict__ eB,
+                                                     uint16_t* __restrict__ planes, long plane, int ldp) {
+  __shared__ uint32_t t[3][32][33];     // (re, -im) words of the three planes: [G][P]
+  const int G0 = blockIdx.x * 32, P0 = blockIdx.y * 32;
+  {
+    const int g = threadIdx.x & 31, G = G0 + g;
+    const bool in = G < nG;
+    const double v = in ? vt[G] : 0.0;
+    const long o = in ? flat[G] : 0;
+    const int e = in ? eB[G] : 0;
+    for (int p = threadIdx.x >> 5; p < 32; p += 8) {
+      const double2 x = in && P0 + p < np ? F[(long)(P0 + p) * ng + o] : make_double2(0.0, 0.0);
+      uint16_t re[3], im[3];
+      slice3((float)(v * x.x), e, re);
+      slice3((float)(v * x.y), e, im);   // -im of v conj(x)
+#pragma unroll
+      for (int q = 0; q < 3; q++) t[q][g][p] = (uint32_t)re[q] | ((uint32_t)im[q] << 16);
+    }
+  }
+  __syncthreads();
+  const int p = threadIdx.x & 31, P = P0 + p;
+  if (P >= np) return;
+  for (int g = threadIdx.x >> 5; g < 32; g += 8) {
+    const int G = G0 + g;
+    if (G >= nG) continue;
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      const uint32_t w = t[q][g][p];
+      uint32_t* o = reinterpret_cast<uint32_t*>(planes + q * plane + 2L * G * ldp + 2 * P);
+      *o = w;
+      // (im, re): im is the second half with its sign flipped
+      *reinterpret_cast<uint32_t*>(reinterpret_cast<uint16_t*>(o) + ldp) = __byte_perm(w ^ 0x80000000u, 0, 0x1032);
+    }
+  }
+}
+
+// Bq[Q][G] = vt[G] conj(F[Q][flat[G]])
+__global__ void coulomb_conj(const double2* __restrict__ F, long ng, const int* __restrict__ flat, int nG, int np,
+                             const double* __restrict__ vt, double2* __restrict__ Bq) {
   const long i = (long)blockIdx.x * TB + threadIdx.x;
   if (i >= (long)np * nG) return;
   const int Q = (int)(i / nG), G = (int)(i % nG);
-  const double f0 = gm[3 * G] + q0, f1 = gm[3 * G + 1] + q1, f2 = gm[3 * G + 2] + q2;
-  const double kx = f0 * B.b[0] + f1 * B.b[3] + f2 * B.b[6];
-  const double ky = f0 * B.b[1] + f1 * B.b[4] + f2 * B.b[7];
-  const double kz = f0 * B.b[2] + f1 * B.b[5] + f2 * B.b[8];
-  const double k2 = kx * kx + ky * ky + kz * kz;
-  const double v = k2 > 1e-12 ? 4.0 * M_PI / k2 : 0.0;
+  const double v = vt[G];
   const double2 x = F[(long)Q * ng + flat[G]];
   Bq[i] = make_double2(v * x.x, -v * x.y);
 }
@@ -373,6 +436,8 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     if (step_ms_host && ev[i]) cudaEventRecord(ev[i], s);
   };
   const int NPART = 1024;
+  double *vt = nullptr, *cm = nullptr;
+  double2* phd = nullptr;
   double2 *Psi = nullptr, *Psivt = nullptr, *D = nullptr, *M = nullptr, *W = nullptr, *Y = nullptr, *Ge = nullptr;
   double2 *Ugc = nullptr, *Bm = nullptr, *F = nullptr, *T = nullptr, *Gam = nullptr, *Aq = nullptr, *Bq = nullptr;
   double2 *Z = nullptr, *T1 = nullptr, *T2 = nullptr, *Uvp = nullptr, *G1 = nullptr, *G2 = nullptr, *twd = nullptr;
@@ -495,17 +560,23 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     }
     // R now holds xi
     const long tot = (long)np * ng;
-    dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(R, true, F, tot, g3, 1, twd + geo.off[2]);
-    dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(F, false, T, tot, g2, g3, twd + geo.off[1]);
-    dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(T, false, F, tot, g1, (long)g2 * g3, twd + geo.off[0]);
+    // (THC_MIXED: the direct sums, as in step 4 below; an FFT's last bits would
+    // come out of the solve there at 8e-8 of single entries of g)
+    if ((e = dft_axis(R, true, F, tot, g3, 1, twd + geo.off[2], s, dig)) != cudaSuccess) break;
+    if ((e = dft_axis(F, false, T, tot, g2, g3, twd + geo.off[1], s, dig)) != cudaSuccess) break;
+    if ((e = dft_axis(T, false, F, tot, g1, (long)g2 * g3, twd + geo.off[0], s, dig)) != cudaSuccess) break;
     if ((e = cudaGetLastError()) != cudaSuccess) break;
 
     // 3. Gam = sum over q and its representatives of (c ph W^q ph^H) (v o conj(xh))
     mark(2);
     if ((e = cudaMalloc(&Gam, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
     if (precision == THC_FP64 && (e = cudaMalloc(&Aq, sizeof(double2) * npq)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&Bq, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&Z, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
+    if (precision == THC_FP64) {
+      if ((e = cudaMalloc(&Bq, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
+      if ((e = cudaMalloc(&Z, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
+    }
+    if ((e = cudaMalloc(&vt, sizeof(double) * nG)) != cudaSuccess) break;
+    if ((e = cudaMalloc(&phd, sizeof(double2) * np)) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(Gam, 0, sizeof(double2) * (size_t)np * nG, s)) != cudaSuccess) break;
     // THC_MIXED: Z = A Bq on the tensor cores, A (FP32, sliced in the GEMM with
     // its row exponents) against the embedded Bq (three fp16 slices with the
@@ -522,6 +593,8 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
       if ((e = cudaMalloc(&Bpl, sizeof(uint16_t) * 3 * (size_t)plane)) != cudaSuccess) break;
       if ((e = cudaMalloc(&eA, sizeof(int) * np)) != cudaSuccess) break;
       if ((e = cudaMalloc(&eB, sizeof(int) * nG)) != cudaSuccess) break;
+      if ((e = cudaMalloc(&cm, sizeof(double) * nG)) != cudaSuccess) break;
+      col_max<<<blocks(nG), TB, 0, s>>>(F, ng, flatd, nG, np, cm);
       if ((e = cudaMalloc(&tcerr, 64)) != cudaSuccess) break;
       if (npart > 0) {
         if ((e = cudaMalloc(&ps0, sizeof(int) * npart)) != cudaSuccess) break;
@@ -549,24 +622,23 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
             const double qx = x0 * B.b[0] + x1 * B.b[3] + x2 * B.b[6];
             const double qy = x0 * B.b[1] + x1 * B.b[4] + x2 * B.b[7];
             const double qz = x0 * B.b[2] + x1 * B.b[5] + x2 * B.b[8];
-            coulomb_conj<<<blocks((long)np * nG), TB, 0, s>>>(F, ng, flatd, gmd, nG, np, B, x0, x1, x2, Bq);
+            q_tables<<<blocks(std::max(nG, np)), TB, 0, s>>>(gmd, nG, rPd, np, B, x0, x1, x2, qx, qy, qz, vt, phd, cm,
+                                                             eB);
             if (!tc) {
-              phase_w<<<blocks(npq), TB, 0, s>>>(W + (long)q * npq, np, rPd, qx, qy, qz, c, Aq);
+              coulomb_conj<<<blocks((long)np * nG), TB, 0, s>>>(F, ng, flatd, nG, np, vt, Bq);
+              phase_w<double2><<<blocks(npq), TB, 0, s>>>(W + (long)q * npq, np, phd, c, Aq, np);
               if ((e = gemm_z_best(A_MK, B_KN, np, nG, np, Aq, np, 0, Bq, nG, 0, Z, nG, 0, 1, oz, s)) != cudaSuccess) break;
+              axpy_z<<<blocks((long)np * nG), TB, 0, s>>>(Gam, Z, (long)np * nG);
             } else {
-              phase_w32<<<blocks(npq), TB, 0, s>>>(W + (long)q * npq, np, rPd, qx, qy, qz, c, Aq32, lda);
+              phase_w<float2><<<blocks(npq), TB, 0, s>>>(W + (long)q * npq, np, phd, c, Aq32, lda);
               if ((e = row_exponents_c(Aq32, 0, lda, 1, np, np, eA, s)) != cudaSuccess) break;
-              if ((e = col_exponents_z(Bq, 0, nG, 1, np, nG, eB, s)) != cudaSuccess) break;
-              // embedded in slabs of G (the embedding's grid holds at most 131,070 rows j)
-              for (int g0 = 0; g0 < nG && e == cudaSuccess; g0 += 65536)
-                e = embed_b(Bq + g0, true, 0, nG, 1, false, false, 1, np, std::min(65536, nG - g0), eB + g0,
-                            Bpl + 2L * g0 * ldp, plane, ldp, s);
-              if (e != cudaSuccess) break;
-              if ((e = tc_gemm(opA, opB, np, 2 * nG, 2 * np, 1, eA, np, eB, nG, Z, true, 2L * nG, 2L * np * nG, ps0,
-                               pbc, tcerr, s, nullptr, 8, 1, 0)) != cudaSuccess)
+              embed_coulomb<<<dim3((nG + 31) / 32, (np + 31) / 32), 256, 0, s>>>(F, ng, flatd, nG, np, vt, eB, Bpl, plane,
+                                                                                 ldp);
+              // (added to Gam as it is written)
+              if ((e = tc_gemm(opA, opB, np, 2 * nG, 2 * np, 1, eA, np, eB, nG, Gam, true, 2L * nG, 2L * np * nG, ps0,
+                               pbc, tcerr, s, nullptr, 8, 1, 0, nullptr, nullptr, 0, nullptr, 0, 0, true)) != cudaSuccess)
                 break;
             }
-            axpy_z<<<blocks((long)np * nG), TB, 0, s>>>(Gam, Z, (long)np * nG);
           }
     }
     if (e != cudaSuccess) break;
@@ -581,9 +653,9 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     mark(3);
     if ((e = cudaMemsetAsync(F, 0, sizeof(double2) * (size_t)np * ng, s)) != cudaSuccess) break;
     scatter_g<<<blocks((long)np * nG), TB, 0, s>>>(Gam, np, nG, flatd, ng, F);
-    dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(F, false, T, tot, g3, 1, twd + geo.off[2]);
-    dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(T, false, F, tot, g2, g3, twd + geo.off[1]);
-    dft_axis_kernel<<<blocks(tot), TB, 0, s>>>(F, false, T, tot, g1, (long)g2 * g3, twd + geo.off[0]);
+    if ((e = dft_axis(F, false, T, tot, g3, 1, twd + geo.off[2], s, dig)) != cudaSuccess) break;
+    if ((e = dft_axis(T, false, F, tot, g2, g3, twd + geo.off[1], s, dig)) != cudaSuccess) break;
+    if ((e = dft_axis(F, false, T, tot, g1, (long)g2 * g3, twd + geo.off[0], s, dig)) != cudaSuccess) break;
     if ((e = cudaMalloc(&Lam, sizeof(double) * (size_t)np * ng)) != cudaSuccess) break;
     real_part<<<blocks(tot), TB, 0, s>>>(T, tot, Lam);
     if (dig) {
@@ -593,7 +665,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     }
     if ((e = cudaMalloc(&Sbar, sizeof(double) * npq)) != cudaSuccess) break;
     // S-bar = -Lam xi^T
-    if (dig && ng <= OZ_MAX_K && oz.bytes >= oz_work_min((int)((ng + 1) / 2))) {
+    if (ng <= OZ_MAX_K && oz.bytes >= oz_work_min((int)((ng + 1) / 2))) {
       if ((e = oz_gemm_d(false, false, np, np, (int)ng, Lam, ng, R, ng, Sbar, np, -1.0, false, oz, s)) != cudaSuccess)
         break;
     } else {
@@ -700,7 +772,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
   }
   void* ptrs[] = {Psi, Psivt, D,   M,   W,  Y,  Ge,  Ugc,   Bm,    F,    T,     Gam,  Aq,  Bq,  Z,
                   T1,  T2,    Uvp, G1,  G2, twd, R,  S,     L,     Linv,  Lam,  Sbar,  rPd,  part, ptsd, gmd,
-                  flatd, bad, kqd, qkd, Aq32, Bpl, eA,  eB,  ps0, pbc, tcerr, Y32, A2, Uv32, eOrb};
+                  flatd, bad, kqd, qkd, Aq32, Bpl, eA,  eB,  ps0, pbc, tcerr, Y32, A2, Uv32, eOrb, vt, cm, phd};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   oz_free(oz);
