@@ -203,10 +203,10 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
   const int nchunk = (g.nst + CHUNK_ST - 1) / CHUNK_ST;
   // unit -> (batch entry, lane tile, column tile), column tiles fastest: CTAs side by side share the lane tile
   auto decode = [&](long u, int& b, int& li, int& ni) {
-    ni = (int)(u % g.tn);
-    const long r = u / g.tn;
-    li = (int)(r % g.tl);
-    b = (int)(r / g.tl);
+    const unsigned r = (unsigned)u / (unsigned)g.tn;
+    ni = (int)((unsigned)u - r * (unsigned)g.tn);
+    b = (int)(r / (unsigned)g.tl);
+    li = (int)(r - (unsigned)b * (unsigned)g.tl);
   };
 
   // (warps 0 and 1 keep all lanes in their loops and elect one per batch of
@@ -603,6 +603,7 @@ template <int CX>
 cudaError_t launch(const OzMaps& maps, const OzShape& g, const int* eL, const int* eN, double* out, const OzWork& w,
                    cudaStream_t s) {
   int dev = 0, nsm = 0;
+  if (g.units >= (1L << 31)) return cudaErrorInvalidValue;   // counted in 32 bits
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
@@ -724,10 +725,13 @@ void oz_free(OzWork& w) {
   w = OzWork{};
 }
 
-// Below about 2e6 complex multiply-adds the five launches of the digit form
-// cost more than the product on the FP64 pipe.
+// The FP64 kernel takes 4.3 us per unit of K and round of its 64 x 64 tiles
+// over the SMs (two multiply-adds a clock on each): 35 us for one tile of
+// K = 8, and 0.3 ms for one of K = 71.  The digit form's five launches are
+// about 35 us in all.
 bool oz_wins(int M, int N, int K, int batch) {
-  return (double)M * N * K * batch > 2e6 && 2L * K <= OZ_MAX_K;
+  const double tiles = ((M + 63) / 64) * (double)((N + 63) / 64) * batch;
+  return ceil(tiles / 152.0) * K >= 10.0 && 2L * K <= OZ_MAX_K;
 }
 
 cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,

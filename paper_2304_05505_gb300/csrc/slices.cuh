@@ -29,18 +29,56 @@ __device__ __forceinline__ void slice3_planes(float y, float* p) {
   p[2] = s2 * 256.0f;
 }
 
-// The same for y + l with |l| far below the leading slice's unit: the
-// leading slice is rint(y), and l joins the first remainder before it is
-// rounded to the second and third slices.
-__device__ __forceinline__ void slice3_planes_x(float y, float l, float* p) {
-  const float s0 = __fsub_rn(__fadd_rn(y, 0x1.8p23f), 0x1.8p23f);
-  float r = __fadd_rn(__fsub_rn(y, s0), l);
-  const float s1 = __fsub_rn(__fadd_rn(r, 0x1.8p12f), 0x1.8p12f);
-  r = __fsub_rn(r, s1);
-  const float s2 = __fsub_rn(__fadd_rn(r, 0x1.8p1f), 0x1.8p1f);
-  p[0] = s0 * 256.0f;
-  p[1] = s1 * 256.0f;
-  p[2] = s2 * 256.0f;
+// Two FP32 values in one register pair, added and multiplied by one
+// instruction (sm_100 and later).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// slice3_planes of two values at once, each plane as a word of two fp16
+// numbers (the first value in the low half); y and l already times 2^8, so
+// that the rounded parts are the planes themselves.  EXT: the value is y + l
+// with |l| far below the leading slice's unit: the leading slice is rint(y),
+// and l joins the first remainder before it is rounded on.
+template <bool EXT>
+__device__ __forceinline__ void slice3_words(f32x2 y, f32x2 l, uint32_t& w0, uint32_t& w1, uint32_t& w2) {
+  const f32x2 m0 = pack2(0x1.8p31f, 0x1.8p31f), m1 = pack2(0x1.8p20f, 0x1.8p20f), m2 = pack2(0x1.8p9f, 0x1.8p9f);
+  const f32x2 s0 = sub2(add2(y, m0), m0);
+  f32x2 r = sub2(y, s0);
+  if (EXT) r = add2(r, l);
+  const f32x2 s1 = sub2(add2(r, m1), m1);
+  r = sub2(r, s1);
+  const f32x2 s2 = sub2(add2(r, m2), m2);
+  auto word = [](f32x2 v) {
+    float a, b;
+    unpack2(v, a, b);
+    const __half2 h = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+  };
+  w0 = word(s0);
+  w1 = word(s1);
+  w2 = word(s2);
 }
 
 // The fp16 bits of the three planes of x with row exponent e.  The scale

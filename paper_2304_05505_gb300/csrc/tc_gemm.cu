@@ -251,38 +251,85 @@ __device__ __forceinline__ int row_exp(const int* e, long i) {
 
 // The three fp16 planes of 8 consecutive reals x[0..8) of one row (scale sc =
 // 2^(7 - e_row)), packed two reals per word: w[p][j] holds reals 2j, 2j + 1 of
-// plane p.
+// plane p.  Two reals per instruction: 13 for a pair, against 27 one by one.
 __device__ __forceinline__ void slice8_f16(const float* x, float sc, uint32_t w[NPL][4]) {
+  const f32x2 s2 = pack2(sc, sc), k2 = pack2(256.f, 256.f);
 #pragma unroll
-  for (int j = 0; j < 8; j += 2) {
-    float lo[NPL], hi[NPL];
-    slice3_planes(x[j] * sc, lo);
-    slice3_planes(x[j + 1] * sc, hi);
+  for (int j = 0; j < 4; j++)
+    slice3_words<false>(mul2(mul2(pack2(x[2 * j], x[2 * j + 1]), s2), k2), 0, w[0][j], w[1][j], w[2][j]);
+}
+
+// The same for values given as an FP32 part x and a remainder, the fp16
+// multiple q of the unit in the last place of x (word j of q: the pair j):
+// q 2^(eh - 150) for x of biased exponent eh, none where eh < 24.
+__device__ __forceinline__ void slice8_f16x(const float* x, const uint32_t* q, float sc, uint32_t w[NPL][4]) {
+  const f32x2 s2 = pack2(sc, sc), k2 = pack2(256.f, 256.f), u2 = pack2(0x1p-15f, 0x1p-15f);
 #pragma unroll
-    for (int p = 0; p < NPL; p++) {
-      const __half2 h = __floats2half2_rn(lo[p], hi[p]);
-      w[p][j >> 1] = *reinterpret_cast<const uint32_t*>(&h);
-    }
+  for (int j = 0; j < 4; j++) {
+    // 2^(eh - 127) 2^(7 - e_row) 2^-15: the unit times the row's scale and 2^8
+    const uint32_t e0 = __float_as_uint(x[2 * j]) & 0x7f800000u, e1 = __float_as_uint(x[2 * j + 1]) & 0x7f800000u;
+    const f32x2 u = mul2(mul2(pack2(__uint_as_float(e0), __uint_as_float(e1)), u2), s2);
+    const float2 h = __half22float2(*reinterpret_cast<const __half2*>(q + j));
+    const f32x2 l = mul2(u, pack2(e0 >= (24u << 23) ? h.x : 0.f, e1 >= (24u << 23) ? h.y : 0.f));
+    slice3_words<true>(mul2(mul2(pack2(x[2 * j], x[2 * j + 1]), s2), k2), l, w[0][j], w[1][j], w[2][j]);
   }
 }
 
-// The same for values given as an FP32 part x and a small remainder lo
-// (already scaled by the row's scale): the leading slice comes from x alone,
-// the remainder joins the first remainder (exact up to an FP32 rounding far
-// below the last slice).
-__device__ __forceinline__ void slice8_f16x(const float* x, const float* lo, float sc, uint32_t w[NPL][4]) {
-#pragma unroll
-  for (int j = 0; j < 8; j += 2) {
-    float p0[NPL], p1[NPL];
-    slice3_planes_x(x[j] * sc, lo[j], p0);
-    slice3_planes_x(x[j + 1] * sc, lo[j + 1], p1);
-#pragma unroll
-    for (int p = 0; p < NPL; p++) {
-      const __half2 h = __floats2half2_rn(p0[p], p1[p]);
-      w[p][j >> 1] = *reinterpret_cast<const uint32_t*>(&h);
+// Walks the units of one CTA: unit -> (b, m tile, n tile, K chunk), K chunk
+// fastest, then n; Hermitian products: per batch entry the tiles n >=
+// herm_n0(m), m ascending.  Every warp steps through the units by itself, so
+// a step is additions with carries (divisions once, at the start).
+struct UnitWalk {
+  int b, mi, ni, kc;
+  int db, dm, dn, dk;   // the step in mixed-radix digits (Hermitian: dn = the step)
+  __device__ __forceinline__ UnitWalk(const Geometry& g, unsigned u, unsigned step) {
+    if (g.herm) {
+      kc = db = dm = dk = 0;
+      dn = (int)step;
+      b = (int)(u / (unsigned)g.upb);
+      int r = (int)(u - (unsigned)b * (unsigned)g.upb);
+      for (mi = 0; mi < g.mt - 1; mi++) {
+        const int cnt = g.nt - herm_n0(mi);
+        if (r < cnt) break;
+        r -= cnt;
+      }
+      ni = herm_n0(mi) + r;
+    } else {
+      split(g, u, b, mi, ni, kc);
+      split(g, step, db, dm, dn, dk);
     }
   }
-}
+  static __device__ __forceinline__ void split(const Geometry& g, unsigned u, int& b, int& m, int& n, int& k) {
+    k = (int)(u % (unsigned)g.nchunk);
+    u /= (unsigned)g.nchunk;
+    n = (int)(u % (unsigned)g.nt);
+    u /= (unsigned)g.nt;
+    m = (int)(u % (unsigned)g.mt);
+    b = (int)(u / (unsigned)g.mt);
+  }
+  __device__ __forceinline__ void next(const Geometry& g) {
+    if (g.herm) {
+      int left = dn;
+      while (left >= g.nt - ni) {
+        left -= g.nt - ni;
+        if (++mi == g.mt) {
+          mi = 0;
+          b++;
+        }
+        ni = herm_n0(mi);
+      }
+      ni += left;
+      return;
+    }
+    int c = (kc += dk) >= g.nchunk;
+    if (c) kc -= g.nchunk;
+    c = (ni += dn + c) >= g.nt;
+    if (c) ni -= g.nt;
+    c = (mi += dm + c) >= g.mt;
+    if (c) mi -= g.mt;
+    b += db + c;
+  }
+};
 
 // A warp's 32-row x 16-column staging tile into a partial-sum buffer: lane ->
 // (row, 4 columns), 8 rows x 64 B per instruction.
@@ -420,30 +467,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
   const long u_begin = AR ? g.units * blockIdx.x / gridDim.x : (long)blockIdx.x;
   const long u_end = AR ? g.units * (blockIdx.x + 1) / gridDim.x : g.units;
   const long u_step = AR ? 1 : gridDim.x;
-  // unit u -> (b, m tile, n tile, K chunk), K chunk fastest, then n
-  auto decode = [&](long u, int& b, int& mi, int& ni, int& kc) {
-    if (g.herm) {   // one chunk; per batch entry the tiles n >= herm_n0(m), m ascending
-      kc = 0;
-      b = (int)(u / g.upb);
-      long r = u - (long)b * g.upb;
-      int m = 0;
-      for (; m < g.mt - 1; m++) {
-        const long cnt = g.nt - herm_n0(m);
-        if (r < cnt) break;
-        r -= cnt;
-      }
-      mi = m;
-      ni = herm_n0(m) + (int)r;
-      return;
-    }
-    kc = (int)(u % g.nchunk);
-    long r = u / g.nchunk;
-    ni = (int)(r % g.nt);
-    r /= g.nt;
-    mi = (int)(r % g.mt);
-    b = (int)(r / g.mt);
-  };
-
+  UnitWalk uw(g, (unsigned)u_begin, (unsigned)u_step);
   // Warps 0 and 1 run their loops with all lanes (the loop state is uniform)
   // and elect one lane for each batch of instructions.  In a branch of one
   // lane the operands of a tcgen05.mma or a TMA copy are moved to the uniform
@@ -459,9 +483,8 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
       uint32_t it = 0, agen = 0, nfull = 0, nsa = 0;   // K blocks; B (or A and B) and FP32 A copies issued
       long gprev = -1;
       bool ok = true;
-      for (long u = u_begin; u < u_end && ok; u += u_step) {
-        int b, mi, ni, kc;
-        decode(u, b, mi, ni, kc);
+      for (long u = u_begin; u < u_end && ok; u += u_step, uw.next(g)) {
+        const int b = uw.b, mi = uw.mi, ni = uw.ni, kc = uw.kc;
         const int bz = b + g.b0;   // the batch coordinate in the operands' tensor maps
         if constexpr (AR) {
           const long grp = (long)b * g.mt + mi;
@@ -554,9 +577,8 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
       uint32_t it = 0, local = 0, agen = 0;
       long gprev = -1;
       bool ok = true;
-      for (long u = u_begin; u < u_end && ok; u += u_step, local++) {
-        int b, mi, ni, kc;
-        decode(u, b, mi, ni, kc);
+      for (long u = u_begin; u < u_end && ok; u += u_step, local++, uw.next(g)) {
+        const int b = uw.b, mi = uw.mi, ni = uw.ni, kc = uw.kc;
         if constexpr (AR) {
           const long grp = (long)b * g.mt + mi;
           if (grp != gprev) {
@@ -672,9 +694,8 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
     const uint32_t tdst = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + TA_COL + 8 * hf;
     uint32_t it = 0;
     bool ok = true;
-    for (long u = u_begin; u < u_end && ok; u += u_step) {
-      int b, mi, ni, kc;
-      decode(u, b, mi, ni, kc);
+    for (long u = u_begin; u < u_end && ok; u += u_step, uw.next(g)) {
+      const int b = uw.b, mi = uw.mi, ni = uw.ni, kc = uw.kc;
       const int row = mi * BM + r;
       // 2^(7 - e): the row's scale, exact
       const int erow = row < g.M ? row_exp(eA, (long)b * seA + row) : 0;
@@ -712,15 +733,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
             // unit in the last place (64B-swizzled row r of the fp16 tile)
             const uint4 q = *reinterpret_cast<const uint4*>(src + SA_HI + r * 64 + 16 * (pc ^ ((r >> 1) & 3)));
             const uint32_t qw[4] = {q.x, q.y, q.z, q.w};
-            float lo[8];
-#pragma unroll
-            for (int j = 0; j < 8; j++) {
-              const uint16_t h16 = (uint16_t)(qw[j >> 1] >> (16 * (j & 1)));
-              const int eh = (int)((__float_as_uint(x[j]) >> 23) & 0xffu);
-              // q 2^(eh - 150) (the unit in the last place of x[j]) times the row's scale
-              lo[j] = eh >= 24 ? __half2float(__ushort_as_half(h16)) * pow2f(eh - 150 + 7 - erow) : 0.f;
-            }
-            slice8_f16x(x, lo, sc, wd);
+            slice8_f16x(x, qw, sc, wd);
           } else {
             slice8_f16(x, sc, wd);
           }
@@ -747,9 +760,8 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
     const uint32_t lane_off = (uint32_t)(32 * q) << 16;
     float* stg = epi_stage + (warp - EPI_W0) * EPI_TILE;
     uint32_t local = 0;
-    for (long u = u_begin; u < u_end; u += u_step, local++) {
-      int b, mi, ni, kc;
-      decode(u, b, mi, ni, kc);
+    for (long u = u_begin; u < u_end; u += u_step, local++, uw.next(g)) {
+      const int b = uw.b, mi = uw.mi, ni = uw.ni, kc = uw.kc;
       const int row0 = mi * BM + 32 * q;          // first row of this warp's blocks
       const int cbase = ni * BN + EPI_COLS * h;   // first column of this warp
       // exponents before the accumulator is ready: this lane's row, and the
@@ -759,6 +771,8 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
         if (row0 + lane < g.M) ea = row_exp(eA, (long)b * seA + row0 + lane);
         if (lane < EPI_COLS / 2 && cbase + 2 * lane < g.Nr) ebl = eB[(long)b * seB + (cbase >> 1) + lane];
       }
+      // exponents whose scales are plain FP32 powers of two, whatever the pair (the usual case)
+      const bool plain = OUT == 0 && __all_sync(0xffffffffu, ea > -45 && ea < 60 && ebl > -45 && ebl < 60);
       const int set = CV ? 0 : local & 1;
       const uint32_t accA = tmem + lane_off + 256 * set, accBC = accA + 128;
       // CV: both halves of the warp's columns into registers as soon as each
@@ -767,7 +781,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
       float ca[CV ? 32 : 1];
       if constexpr (CV != 0) {
         static_assert(EPI_COLS == 32, "columns of an epilogue warp");
-        if (!__all_sync(0xffffffffu, mbar_wait(AFULL(0), local & 1, err, 16))) break;
+        if (!mbar_wait_uniform(AFULL(0), local & 1, err, 16)) break;
         fence_after();
         tmem_ld32(accA + EPI_COLS * h, ca);
         fence_before();
@@ -791,7 +805,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
             }
           }
         }
-        if (!__all_sync(0xffffffffu, mbar_wait(AFULL(1), local & 1, err, 16))) break;
+        if (!mbar_wait_uniform(AFULL(1), local & 1, err, 16)) break;
         fence_after();
         if constexpr (OUT == 2) {
           tmem_ld32(accBC + EPI_COLS * h, ca);
@@ -826,7 +840,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
           continue;
         }
       } else {
-        if (!mbar_wait_warp(AFULL(set), (local >> 1) & 1, err, 16)) break;
+        if (!mbar_wait_uniform(AFULL(set), (local >> 1) & 1, err, 16)) break;
         fence_after();
       }
 #pragma unroll
@@ -890,8 +904,10 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
             float y[16];
 #pragma unroll
             for (int j = 0; j < 16; j += 4) {
-              const float s0 = pow2f(ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1)) - 30);
-              const float s1 = pow2f(ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1) + 1) - 30);
+              const int e0 = ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1)) - 30;
+              const int e1 = ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1) + 1) - 30;
+              const float s0 = plain ? __int_as_float((e0 + 127) << 23) : pow2f(e0);
+              const float s1 = plain ? __int_as_float((e1 + 127) << 23) : pow2f(e1);
               // va is exact: one rounding in the add (CV: added when vb was read)
               y[j] = (CV ? va[j] : va[j] + vb[j]) * s0;
               y[j + 1] = (CV ? va[j + 1] : va[j + 1] + vb[j + 1]) * s0;
@@ -919,6 +935,15 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
           const int f = lane >> 3;
           const int col = col0 + 4 * f;
           const bool vec = (OUT == 2) ? (g.Nr % 4 == 0) : ((ldo % 4) == 0 && (sbo % 4) == 0);
+          if (OUT == 0 && vec && row0 + 32 <= g.M && col0 + 16 <= g.Nr && (!g.herm || (col0 >> 1) > row0 + 31)) {
+            // a block inside the result, above the diagonal: no element to leave out
+            float* o = (float*)out + (long)b * sbo + (long)(row0 + (lane & 7)) * ldo + col;
+#pragma unroll
+            for (int it = 0; it < 4; it++, o += 8 * ldo)
+              *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(stg + stage_off((lane & 7) + 8 * it, f));
+            __syncwarp();   // the tile is rewritten by the next block
+            continue;
+          }
 #pragma unroll
           for (int pass = 0; pass < (OUT == 2 ? 2 : 1); pass++) {
             if (pass == 1) {   // FP32 remainders of the chunk through the same tile
@@ -1239,6 +1264,7 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
     g.units = (long)batch * g.upb;
   }
   if (g.units <= 0) return cudaSuccess;
+  if (g.units >= (1L << 31)) return cudaErrorInvalidValue;   // the units are counted in 32 bits
   const bool split = g.nchunk > 1;
   if (split && (!ps0 || !pbc)) return cudaErrorInvalidValue;
   if (g.nchunk > 127) return cudaErrorInvalidValue;   // the combined leading sums stay below 2^31
