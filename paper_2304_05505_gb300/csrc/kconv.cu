@@ -36,6 +36,7 @@
 //
 #include "thc_internal.cuh"
 #include "mbarrier.cuh"
+#include "pdl.cuh"
 #include "tc_gemm.cuh"
 
 #include <cuda.h>
@@ -182,6 +183,7 @@ template <typename R>
 __global__ void kconv_kernel(const typename cplx<R>::type* __restrict__ D,
                              const typename cplx<R>::type* __restrict__ Vh,
                              typename cplx<R>::type* __restrict__ M, long npq, Twiddles tw) {
+  pdl_begin();
   typedef typename cplx<R>::type CT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CT* buf = reinterpret_cast<CT*>(smem_raw);
@@ -276,6 +278,7 @@ template <int N1, int N2, int N3>
 __global__ void __launch_bounds__(256, 2) kconv_lanes_kernel(const float2* __restrict__ D,
                                                           const float2* __restrict__ Vh, float2* __restrict__ M,
                                                           long npq, Twiddles tw) {
+  pdl_begin();
   constexpr int L = N2 * N3, EPW = 32 / N1, EPB = EPW * 8;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int slot = lane / EPW;                       // first mesh index of this lane's values
@@ -329,6 +332,7 @@ __global__ void __launch_bounds__(256, 2) kconv_pipe_kernel(const __grid_constan
                                                          float2* __restrict__ M, long npq, long nbatch,
                                                          Twiddles tw, unsigned* __restrict__ rowkey, int np,
                                                          int* err) {
+  pdl_begin();
   constexpr int L = N2 * N3, NK = N1 * L, EPW = 32 / N1, EPB = EPW * 8, LP = (L + 1) / 2;
   constexpr uint32_t BOX = NK * EPB * sizeof(float2);
   extern __shared__ __align__(128) unsigned char kc_smem[];   // [D box][Vh box][scratch][mbarrier]
@@ -508,6 +512,7 @@ __global__ void __launch_bounds__(256) kconv_tile_kernel(const __grid_constant__
                                                       const __grid_constant__ CUtensorMap mapV,
                                                       float2* __restrict__ M, long npq, long nbatch, Twiddles tw,
                                                       unsigned* __restrict__ rowkey, int np, int* err) {
+  pdl_begin();
   const int nk = tw.n[0] * tw.n[1] * tw.n[2];
   const uint32_t box_bytes = (uint32_t)nk * TILE_EPB * sizeof(float2);
   extern __shared__ __align__(128) unsigned char kt_smem[];   // [D box][Vh box][row maxima][mbarrier]
@@ -690,6 +695,7 @@ __global__ void __launch_bounds__(256, 2) kconv_herm_kernel(const __grid_constan
                                                          uint32_t* __restrict__ rowk, uint32_t* __restrict__ colk,
                                                          const int* __restrict__ tcum, int* err,
                                                          uint32_t* __restrict__ Mlo) {
+  pdl_begin();
   static_assert(!X || N1 == 2 || N1 == 4, "the extended form needs radix-2/4 meshes");
   constexpr int L = N2 * N3, NK = N1 * L, EPW = 32 / N1, EPB = EPW * 8, LP = (L + 1) / 2, KWR = N1 * LP;
   constexpr uint32_t BOX = NK * EPB * sizeof(float2);
@@ -953,6 +959,7 @@ template <int N1, int N2, int N3>
 __global__ void __launch_bounds__(128) herm_keys_to_exponents(const uint32_t* __restrict__ rowk,
                                                               const uint32_t* __restrict__ colk, int np,
                                                               int* __restrict__ e) {
+  pdl_begin();
   constexpr int L = N2 * N3, EPW = 32 / N1, LP = (L + 1) / 2, KWR = N1 * LP;
   __shared__ uint32_t part[4][32];
   const int nqb = (np + EPW - 1) / EPW, npb = (np + 7) / 8;
@@ -1000,6 +1007,7 @@ __global__ void herm_tile_prefix(int* tcum, int np, int epw) {
 // at least 2^-133 its frexp exponent (normal: biased exponent - 126;
 // subnormal: bit length of the 7 kept mantissa bits - 133), else 0.
 __global__ void rowkey_to_exponents(unsigned* v, long n) {
+  pdl_begin();
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     const unsigned k = v[i];
     const int e = k >= 0x80u ? (int)(k >> 7) - 126 : k ? (32 - __clz((int)k)) - 133 : 0;
@@ -1073,7 +1081,7 @@ template <int N1, int N2, int N3>
 cudaError_t kconv_lanes_launch(const float2* D, const float2* Vh, float2* M, long npq, cudaStream_t s) {
   constexpr int EPB = (32 / N1) * 8;
   const long blocks = (npq + EPB - 1) / EPB;
-  kconv_lanes_kernel<N1, N2, N3><<<(unsigned)blocks, 256, 0, s>>>(D, Vh, M, npq, make_twiddles(N1, N2, N3));
+  launch_pdl(kconv_lanes_kernel<N1, N2, N3>, (unsigned)blocks, 256, 0, s, D, Vh, M, npq, make_twiddles(N1, N2, N3));
   return cudaGetLastError();
 }
 
@@ -1094,7 +1102,7 @@ cudaError_t kconv_launch(const typename cplx<R>::type* D, const typename cplx<R>
   cudaError_t e = cudaFuncSetAttribute(kconv_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   const long blocks = (npq + T - 1) / T;
-  kconv_kernel<R><<<(unsigned)blocks, T, sm, s>>>(D, Vh, M, npq, make_twiddles(n1, n2, n3));
+  launch_pdl(kconv_kernel<R>, (unsigned)blocks, T, sm, s, D, Vh, M, npq, make_twiddles(n1, n2, n3));
   return cudaGetLastError();
 }
 
@@ -1124,7 +1132,7 @@ cudaError_t kconv_pipe_launch(const float2* D, const float2* Vh, float2* M, int 
   if (e != cudaSuccess) return e;
   const long nbatch = (npq + EPB - 1) / EPB;
   const unsigned grid = (unsigned)std::min<long>(nbatch, 2L * nsm);
-  kconv_pipe_kernel<N1, N2, N3><<<grid, 256, SMEM, s>>>(mapD, mapV, M, npq, nbatch, make_twiddles(N1, N2, N3),
+  launch_pdl(kconv_pipe_kernel<N1, N2, N3>, grid, 256, SMEM, s, mapD, mapV, M, npq, nbatch, make_twiddles(N1, N2, N3),
                                                          rowkey, np, err);
   return cudaGetLastError();
 }
@@ -1159,12 +1167,12 @@ cudaError_t kconv_herm_launch(const float2* D, const float2* Vh, float2* M, int 
   uint32_t* colk = keys + (long)nqb * np * KWR;
   const int* tcum = reinterpret_cast<const int*>(colk + (long)npb * np * KWR);
   const unsigned grid = (unsigned)std::min<long>(ntile, 2L * nsm);
-  kconv_herm_kernel<N1, N2, N3, X><<<grid, 256, SMEM, s>>>(mapD, mapV, M, np, ntile, make_twiddles(N1, N2, N3),
+  launch_pdl(kconv_herm_kernel<N1, N2, N3, X>, grid, 256, SMEM, s, mapD, mapV, M, np, ntile, make_twiddles(N1, N2, N3),
                                                          rowk, colk, tcum, err, Mlo);
   r = cudaGetLastError();
   if (r == cudaSuccess && conv_done) r = cudaEventRecord(conv_done, s);
   if (r != cudaSuccess) return r;
-  herm_keys_to_exponents<N1, N2, N3><<<(unsigned)std::min(np, 152 * 16), 128, 0, s>>>(rowk, colk, np, e);
+  launch_pdl(herm_keys_to_exponents<N1, N2, N3>, (unsigned)std::min(np, 152 * 16), 128, 0, s, rowk, colk, np, e);
   return cudaGetLastError();
 }
 
@@ -1228,7 +1236,7 @@ cudaError_t kconv_tile_launch(const float2* D, const float2* Vh, float2* M, int 
   const long nbatch = (npq + TILE_EPB - 1) / TILE_EPB;
   const int per_sm = sm <= 113 * 1024 ? 2 : 1;
   const unsigned grid = (unsigned)std::min<long>(nbatch, (long)per_sm * nsm);
-  kconv_tile_kernel<<<grid, 256, sm, s>>>(mapD, mapV, M, npq, nbatch, make_twiddles(n1, n2, n3), rowkey, np, err);
+  launch_pdl(kconv_tile_kernel, grid, 256, sm, s, mapD, mapV, M, npq, nbatch, make_twiddles(n1, n2, n3), rowkey, np, err);
   return cudaGetLastError();
 }
 
@@ -1250,7 +1258,7 @@ cudaError_t kconv_c_rowexp(const float2* D, const float2* Vh, float2* M, int np,
     if (r == cudaSuccess) r = kconv_tile_launch(D, Vh, M, np, n1, n2, n3, key, err, s);
     if (r == cudaSuccess && conv_done) r = cudaEventRecord(conv_done, s);
     if (r != cudaSuccess) return r;
-    rowkey_to_exponents<<<(unsigned)std::min<long>((rows + 255) / 256, 152L * 8), 256, 0, s>>>(key, rows);
+    launch_pdl(rowkey_to_exponents, (unsigned)std::min<long>((rows + 255) / 256, 152L * 8), 256, 0, s, key, rows);
     r = cudaGetLastError();
     *done = r == cudaSuccess;
     return r;
@@ -1271,7 +1279,7 @@ cudaError_t kconv_c_rowexp(const float2* D, const float2* Vh, float2* M, int np,
   else r = kconv_pipe_launch<2, 2, 2>(D, Vh, M, np, key, err, s);
   if (r == cudaSuccess && conv_done) r = cudaEventRecord(conv_done, s);
   if (r != cudaSuccess) return r;
-  rowkey_to_exponents<<<(unsigned)std::min<long>((rows + 255) / 256, 152L * 8), 256, 0, s>>>(key, rows);
+  launch_pdl(rowkey_to_exponents, (unsigned)std::min<long>((rows + 255) / 256, 152L * 8), 256, 0, s, key, rows);
   r = cudaGetLastError();
   *done = r == cudaSuccess;
   return r;

@@ -8,6 +8,9 @@
 // float-float (two-sum) pair, which is carried into FP64 before any sum across
 // threads; every sum across threads and blocks is FP64.
 #include "thc_internal.cuh"
+#include "pdl.cuh"
+
+#include <algorithm>
 
 namespace {
 
@@ -34,6 +37,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 __global__ void __launch_bounds__(RT) ex_partial_z(const double2* __restrict__ Psi,
                                                     const double2* __restrict__ Y, long n,
                                                     double* __restrict__ partial) {
+  pdl_begin();
   __shared__ double sh[RT / 32];
   double re = 0.0, im = 0.0;
   for (long i = (long)blockIdx.x * RT + threadIdx.x; i < n; i += (long)gridDim.x * RT) {
@@ -52,6 +56,7 @@ __global__ void __launch_bounds__(RT) ex_partial_z(const double2* __restrict__ P
 __global__ void __launch_bounds__(RT) ex_partial_c(const float2* __restrict__ Psi,
                                                     const float2* __restrict__ Y, long n,
                                                     double* __restrict__ partial) {
+  pdl_begin();
   __shared__ double sh[RT / 32];
   float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
   // unrolled so that the loads of several iterations are in flight together
@@ -75,6 +80,7 @@ __global__ void __launch_bounds__(RT) ex_partial_c(const float2* __restrict__ Ps
 // One block; thread t adds partials t, t + RT, ... and the block tree adds
 // the thread sums: a fixed order, so the result is reproducible.
 __global__ void __launch_bounds__(RT) ex_final(const double* __restrict__ partial, int np, int nk, double* ex) {
+  pdl_begin();
   __shared__ double sh[RT / 32];
   double re = 0.0, im = 0.0;
   for (int i = threadIdx.x; i < np; i += RT) {
@@ -124,22 +130,28 @@ unsigned grid_for(long n, int t) {
 
 }  // namespace
 
+// Blocks of a partial sum: no more than there are elements for (a small cell's
+// final sum over 1216 pairs took as long as two of its GEMMs).
+static int ex_blocks(long n, int npartial) { return (int)std::max<long>(1, std::min<long>(npartial, (n + 1023) / 1024)); }
+
 cudaError_t ex_reduce_z(const double2* Psi, const double2* Y, long n, int nk, double* partial,
                         int npartial, double* ex, cudaStream_t s) {
-  ex_partial_z<<<npartial, RT, 0, s>>>(Psi, Y, n, partial);
-  ex_final<<<1, RT, 0, s>>>(partial, npartial, nk, ex);
+  npartial = ex_blocks(n, npartial);
+  launch_pdl(ex_partial_z, npartial, RT, 0, s, Psi, Y, n, partial);
+  launch_pdl(ex_final, 1, RT, 0, s, partial, npartial, nk, ex);
   return cudaGetLastError();
 }
 
 cudaError_t ex_finalize(const double* partial, int npartial, int nk, double* ex, cudaStream_t s) {
-  ex_final<<<1, RT, 0, s>>>(partial, npartial, nk, ex);
+  launch_pdl(ex_final, 1, RT, 0, s, partial, npartial, nk, ex);
   return cudaGetLastError();
 }
 
 cudaError_t ex_reduce_c(const float2* Psi, const float2* Y, long n, int nk, double* partial,
                         int npartial, double* ex, cudaStream_t s) {
-  ex_partial_c<<<npartial, RT, 0, s>>>(Psi, Y, n, partial);
-  ex_final<<<1, RT, 0, s>>>(partial, npartial, nk, ex);
+  npartial = ex_blocks(n, npartial);
+  launch_pdl(ex_partial_c, npartial, RT, 0, s, Psi, Y, n, partial);
+  launch_pdl(ex_final, 1, RT, 0, s, partial, npartial, nk, ex);
   return cudaGetLastError();
 }
 

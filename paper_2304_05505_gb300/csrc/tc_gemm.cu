@@ -77,6 +77,7 @@
 #include "tc_gemm.cuh"
 #include "slices.cuh"
 #include "mbarrier.cuh"
+#include "pdl.cuh"
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -418,10 +419,6 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
   static_assert(2 * SA_STAGES + 2 * B_STAGES <= 48, "barrier slots 14 .. 61");
 
   __shared__ int abort_flag;
-  if (threadIdx.x == 0) abort_flag = *(volatile int*)err;
-  __syncthreads();
-  if (abort_flag) return;   // an earlier CTA gave up a wait: skip the work
-
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -457,6 +454,9 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // (barriers and TMEM are set up while the kernel before this one finishes)
+  pdl_begin();
+  if (threadIdx.x == 0) abort_flag = *(volatile int*)err;
   fence_before();
   __syncthreads();
   fence_after();
@@ -465,7 +465,8 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
   // units of this CTA: strided (CTAs running side by side share the A tile
   // through L2) or, A resident, one contiguous range
   const long u_begin = AR ? g.units * blockIdx.x / gridDim.x : (long)blockIdx.x;
-  const long u_end = AR ? g.units * (blockIdx.x + 1) / gridDim.x : g.units;
+  // (none after an earlier CTA gave up a wait)
+  const long u_end = abort_flag ? u_begin : AR ? g.units * (blockIdx.x + 1) / gridDim.x : g.units;
   const long u_step = AR ? 1 : gridDim.x;
   UnitWalk uw(g, (unsigned)u_begin, (unsigned)u_step);
   // Warps 0 and 1 run their loops with all lanes (the loop state is uniform)
@@ -1021,6 +1022,7 @@ __global__ void __launch_bounds__(256) tc_combine_kernel(const int* __restrict__
                                                          const int* __restrict__ eB, long seB, void* out, long ldo,
                                                          long sbo, const float* __restrict__ w, double* dot,
                                                          int acc) {
+  pdl_begin();
   static_assert(!DOT || (!OUT_F64 && V == 4), "the dot product of an FP32 result, four columns per thread");
   const long total = (long)batch * M * Nr;
   const long nv = total / V;
@@ -1281,7 +1283,7 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
     e = cudaFuncSetAttribute(tc_gemm_kernel<OUTK, NPK, ARK, CVK>,                                         \
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem<CVK>::BYTES);               \
     if (e != cudaSuccess) return e;                                                                       \
-    tc_gemm_kernel<OUTK, NPK, ARK, CVK><<<grid, Roles<CVK>::NT, Smem<CVK>::BYTES, s>>>(maps, g, eA, seA, eB, seB, \
+    launch_pdl(tc_gemm_kernel<OUTK, NPK, ARK, CVK>, grid, Roles<CVK>::NT, Smem<CVK>::BYTES, s, maps, g, eA, seA, eB, seB, \
                                                                            out, ldo, sbo, ps0, pbc, err); \
   }
 #define BY_OUT(NPK, ARK, CVK) \
@@ -1313,7 +1315,7 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
                    sbo == (long)M * Nr && ((uintptr_t)dot_with & 15) == 0;
   if (dot) cg = std::min<unsigned>(cg, (unsigned)dot_max);
 #define COMBINE(F64, V, D)                                                                                 \
-  tc_combine_kernel<F64, V, D><<<cg, 256, 0, s>>>(ps0, pbc, g.nchunk, batch, M, Nr, eA, seA, eB, seB, out, ldo, \
+  launch_pdl(tc_combine_kernel<F64, V, D>, cg, 256, 0, s, ps0, pbc, g.nchunk, batch, M, Nr, eA, seA, eB, seB, out, ldo, \
                                                   sbo, dot_with, dot_partial, (int)accumulate)
   if (out_f64) {
     if (v4) COMBINE(true, 4, false); else COMBINE(true, 1, false);

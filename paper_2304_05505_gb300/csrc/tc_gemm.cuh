@@ -116,3 +116,7 @@ cudaError_t embed_b(const void* src, bool src_f64, long sbs, long ldk, long ldj,
                     int batch, int K, int J, const int* e, uint16_t* planes, long plane, int ldp,
                     cudaStream_t s);
 
+// The column exponents e[b * J + j] (col_exponents_*) and the embedded planes
+// (embed_b) of B(k, j) = src[b * sbs + k * lds + j], in one kernel.
+cudaError_t col_embed(const void* src, bool src_f64, long sbs, int lds, bool conj_a, int batch, int K, int J, int* e,
+                      uint16_t* planes, long plane, int ldp, cudaStream_t s);

@@ -581,9 +581,8 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
     const int b0 = kb(h), nb = kb(h + 1) - kb(h);
     if (io) CKC(c, cudaStreamWaitEvent(s, c->cev[1 + h], 0));
     // S1  Psi = X^T C on tensor cores: B = embedded C, one exponent per orbital
-    CKC(c, col_exponents_z(C + b0 * Nn, Nn, n, nb, N, n, c->eC + b0 * n, s));
-    CKC(c, embed_b(C + b0 * Nn, true, Nn, n, 1, false, false, nb, N, n, c->eC + b0 * n,
-                   c->Bc_pl + (long)b0 * 2 * n * c->ldC, c->plBc, c->ldC, s));
+    CKC(c, col_embed(C + b0 * Nn, true, Nn, n, false, nb, N, n, c->eC + b0 * n,
+                     c->Bc_pl + (long)b0 * 2 * n * c->ldC, c->plBc, c->ldC, s));
     if (h == 0) CKC(c, record_core(c, 0, 0, s));
     // A = X^T, read from FP32 X [mu][P] and sliced (transposed) inside the GEMM
     CKC(c, tc_gemm(c->opXT, c->opBc, P, 2 * n, 2 * N, nb, c->eXT + (long)b0 * P, P, c->eC + b0 * n, n,
@@ -644,8 +643,7 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
                    2 * N, 2L * P * N, c->ps0_ao, c->pbc_ao, c->tc_err, s, core_event(c, 3, 1), 8,
                    !a_f32 ? 0 : (herm && c->Mlo) ? 3 : 1));
     CKC(c, mark(c, 4, s, false));
-    CKC(c, col_exponents_c(c->Zao, (long)P * N, N, nk, P, N, c->eZ, s));
-    CKC(c, embed_b(c->Zao, false, (long)P * N, N, 1, false, true, nk, P, N, c->eZ, c->Bz_pl, c->plAO, c->ldAO, s));
+    CKC(c, col_embed(c->Zao, false, (long)P * N, N, true, nk, P, N, c->eZ, c->Bz_pl, c->plAO, c->ldAO, s));
     CKC(c, record_core(c, 4, 0, s));
     CKC(c, tc_gemm(c->opXn, c->opBz, N, 2 * N, 2 * P, nk, c->eXn, N, c->eZ, N, Kao, true, 2 * N, 2L * N * N,
                    c->ps0_ao, c->pbc_ao, c->tc_err, s, core_event(c, 4, 1), 8, 1));
@@ -665,8 +663,7 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
   } else {
     CKC(c, slice_rows_exact(M, P, (long)nk * P, c->eM, c->M_pl, c->plM, c->ldM, s));
   }
-  CKC(c, col_exponents_c(Psi, Pn, n, nk, P, n, c->eY, s));
-  CKC(c, embed_b(Psi, false, Pn, n, 1, false, false, nk, P, n, c->eY, c->By_pl, c->plBy, c->ldM, s));
+  CKC(c, col_embed(Psi, false, Pn, n, false, nk, P, n, c->eY, c->By_pl, c->plBy, c->ldM, s));
   CKC(c, record_core(c, 3, 0, s));
   // (THC_MIXED_EXT with the Hermitian form: M's fp16 remainders join its FP32 values)
   const int m_conv = !a_f32 ? 0 : (herm && c->Mlo) ? 3 : 1;
@@ -678,8 +675,7 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
   CKC(c, mark(c, 4, s, false));
   // S4b KC = conj(X) Y on tensor cores: A = X (FP32, sliced inside the GEMM),
   // B = embedded Y (conj-A form)
-  CKC(c, col_exponents_c(Y, Pn, n, nk, P, n, c->eY, s));
-  CKC(c, embed_b(Y, false, Pn, n, 1, false, true, nk, P, n, c->eY, c->By_pl, c->plBy, c->ldM, s));
+  CKC(c, col_embed(Y, false, Pn, n, true, nk, P, n, c->eY, c->By_pl, c->plBy, c->ldM, s));
   CKC(c, record_core(c, 4, 0, s));
   // (host-buffer build: per half of the k points, its KC going out on the
   // copy stream while the next half is computed)
@@ -1012,18 +1008,18 @@ thc_status thc_launches_per_build(const thc_ctx* c, int* launches) {
   // FP64 and CUDA-core forms: S1, S2, S3, S4a, S4b, E_x partial, E_x final
   // (FP64 after a build: that build's count; a product from digits is five
   // kernels, per slab).
-  // Tensor-core form: S1 3 (exponents, embed, GEMM), S2 2 (slices with their
-  // row exponents and the embedded Psi^H, GEMM), S3 + S4a 5 (the convolution, the row
+  // Tensor-core form: S1 2 (exponents and embedding, GEMM), S2 2 (slices with their
+  // row exponents and the embedded Psi^H, GEMM), S3 + S4a 4 (the convolution, the row
   // exponents of M: in the convolution plus a conversion kernel on the
-  // 2^3 .. 4^3 meshes, else a kernel of their own; exponents of Psi, embed,
-  // GEMM), S4b 3, E_x 2; S1, S4a and S4b add a combine kernel when split
+  // 2^3 .. 4^3 meshes, else a kernel of their own; exponents of Psi and its
+  // embedding, GEMM), S4b 2, E_x 2; S1, S4a and S4b add a combine kernel when split
   // along K, and S4a's combine then forms the partial sums of E_x (E_x 1)
   // when its result rows are 16-byte strided (n_occ even).
   if (tc_form(c->precision)) {
     const int s1 = tc_partial_elems(c->nisdf, 2 * c->nocc, 2 * c->nbas, c->nk) > 0 ? 1 : 0;
     const int s4a = tc_partial_elems(c->nisdf, 2 * c->nocc, 2 * c->nisdf, c->nk) > 0 ? 1 : 0;
     const int s4b = tc_partial_elems(c->nbas, 2 * c->nocc, 2 * c->nisdf, c->nk) > 0 ? 1 : 0;
-    *launches = 3 + s1 + 2 + 1 + 4 + s4a + 3 + s4b + (s4a && c->nocc % 2 == 0 ? 1 : 2);
+    *launches = 2 + s1 + 2 + 1 + 3 + s4a + 2 + s4b + (s4a && c->nocc % 2 == 0 ? 1 : 2);
   } else {
     *launches = c->precision == THC_FP64 && c->n_launch ? c->n_launch : 7;
   }
