@@ -115,10 +115,11 @@ thc_status thc_set_kernel(thc_ctx* ctx, const double* V);
  * imaginary part of the S5 sum (a residual, zero for Hermitian V).
  * Asynchronous on the context's stream.  In the tensor-core forms a build
  * that is not being profiled runs as one CUDA graph launch: its kernels are
- * captured from the stream on the first build with these (C, KC, ex)
- * pointers and replayed on later ones (the contents of C may change between
- * builds; new pointers, thc_set_collocation or thc_set_kernel capture anew;
- * a capture the driver refuses falls back to launching the kernels). */
+ * captured from the stream on the first build after thc_set_collocation or
+ * thc_set_kernel and replayed on later ones, with any buffers (their addresses
+ * are written on the stream when they change).  A capture the driver refuses, a
+ * KC that is not 32-byte aligned, or a stream that is itself being captured
+ * gets the kernels directly. */
 thc_status thc_build(thc_ctx* ctx, const double* C, double* KC, double* ex);
 
 /* The same build from and to host memory: copies C_host in, runs the build,

@@ -79,8 +79,10 @@ __global__ void __launch_bounds__(RT) ex_partial_c(const float2* __restrict__ Ps
 
 // One block; thread t adds partials t, t + RT, ... and the block tree adds
 // the thread sums: a fixed order, so the result is reproducible.
-__global__ void __launch_bounds__(RT) ex_final(const double* __restrict__ partial, int np, int nk, double* ex) {
+__global__ void __launch_bounds__(RT) ex_final(const double* __restrict__ partial, int np, int nk, double* ex,
+                                               double* const* ex_at) {
   pdl_begin();
+  if (ex_at) ex = *ex_at;
   __shared__ double sh[RT / 32];
   double re = 0.0, im = 0.0;
   for (int i = threadIdx.x; i < np; i += RT) {
@@ -138,20 +140,20 @@ cudaError_t ex_reduce_z(const double2* Psi, const double2* Y, long n, int nk, do
                         int npartial, double* ex, cudaStream_t s) {
   npartial = ex_blocks(n, npartial);
   launch_pdl(ex_partial_z, npartial, RT, 0, s, Psi, Y, n, partial);
-  launch_pdl(ex_final, 1, RT, 0, s, partial, npartial, nk, ex);
+  launch_pdl(ex_final, 1, RT, 0, s, partial, npartial, nk, ex, nullptr);
   return cudaGetLastError();
 }
 
-cudaError_t ex_finalize(const double* partial, int npartial, int nk, double* ex, cudaStream_t s) {
-  launch_pdl(ex_final, 1, RT, 0, s, partial, npartial, nk, ex);
+cudaError_t ex_finalize(const double* partial, int npartial, int nk, double* ex, cudaStream_t s, double* const* ex_at) {
+  launch_pdl(ex_final, 1, RT, 0, s, partial, npartial, nk, ex, ex_at);
   return cudaGetLastError();
 }
 
 cudaError_t ex_reduce_c(const float2* Psi, const float2* Y, long n, int nk, double* partial,
-                        int npartial, double* ex, cudaStream_t s) {
+                        int npartial, double* ex, cudaStream_t s, double* const* ex_at) {
   npartial = ex_blocks(n, npartial);
   launch_pdl(ex_partial_c, npartial, RT, 0, s, Psi, Y, n, partial);
-  launch_pdl(ex_final, 1, RT, 0, s, partial, npartial, nk, ex);
+  launch_pdl(ex_final, 1, RT, 0, s, partial, npartial, nk, ex, ex_at);
   return cudaGetLastError();
 }
 

@@ -369,8 +369,8 @@ __device__ __forceinline__ void put_block(float* __restrict__ part, const float*
 template <int OUT, int NP, bool AR, int CV>
 __global__ void __launch_bounds__(Roles<CV>::NT, 1)
 tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restrict__ eA, long seA,
-               const int* __restrict__ eB, long seB, void* out, long ldo, long sbo, int* __restrict__ ps0,
-               float* __restrict__ pbc, int* err) {
+               const int* __restrict__ eB, long seB, void* out, void* const* out_at, long ldo, long sbo,
+               int* __restrict__ ps0, float* __restrict__ pbc, int* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   static_assert(NP == 6 || NP == 8, "slice products");
@@ -457,6 +457,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
   // (barriers and TMEM are set up while the kernel before this one finishes)
   pdl_begin();
   if (threadIdx.x == 0) abort_flag = *(volatile int*)err;
+  if (out_at) out = *out_at;
   fence_before();
   __syncthreads();
   fence_after();
@@ -1019,10 +1020,11 @@ template <bool OUT_F64, int V, bool DOT>
 __global__ void __launch_bounds__(256) tc_combine_kernel(const int* __restrict__ ps0, const float* __restrict__ pbc,
                                                          int nchunk, int batch, int M, int Nr,
                                                          const int* __restrict__ eA, long seA,
-                                                         const int* __restrict__ eB, long seB, void* out, long ldo,
-                                                         long sbo, const float* __restrict__ w, double* dot,
+                                                         const int* __restrict__ eB, long seB, void* out,
+                                                         void* const* out_at, long ldo, long sbo, const float* __restrict__ w, double* dot,
                                                          int acc) {
   pdl_begin();
+  if (out_at) out = *out_at;
   static_assert(!DOT || (!OUT_F64 && V == 4), "the dot product of an FP32 result, four columns per thread");
   const long total = (long)batch * M * Nr;
   const long nv = total / V;
@@ -1234,7 +1236,8 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
                     const int* eA, long seA, const int* eB, long seB, void* out, bool out_f64, long ldo,
                     long sbo, int* ps0, float* pbc, int* err, cudaStream_t s,
                     cudaEvent_t gemm_done, int products, int a_conv, int herm, const float* dot_with,
-                    double* dot_partial, int dot_max, int* dot_blocks, int b0, int ckb, bool accumulate) {
+                    double* dot_partial, int dot_max, int* dot_blocks, int b0, int ckb, bool accumulate,
+                    void* const* out_at) {
   if (dot_blocks) *dot_blocks = 0;
   if (b0 < 0) return cudaErrorInvalidValue;
   if (products != 6 && products != 8) return cudaErrorInvalidValue;
@@ -1284,7 +1287,7 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem<CVK>::BYTES);               \
     if (e != cudaSuccess) return e;                                                                       \
     launch_pdl(tc_gemm_kernel<OUTK, NPK, ARK, CVK>, grid, Roles<CVK>::NT, Smem<CVK>::BYTES, s, maps, g, eA, seA, eB, seB, \
-                                                                           out, ldo, sbo, ps0, pbc, err); \
+                                                                           out, out_at, ldo, sbo, ps0, pbc, err); \
   }
 #define BY_OUT(NPK, ARK, CVK) \
   { if (split) LAUNCH(2, NPK, ARK, CVK) else if (out_f64) LAUNCH(1, NPK, ARK, CVK) else LAUNCH(0, NPK, ARK, CVK) }
@@ -1315,8 +1318,8 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
                    sbo == (long)M * Nr && ((uintptr_t)dot_with & 15) == 0;
   if (dot) cg = std::min<unsigned>(cg, (unsigned)dot_max);
 #define COMBINE(F64, V, D)                                                                                 \
-  launch_pdl(tc_combine_kernel<F64, V, D>, cg, 256, 0, s, ps0, pbc, g.nchunk, batch, M, Nr, eA, seA, eB, seB, out, ldo, \
-                                                  sbo, dot_with, dot_partial, (int)accumulate)
+  launch_pdl(tc_combine_kernel<F64, V, D>, cg, 256, 0, s, ps0, pbc, g.nchunk, batch, M, Nr, eA, seA, eB, seB, out, \
+             out_at, ldo, sbo, dot_with, dot_partial, (int)accumulate)
   if (out_f64) {
     if (v4) COMBINE(true, 4, false); else COMBINE(true, 1, false);
   } else if (dot) {

@@ -46,13 +46,16 @@ cudaError_t make_plane_map(void* map_out, const void* base, int batch, int rows,
 // the caller offsets them).  ckb > 0: K blocks per chunk instead of
 // tc_chunk_blocks' choice for this shape (a sub-batch then sums in the whole
 // product's order; at most 32).  accumulate (FP64 output): the result is added
-// to what out holds.
+// to what out holds.  out_at (may be null): device memory that holds the
+// address of out when the kernels run, in place of out (which then only has
+// to share its alignment).
 cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int Kr, int batch,
                     const int* eA, long seA, const int* eB, long seB, void* out, bool out_f64, long ldo,
                     long sbo, int* ps0, float* pbc, int* err, cudaStream_t s,
                     cudaEvent_t gemm_done = nullptr, int products = 8, int a_conv = 0, int herm = 0,
                     const float* dot_with = nullptr, double* dot_partial = nullptr, int dot_max = 0,
-                    int* dot_blocks = nullptr, int b0 = 0, int ckb = 0, bool accumulate = false);
+                    int* dot_blocks = nullptr, int b0 = 0, int ckb = 0, bool accumulate = false,
+                    void* const* out_at = nullptr);
 
 // Map of an FP32 matrix [batch][rows][ld floats] (cols valid) in 32-float K
 // boxes of 128 rows with 128B swizzle (ld * 4 bytes a multiple of 16).
@@ -118,5 +121,9 @@ cudaError_t embed_b(const void* src, bool src_f64, long sbs, long ldk, long ldj,
 
 // The column exponents e[b * J + j] (col_exponents_*) and the embedded planes
 // (embed_b) of B(k, j) = src[b * sbs + k * lds + j], in one kernel.
+// src_at (may be null): device memory that holds the address of src when the
+// kernel runs, in place of src (a captured build then serves any buffers);
+// only where the columns fit shared memory (col_embed_fits).
+bool col_embed_fits(int K);
 cudaError_t col_embed(const void* src, bool src_f64, long sbs, int lds, bool conj_a, int batch, int K, int J, int* e,
-                      uint16_t* planes, long plane, int ldp, cudaStream_t s);
+                      uint16_t* planes, long plane, int ldp, cudaStream_t s, const void* const* src_at = nullptr);

@@ -133,10 +133,11 @@ __global__ void embed_kernel(const CT* __restrict__ src, long sbs, long ldk, lon
 // k, N_P = 1200, n = 60).
 constexpr int EJ = 8;
 template <typename CT>
-__global__ void __launch_bounds__(256) colembed_kernel(const CT* __restrict__ src, long sbs, int lds, bool conj_a, int K,
-                                                       int J, int* __restrict__ e, uint16_t* __restrict__ planes,
-                                                       long plane, int ldp) {
+__global__ void __launch_bounds__(256) colembed_kernel(const CT* src, const void* const* src_at, long sbs, int lds,
+                                                       bool conj_a, int K, int J, int* __restrict__ e,
+                                                       uint16_t* __restrict__ planes, long plane, int ldp) {
   pdl_begin();
+  if (src_at) src = (const CT*)*src_at;
   typedef typename AbsBits<CT>::T T;
   extern __shared__ __align__(16) unsigned char ce_smem[];
   float2* x = reinterpret_cast<float2*>(ce_smem);     // [column][K + 1]
@@ -367,11 +368,14 @@ cudaError_t embed_b(const void* src, bool src_f64, long sbs, long ldk, long ldj,
   return cudaGetLastError();
 }
 
+bool col_embed_fits(int K) { return sizeof(float2) * EJ * ((size_t)K + 1) <= 200 * 1024; }
+
 cudaError_t col_embed(const void* src, bool src_f64, long sbs, int lds, bool conj_a, int batch, int K, int J, int* e,
-                      uint16_t* planes, long plane, int ldp, cudaStream_t s) {
+                      uint16_t* planes, long plane, int ldp, cudaStream_t s, const void* const* src_at) {
   if ((long)batch * J * K == 0) return cudaSuccess;
   const size_t sm = sizeof(float2) * EJ * ((size_t)K + 1);
-  if (sm > 200 * 1024 || batch > 65535) {   // columns too long for shared memory: exponents, then planes
+  if (!col_embed_fits(K) || batch > 65535) {   // columns too long for shared memory: exponents, then planes
+    if (src_at) return cudaErrorInvalidValue;
     cudaError_t r = src_f64 ? col_exponents_z((const double2*)src, sbs, lds, batch, K, J, e, s)
                             : col_exponents_c((const float2*)src, sbs, lds, batch, K, J, e, s);
     if (r != cudaSuccess) return r;
@@ -381,11 +385,13 @@ cudaError_t col_embed(const void* src, bool src_f64, long sbs, int lds, bool con
   if (src_f64) {
     const cudaError_t r = cudaFuncSetAttribute(colembed_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (r != cudaSuccess) return r;
-    launch_pdl(colembed_kernel<double2>, grid, 256, sm, s, (const double2*)src, sbs, lds, conj_a, K, J, e, planes, plane, ldp);
+    launch_pdl(colembed_kernel<double2>, grid, 256, sm, s, (const double2*)src, src_at, sbs, lds, conj_a, K, J, e, planes,
+               plane, ldp);
   } else {
     const cudaError_t r = cudaFuncSetAttribute(colembed_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (r != cudaSuccess) return r;
-    launch_pdl(colembed_kernel<float2>, grid, 256, sm, s, (const float2*)src, sbs, lds, conj_a, K, J, e, planes, plane, ldp);
+    launch_pdl(colembed_kernel<float2>, grid, 256, sm, s, (const float2*)src, src_at, sbs, lds, conj_a, K, J, e, planes,
+               plane, ldp);
   }
   return cudaGetLastError();
 }

@@ -551,8 +551,10 @@ struct HostIO {
   double2* KC;
 };
 
+// at (may be null): device addresses of C, KC and ex, read by the kernels as
+// they run, in place of the arguments.
 static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex, double2* Kao = nullptr,
-                           const HostIO* io = nullptr) {
+                           const HostIO* io = nullptr, void** at = nullptr) {
   const int* kProducts = c->precision == THC_MIXED_EXT ? kProductsExt : ::kProducts;
   const int nk = c->nk, N = c->nbas, n = c->nocc, P = c->nisdf;
   const long PP = (long)P * P, Pn = (long)P * n, Nn = (long)N * n;
@@ -582,7 +584,7 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
     if (io) CKC(c, cudaStreamWaitEvent(s, c->cev[1 + h], 0));
     // S1  Psi = X^T C on tensor cores: B = embedded C, one exponent per orbital
     CKC(c, col_embed(C + b0 * Nn, true, Nn, n, false, nb, N, n, c->eC + b0 * n,
-                     c->Bc_pl + (long)b0 * 2 * n * c->ldC, c->plBc, c->ldC, s));
+                     c->Bc_pl + (long)b0 * 2 * n * c->ldC, c->plBc, c->ldC, s, at));
     if (h == 0) CKC(c, record_core(c, 0, 0, s));
     // A = X^T, read from FP32 X [mu][P] and sliced (transposed) inside the GEMM
     CKC(c, tc_gemm(c->opXT, c->opBc, P, 2 * n, 2 * N, nb, c->eXT + (long)b0 * P, P, c->eC + b0 * n, n,
@@ -684,7 +686,7 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
     CKC(c, tc_gemm(c->opXn, c->opBy, N, 2 * n, 2 * P, nb, c->eXn + (long)b0 * N, N, c->eY + b0 * n, n,
                    KC + b0 * Nn, true, 2 * n, 2 * Nn, c->part_s0, c->part_bc, c->tc_err, s,
                    h == nh - 1 ? core_event(c, 4, 1) : nullptr, kProducts[3], 1, 0, nullptr, nullptr, 0, nullptr,
-                   b0, tc_chunk_blocks(N, 2 * n, 2 * P, nk)));
+                   b0, tc_chunk_blocks(N, 2 * n, 2 * P, nk), false, at ? at + 1 : nullptr));
     if (io) {
       CKC(c, cudaEventRecord(c->cev[3 + h], s));
       CKC(c, cudaStreamWaitEvent(cs, c->cev[3 + h], 0));
@@ -694,9 +696,10 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
   CKC(c, mark(c, 5, s, false));
   CKC(c, record_core(c, 5, 0, s));
   if (ex_blocks > 0)
-    CKC(c, ex_finalize(c->partial, ex_blocks, nk, ex, s));
+    CKC(c, ex_finalize(c->partial, ex_blocks, nk, ex, s, at ? (double* const*)(at + 2) : nullptr));
   else
-    CKC(c, ex_reduce_c(Psi, Y, (long)nk * P * n, nk, c->partial, c->n_partial, ex, s));
+    CKC(c, ex_reduce_c(Psi, Y, (long)nk * P * n, nk, c->partial, c->n_partial, ex, s,
+                       at ? (double* const*)(at + 2) : nullptr));
   CKC(c, record_core(c, 5, 1, s));
   CKC(c, mark(c, 6, s, false));
   if (io) {   // the copies out joined to the context's stream
@@ -706,29 +709,48 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
   return THC_OK;
 }
 
-// The tensor-core build as one CUDA graph launch: its 16-odd kernels (and the
-// stage-boundary events) are captured from the stream once per (C, KC, ex)
-// triple and replayed.  If the capture fails the build runs directly.
+__global__ void set_buffers(void** at, const void* C, void* KC, void* ex) {
+  at[0] = (void*)C;
+  at[1] = KC;
+  at[2] = ex;
+}
+
+// The tensor-core build as one CUDA graph launch: its kernels are captured
+// from the stream once per collocation and kernel, and find the caller's
+// buffers through three addresses in device memory, which one small kernel
+// writes on the stream when they are others than the last build's (a capture
+// per set of buffers cost 0.2 ms, twice a small cell's build).  If the capture
+// fails the build runs directly.
 static thc_status build_tc_graph(thc_ctx* c, const double2* C, double2* KC, double* ex) {
-  if (!c->gexec || c->g_C != C || c->g_KC != KC || c->g_ex != ex) {
-    drop_graph(c);
+  // (the GEMM's stores are chosen by the alignment of KC; basis sets too long
+  // for the embedding's shared memory take their C directly)
+  // (a stream that the caller is capturing takes the kernels themselves: the
+  // addresses noted as written would otherwise only be written at a replay)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
+  if (cap != cudaStreamCaptureStatusNone || !col_embed_fits(c->nbas) || ((uintptr_t)KC & 31))
+    return build_tc(c, C, KC, ex);
+  void** at = (void**)((char*)c->flag + 16);
+  if (!c->gexec) {
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
       cudaGetLastError();
       return build_tc(c, C, KC, ex);
     }
-    const thc_status st = build_tc(c, C, KC, ex);
+    const thc_status st = build_tc(c, C, KC, ex, nullptr, nullptr, at);
     const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
     cudaGraphExec_t x = nullptr;
-    if (st == THC_OK && e == cudaSuccess && g && cudaGraphInstantiate(&x, g, 0) == cudaSuccess) {
-      c->gexec = x;
-      c->g_C = C;
-      c->g_KC = KC;
-      c->g_ex = ex;
-    }
+    if (st == THC_OK && e == cudaSuccess && g && cudaGraphInstantiate(&x, g, 0) == cudaSuccess) c->gexec = x;
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();   // a failed capture leaves no sticky error: run the build directly
     if (!c->gexec) return build_tc(c, C, KC, ex);
+  }
+  if (c->g_C != C || c->g_KC != KC || c->g_ex != ex) {
+    set_buffers<<<1, 1, 0, c->stream>>>(at, C, KC, ex);
+    CKC(c, cudaGetLastError());
+    c->g_C = C;
+    c->g_KC = KC;
+    c->g_ex = ex;
   }
   CKC(c, cudaGraphLaunch(c->gexec, c->stream));
   return THC_OK;

@@ -64,7 +64,9 @@ struct thc_ctx {
   bool oz_asked;
   int n_launch;     // kernels of the last FP64 build (0: none yet)
   // the tensor-core build replayed as a CUDA graph while not profiled: its
-  // executable graph and the caller buffers it was captured with
+  // executable graph, which finds the caller's buffers through three
+  // addresses in device memory (in the flag word's block), and the addresses
+  // last put there on the stream
   cudaGraphExec_t gexec;
   const void *g_C, *g_KC, *g_ex;
   // thc_build_host: a copy stream that moves C in and KC out in halves beside
@@ -227,9 +229,12 @@ cudaError_t ex_reduce_z(const double2* Psi, const double2* Y, long n, int nk, do
 // E_x from block partial sums of <Psi, Y> already written (2 doubles each,
 // real and imaginary part), added in a fixed order: ex[0] = -re / nk,
 // ex[1] = -im / nk.
-cudaError_t ex_finalize(const double* partial, int npartial, int nk, double* ex, cudaStream_t s);
+// ex_at (may be null): device memory that holds the address of ex when the
+// kernel runs, in place of ex.
+cudaError_t ex_finalize(const double* partial, int npartial, int nk, double* ex, cudaStream_t s,
+                        double* const* ex_at = nullptr);
 cudaError_t ex_reduce_c(const float2* Psi, const float2* Y, long n, int nk, double* partial,
-                        int npartial, double* ex, cudaStream_t s);
+                        int npartial, double* ex, cudaStream_t s, double* const* ex_at = nullptr);
 
 // Message returned by thc_last_error(NULL) for calls made without a context.
 void set_global_error(const std::string& msg);
