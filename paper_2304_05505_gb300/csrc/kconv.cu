@@ -178,11 +178,27 @@ __device__ __forceinline__ void dft3(typename cplx<R>::type* x, int T, const Twi
   dft_axis<R>(x, T, tw, 2, sign);
 }
 
+// Row-exponent key of a value pair's max(|re|, |im|): the top 16 bits of its
+// FP32 pattern (sign 0, exponent, 7 mantissa bits), which orders as the value
+// does and fixes its frexp exponent whenever the value is at least 2^-133.
+__device__ __forceinline__ uint32_t abs_bits(float2 v) {
+  return max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu);
+}
+
+// Where M goes: flat [k][npq], and/or (odd N_P) rows padded to N_P + 1 complex
+// values, [k][np][np + 1], which TMA can read.
+template <typename CT>
+struct ConvOut {
+  CT* M;    // flat, or null
+  CT* Mp;   // padded, or null
+  int np;
+};
+
 // M = IDFT(DFT(D) o Vh), one element per thread, values in shared memory.
 template <typename R>
 __global__ void kconv_kernel(const typename cplx<R>::type* __restrict__ D,
                              const typename cplx<R>::type* __restrict__ Vh,
-                             typename cplx<R>::type* __restrict__ M, long npq, Twiddles tw) {
+                             ConvOut<typename cplx<R>::type> out, long npq, Twiddles tw) {
   pdl_begin();
   typedef typename cplx<R>::type CT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -202,8 +218,12 @@ __global__ void kconv_kernel(const typename cplx<R>::type* __restrict__ D,
     x[(long)a * T] = cmul(x[(long)a * T], v);
   }
   dft3<R>(x, T, tw, +1);
-  if (ok)
-    for (int k = 0; k < nk; k++) M[(long)k * npq + e] = x[(long)k * T];
+  if (out.M && ok)
+    for (int k = 0; k < nk; k++) out.M[(long)k * npq + e] = x[(long)k * T];
+  if (out.Mp && ok) {
+    const long pl = npq + out.np, o = e + e / out.np;
+    for (int k = 0; k < nk; k++) out.Mp[(long)k * pl + o] = x[(long)k * T];
+  }
 }
 
 // Lane-split FP32 form for the meshes 2^3, 3^3 and 4^3 (compile-time N1, N2,
@@ -276,7 +296,7 @@ __device__ __forceinline__ void lanes_convolve(float2* x, const float2* vh, cons
 
 template <int N1, int N2, int N3>
 __global__ void __launch_bounds__(256, 2) kconv_lanes_kernel(const float2* __restrict__ D,
-                                                          const float2* __restrict__ Vh, float2* __restrict__ M,
+                                                          const float2* __restrict__ Vh, ConvOut<float2> out,
                                                           long npq, Twiddles tw) {
   pdl_begin();
   constexpr int L = N2 * N3, EPW = 32 / N1, EPB = EPW * 8;
@@ -293,17 +313,16 @@ __global__ void __launch_bounds__(256, 2) kconv_lanes_kernel(const float2* __res
 #pragma unroll
   for (int j = 0; j < L; j++) vh[j] = ok ? __ldcs(Vh + off + (long)j * npq) : make_float2(0.f, 0.f);
   lanes_convolve<N1, N2, N3>(x, vh, tw, slot, el);
-  if (ok) {
+  if (out.M && ok) {
 #pragma unroll
-    for (int j = 0; j < L; j++) M[off + (long)j * npq] = x[j];
+    for (int j = 0; j < L; j++) out.M[off + (long)j * npq] = x[j];
   }
-}
-
-// Row-exponent key of a value pair's max(|re|, |im|): the top 16 bits of its
-// FP32 pattern (sign 0, exponent, 7 mantissa bits), which orders as the value
-// does and fixes its frexp exponent whenever the value is at least 2^-133.
-__device__ __forceinline__ uint32_t abs_bits(float2 v) {
-  return max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu);
+  if (out.Mp && ok) {
+    const long pl = npq + out.np;
+    float2* d = out.Mp + (long)slot * L * pl + e + e / out.np;
+#pragma unroll
+    for (int j = 0; j < L; j++) d[(long)j * pl] = x[j];
+  }
 }
 
 // Persistent, TMA-fed form of the lane-split convolution (N_P^2 even).  A
@@ -1015,6 +1034,14 @@ __global__ void rowkey_to_exponents(unsigned* v, long n) {
   }
 }
 
+// complex128 copy of rows padded to np + 1 values
+__global__ void unpad_kernel(const float2* __restrict__ Mp, double2* __restrict__ out, int np, long n) {
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+    const float2 v = Mp[i + i / np];
+    out[i] = make_double2((double)v.x, (double)v.y);
+  }
+}
+
 // Vh[a] = (1/N_k) sum_q w^{+a.q} V[q], FP64; stored FP64 and/or FP32.
 __global__ void prepare_kernel(const double2* __restrict__ V, double2* __restrict__ Vh64,
                                float2* __restrict__ Vh32, long npq, Twiddles tw) {
@@ -1078,31 +1105,32 @@ int pick_threads(int nk, size_t elem) {
 }
 
 template <int N1, int N2, int N3>
-cudaError_t kconv_lanes_launch(const float2* D, const float2* Vh, float2* M, long npq, cudaStream_t s) {
+cudaError_t kconv_lanes_launch(const float2* D, const float2* Vh, const ConvOut<float2>& out, long npq, cudaStream_t s) {
   constexpr int EPB = (32 / N1) * 8;
   const long blocks = (npq + EPB - 1) / EPB;
-  launch_pdl(kconv_lanes_kernel<N1, N2, N3>, (unsigned)blocks, 256, 0, s, D, Vh, M, npq, make_twiddles(N1, N2, N3));
+  launch_pdl(kconv_lanes_kernel<N1, N2, N3>, (unsigned)blocks, 256, 0, s, D, Vh, out, npq, make_twiddles(N1, N2, N3));
   return cudaGetLastError();
 }
 
 template <typename R>
 cudaError_t kconv_launch(const typename cplx<R>::type* D, const typename cplx<R>::type* Vh,
-                         typename cplx<R>::type* M, long npq, int n1, int n2, int n3, cudaStream_t s) {
-  if constexpr (sizeof(R) == sizeof(float)) {
-    if (n1 == n2 && n2 == n3) {
-      if (n1 == 4) return kconv_lanes_launch<4, 4, 4>(D, Vh, M, npq, s);
-      if (n1 == 3) return kconv_lanes_launch<3, 3, 3>(D, Vh, M, npq, s);
-      if (n1 == 2) return kconv_lanes_launch<2, 2, 2>(D, Vh, M, npq, s);
-    }
-  }
+                         const ConvOut<typename cplx<R>::type>& out, long npq, int n1, int n2, int n3,
+                         cudaStream_t s) {
   const int nk = n1 * n2 * n3;
   const size_t el = sizeof(typename cplx<R>::type);
+  if constexpr (sizeof(R) == sizeof(float)) {
+    if (n1 == n2 && n2 == n3) {
+      if (n1 == 4) return kconv_lanes_launch<4, 4, 4>(D, Vh, out, npq, s);
+      if (n1 == 3) return kconv_lanes_launch<3, 3, 3>(D, Vh, out, npq, s);
+      if (n1 == 2) return kconv_lanes_launch<2, 2, 2>(D, Vh, out, npq, s);
+    }
+  }
   const int T = pick_threads(nk, el);
   const size_t sm = (size_t)T * nk * el;
   cudaError_t e = cudaFuncSetAttribute(kconv_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   const long blocks = (npq + T - 1) / T;
-  launch_pdl(kconv_kernel<R>, (unsigned)blocks, T, sm, s, D, Vh, M, npq, make_twiddles(n1, n2, n3));
+  launch_pdl(kconv_kernel<R>, (unsigned)blocks, T, sm, s, D, Vh, out, npq, make_twiddles(n1, n2, n3));
   return cudaGetLastError();
 }
 
@@ -1293,12 +1321,22 @@ cudaError_t mlo_combine_c2z(const float2* M, const uint32_t* Mlo, double2* out, 
 cudaError_t kconv_z(const double2* D, const double2* Vh, double2* M, long npq, int n1, int n2,
                     int n3, cudaStream_t s) {
   if (kconv_fix_applies(n1, n2, n3)) return kconv_fix_z(D, Vh, M, npq, n1, n2, n3, s);
-  return kconv_launch<double>(D, Vh, M, npq, n1, n2, n3, s);
+  return kconv_launch<double>(D, Vh, ConvOut<double2>{M, nullptr, 0}, npq, n1, n2, n3, s);
 }
 
 cudaError_t kconv_c(const float2* D, const float2* Vh, float2* M, long npq, int n1, int n2,
                     int n3, cudaStream_t s) {
-  return kconv_launch<float>(D, Vh, M, npq, n1, n2, n3, s);
+  return kconv_launch<float>(D, Vh, ConvOut<float2>{M, nullptr, 0}, npq, n1, n2, n3, s);
+}
+
+cudaError_t kconv_c_padded(const float2* D, const float2* Vh, float2* M, float2* Mp, int np, int n1, int n2, int n3,
+                           cudaStream_t s) {
+  return kconv_launch<float>(D, Vh, ConvOut<float2>{M, Mp, np}, (long)np * np, n1, n2, n3, s);
+}
+
+cudaError_t unpad_c2z(const float2* Mp, double2* out, int np, long rows, cudaStream_t s) {
+  unpad_kernel<<<(unsigned)std::min<long>((rows * np + 255) / 256, 152L * 16), 256, 0, s>>>(Mp, out, np, rows * np);
+  return cudaGetLastError();
 }
 
 cudaError_t prepare_kernel_z(const double2* V, double2* Vh64, float2* Vh32, long npq, int n1,

@@ -53,7 +53,8 @@ struct Sizes {
   int ldX;
   long x32;
   int ldC, ldM, ldPs;
-  long plPs, plBc, plBd, plBy, plM;
+  long plPs, plBc, plBd, plBy;
+  long mpad;  // bytes of M's padded rows (odd N_P)
   long nexp;  // exponents: eXn + eXT + ePsi + eC + eY + eM
   long npart; // split-K partial elements (max over the tensor-core GEMMs)
   long hkey;  // key words of the Hermitian convolution (0 where it does not apply)
@@ -79,7 +80,10 @@ Sizes sizes_of(const thc_dims* d, int precision) {
   s.plBc = s.nk * 2 * d->nocc * s.ldC;
   s.plBd = s.nk * 2L * d->nisdf * s.ldPs;
   s.plBy = s.nk * 2 * d->nocc * (long)s.ldM;
-  s.plM = (d->nisdf % 2) ? s.nk * d->nisdf * (long)s.ldM : 0;   // M's slices only for odd N_P
+  // odd N_P: M in rows of N_P + 1 complex values, 8 (N_P + 1) bytes each.  The
+  // 6 ldM >= 8 (N_P + 1) bytes a row that are set aside are the size that
+  // thc_memory_bytes states for odd N_P.
+  s.mpad = (d->nisdf % 2) ? 6 * s.nk * d->nisdf * (long)s.ldM : 0;
   s.nexp = s.nk * (d->nbas + 3L * d->nisdf + 2L * d->nocc);
   s.npart = std::max({tc_partial_elems(d->nisdf, 2 * d->nocc, 2 * d->nbas, (int)s.nk),
                       tc_partial_elems(d->nisdf, 2 * d->nisdf, 2 * d->nocc, (int)s.nk),
@@ -114,7 +118,7 @@ size_t memory_bytes(const thc_dims* d, int precision) {
   if (tc_form(precision)) {
     b += sizeof(uint32_t) * s.mlo;                                           // remainders of M (THC_MIXED_EXT)
     b += s.x32 * sizeof(float2);                                             // X in FP32
-    b += 3 * 2 * (s.plPs + s.plBc + s.plBd + s.plBy + s.plM);               // fp16 slices
+    b += 3 * 2 * (s.plPs + s.plBc + s.plBd + s.plBy) + s.mpad;               // fp16 slices, M's padded rows
     b += sizeof(int) * s.nexp + 64;                                         // exponents, error word
     b += (sizeof(int) + sizeof(float)) * s.npart;                           // split-K partial sums
     b += sizeof(uint32_t) * s.hkey;                                          // Hermitian convolution keys
@@ -130,7 +134,7 @@ void free_all(thc_ctx* c) {
   void* ptrs[] = {c->X64, c->Vh64, c->X32, c->Vh32, c->Psi, c->D, c->M, c->Y,
                   c->Cdev, c->KCdev, c->exdev, c->partial, c->flag,
                   c->PsiA_pl, c->Bc_pl, c->Bd_pl, c->By_pl, c->ex_pl, c->tc_err, c->part_s0,
-                  c->part_bc, c->M_pl, c->hkeys, c->Zao, c->Wao, c->BxT_pl, c->Bz_pl, c->eZ, c->ps0_ao,
+                  c->part_bc, c->Mp, c->hkeys, c->Zao, c->Wao, c->BxT_pl, c->Bz_pl, c->eZ, c->ps0_ao,
                   c->pbc_ao, c->Mlo};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -219,7 +223,7 @@ thc_status thc_create(thc_ctx** out, const thc_dims* d, int precision, void* str
     W(&c->M, s.v * s.el);
     if (s.mlo) W((void**)&c->Mlo, sizeof(uint32_t) * s.mlo);
     W((void**)&c->X32, s.x32 * sizeof(float2));
-    if (s.plM) W((void**)&c->M_pl, 3 * 2 * s.plM);
+    if (s.mpad) W((void**)&c->Mp, s.mpad);
     W((void**)&c->PsiA_pl, 3 * 2 * s.plPs);
     W((void**)&c->Bc_pl, 3 * 2 * s.plBc);
     W((void**)&c->Bd_pl, 3 * 2 * s.plBd);
@@ -259,7 +263,7 @@ thc_status thc_create(thc_ctx** out, const thc_dims* d, int precision, void* str
   if (tc_form(precision)) {
     c->ldX = s.ldX; c->ldC = s.ldC; c->ldM = s.ldM; c->ldPs = s.ldPs;
     c->plPs = s.plPs;
-    c->plBc = s.plBc; c->plBd = s.plBd; c->plBy = s.plBy; c->plM = s.plM;
+    c->plBc = s.plBc; c->plBd = s.plBd; c->plBy = s.plBy;
     const int nk = (int)s.nk, N = d->nbas, n = d->nocc, P = d->nisdf;
     c->eXn = c->ex_pl;
     c->eXT = c->eXn + (long)nk * N;
@@ -287,11 +291,9 @@ thc_status thc_create(thc_ctx** out, const thc_dims* d, int precision, void* str
           return e == cudaErrorNotSupported ? THC_ERR_UNSUPPORTED : THC_ERR_CUDA;
         }
       }
-    if (s.plM)
-      for (int p = 0; p < 3 && e == cudaSuccess; p++)
-        e = make_plane_map(c->opM.map[p], c->M_pl + p * s.plM, nk, P, 2 * P, s.ldM);
-    else
-      e = make_f32_map(c->opMf.map[0], c->M, nk, P, 2 * P, 2 * P);
+    e = e != cudaSuccess ? e
+        : c->Mp          ? make_f32_map(c->opMf.map[0], c->Mp, nk, P, 2 * P, 2 * (P + 1))
+                         : make_f32_map(c->opMf.map[0], c->M, nk, P, 2 * P, 2 * P);
     if (e == cudaSuccess && c->Mlo) e = make_plane_map(c->opMf.map[1], c->Mlo, nk, P, 2 * P, 2 * P);
     if (e == cudaSuccess && c->hkeys) {
       e = kconv_herm_prepare(c->hkeys, P, d->n1, d->n2, d->n3, c->stream);
@@ -601,8 +603,7 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
   // D is Hermitian, so only the tiles that reach the diagonal are multiplied
   // (Hermitian V: M^k is Hermitian too, and S3 reads D on and above the
   // diagonal only, so S2 leaves the part below it unwritten)
-  const bool a_f32 = c->plM == 0;
-  const bool herm = c->herm_v && c->hkeys && a_f32;
+  const bool herm = c->herm_v && c->hkeys;   // (no keys for odd N_P)
   // (THC-AO-K reads all of D for its energy, so D is written whole there)
   const bool upper = herm && !Kao;
   CKC(c, tc_gemm(c->opPs, c->opBd, P, 2 * P, 2 * n, nk, c->ePsi, P, c->ePsi, P, D, false, 2 * P, 2 * PP,
@@ -614,36 +615,36 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
   // (2^3, 3^3 and 4^3 meshes: the convolution also finds the exact row
   // exponents of M that S4a slices it with)
   bool have_eM = false;
+  // the rows of M as the GEMM reads them (the pad of odd N_P is zero from thc_create on)
+  const float2* Mr = c->Mp ? c->Mp : M;
+  const int ldMr = P + (c->Mp != nullptr);
   if (herm) {
     CKC(c, kconv_c_herm(D, c->Vh32, M, P, c->n1, c->n2, c->n3, c->hkeys, c->eM, c->tc_err, core_event(c, 2, 0),
                         core_event(c, 2, 1), s, c->Mlo));
     have_eM = true;
-  } else if (a_f32) {
+  } else if (!c->Mp) {
     CKC(c, kconv_c_rowexp(D, c->Vh32, M, P, c->n1, c->n2, c->n3, c->eM, &have_eM, c->tc_err,
                           core_event(c, 2, 0), core_event(c, 2, 1), s));
   } else {
+    // odd N_P: padded rows, which S4a's GEMM reads as it reads M for even N_P
     CKC(c, record_core(c, 2, 0, s));
-    CKC(c, kconv_c(D, c->Vh32, M, PP, c->n1, c->n2, c->n3, s));
+    CKC(c, kconv_c_padded(D, c->Vh32, Kao ? M : nullptr, c->Mp, P, c->n1, c->n2, c->n3, s));
     CKC(c, record_core(c, 2, 1, s));
   }
   CKC(c, mark(c, 3, s, false));
   if (Kao) {
     // THC-AO-K: Z = M X^T (A = M as in S4a; B = the embedded X^T, made once
     // per collocation), then K = conj(X) Z (A = X as in S4b; B = embedded Z)
-    if (a_f32) {
-      if (!have_eM) CKC(c, row_exponents_rows(M, P, (long)nk * P, c->eM, s));
-    } else {
-      CKC(c, slice_rows_exact(M, P, (long)nk * P, c->eM, c->M_pl, c->plM, c->ldM, s));
-    }
+    if (!have_eM) CKC(c, row_exponents_rows(Mr, ldMr, (long)nk * P, c->eM, s));
     if (!c->bxt_valid) {
       CKC(c, embed_b(c->X32, false, (long)N * c->ldX, 1, c->ldX, false, false, nk, P, N, c->eXn, c->BxT_pl, c->plAO,
                      c->ldAO, s));
       c->bxt_valid = true;
     }
     CKC(c, record_core(c, 3, 0, s));
-    CKC(c, tc_gemm(a_f32 ? c->opMf : c->opM, c->opBxT, P, 2 * N, 2 * P, nk, c->eM, P, c->eXn, N, c->Zao, false,
+    CKC(c, tc_gemm(c->opMf, c->opBxT, P, 2 * N, 2 * P, nk, c->eM, P, c->eXn, N, c->Zao, false,
                    2 * N, 2L * P * N, c->ps0_ao, c->pbc_ao, c->tc_err, s, core_event(c, 3, 1), 8,
-                   !a_f32 ? 0 : (herm && c->Mlo) ? 3 : 1));
+                   herm && c->Mlo ? 3 : 1));
     CKC(c, mark(c, 4, s, false));
     CKC(c, col_embed(c->Zao, false, (long)P * N, N, true, nk, P, N, c->eZ, c->Bz_pl, c->plAO, c->ldAO, s));
     CKC(c, record_core(c, 4, 0, s));
@@ -659,19 +660,14 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
   // S4a Y = M Psi on tensor cores: A = M in FP32, cut into its slices inside
   // the GEMM with the exact row exponents of M; B = embedded Psi with one
   // exponent per orbital
-  // (odd N_P: M's slices go through HBM, written by the warp-per-row kernel)
-  if (a_f32) {
-    if (!have_eM) CKC(c, row_exponents_rows(M, P, (long)nk * P, c->eM, s));
-  } else {
-    CKC(c, slice_rows_exact(M, P, (long)nk * P, c->eM, c->M_pl, c->plM, c->ldM, s));
-  }
+  if (!have_eM) CKC(c, row_exponents_rows(Mr, ldMr, (long)nk * P, c->eM, s));
   CKC(c, col_embed(Psi, false, Pn, n, false, nk, P, n, c->eY, c->By_pl, c->plBy, c->ldM, s));
   CKC(c, record_core(c, 3, 0, s));
   // (THC_MIXED_EXT with the Hermitian form: M's fp16 remainders join its FP32 values)
-  const int m_conv = !a_f32 ? 0 : (herm && c->Mlo) ? 3 : 1;
+  const int m_conv = herm && c->Mlo ? 3 : 1;
   // (the split-K combine that writes Y also forms the block sums of <Psi, Y> for S5)
   int ex_blocks = 0;
-  CKC(c, tc_gemm(a_f32 ? c->opMf : c->opM, c->opBy, P, 2 * n, 2 * P, nk, c->eM, P, c->eY, n, Y, false, 2 * n,
+  CKC(c, tc_gemm(c->opMf, c->opBy, P, 2 * n, 2 * P, nk, c->eM, P, c->eY, n, Y, false, 2 * n,
                  2 * Pn, c->part_s0, c->part_bc, c->tc_err, s, core_event(c, 3, 1), kProducts[2], m_conv, 0,
                  (const float*)Psi, c->partial, c->n_partial, &ex_blocks));
   CKC(c, mark(c, 4, s, false));
@@ -950,6 +946,8 @@ thc_status thc_get_intermediate(thc_ctx* c, int which, double* out) {
   void* src = which == 0 ? c->Psi : which == 1 ? c->D : which == 2 ? c->M : c->Y;
   if (which == 2 && c->Mlo && c->m_ext)
     CKC(c, mlo_combine_c2z((const float2*)src, c->Mlo, (double2*)out, n, c->stream));
+  else if (which == 2 && c->Mp)
+    CKC(c, unpad_c2z(c->Mp, (double2*)out, c->nisdf, (long)c->nk * c->nisdf, c->stream));
   else if (which == 1 && tc_form(c->precision) && c->d_upper)
     CKC(c, hermitian_fill_c2z((const float2*)src, (double2*)out, c->nisdf, c->nk, c->stream));
   else if (c->precision == THC_FP64)
@@ -1021,7 +1019,7 @@ thc_status thc_profile_kernels(const thc_ctx* c, float core_ms[6]) {
 thc_status thc_hermitian_kernel(const thc_ctx* c, int* hermitian) {
   if (!c || !hermitian) return THC_ERR_ARG;
   if (!c->have_v) return THC_ERR_STATE;
-  *hermitian = (tc_form(c->precision) && c->herm_v && c->hkeys && c->plM == 0) ? 1 : 0;
+  *hermitian = (tc_form(c->precision) && c->herm_v && c->hkeys) ? 1 : 0;
   return THC_OK;
 }
 

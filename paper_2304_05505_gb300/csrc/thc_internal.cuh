@@ -107,17 +107,18 @@ struct thc_ctx {
   uint16_t* By_pl;    // [nk][2 nocc][ldM]   embedded Psi, B of S4a, then embedded Y, B of S4b
                       //                     (column exponents of Psi, then of Y, in eY [nk][nocc])
                       // M (FP32 workspace) is A of S4a, sliced inside the GEMM   eM [nk][nisdf]
-  uint16_t* M_pl;     // [nk][nisdf][ldM] M's slices, only for odd nisdf (FP32 rows of 8 nisdf
-                      // bytes are not 16-byte strided, which the FP32 tensor map needs)
+  float2* Mp;         // [nk][nisdf][nisdf + 1] M in rows padded to an even length, only for odd
+                      // nisdf (FP32 rows of 8 nisdf bytes are not 16-byte strided, which the
+                      // FP32 tensor map needs); M itself is then written only where the energy
+                      // of thc_build_K reads it
   int* ex_pl;         // eXn | eXT | ePsi | eC | eY | eM
   int* part_s0;       // split-K partial sums of the tensor-core GEMMs (exact leading class)
   float* part_bc;     // and their FP32 remainders
   int *eXn, *eXT, *ePsi, *eC, *eY, *eM;
-  long plPs, plBc, plBd, plBy, plM;
+  long plPs, plBc, plBd, plBy;
   int ldC, ldM, ldPs;
   TcOperand opXT, opPs, opXn, opBc, opBd, opBy;   // opXT, opXn: FP32 maps of X32
-  TcOperand opMf;     // map[0]: FP32 map of M (A of S4a, converted in the GEMM), even nisdf
-  TcOperand opM;      // M's slices, odd nisdf
+  TcOperand opMf;     // map[0]: FP32 map of M, or of Mp (A of S4a, converted in the GEMM)
   // THC-AO-K (thc_build_K), allocated by its first call: Z = M X^T and, for
   // the tensor-core form, the embedded planes of X^T (static) and of Z, the
   // column exponents of Z and split-K partials of the two products; for the
@@ -179,6 +180,13 @@ cudaError_t kconv_z(const double2* D, const double2* Vh, double2* M, long npq, i
                     int n3, cudaStream_t s);
 cudaError_t kconv_c(const float2* D, const float2* Vh, float2* M, long npq, int n1, int n2,
                     int n3, cudaStream_t s);
+// As kconv_c with npq = np^2 for odd np: M goes to rows padded to np + 1
+// values, Mp[k][p][np + 1] (16-byte strided, so TMA reads them; the last value
+// of a row is not written), and to M as well where that is not null.
+cudaError_t kconv_c_padded(const float2* D, const float2* Vh, float2* M, float2* Mp, int np, int n1, int n2, int n3,
+                           cudaStream_t s);
+// complex128 copy out[rows][np] of Mp[rows][np + 1].
+cudaError_t unpad_c2z(const float2* Mp, double2* out, int np, long rows, cudaStream_t s);
 // As kconv_c with npq = np^2.  On the 2^3, 3^3 and 4^3 meshes with npq even
 // (and err non-null) it runs the TMA-fed convolution, which also writes the
 // row exponents of M: e[k * np + p] = the smallest e with
