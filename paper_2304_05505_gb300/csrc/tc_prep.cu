@@ -131,7 +131,7 @@ __global__ void embed_kernel(const CT* __restrict__ src, long sbs, long ldk, lon
 // and writes the planes along K.  The two kernels it replaces read the columns
 // one value per 32-byte sector the second time (0.040 ms for Psi at 4 x 4 x 4
 // k, N_P = 1200, n = 60).
-constexpr int EJ = 8;
+constexpr int EJ = 4;
 template <typename CT>
 __global__ void __launch_bounds__(256) colembed_kernel(const CT* src, const void* const* src_at, long sbs, int lds,
                                                        bool conj_a, int K, int J, int* __restrict__ e,
@@ -141,48 +141,67 @@ __global__ void __launch_bounds__(256) colembed_kernel(const CT* src, const void
   typedef typename AbsBits<CT>::T T;
   extern __shared__ __align__(16) unsigned char ce_smem[];
   float2* x = reinterpret_cast<float2*>(ce_smem);     // [column][K + 1]
-  __shared__ T red[32][EJ + 1];
+  __shared__ T red[8][EJ + 1];
   __shared__ int se[EJ];
   const int b = blockIdx.y, j0 = blockIdx.x * EJ, KP = K + 1;
   const int c = threadIdx.x & (EJ - 1), r = threadIdx.x / EJ;
   const CT* p = src + (long)b * sbs + j0 + c;
   T m = 0;
   if (j0 + c < J) {
-#pragma unroll 4
+#pragma unroll 8
     for (int k = r; k < K; k += 256 / EJ) {
       const CT v = p[(long)k * lds];
       m = max(m, AbsBits<CT>::of(v));
       x[c * KP + k] = make_float2((float)v.x, (float)v.y);
     }
   }
-  red[r][c] = m;
+  // maxima over the lanes of a warp that hold the same column, then over the warps
+#pragma unroll
+  for (int o = EJ; o < 32; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) < EJ) red[threadIdx.x >> 5][c] = m;
   __syncthreads();
   if (threadIdx.x < EJ) {
-    for (int i = 1; i < 256 / EJ; i++) m = max(m, red[i][threadIdx.x]);
+#pragma unroll
+    for (int i = 0; i < 8; i++) m = max(m, red[i][threadIdx.x]);
     const int ex = row_exponent(AbsBits<CT>::value(m));
     se[threadIdx.x] = ex;
     if (j0 + (int)threadIdx.x < J) e[(long)b * J + j0 + threadIdx.x] = ex;
   }
   __syncthreads();
+  // 64 threads per column, two values of K (8 bytes of each plane row) per step
+  const int cc = threadIdx.x / (256 / EJ);
+  if (j0 + cc >= J) return;
   const f32x2 k2 = pack2(256.f, 256.f);
-  for (int cc = 0; cc < EJ && j0 + cc < J; cc++) {
-    const int sh = 7 - se[cc];
-    const bool plain = sh >= -126 && sh <= 127;
-    const float sc = plain ? __int_as_float((sh + 127) << 23) : 1.f;
-    const f32x2 s2 = pack2(sc, sc);
-    uint16_t* o = planes + ((long)b * 2 * J + 2L * (j0 + cc)) * ldp;
-    for (int k = threadIdx.x; k < K; k += 256) {
-      float2 v = x[cc * KP + k];
-      if (!plain) v = make_float2(ldexpf(v.x, sh), ldexpf(v.y, sh));
-      uint32_t w[3];
-      slice3_words<false>(mul2(mul2(pack2(v.x, v.y), s2), k2), 0, w[0], w[1], w[2]);
+  const int sh = 7 - se[cc];
+  const bool plain = sh >= -126 && sh <= 127;
+  const float sc = plain ? __int_as_float((sh + 127) << 23) : 1.f;
+  const f32x2 s2 = pack2(sc, sc);
+  uint16_t* o = planes + ((long)b * 2 * J + 2L * (j0 + cc)) * ldp;
+  const float2* xc = x + cc * KP;
+#pragma unroll 2
+  for (int k = 2 * (threadIdx.x & (256 / EJ - 1)); k < K; k += 2 * (256 / EJ)) {
+    const bool two = k + 1 < K;
+    float2 v0 = xc[k], v1 = two ? xc[k + 1] : make_float2(0.f, 0.f);
+    if (!plain) {
+      v0 = make_float2(ldexpf(v0.x, sh), ldexpf(v0.y, sh));
+      v1 = make_float2(ldexpf(v1.x, sh), ldexpf(v1.y, sh));
+    }
+    uint32_t w0[3], w1[3];
+    slice3_words<false>(mul2(mul2(pack2(v0.x, v0.y), s2), k2), 0, w0[0], w0[1], w0[2]);
+    slice3_words<false>(mul2(mul2(pack2(v1.x, v1.y), s2), k2), 0, w1[0], w1[1], w1[2]);
+    // [[re, -im], [im, re]], or for conj(A) [[re, im], [im, -re]]
+    const uint32_t neg0 = conj_a ? 0u : 0x80000000u, neg1 = conj_a ? 0x80000000u : 0u;
 #pragma unroll
-      for (int q = 0; q < 3; q++) {
-        const uint32_t t = __byte_perm(w[q], 0, 0x1032);   // (im, re)
-        uint16_t* d = o + q * plane + 2 * k;
-        // [[re, -im], [im, re]], or for conj(A) [[re, im], [im, -re]]
-        *reinterpret_cast<uint32_t*>(d) = conj_a ? w[q] : w[q] ^ 0x80000000u;
-        *reinterpret_cast<uint32_t*>(d + ldp) = conj_a ? t ^ 0x80000000u : t;
+    for (int q = 0; q < 3; q++) {
+      uint16_t* d = o + q * plane + 2 * k;
+      const uint2 a = make_uint2(w0[q] ^ neg0, w1[q] ^ neg0);
+      const uint2 t = make_uint2(__byte_perm(w0[q], 0, 0x1032) ^ neg1, __byte_perm(w1[q], 0, 0x1032) ^ neg1);
+      if (two) {
+        *reinterpret_cast<uint2*>(d) = a;
+        *reinterpret_cast<uint2*>(d + ldp) = t;
+      } else {
+        *reinterpret_cast<uint32_t*>(d) = a.x;
+        *reinterpret_cast<uint32_t*>(d + ldp) = t.x;
       }
     }
   }
