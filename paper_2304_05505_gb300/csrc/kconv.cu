@@ -973,35 +973,44 @@ __global__ void __launch_bounds__(256, 2) kconv_herm_kernel(const __grid_constan
 // e[k * np + P] from the keys of the tiles that hold row P (rowk[P][qb], qb
 // from the first tile of row band P / 8 that reaches the diagonal) and of
 // those whose mirrored part lands in row P (colk[P][pb], the tiles of column
-// band P / EPW): one block of four warps per row, lanes over the key words.
+// band P / EPW): one block per row.  Both are one run of words, KWR to a tile,
+// which the block reads flat, a thread always at the same word of a tile and
+// eight loads in flight (the keys of 4 x 4 x 4 k, N_P = 1200 are 23 MB; with a
+// warp to a tile and two loads in flight they took 21.9 us, 13.0 at 3 x 3 x 3
+// with N_P = 600, where 15 of a warp's 32 lanes had a word).
 template <int N1, int N2, int N3>
 __global__ void __launch_bounds__(128) herm_keys_to_exponents(const uint32_t* __restrict__ rowk,
                                                               const uint32_t* __restrict__ colk, int np,
                                                               int* __restrict__ e) {
   pdl_begin();
-  constexpr int L = N2 * N3, EPW = 32 / N1, LP = (L + 1) / 2, KWR = N1 * LP;
-  __shared__ uint32_t part[4][32];
+  constexpr int L = N2 * N3, EPW = 32 / N1, LP = (L + 1) / 2, KWR = N1 * LP, G = 128 / KWR, STEP = G * KWR;
+  __shared__ uint32_t part[128];
   const int nqb = (np + EPW - 1) / EPW, npb = (np + 7) / 8;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tid = threadIdx.x;
   for (int P = blockIdx.x; P < np; P += gridDim.x) {
-    uint32_t m0 = 0u, m1 = 0u;
-    if (lane < KWR) {
-      const uint32_t* r = rowk + (long)P * nqb * KWR + lane;
-      int qb = herm_qb0(P / 8, EPW) + warp;
-      for (; qb + 4 < nqb; qb += 8) {
-        m0 = __vmaxu2(m0, r[(long)qb * KWR]);
-        m1 = __vmaxu2(m1, r[(long)(qb + 4) * KWR]);
+    uint32_t m = 0u;
+    auto run = [&](const uint32_t* p, int n) {
+      for (int t = tid; t < n; t += 8 * STEP) {
+        uint32_t w[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) w[j] = t + j * STEP < n ? __ldcs(p + t + j * STEP) : 0u;
+#pragma unroll
+        for (int j = 0; j < 8; j++) m = __vmaxu2(m, w[j]);
       }
-      if (qb < nqb) m0 = __vmaxu2(m0, r[(long)qb * KWR]);
-      const uint32_t* c = colk + (long)P * npb * KWR + lane;
-      const int qbP = P / EPW;
-      for (int pb = warp; pb < npb && herm_qb0(pb, EPW) <= qbP; pb += 4) m1 = __vmaxu2(m1, c[(long)pb * KWR]);
+    };
+    if (tid < STEP) {
+      const int q0 = herm_qb0(P / 8, EPW), qbP = P / EPW;
+      // the row bands pb with herm_qb0(pb) <= qbP
+      const int pbs = min(npb, (EPW * qbP + EPW - 1) / 8 + 1);
+      run(rowk + ((long)P * nqb + q0) * KWR, (nqb - q0) * KWR);
+      run(colk + (long)P * npb * KWR, pbs * KWR);
     }
-    part[warp][lane] = __vmaxu2(m0, m1);
+    part[tid] = m;
     __syncthreads();
-    if (warp == 0 && lane < KWR) {
-      const uint32_t m = __vmaxu2(__vmaxu2(part[0][lane], part[1][lane]), __vmaxu2(part[2][lane], part[3][lane]));
-      const int s = lane / LP, i = lane - s * LP;
+    if (tid < KWR) {
+#pragma unroll
+      for (int g = 1; g < G; g++) m = __vmaxu2(m, part[g * KWR + tid]);
+      const int s = tid / LP, i = tid - s * LP;
       e[(long)(s * L + 2 * i) * np + P] = key_exponent(m & 0xffffu);
       if (2 * i + 1 < L) e[(long)(s * L + 2 * i + 1) * np + P] = key_exponent(m >> 16);
     }

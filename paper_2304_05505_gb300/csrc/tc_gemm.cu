@@ -1031,10 +1031,18 @@ __global__ void __launch_bounds__(256) tc_combine_kernel(const int* __restrict__
   float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
   for (long iv = (long)blockIdx.x * blockDim.x + threadIdx.x; iv < nv; iv += (long)gridDim.x * blockDim.x) {
     const long i = iv * V;
-    const int col = (int)(i % Nr);
-    const long bm = i / Nr;
-    const int m = (int)(bm % M);
-    const int b = (int)(bm / M);
+    int col, m, b;
+    if (total <= 0x7fffffffL) {   // (a 64-bit division is a hundred instructions)
+      const unsigned bm = (unsigned)i / (unsigned)Nr;
+      col = (int)((unsigned)i - bm * (unsigned)Nr);
+      b = (int)(bm / (unsigned)M);
+      m = (int)(bm - (unsigned)b * (unsigned)M);
+    } else {
+      const long bm = i / Nr;
+      col = (int)(i - bm * Nr);
+      b = (int)(bm / M);
+      m = (int)(bm - (long)b * M);
+    }
     long s0[V];
     float bc[V];
 #pragma unroll
@@ -1042,15 +1050,38 @@ __global__ void __launch_bounds__(256) tc_combine_kernel(const int* __restrict__
       s0[j] = 0;
       bc[j] = 0.f;
     }
-    for (int c = 0; c < nchunk; c++) {
+    // four chunks' loads in flight (three or four chunks are the usual split)
+    for (int c0 = 0; c0 < nchunk; c0 += 4) {
       if constexpr (V == 4) {
-        const int4 a = __ldcs(reinterpret_cast<const int4*>(ps0 + (long)c * total + i));
-        const float4 f = __ldcs(reinterpret_cast<const float4*>(pbc + (long)c * total + i));
-        s0[0] += a.x; s0[1] += a.y; s0[2] += a.z; s0[3] += a.w;
-        bc[0] += f.x; bc[1] += f.y; bc[2] += f.z; bc[3] += f.w;
+        int4 a[4];
+        float4 f[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+          if (c0 + q < nchunk) {
+            a[q] = __ldcs(reinterpret_cast<const int4*>(ps0 + (long)(c0 + q) * total + i));
+            f[q] = __ldcs(reinterpret_cast<const float4*>(pbc + (long)(c0 + q) * total + i));
+          }
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+          if (c0 + q < nchunk) {
+            s0[0] += a[q].x; s0[1] += a[q].y; s0[2] += a[q].z; s0[3] += a[q].w;
+            bc[0] += f[q].x; bc[1] += f[q].y; bc[2] += f[q].z; bc[3] += f[q].w;
+          }
       } else {
-        s0[0] += ps0[(long)c * total + i];
-        bc[0] += pbc[(long)c * total + i];
+        int a[4];
+        float f[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+          if (c0 + q < nchunk) {
+            a[q] = ps0[(long)(c0 + q) * total + i];
+            f[q] = pbc[(long)(c0 + q) * total + i];
+          }
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+          if (c0 + q < nchunk) {
+            s0[0] += a[q];
+            bc[0] += f[q];
+          }
       }
     }
     const int ea = row_exp(eA, (long)b * seA + m) - 14;
