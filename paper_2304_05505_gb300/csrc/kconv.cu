@@ -707,8 +707,16 @@ __global__ void mlo_combine_kernel(const float2* __restrict__ M, const uint32_t*
 // 16-bit keys); herm_keys_to_exponents takes the maxima.
 // X (extended form, N1 = 2 or 4): also writes Mlo, the fp16 remainders of M
 // (mlo_scale), [N_k][np][np] pairs (re, im).
+constexpr int CK_ROW = 36;   // words of a key row (32 lanes): 4 i + lane are distinct banks for the column keys' reads
+
+// Blocks to an SM: what shared memory holds of the 64-point form (107 KB a
+// block); the smaller meshes take more, for the latency of their chains of
+// barriers (3 x 3 x 3, N_P = 600: 2 blocks left 46 % of the issue slots empty;
+// 44.4 us with two, 38.2 with three).
+__host__ __device__ constexpr int herm_blocks(int n1, bool x) { return n1 == 4 ? 2 : n1 == 3 ? 3 : x ? 2 : 4; }
+
 template <int N1, int N2, int N3, bool X>
-__global__ void __launch_bounds__(256, 2) kconv_herm_kernel(const __grid_constant__ CUtensorMap mapD,
+__global__ void __launch_bounds__(256, herm_blocks(N1, X)) kconv_herm_kernel(const __grid_constant__ CUtensorMap mapD,
                                                          const __grid_constant__ CUtensorMap mapV,
                                                          float2* __restrict__ M, int np, long ntile, Twiddles tw,
                                                          uint32_t* __restrict__ rowk, uint32_t* __restrict__ colk,
@@ -722,9 +730,9 @@ __global__ void __launch_bounds__(256, 2) kconv_herm_kernel(const __grid_constan
   const float2* sD = reinterpret_cast<const float2*>(kc_smem);
   const float2* sV = reinterpret_cast<const float2*>(kc_smem + BOX);
   float2* scr = reinterpret_cast<float2*>(kc_smem + 2 * BOX);
-  uint32_t* ckey = reinterpret_cast<uint32_t*>(kc_smem + 3 * BOX);   // [warp][lane][LP]
-  const uint32_t bar = smem_u32(kc_smem + 3 * BOX + 8 * 32 * LP * 4);
-  int* tnext = reinterpret_cast<int*>(kc_smem + 3 * BOX + 8 * 32 * LP * 4 + 8);   // (pb, qb) of the next tile
+  uint32_t* ckey = reinterpret_cast<uint32_t*>(kc_smem + 3 * BOX);   // [warp][LP][CK_ROW]
+  const uint32_t bar = smem_u32(kc_smem + 3 * BOX + 8 * CK_ROW * LP * 4);
+  int* tnext = reinterpret_cast<int*>(kc_smem + 3 * BOX + 8 * CK_ROW * LP * 4 + 8);   // (pb, qb) of the next tile
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int slot = lane / EPW, el = lane - slot * EPW;
   const bool live = slot < N1;
@@ -765,6 +773,11 @@ __global__ void __launch_bounds__(256, 2) kconv_herm_kernel(const __grid_constan
   }
   __syncthreads();
   const long npq = (long)np * np;
+  // the mirror image: a thread keeps its row and column of the tile and takes
+  // every KPP-th k plane
+  constexpr int KPP = 256 / (8 * EPW);
+  static_assert(NK % KPP == 0, "whole passes over the k planes");
+  const int mr = threadIdx.x & 7, mc = (threadIdx.x >> 3) % EPW, mk = (threadIdx.x >> 3) / EPW;
   bool good = true;
   uint32_t fail_parity = 0;
   long it = 0;
@@ -902,7 +915,7 @@ __global__ void __launch_bounds__(256, 2) kconv_herm_kernel(const __grid_constan
       const uint32_t k = __byte_perm(abs_bits(x[2 * i]), 2 * i + 1 < L ? abs_bits(x[2 * i + 1 < L ? 2 * i + 1 : 0]) : 0u,
                                      0x7632);
       w[i] = direct ? k : 0u;
-      ckey[(warp * 32 + lane) * LP + i] = mirror ? k : 0u;
+      ckey[(warp * LP + i) * CK_ROW + lane] = mirror ? k : 0u;
     }
 #pragma unroll
     for (int o = 1; o < EPW; o <<= 1) {
@@ -929,12 +942,17 @@ __global__ void __launch_bounds__(256, 2) kconv_herm_kernel(const __grid_constan
       }
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < NK * EPW * 8; idx += blockDim.x) {
-      const int r = idx & 7, c = (idx >> 3) % EPW, k = idx / (8 * EPW);
-      const int mP = 8 * pb + r, mQ = EPW * qb + c;
-      if (mQ > mP && mQ < np) {
-        const float2 v = scr[(k * EPW + c) * 8 + (r ^ tsw(k, c))];
-        __stcs(M + ((long)k * np + mQ) * np + mP, make_float2(v.x, -v.y));
+    const int mP = 8 * pb + mr, mQ = EPW * qb + mc;
+    const bool mout = mk < KPP && mQ > mP && mQ < np;
+    if (mout) {
+      float2* d = M + ((long)mk * np + mQ) * np + mP;
+      // (unrolled, the stores of sixteen planes leave in one burst between the
+      // other block's loads: 0.330 ms instead of 0.300 at 4 x 4 x 4, N_P = 1200)
+#pragma unroll 1
+      for (int i = 0; i < NK / KPP; i++) {
+        const int k = mk + i * KPP;
+        const float2 v = scr[(k * EPW + mc) * 8 + (mr ^ tsw(k, mc))];
+        __stcs(d + (long)i * KPP * npq, make_float2(v.x, -v.y));
       }
     }
     if constexpr (X) {
@@ -950,11 +968,13 @@ __global__ void __launch_bounds__(256, 2) kconv_herm_kernel(const __grid_constan
         }
       }
       __syncthreads();
-      for (int idx = threadIdx.x; idx < NK * EPW * 8; idx += blockDim.x) {
-        const int r = idx & 7, c = (idx >> 3) % EPW, k = idx / (8 * EPW);
-        const int mP = 8 * pb + r, mQ = EPW * qb + c;
-        if (mQ > mP && mQ < np)
-          __stcs(Mlo + ((long)k * np + mQ) * np + mP, scr32[(k * EPW + c) * 8 + (r ^ tsw(k, c))] ^ 0x80000000u);
+      if (mout) {
+        uint32_t* d = Mlo + ((long)mk * np + mQ) * np + mP;
+#pragma unroll
+        for (int i = 0; i < NK / KPP; i++) {
+          const int k = mk + i * KPP;
+          __stcs(d + (long)i * KPP * npq, scr32[(k * EPW + mc) * 8 + (mr ^ tsw(k, mc))] ^ 0x80000000u);
+        }
       }
     }
     for (int idx = threadIdx.x; idx < N1 * EPW * LP; idx += blockDim.x) {
@@ -963,7 +983,7 @@ __global__ void __launch_bounds__(256, 2) kconv_herm_kernel(const __grid_constan
       if (cq >= np) continue;
       uint32_t m = 0u;
 #pragma unroll
-      for (int v = 0; v < 8; v++) m = __vmaxu2(m, ckey[(v * 32 + ln) * LP + i]);
+      for (int v = 0; v < 8; v++) m = __vmaxu2(m, ckey[(v * LP + i) * CK_ROW + ln]);
       colk[((long)cq * npb + pb) * KWR + cs * LP + i] = m;
     }
   }
@@ -1179,7 +1199,7 @@ cudaError_t kconv_herm_launch(const float2* D, const float2* Vh, float2* M, int 
                               int* err, cudaEvent_t conv_done, cudaStream_t s, uint32_t* Mlo) {
   constexpr int L = N2 * N3, NK = N1 * L, EPW = 32 / N1, EPB = EPW * 8, LP = (L + 1) / 2, KWR = N1 * LP;
   constexpr uint32_t BOX = NK * EPB * sizeof(float2);
-  constexpr uint32_t SMEM = 3 * BOX + 8 * 32 * LP * 4 + 16;   // + mbarrier and the next tile's (pb, qb)
+  constexpr uint32_t SMEM = 3 * BOX + 8 * CK_ROW * LP * 4 + 16;   // + mbarrier and the next tile's (pb, qb)
   static_assert(BOX % 128 == 0, "boxes start on 128-byte boundaries");
   const long npq = (long)np * np;
   alignas(64) unsigned char mD[128], mV[128];
@@ -1203,7 +1223,7 @@ cudaError_t kconv_herm_launch(const float2* D, const float2* Vh, float2* M, int 
   uint32_t* rowk = keys;
   uint32_t* colk = keys + (long)nqb * np * KWR;
   const int* tcum = reinterpret_cast<const int*>(colk + (long)npb * np * KWR);
-  const unsigned grid = (unsigned)std::min<long>(ntile, 2L * nsm);
+  const unsigned grid = (unsigned)std::min<long>(ntile, (long)herm_blocks(N1, X) * nsm);
   launch_pdl(kconv_herm_kernel<N1, N2, N3, X>, grid, 256, SMEM, s, mapD, mapV, M, np, ntile, make_twiddles(N1, N2, N3),
                                                          rowk, colk, tcum, err, Mlo);
   r = cudaGetLastError();
