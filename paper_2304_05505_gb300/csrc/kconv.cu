@@ -585,6 +585,9 @@ __global__ void __launch_bounds__(256) kconv_tile_kernel(const __grid_constant__
         if (rfirst == rlast) {
           key = __reduce_max_sync(0xffffffffu, key);
           if (lane == 0) rmax[k] = max(rmax[k], key);
+        } else if (rlast > rfirst + 1) {
+          // rows shorter than a batch
+          if (key) atomicMax(rowkey + (long)k * np + e / np, key);
         } else {
           // a batch across a row boundary: each row's part straight to memory
           const bool first = e / np == rfirst;
@@ -1038,6 +1041,196 @@ __global__ void __launch_bounds__(128) herm_keys_to_exponents(const uint32_t* __
   }
 }
 
+// Hermitian form of the shared-memory convolution, for meshes with axes of 1, 2,
+// 3, 4 and 6 points (compile-time N2, N3).  A tile is 4 rows P by 8
+// columns Q, one element to a lane; only the tiles that reach the diagonal are
+// loaded, and the lanes of the upper part write their value of M at (P, Q) and
+// its conjugate at (Q, P), which halves the bytes read and the transforms.
+// Warp i1 holds the plane of the mesh with first index i1: the transforms along
+// the second and third axis run in its registers (N2 N3 values a lane), those
+// along the first in shared memory, in the same order as the flat form, so M
+// has the same bits for Hermitian input.  D comes by TMA; Vh never goes through
+// shared memory: the lanes load it at the product, from L2, into which a
+// prefetch of its box was issued with the load of D.  A value so crosses shared
+// memory 8 times instead of 18, which is what bounds the flat form (6 x 6 x 6 k,
+// N_P = 2400: 9.0 ms, where the bytes take 4.4 at the measured copy rate).
+// Row keys go to scratch as in kconv_herm_kernel: rowk[P][qb][KWR] from the
+// elements with Q >= P, colk[Q][pb][KWR] from their mirror image.
+constexpr int TH_R = 4, TH_C = 8;
+
+// Order of the tiles: squares of TH_B x TH_B blocks of 8 x 8 elements (two tiles
+// each), about what is in flight at a time.  Along whole rows of tiles the
+// mirror image of what is in flight would be 64 bytes in each of thousands of
+// rows of M, far apart in memory, with the neighbouring bytes of a row only
+// after the whole row of tiles has passed through L2.
+constexpr int TH_B = 12;
+// Positions before the coarse row g of the squares (upper triangle, nc to a side).
+__host__ __device__ __forceinline__ long tile_herm_before(long g, long nc) {
+  return (g * nc - g * (g - 1) / 2) * (2 * TH_B * TH_B);
+}
+
+// (36 values a lane: two blocks an SM, without spills, are faster than three)
+template <int N2, int N3>
+__global__ void __launch_bounds__(192, N2 * N3 > 18 ? 2 : 3) kconv_tile_herm_kernel(const __grid_constant__ CUtensorMap mapD,
+                                                              const float2* __restrict__ Vh, float2* __restrict__ M,
+                                                              int np, long npos, Twiddles tw,
+                                                              uint32_t* __restrict__ rowk, uint32_t* __restrict__ colk,
+                                                              int* err) {
+  pdl_begin();
+  constexpr int L = N2 * N3, LP = (L + 1) / 2;
+  const int n1 = tw.n[0], KWR = n1 * LP;
+  const uint32_t box = (uint32_t)(n1 * L * TILE_EPB * sizeof(float2));
+  extern __shared__ __align__(128) unsigned char kt_smem[];   // [k][32] of D, mbarrier, (pb, qb) of the tile
+  float2* sD = reinterpret_cast<float2*>(kt_smem);
+  const uint32_t bar = smem_u32(kt_smem + box);
+  int* tnext = reinterpret_cast<int*>(kt_smem + box + 8);
+  const int lane = threadIdx.x & 31, i1 = threadIdx.x >> 5;
+  const int r = lane / TH_C, c = lane % TH_C;
+  const long npq = (long)np * np;
+  const int nqb = (np + TH_C - 1) / TH_C, npb = (np + TH_R - 1) / TH_R;
+  // thread 0: the next tile from position t on that reaches the diagonal, its
+  // loads and (pb, qb), pb = -1 at the end
+  const int nc = (nqb + TH_B - 1) / TH_B;
+  long t0 = blockIdx.x;
+  auto issue = [&]() {
+    tnext[0] = -1;
+    for (; t0 < npos; t0 += gridDim.x) {
+      int lo = 0, hi = nc - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (tile_herm_before(mid, nc) <= t0) lo = mid;
+        else hi = mid - 1;
+      }
+      const long u = t0 - tile_herm_before(lo, nc);
+      const int in = (int)(u % (2 * TH_B * TH_B));
+      const int g = TH_B * lo + (in >> 1) / TH_B, qb = TH_B * (lo + (int)(u / (2 * TH_B * TH_B))) + (in >> 1) % TH_B;
+      const int pb = 2 * g + (in & 1);
+      if (qb < g || qb >= nqb || pb >= npb) continue;
+      tnext[0] = pb;
+      tnext[1] = qb;
+      mbar_expect_tx(bar, box);
+      tma_load_3d(smem_u32(sD), &mapD, bar, 2 * TH_C * qb, TH_R * pb, 0);
+      t0 += gridDim.x;
+      break;
+    }
+  };
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    mbar_fence_init();
+    issue();
+  }
+  bool good = true;
+  uint32_t parity = 0;
+  // the lines along the first axis: warp w takes w, w + n1, ...
+  auto first_axis = [&](int sign) {
+    if (n1 > 1)
+      for (int l = i1; l < L; l += n1) smem_line<float>(sD + l * TILE_EPB + lane, n1, L * TILE_EPB, tw, 0, sign);
+    __syncthreads();
+  };
+  for (long it = 0;; it++) {
+    __syncthreads();
+    const int pb = tnext[0], qb = tnext[1];
+    if (pb < 0) break;
+    parity = (uint32_t)(it & 1);
+    good = mbar_wait_warp(bar, parity, err, 8192);
+    good = __syncthreads_and(good);
+    if (!good) break;
+    const int P = TH_R * pb + r, Q = TH_C * qb + c;
+    const bool direct = P < np && Q < np && Q >= P, mirror = direct && Q > P;
+    float2* plane = sD + i1 * L * TILE_EPB + lane;
+    first_axis(-1);
+    float2 x[L];
+#pragma unroll
+    for (int j = 0; j < L; j++) x[j] = plane[j * TILE_EPB];
+    local_dfts<N2, N3>(x, tw, -1);
+    const float2* v = Vh + (long)i1 * L * npq + (long)P * np + Q;
+    constexpr int G = L % 12 == 0 ? 12 : L % 9 == 0 ? 9 : L % 8 == 0 ? 8 : L % 6 == 0 ? 6 : L % 4 == 0 ? 4 : L;
+    static_assert(L % G == 0, "whole groups of Vh loads");
+#pragma unroll
+    for (int j0 = 0; j0 < L; j0 += G) {
+      float2 vh[G];
+#pragma unroll
+      for (int j = 0; j < G; j++) vh[j] = direct ? __ldcs(v + (long)(j0 + j) * npq) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < G; j++) plane[(j0 + j) * TILE_EPB] = cmul(x[j0 + j], vh[j]);
+    }
+    __syncthreads();
+    first_axis(+1);
+#pragma unroll
+    for (int j = 0; j < L; j++) x[j] = plane[j * TILE_EPB];
+    __syncthreads();                                     // the box (and tnext) are free for the next tile
+    if (threadIdx.x == 0) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      issue();
+    }
+    local_dfts<N2, N3>(x, tw, +1);
+    if (direct) {
+      float2* d = M + (long)i1 * L * npq + (long)P * np + Q;
+#pragma unroll
+      for (int j = 0; j < L; j++) __stcs(d + (long)j * npq, x[j]);
+    }
+    if (mirror) {
+      float2* d = M + (long)i1 * L * npq + (long)Q * np + P;
+#pragma unroll
+      for (int j = 0; j < L; j++) __stcs(d + (long)j * npq, make_float2(x[j].x, -x[j].y));
+    }
+    // keys: rows over the lanes of a row, columns over the lanes of a column
+    uint32_t* rk = rowk + ((long)P * nqb + qb) * KWR + i1 * LP;
+    uint32_t* ck = colk + ((long)Q * npb + pb) * KWR + i1 * LP;
+#pragma unroll
+    for (int i = 0; i < LP; i++) {
+      const uint32_t k = __byte_perm(abs_bits(x[2 * i]), 2 * i + 1 < L ? abs_bits(x[2 * i + 1 < L ? 2 * i + 1 : 0]) : 0u,
+                                     0x7632);
+      uint32_t a = direct ? k : 0u, b = mirror ? k : 0u;
+#pragma unroll
+      for (int o = 1; o < TH_C; o <<= 1) a = __vmaxu2(a, __shfl_xor_sync(0xffffffffu, a, o));
+#pragma unroll
+      for (int o = TH_C; o < 32; o <<= 1) b = __vmaxu2(b, __shfl_xor_sync(0xffffffffu, b, o));
+      if (c == (i & (TH_C - 1)) && P < np) rk[i] = a;
+      if (r == (i & (TH_R - 1)) && Q < np) ck[i] = b;
+    }
+  }
+  // the copy of the tile whose wait gave up may still be in flight
+  if (!good && threadIdx.x == 0) mbar_drain(bar, parity);
+}
+
+// The exponents from the keys of kconv_tile_herm_kernel, as
+// herm_keys_to_exponents (KWR <= 128 words to a tile).
+__global__ void __launch_bounds__(128) tile_keys_to_exponents(const uint32_t* __restrict__ rowk,
+                                                              const uint32_t* __restrict__ colk, int np, int n1, int L,
+                                                              int* __restrict__ e) {
+  pdl_begin();
+  __shared__ uint32_t part[128];
+  const int LP = (L + 1) / 2, KWR = n1 * LP, G = 128 / KWR, STEP = G * KWR;
+  const int nqb = (np + TH_C - 1) / TH_C, npb = (np + TH_R - 1) / TH_R;
+  const int tid = threadIdx.x;
+  for (int P = blockIdx.x; P < np; P += gridDim.x) {
+    uint32_t m = 0u;
+    auto run = [&](const uint32_t* p, int n) {
+      for (int t = tid; t < n; t += 8 * STEP) {
+        uint32_t w[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) w[j] = t + j * STEP < n ? __ldcs(p + t + j * STEP) : 0u;
+#pragma unroll
+        for (int j = 0; j < 8; j++) m = __vmaxu2(m, w[j]);
+      }
+    };
+    if (tid < STEP) {
+      run(rowk + ((long)P * nqb + P / TH_C) * KWR, (nqb - P / TH_C) * KWR);
+      run(colk + (long)P * npb * KWR, min(npb, 2 * (P / TH_C) + 2) * KWR);
+    }
+    part[tid] = m;
+    __syncthreads();
+    if (tid < KWR) {
+      for (int g = 1; g < G; g++) m = __vmaxu2(m, part[g * KWR + tid]);
+      const int s = tid / LP, i = tid - s * LP;
+      e[(long)(s * L + 2 * i) * np + P] = key_exponent(m & 0xffffu);
+      if (2 * i + 1 < L) e[(long)(s * L + 2 * i + 1) * np + P] = key_exponent(m >> 16);
+    }
+    __syncthreads();
+  }
+}
+
 // tcum[pb] = the tiles of the row bands before pb that reach the diagonal
 // (tcum[npb] = all of them).
 __global__ void herm_tile_prefix(int* tcum, int np, int epw) {
@@ -1340,6 +1533,65 @@ cudaError_t kconv_c_rowexp(const float2* D, const float2* Vh, float2* M, int np,
   r = cudaGetLastError();
   *done = r == cudaSuccess;
   return r;
+}
+
+// Key scratch (bytes) of the Hermitian shared-memory form: of rows, of columns.
+static size_t tile_herm_row_bytes(int np, int kwr) { return 4 * (size_t)kwr * np * ((np + TH_C - 1) / TH_C); }
+static size_t tile_herm_col_bytes(int np, int kwr) { return 4 * (size_t)kwr * np * ((np + TH_R - 1) / TH_R); }
+
+bool kconv_tile_herm_applies(int np, int n1, int n2, int n3, size_t row_scratch, size_t col_scratch) {
+  auto in = [](int n) { return n == 1 || n == 2 || n == 3 || n == 4 || n == 6; };
+  const int kwr = n1 * ((n2 * n3 + 1) / 2);
+  return np >= 2 && np % 2 == 0 && (long)np * np < (1L << 29) && in(n1) && in(n2) && in(n3) &&
+         tile_herm_row_bytes(np, kwr) <= row_scratch && tile_herm_col_bytes(np, kwr) <= col_scratch;
+}
+
+template <int N2, int N3>
+static cudaError_t kconv_tile_herm_launch(const float2* D, const float2* Vh, float2* M, int np, int n1, uint32_t* rowk,
+                                          uint32_t* colk, int* e, int* err, cudaEvent_t conv_done, cudaStream_t s) {
+  constexpr int L = N2 * N3;
+  const long npq = (long)np * np;
+  alignas(64) unsigned char mD[128];
+  cudaError_t r = make_f32_map_3d(mD, D, 2L * np, np, n1 * L, 8L * np, 8 * npq, 2 * TH_C, TH_R, n1 * L);
+  if (r != cudaSuccess) return r;
+  CUtensorMap mapD;
+  memcpy(&mapD, mD, sizeof mapD);
+  const int nqb = (np + TH_C - 1) / TH_C;
+  const size_t sm = (size_t)n1 * L * TILE_EPB * sizeof(float2) + 16;
+  auto kernel = kconv_tile_herm_kernel<N2, N3>;
+  r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (r != cudaSuccess) return r;
+  int per_sm = 0, dev = 0, nsm = 0;
+  r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * n1, sm);
+  if (r == cudaSuccess) r = cudaGetDevice(&dev);
+  if (r == cudaSuccess) r = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (r != cudaSuccess) return r;
+  const int nc = (nqb + TH_B - 1) / TH_B;
+  const long npos = tile_herm_before(nc, nc);
+  const unsigned grid = (unsigned)std::min<long>(npos, (long)std::max(per_sm, 1) * nsm);
+  launch_pdl(kernel, grid, 32 * n1, sm, s, mapD, Vh, M, np, npos, make_twiddles(n1, N2, N3), rowk, colk, err);
+  r = cudaGetLastError();
+  if (r == cudaSuccess && conv_done) r = cudaEventRecord(conv_done, s);
+  if (r != cudaSuccess) return r;
+  launch_pdl(tile_keys_to_exponents, (unsigned)std::min(np, 152 * 16), 128, 0, s, rowk, colk, np, n1, L, e);
+  return cudaGetLastError();
+}
+
+cudaError_t kconv_c_tile_herm(const float2* D, const float2* Vh, float2* M, int np, int n1, int n2, int n3, void* rows,
+                              void* cols, int* e, int* err, cudaEvent_t started, cudaEvent_t conv_done,
+                              cudaStream_t s) {
+  if (started) {
+    const cudaError_t r = cudaEventRecord(started, s);
+    if (r != cudaSuccess) return r;
+  }
+  uint32_t *rowk = reinterpret_cast<uint32_t*>(rows), *colk = reinterpret_cast<uint32_t*>(cols);
+#define TH3(A, B) \
+  if (n2 == A && n3 == B) return kconv_tile_herm_launch<A, B>(D, Vh, M, np, n1, rowk, colk, e, err, conv_done, s);
+#define TH2(A) TH3(A, 1) TH3(A, 2) TH3(A, 3) TH3(A, 4) TH3(A, 6)
+  TH2(1) TH2(2) TH2(3) TH2(4) TH2(6)
+#undef TH2
+#undef TH3
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t mlo_combine_c2z(const float2* M, const uint32_t* Mlo, double2* out, long n, cudaStream_t s) {

@@ -410,6 +410,14 @@ thc_status thc_set_collocation(thc_ctx* c, const double* X) {
   return THC_OK;
 }
 
+// The Hermitian convolution of the meshes without hkeys can be used (even N_P,
+// its keys fit in the planes of the B operands of S2, already read then, and of
+// S4a, written after: about N_P <= 48 n_occ).
+static bool herm_tile_form(const thc_ctx* c) {
+  return tc_form(c->precision) && !c->hkeys &&
+         kconv_tile_herm_applies(c->nisdf, c->n1, c->n2, c->n3, 3 * 2 * (size_t)c->plBd, 3 * 2 * (size_t)c->plBy);
+}
+
 thc_status thc_set_kernel(thc_ctx* c, const double* V) {
   if (!c || !V || !aligned16(V)) return THC_ERR_ARG;
   const long npq = (long)c->nisdf * c->nisdf;
@@ -419,7 +427,7 @@ thc_status thc_set_kernel(thc_ctx* c, const double* V) {
   drop_graph(c);
   CKC(c, prepare_kernel_z(v, c->Vh64, c->Vh32, npq, c->n1, c->n2, c->n3, c->stream));
   c->herm_v = false;
-  if (c->hkeys) {
+  if (c->hkeys || herm_tile_form(c)) {
     // every V^q Hermitian to 1e-12 of max |V|: then M^k is Hermitian and the
     // build convolves the part of D on and above the diagonal only
     unsigned long long* dv = reinterpret_cast<unsigned long long*>(c->partial);
@@ -604,8 +612,9 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
   // (Hermitian V: M^k is Hermitian too, and S3 reads D on and above the
   // diagonal only, so S2 leaves the part below it unwritten)
   const bool herm = c->herm_v && c->hkeys;   // (no keys for odd N_P)
+  const bool herm_tile = c->herm_v && herm_tile_form(c);
   // (THC-AO-K reads all of D for its energy, so D is written whole there)
-  const bool upper = herm && !Kao;
+  const bool upper = (herm || herm_tile) && !Kao;
   CKC(c, tc_gemm(c->opPs, c->opBd, P, 2 * P, 2 * n, nk, c->ePsi, P, c->ePsi, P, D, false, 2 * P, 2 * PP,
                  c->part_s0, c->part_bc, c->tc_err, s, core_event(c, 1, 1), kProducts[1], 0, upper ? 2 : 1));
   c->d_upper = upper;
@@ -621,6 +630,10 @@ static thc_status build_tc(thc_ctx* c, const double2* C, double2* KC, double* ex
   if (herm) {
     CKC(c, kconv_c_herm(D, c->Vh32, M, P, c->n1, c->n2, c->n3, c->hkeys, c->eM, c->tc_err, core_event(c, 2, 0),
                         core_event(c, 2, 1), s, c->Mlo));
+    have_eM = true;
+  } else if (herm_tile) {
+    CKC(c, kconv_c_tile_herm(D, c->Vh32, M, P, c->n1, c->n2, c->n3, c->Bd_pl, c->By_pl, c->eM, c->tc_err, core_event(c, 2, 0),
+                             core_event(c, 2, 1), s));
     have_eM = true;
   } else if (!c->Mp) {
     CKC(c, kconv_c_rowexp(D, c->Vh32, M, P, c->n1, c->n2, c->n3, c->eM, &have_eM, c->tc_err,

@@ -211,6 +211,13 @@ cudaError_t kconv_herm_prepare(uint32_t* keys, int np, int n1, int n2, int n3, c
 cudaError_t kconv_c_herm(const float2* D, const float2* Vh, float2* M, int np, int n1, int n2, int n3,
                          uint32_t* keys, int* e, int* err, cudaEvent_t started, cudaEvent_t conv_done,
                          cudaStream_t s, uint32_t* Mlo = nullptr);
+// The same for other meshes: kconv_tile_herm_applies for np even, axes of 1, 2,
+// 3, 4 and 6 points and keys that fit in the two scratch buffers (bytes;
+// 4-byte aligned, overwritten).
+bool kconv_tile_herm_applies(int np, int n1, int n2, int n3, size_t row_scratch, size_t col_scratch);
+cudaError_t kconv_c_tile_herm(const float2* D, const float2* Vh, float2* M, int np, int n1, int n2, int n3, void* rows,
+                              void* cols, int* e, int* err, cudaEvent_t started, cudaEvent_t conv_done,
+                              cudaStream_t s);
 cudaError_t kconv_c_rowexp(const float2* D, const float2* Vh, float2* M, int np, int n1, int n2, int n3,
                            int* e, bool* done, int* err, cudaEvent_t started, cudaEvent_t conv_done,
                            cudaStream_t s);
