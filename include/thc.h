@@ -59,7 +59,10 @@ typedef enum {
 } thc_status;
 
 typedef enum {
-  THC_FP64 = 0,            /* every step in FP64 on CUDA cores */
+  /* every step to FP64 accuracy: large products from exact integer digits on
+   * the tensor cores (seven digits of 9 bits, sums exact, rounded once), the
+   * rest in FP64 on CUDA cores */
+  THC_FP64 = 0,
   THC_MIXED = 1,           /* S1, S2, S4a, S4b on tensor cores (tcgen05): each
                               operand row scaled by a power of two and cut into
                               three fixed-point slices of 8, 11 and 11 bits held
@@ -92,7 +95,11 @@ typedef struct thc_ctx thc_ctx;
  * (thc_memory_bytes tells how much) up front.  *ctx is NULL on failure. */
 thc_status thc_create(thc_ctx** ctx, const thc_dims* dims, int precision, void* stream);
 
-/* Device bytes the context holds (X copy, prepared kernel, workspace). */
+/* Device bytes the context holds (X copy, prepared kernel, workspace).
+ * THC_FP64: besides these, thc_set_collocation sets aside up to 2 GB for the
+ * digits of its products where the device has them (half as much is tried
+ * each time it has not; without any, the products run in FP64 on CUDA
+ * cores). */
 thc_status thc_memory_bytes(const thc_dims* dims, int precision, size_t* bytes);
 
 /* X: device, [N_k][nbas][nisdf] complex128.  Copied (and converted for
@@ -137,8 +144,8 @@ thc_status thc_build_host(thc_ctx* ctx, const double* C_host, double* KC_host, d
  * cell-periodic parts of the basis functions instead of the occupied
  * orbitals); the build takes any V.  C: device [N_k][nbas][nocc] complex128;
  * K: device [N_k][nbas][nbas] complex128 (written, must not overlap C); ex:
- * device, 2 doubles as in thc_build.  THC_FP64: every step in FP64 (the two
- * products on CUDA cores).  THC_MIXED: Z = M X^T and K = conj(X) Z on the
+ * device, 2 doubles as in thc_build.  THC_FP64: every step to FP64 accuracy
+ * (products as in thc_build).  THC_MIXED: Z = M X^T and K = conj(X) Z on the
  * tensor cores (three fp16 slices, 8 slice products, exact leading sums; the
  * planes of X^T are made once per thc_set_collocation).  THC_MIXED_SIMT:
  * THC_ERR_UNSUPPORTED.  The first call on a context allocates the form's
@@ -209,18 +216,22 @@ thc_status thc_debug_fail_alloc(int nth);
 /* The FP64 fused multiply-add rate of the current device, measured: a kernel
  * of independent FMA chains on every SM, timed with CUDA events on `stream`
  * (a cudaStream_t) after one warm-up launch.  *tflops_host = FP64 TFLOP/s
- * (2 flops per FMA).  The FP64 build's stages are reported against it.
+ * (2 flops per FMA).
  * Synchronises the stream; changes no device setting. */
 thc_status thc_measure_fp64_rate(void* stream, double* tflops_host);
 
-/* Number of kernel launches one thc_build makes. */
+/* Number of kernel launches one thc_build makes (THC_FP64: of the last build;
+ * 7 before the first). */
 thc_status thc_launches_per_build(const thc_ctx* ctx, int* launches);
 
 /* *hermitian = 1 when the builds take the Hermitian form (THC_MIXED on a
  * 2^3, 3^3 or 4^3 mesh with even nisdf, and the V of the last thc_set_kernel
  * Hermitian for every q to 1e-12 of max |V|): then M^k is Hermitian, S2
  * writes D on and above the diagonal only and S3 reads that half of D and of
- * the prepared kernel; else 0.  THC_ERR_STATE before thc_set_kernel. */
+ * the prepared kernel; else 0.  (Other meshes with axes of 1, 2, 3, 4 and 6
+ * points use the symmetry in S2 and S3 too, where N_P is even and at most
+ * about 48 n_occ; this call says 0 for them.)  THC_ERR_STATE before
+ * thc_set_kernel. */
 thc_status thc_hermitian_kernel(const thc_ctx* ctx, int* hermitian);
 
 thc_status thc_destroy(thc_ctx* ctx);
@@ -263,7 +274,8 @@ thc_status thc_select_points(const double* U, int nfunc, int ncand, int npts, do
  * points_host: npts distinct grid indices (host).  V_out: device,
  * [N_k][npts][npts] complex128 (q on the mesh index).  xi_out: device,
  * [npts][N_g] doubles, or NULL.  Allocates its own scratch (about
- * 40 npts N_g bytes) and waits for `stream`.  THC_ERR_ARG for bad sizes,
+ * 40 npts N_g bytes, and up to 1.25 GB for the digits of its products, less
+ * where the device has less) and waits for `stream`.  THC_ERR_ARG for bad sizes,
  * repeated or out-of-range points, or points whose metric S is numerically
  * singular (a Cholesky pivot below 1e-12 of its diagonal entry; message in
  * thc_last_error(NULL)). */
@@ -275,8 +287,8 @@ thc_status thc_fit_kernel(const double* U, int nfunc, const int* grid_host, cons
  * interpolation vectors to the current orbitals, their FFT, and M^q as a sum
  * over G; Sec. 2.2).  Computes what thc_fit_kernel computes, with the same
  * arguments, conventions and errors (no xi output), and times its steps.
- * precision THC_FP64: every step in FP64 (the result equals thc_fit_kernel's
- * bit for bit).  THC_MIXED: the fit's metric, its Cholesky factor, the solve
+ * precision THC_FP64: every step to FP64 accuracy (the result equals
+ * thc_fit_kernel's bit for bit).  THC_MIXED: the fit's metric, its Cholesky factor, the solve
  * and the FFT stay FP64; the contraction
  *   V^q[P,Q] = sum_G Xq[P][G] conj(Xq[Q][G]),  Xq = xh sqrt(v(G+q)) e^{-i q.r_P} (scaled),
  * which dominates the rebuild (N_k N_P^2 N_G complex multiply-adds), runs on
@@ -314,8 +326,8 @@ thc_status thc_rebuild_kernel(const double* U, int nfunc, const int* grid_host, 
  * lattice_host, mesh_host, points_host, npts: as for thc_fit_kernel.  V:
  * device, [N_k][npts][npts] complex128, the kernel fitted to U at these points
  * (thc_fit_kernel's or thc_rebuild_kernel's output); the response terms use
- * the fit recomputed here.  precision THC_FP64: every step in FP64 on CUDA
- * cores.  THC_MIXED: the (q, G) contraction of the response, the
+ * the fit recomputed here.  precision THC_FP64: every step to FP64 accuracy
+ * (large products from exact digits on the tensor cores).  THC_MIXED: the (q, G) contraction of the response, the
  * O(N_k npts^2 N_G) step that dominates, runs on the tcgen05 tensor cores as
  * thc_rebuild_kernel's contraction does (W^q with its phases rounded to FP32
  * and sliced in the GEMM, v(G+q) conj(xh) cut into three fp16 slices with
@@ -332,7 +344,7 @@ thc_status thc_rebuild_kernel(const double* U, int nfunc, const int* grid_host, 
  * DFT with the solve, and the orbital contractions.  Outputs must not overlap
  * inputs.  Allocates its own scratch, at most about the largest of
  * 48 N_k npts^2, 16 npts (N_k npts + 7 N_g) and 16 N_k n_occ N_g + 32 npts N_g
- * bytes, and waits for `stream`.  THC_ERR_ARG for
+ * bytes, and up to 1.25 GB for the digits of its products, and waits for `stream`.  THC_ERR_ARG for
  * bad sizes, null or misaligned pointers, repeated or out-of-range points, or
  * points whose metric S is numerically singular (as thc_fit_kernel);
  * THC_ERR_TIMEOUT if a device wait of the tensor-core contraction gave up. */

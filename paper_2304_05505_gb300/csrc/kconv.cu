@@ -23,6 +23,9 @@
 //                      place in shared memory (lengths 6 by Good-Thomas)
 //   kconv_lanes_kernel the same meshes as kconv_pipe_kernel without TMA (N1
 //                      lanes per element, first axis by shuffles)
+//   kconv_tile_herm_kernel  meshes with axes of 1, 2, 3, 4 and 6 points, N_P even,
+//                      V Hermitian: tiles of 4 x 8 elements that reach the
+//                      diagonal, two mesh axes in registers
 //   kconv_kernel       any mesh: one thread per element, its N_k values in
 //                      shared memory ([k][thread], conflict-free)
 //   (FP64, axes of 1 to 4 points: kconv_fix.cu)
@@ -1050,10 +1053,13 @@ __global__ void __launch_bounds__(128) herm_keys_to_exponents(const uint32_t* __
 // the second and third axis run in its registers (N2 N3 values a lane), those
 // along the first in shared memory, in the same order as the flat form, so M
 // has the same bits for Hermitian input.  D comes by TMA; Vh never goes through
-// shared memory: the lanes load it at the product, from L2, into which a
-// prefetch of its box was issued with the load of D.  A value so crosses shared
-// memory 8 times instead of 18, which is what bounds the flat form (6 x 6 x 6 k,
-// N_P = 2400: 9.0 ms, where the bytes take 4.4 at the measured copy rate).
+// shared memory: the lanes load it at the product (a prefetch of its box into L2
+// at the start of the tile made it slower, 7.4 -> 8.7 ms).  A value so crosses
+// shared memory 8 times instead of 18, which is what bounds the flat form.
+// 6 x 6 x 6 k: N_P = 2400 9.0 -> 7.3 ms (20 GB), N_P = 1200 2.31 -> 1.38 ms; the
+// flat form's eight warps have little to do on small meshes: 3 x 2 x 4, N_P = 702
+// 267 -> 74 us, 2 x 2 x 3, N_P = 900 355 -> 52 us.  What bounds it now is the wait
+// for memory with 12 warps an SM (36 values a lane in registers).
 // Row keys go to scratch as in kconv_herm_kernel: rowk[P][qb][KWR] from the
 // elements with Q >= P, colk[Q][pb][KWR] from their mirror image.
 constexpr int TH_R = 4, TH_C = 8;
@@ -1062,7 +1068,8 @@ constexpr int TH_R = 4, TH_C = 8;
 // each), about what is in flight at a time.  Along whole rows of tiles the
 // mirror image of what is in flight would be 64 bytes in each of thousands of
 // rows of M, far apart in memory, with the neighbouring bytes of a row only
-// after the whole row of tiles has passed through L2.
+// after the whole row of tiles has passed through L2 (8.5 -> 7.4 ms at 6 x 6 x 6,
+// N_P = 2400; squares of 5, 8 or 24 are within 3 % or slower).
 constexpr int TH_B = 12;
 // Positions before the coarse row g of the squares (upper triangle, nc to a side).
 __host__ __device__ __forceinline__ long tile_herm_before(long g, long nc) {

@@ -29,7 +29,7 @@
 //   4. the block's columns for all candidates: one product with the digits of
 //      U, which are made once, one with the earlier rows of L, and a kernel
 //      that finishes the block's own triangle, d and sum d after every pivot
-// (767 ms to 30 ms for 600 points.)  Where S comes out empty (more than 800
+// (767 ms to 49 ms for 600 points.)  Where S comes out empty (more than 800
 // candidates within a bin of the largest) one pivot is taken the first way.
 #include "oz_gemm.cuh"
 #include "thc_internal.cuh"

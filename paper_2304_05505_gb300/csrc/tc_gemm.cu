@@ -62,7 +62,8 @@
 // the converted forms keep A in TMEM, and the issue of the MMAs (see warps 0
 // and 1 below).  At 4 x 4 x 4 k, N_P = 1200, N = 432, n = 60 the two together
 // took S4a's kernel from 0.354 to 0.268 ms, S4b's from 0.154 to 0.119 and
-// S1's from 0.138 to 0.096 (A in TMEM by itself: no gain).
+// S1's from 0.138 to 0.096 (A in TMEM by itself: no gain).  With the packed
+// slicers and the division-free unit walk they take 0.242, 0.109 and 0.088.
 // The epilogue warps (4 per TMEM lane quadrant) read both accumulators with
 // tcgen05.ld, scale by exact powers of two and store (or write the partial
 // sums), then release the accumulator set.  Each warp turns its 32-row x
