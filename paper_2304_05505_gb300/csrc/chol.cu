@@ -1,5 +1,4 @@
-// Blocked Cholesky factorisation in FP64, the inverse of the factor, and the
-// solve with many right-hand sides as two matrix products.
+// Blocked Cholesky factorisation in FP64.
 //
 // The factor: right-looking in panels of 32 columns.  One warp factors the
 // diagonal block (a row per lane, in registers), the rows below follow by
@@ -10,13 +9,14 @@
 // of chol_column's left-looking sums, which every thread redid from column 0
 // for each of the n dependent launches (34 ms at n = 600, 134 ms at n = 1200).
 //
-// The inverse: [A 0; B C]^-1 = [A^-1 0; -C^-1 B A^-1 C^-1] from the inverted
-// diagonal blocks of 32 upward, all pairs of a level in one launch, the
-// levels of 256 rows and more on the tensor cores.
-//
-// The solve: L^-T (L^-1 X), both products on the tensor cores
-// (oz_gemm.cu), in place of one substitution per thread and right-hand side,
-// which runs at the rate of the FP64 pipe.
+// The solve is a forward and a backward substitution per right-hand side
+// (chol_solve, isdf_common.cuh).  Two products with the inverse of L from
+// digits took 4 ms in place of 70 at n = 600 and 64000 right-hand sides, but
+// are not its equal: a row of L^-1 carries 1 / d_j and a column of the
+// right-hand sides d_j, d_j the scale of point j, so that rounding either at
+// 2^-63 of its largest entry loses the points of low density (xi 1e-9 of its
+// largest entry for densities 1e8 apart, where substitution keeps 2e-15), and
+// the inverse itself is not backward stable.
 #include "chol.cuh"
 
 #include <algorithm>
@@ -82,26 +82,6 @@ __global__ void __launch_bounds__(CB) chol_panel(double* __restrict__ L, int n, 
   for (int r = 0; r < rows; r++) L[(long)(i0 + r) * n + j0 + t] = a[r][t];
 }
 
-// The inverses of the diagonal blocks (a block each, column per lane); Linv is zero elsewhere.
-__global__ void __launch_bounds__(CB) inv_diag(const double* __restrict__ L, double* __restrict__ Linv, int n) {
-  __shared__ double d[CB][CB + 1];
-  const int i = threadIdx.x, j0 = blockIdx.x * CB, m = min(CB, n - j0);
-  for (int r = 0; r < CB; r++)
-    d[r][i] = r < m && i <= r ? L[(long)(j0 + r) * n + j0 + i] : (r == i ? 1.0 : 0.0);
-  __syncwarp();
-  double x[CB];
-#pragma unroll
-  for (int r = 0; r < CB; r++) {
-    double v = r == i ? 1.0 : 0.0;
-#pragma unroll
-    for (int t = 0; t < r; t++) v -= d[r][t] * x[t];
-    x[r] = v / d[r][r];
-  }
-#pragma unroll
-  for (int r = 0; r < CB; r++)
-    if (i <= r && r < m) Linv[(long)(j0 + r) * n + j0 + i] = x[r];
-}
-
 // Trailing update L[i][k] -= sum_t L[i][j0 + t] L[k][j0 + t], i >= k >= j0 + 32, 16 x 16 tiles.
 __global__ void __launch_bounds__(256) chol_update(double* __restrict__ L, int n, int j0) {
   __shared__ double sa[16][CB + 1], sb[16][CB + 1];
@@ -121,34 +101,6 @@ __global__ void __launch_bounds__(256) chol_update(double* __restrict__ L, int n
   L[(long)(i0 + i) * n + k0 + k] = v;
 }
 
-// C = alpha A B for the pairs of one level of the inverse (blockIdx.z = pair), 16 x 16 tiles.  step 0: T = B Ainv
-// (the pair's lower left block of L with the inverse above it); step 1: Linv's block = -Cinv T.
-__global__ void __launch_bounds__(256) inv_level(const double* __restrict__ L, double* __restrict__ Linv,
-                                                 double* __restrict__ T, int n, int h, int step) {
-  __shared__ double sa[16][17], sb[16][17];
-  const int c0 = 2 * h * blockIdx.z, r0 = c0 + h, rows = min(h, n - r0);
-  const int m0 = blockIdx.y * 16, n0 = blockIdx.x * 16, x = threadIdx.x & 15, y = threadIdx.x >> 4;
-  if (m0 >= rows || n0 >= h) return;
-  const int K = step ? rows : h;
-  double v = 0.0;
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    const bool ia = m0 + y < rows && k0 + x < K, ib = k0 + y < K && n0 + x < h;
-    sa[y][x] = ia ? (step ? Linv[(long)(r0 + m0 + y) * n + r0 + k0 + x] : L[(long)(r0 + m0 + y) * n + c0 + k0 + x])
-                  : 0.0;
-    sb[y][x] = ib ? (step ? T[(long)(r0 + k0 + y) * n + c0 + n0 + x] : Linv[(long)(c0 + k0 + y) * n + c0 + n0 + x])
-                  : 0.0;
-    __syncthreads();
-#pragma unroll
-    for (int t = 0; t < 16; t++) v += sa[y][t] * sb[t][x];
-    __syncthreads();
-  }
-  if (m0 + y < rows && n0 + x < h) {
-    const long o = (long)(r0 + m0 + y) * n + c0 + n0 + x;
-    if (step) Linv[o] = -v;
-    else T[o] = v;
-  }
-}
-
 }  // namespace
 
 cudaError_t chol_factor(const double* S, double* L, int n, int* bad, cudaStream_t s) {
@@ -162,35 +114,4 @@ cudaError_t chol_factor(const double* S, double* L, int n, int* bad, cudaStream_
     chol_update<<<dim3(t, t), 256, 0, s>>>(L, n, j);
   }
   return cudaGetLastError();
-}
-
-cudaError_t chol_inverse(const double* L, double* Linv, double* T, int n, const OzWork& w, cudaStream_t s) {
-  cudaError_t e0 = cudaMemsetAsync(Linv, 0, sizeof(double) * (size_t)n * n, s);
-  if (e0 != cudaSuccess) return e0;
-  inv_diag<<<(n + CB - 1) / CB, CB, 0, s>>>(L, Linv, n);
-  for (int h = CB; h < n; h *= 2) {
-    const int pairs = (n - h + 2 * h - 1) / (2 * h);
-    if (h < 256) {
-      const unsigned t = (unsigned)((h + 15) / 16);
-      for (int step = 0; step < 2; step++) inv_level<<<dim3(t, t, pairs), 256, 0, s>>>(L, Linv, T, n, h, step);
-      continue;
-    }
-    for (int p = 0; p < pairs; p++) {
-      const long c0 = 2L * h * p, r0 = c0 + h;
-      const int rows = std::min(h, (int)(n - r0));
-      cudaError_t e = oz_gemm_d(false, true, rows, h, h, L + r0 * n + c0, n, Linv + c0 * n + c0, n, T + r0 * n + c0, n,
-                                1.0, false, w, s);
-      if (e == cudaSuccess)
-        e = oz_gemm_d(false, true, rows, h, rows, Linv + r0 * n + r0, n, T + r0 * n + c0, n, Linv + r0 * n + c0, n,
-                      -1.0, false, w, s);
-      if (e != cudaSuccess) return e;
-    }
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t chol_apply(const double* Linv, double* X, double* Y, int n, int ldx, const OzWork& w, cudaStream_t s) {
-  cudaError_t e = oz_gemm_d(false, true, n, ldx, n, Linv, n, X, ldx, Y, ldx, 1.0, false, w, s);
-  if (e != cudaSuccess) return e;
-  return oz_gemm_d(true, true, n, ldx, n, Linv, n, Y, ldx, X, ldx, 1.0, false, w, s);
 }

@@ -333,12 +333,12 @@ inline bool fit_geometry(const int* grid_host, const double* lattice_host, const
 }
 
 // Scratch of the digit products of a fit and of its adjoint: the whole
-// operands of the metric, the solve and the products of depth kdeep (over the
+// operands of the metric and of the products of depth kdeep (over the
 // grid or its G set, npts x ndeep; 0: none), up to 1.25 GB (larger slabs
-// measured no faster for the metric).  At least what the solve's least slab
-// needs: without room for more the other products run on the FP64 pipe.
+// measured no faster for the metric).  At least what the metric's least slab
+// needs: a product without room for its own runs on the FP64 pipe.
 inline cudaError_t fit_scratch(OzWork& w, int npts, long ng, int nfunc, int ndeep, int kdeep, cudaStream_t s) {
-  const size_t least = oz_work_min(npts);
+  const size_t least = oz_work_min(nfunc);
   size_t want = std::max(oz_work_bytes(npts, (int)ng, nfunc, 1), oz_work_bytes(npts, (int)ng, npts, 1));
   if (ndeep > 0) want = std::max(want, std::max(oz_work_min(kdeep), oz_work_bytes(npts, ndeep, kdeep, 1)));
   return oz_alloc(w, std::max(least, std::min(want, (size_t)5 << 28)), least, s);

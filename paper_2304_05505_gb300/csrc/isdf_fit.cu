@@ -142,7 +142,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
 
   cudaStream_t s = (cudaStream_t)stream;
   // The all-FP64 form takes its products from exact digits on the tensor cores
-  // (metric 397 -> 15 ms, solve 75 -> 4 ms at 3x3x3 k, N_P = 600, 40^3 grid).
+  // (metric 397 -> 15 ms at 3x3x3 k, N_P = 600, 40^3 grid).
   // THC_MIXED keeps the FP64 pipe's sums: the solve passes a change of 1e-15 in
   // the metric on as 1e-12 (cond(S) 1e4), which changes FP32 roundings of the
   // contraction's operands, so that V would move by 1e-10 to 1e-7 per element.
@@ -166,7 +166,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
   double2 *Ugc = nullptr, *Bm = nullptr, *F = nullptr, *Xq = nullptr, *W = nullptr, *twd = nullptr, *phd = nullptr;
   double* svd = nullptr;
   unsigned* rmax = nullptr;
-  double *R = nullptr, *S = nullptr, *L = nullptr, *Linv = nullptr, *rPd = nullptr;
+  double *R = nullptr, *S = nullptr, *L = nullptr, *rPd = nullptr;
   OzWork oz;
   int *ptsd = nullptr, *gmd = nullptr, *flatd = nullptr, *bad = nullptr;
   cudaError_t e = cudaSuccess;
@@ -179,7 +179,6 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     if ((e = cudaMalloc(&R, sizeof(double) * (size_t)npts * ng)) != cudaSuccess) break;
     if ((e = cudaMalloc(&S, sizeof(double) * npq)) != cudaSuccess) break;
     if ((e = cudaMalloc(&L, sizeof(double) * npq)) != cudaSuccess) break;
-    if (dig && (e = cudaMalloc(&Linv, sizeof(double) * npq)) != cudaSuccess) break;
     if (dig && (e = fit_scratch(oz, npts, ng, nfunc, npts, nG, s)) != cudaSuccess) break;
     if ((e = cudaMalloc(&bad, sizeof(int))) != cudaSuccess) break;
     if ((e = cudaMalloc(&twd, sizeof(double2) * tw.size())) != cudaSuccess) break;
@@ -216,13 +215,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
       break;
     }
     mark(2);
-    if (dig) {
-      // (Bm is free once R and S are taken from it: scratch of the inverse and of the products)
-      if ((e = chol_inverse(L, Linv, (double*)Bm, npts, oz, s)) != cudaSuccess) break;
-      if ((e = chol_apply(Linv, R, (double*)Bm, npts, (int)ng, oz, s)) != cudaSuccess) break;
-    } else {
-      chol_solve<<<blocks(ng), TB, 0, s>>>(L, R, npts, ng);
-    }
+    chol_solve<<<blocks(ng), TB, 0, s>>>(L, R, npts, ng);
     mark(3);
     if (xi_out &&
         (e = cudaMemcpyAsync(xi_out, R, sizeof(double) * npts * ng, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
@@ -332,7 +325,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     set_global_error(std::string("thc_fit_kernel: ") + cudaGetErrorString(e));
     st = e == cudaErrorMemoryAllocation ? THC_ERR_OOM : THC_ERR_CUDA;
   }
-  void* ptrs[] = {Ugc, Bm, F, Xq, W, twd, R, S, L, Linv, rPd, phd, svd, rmax, ptsd, gmd, flatd, bad, Xq32, Bpl, eX, ps0, pbc, tcerr};
+  void* ptrs[] = {Ugc, Bm, F, Xq, W, twd, R, S, L, rPd, phd, svd, rmax, ptsd, gmd, flatd, bad, Xq32, Bpl, eX, ps0, pbc, tcerr};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   oz_free(oz);

@@ -442,7 +442,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
   double2 *Ugc = nullptr, *Bm = nullptr, *F = nullptr, *T = nullptr, *Gam = nullptr, *Aq = nullptr, *Bq = nullptr;
   double2 *Z = nullptr, *T1 = nullptr, *T2 = nullptr, *Uvp = nullptr, *G1 = nullptr, *G2 = nullptr, *twd = nullptr;
   OzWork oz;
-  double *R = nullptr, *S = nullptr, *L = nullptr, *Linv = nullptr, *Lam = nullptr, *Sbar = nullptr, *rPd = nullptr, *part = nullptr;
+  double *R = nullptr, *S = nullptr, *L = nullptr, *Lam = nullptr, *Sbar = nullptr, *rPd = nullptr, *part = nullptr;
   int *ptsd = nullptr, *gmd = nullptr, *flatd = nullptr, *bad = nullptr, *kqd = nullptr, *qkd = nullptr;
   // tensor-core state of the (q, G) contraction (THC_MIXED)
   float2* Aq32 = nullptr;
@@ -534,9 +534,6 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     if ((e = cudaMalloc(&R, sizeof(double) * (size_t)np * ng)) != cudaSuccess) break;
     if ((e = cudaMalloc(&S, sizeof(double) * npq)) != cudaSuccess) break;
     if ((e = cudaMalloc(&L, sizeof(double) * npq)) != cudaSuccess) break;
-    if (dig && (e = cudaMalloc(&Linv, sizeof(double) * npq)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&F, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&T, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
     gather_conj<<<blocks((long)np * nf), TB, 0, s>>>(U2, nf, ng, ptsd, np, Ugc);
     if ((e = dig ? gemm_z_best(A_MK, B_KN, np, (int)ng, nf, Ugc, nf, 0, U2, (int)ng, 0, Bm, (int)ng, 0, 1, oz, s)
                  : gemm_z(A_MK, B_KN, np, (int)ng, nf, Ugc, nf, 0, U2, (int)ng, 0, Bm, (int)ng, 0, 1, s)) !=
@@ -552,13 +549,9 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
       set_global_error("thc_vo_gradient: the Gram matrix of the points is not positive definite");
       break;
     }
-    if (dig) {
-      if ((e = chol_inverse(L, Linv, (double*)F, np, oz, s)) != cudaSuccess) break;
-      if ((e = chol_apply(Linv, R, (double*)F, np, (int)ng, oz, s)) != cudaSuccess) break;
-    } else {
-      chol_solve<<<blocks(ng), TB, 0, s>>>(L, R, np, ng);
-    }
-    // R now holds xi
+    chol_solve<<<blocks(ng), TB, 0, s>>>(L, R, np, ng);   // R now holds xi
+    if ((e = cudaMalloc(&F, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
+    if ((e = cudaMalloc(&T, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
     const long tot = (long)np * ng;
     // (THC_MIXED: the direct sums, as in step 4 below; an FFT's last bits would
     // come out of the solve there at 8e-8 of single entries of g)
@@ -658,11 +651,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     if ((e = dft_axis(F, false, T, tot, g1, (long)g2 * g3, twd + geo.off[0], s, dig)) != cudaSuccess) break;
     if ((e = cudaMalloc(&Lam, sizeof(double) * (size_t)np * ng)) != cudaSuccess) break;
     real_part<<<blocks(tot), TB, 0, s>>>(T, tot, Lam);
-    if (dig) {
-      if ((e = chol_apply(Linv, Lam, (double*)F, np, (int)ng, oz, s)) != cudaSuccess) break;
-    } else {
-      chol_solve<<<blocks(ng), TB, 0, s>>>(L, Lam, np, ng);
-    }
+    chol_solve<<<blocks(ng), TB, 0, s>>>(L, Lam, np, ng);
     if ((e = cudaMalloc(&Sbar, sizeof(double) * npq)) != cudaSuccess) break;
     // S-bar = -Lam xi^T
     if (ng <= OZ_MAX_K && oz.bytes >= oz_work_min((int)((ng + 1) / 2))) {
@@ -771,7 +760,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     st = e == cudaErrorMemoryAllocation ? THC_ERR_OOM : THC_ERR_CUDA;
   }
   void* ptrs[] = {Psi, Psivt, D,   M,   W,  Y,  Ge,  Ugc,   Bm,    F,    T,     Gam,  Aq,  Bq,  Z,
-                  T1,  T2,    Uvp, G1,  G2, twd, R,  S,     L,     Linv,  Lam,  Sbar,  rPd,  part, ptsd, gmd,
+                  T1,  T2,    Uvp, G1,  G2, twd, R,  S,     L,     Lam,  Sbar,  rPd,  part, ptsd, gmd,
                   flatd, bad, kqd, qkd, Aq32, Bpl, eA,  eB,  ps0, pbc, tcerr, Y32, A2, Uv32, eOrb, vt, cm, phd};
   for (void* p : ptrs)
     if (p) cudaFree(p);
