@@ -194,7 +194,7 @@ thc_status thc_profile_kernels(const thc_ctx* ctx, float core_ms[6]);
  * are then invalid; the context stays usable), else THC_OK. */
 thc_status thc_sync(thc_ctx* ctx);
 
-/* Test hooks for failure detection (no GPU fault is involved in either).
+/* Test hooks for failure detection (no GPU fault is involved in any).
  *
  * thc_debug_set_wait_limit: the limit, in SM clock cycles, of the bounded
  * device-side waits of the context's kernels (THC_MIXED; THC_ERR_UNSUPPORTED
@@ -212,6 +212,19 @@ thc_status thc_sync(thc_ctx* ctx);
  * nth < 0 disables the hook. */
 thc_status thc_debug_set_wait_limit(thc_ctx* ctx, long long cycles);
 thc_status thc_debug_fail_alloc(int nth);
+
+/* Test hooks of the THC_FP64 products' scratch.
+ *
+ * thc_debug_limit_scratch: from now on the products of calls made on the
+ * calling thread use at most `bytes` of the scratch that they have (they then
+ * go in slabs, and without any in FP64 on CUDA cores); bytes < 0: all of it.
+ *
+ * thc_debug_slab_plan (host only): the slabs of a product
+ * C[M][N] = sum over K A[M][K] B[K][N] of `batch` entries, complex or real,
+ * with `bytes` of scratch: plan[0..2] = batch entries, rows of A and columns of
+ * B in a slab.  THC_ERR_OOM where not even one output tile fits. */
+thc_status thc_debug_limit_scratch(long long bytes);
+thc_status thc_debug_slab_plan(int M, int N, int K, int batch, int real, size_t bytes, int plan[3]);
 
 /* The FP64 fused multiply-add rate of the current device, measured: a kernel
  * of independent FMA chains on every SM, timed with CUDA events on `stream`

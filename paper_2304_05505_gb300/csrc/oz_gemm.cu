@@ -642,6 +642,70 @@ cudaError_t slab(const Side& l, const Side& n, int K, int nb, const int* eL, con
   return launch<CX>(maps, g, eL, eN, out, w, s);
 }
 
+// Whether a complex product embeds A (as the columns) or B (as the lanes).
+// The time of the two choices, in units of 1 / 152 of a tile's 114 cycles per
+// real K: the tiles, and the planes of both operands (22 bytes read and
+// written per real at 6.5 TB/s).
+bool embed_a(int M, int N) {
+  auto cost = [](long lanes, long cols) {
+    return (double)((lanes + TL - 1) / TL) * ((cols + TN - 1) / TN) + 0.009 * (lanes + cols);
+  };
+  return cost(N, 2L * M) <= cost(2L * N, M);
+}
+
+thread_local long long g_limit = -1;   // test hook: most scratch of a product
+
+// Scratch for planes and exponents.
+size_t room_of(const OzWork& w) {
+  const size_t b = g_limit < 0 ? w.bytes : std::min(w.bytes, (size_t)g_limit);
+  return b > HEAD ? b - HEAD : 0;
+}
+
+// Slabs of a product that fit in `room` bytes: batch entries, lane rows and
+// column rows of each (of the sides' own rows).
+struct Slabs {
+  int bs, lrows, nrows;
+};
+
+// Whole batch entries where one fits, as even as they go; else whole tiles of
+// one entry: column tiles in up to half the room, lane tiles in what is left.
+// Rows are rounded down to tiles, so that room for one tile of each side is
+// enough and more of it never fails.
+bool plan_slabs(int lrows, bool lemb, int nrows, bool nemb, int Kr, int batch, size_t room, Slabs& p) {
+  auto lane = [&](int nb, int r) { return side_bytes(r, lemb ? 2L * r : r, Kr, nb); };
+  auto col = [&](int nb, int r) { return side_bytes(r, nemb ? 2L * r : r, Kr, nb); };
+  // the largest n <= most for which fits(n), 0 where there is none
+  auto largest = [](int most, auto fits) {
+    int lo = 0, hi = most + 1;
+    while (lo + 1 < hi) {
+      const int mid = lo + (hi - lo) / 2;
+      if (fits(mid)) lo = mid;
+      else hi = mid;
+    }
+    return lo;
+  };
+  p = Slabs{1, lrows, nrows};
+  const int bs = largest(batch, [&](int nb) { return lane(nb, lrows) + col(nb, nrows) <= room; });
+  if (bs > 0) {
+    const int parts = (batch + bs - 1) / bs;
+    p.bs = (batch + parts - 1) / parts;
+    return true;
+  }
+  const int lt = TL >> lemb, nt = TN >> nemb;   // rows of a tile
+  const size_t lane1 = lane(1, std::min(lt, lrows));
+  if (lane1 + col(1, std::min(nt, nrows)) > room) return false;
+  const int ct = std::max(1, largest((nrows + nt - 1) / nt, [&](int t) {
+    const size_t c = col(1, (int)std::min<long>(nrows, (long)t * nt));
+    return c <= room / 2 && c + lane1 <= room;
+  }));
+  p.nrows = (int)std::min<long>(nrows, (long)ct * nt);
+  const size_t left = room - col(1, p.nrows);
+  const int rt = largest((lrows + lt - 1) / lt,
+                         [&](int t) { return lane(1, (int)std::min<long>(lrows, (long)t * lt)) <= left; });
+  p.lrows = (int)std::min<long>(lrows, (long)rt * lt);
+  return true;
+}
+
 // out(lane i, column j) over batch entries, in slabs that fit the scratch.
 // pairs: the N side is embedded and out is complex [j / 2][i].
 template <int CX>
@@ -649,25 +713,11 @@ cudaError_t product(Side L, Side N, int K, int batch, double* out, long ldo, lon
                     bool acc, const OzWork& w, cudaStream_t s) {
   if (L.rows <= 0 || N.rows <= 0 || batch <= 0) return cudaSuccess;
   if (K <= 0 || (long)K * CX > OZ_MAX_K) return cudaErrorInvalidValue;   // the int64 sums stay below 2^62
-  const int Kr = K * CX, ldp = pad8i(Kr);
-  const size_t room = w.bytes > HEAD ? w.bytes - HEAD : 0;
-  const size_t nb1 = side_bytes(N.rows, plane_rows(N), Kr, 1), lb1 = side_bytes(L.rows, plane_rows(L), Kr, 1);
-  // slabs: whole batch entries when one fits; else rows of the lane side, then of the column side
-  int bs = batch, lrows = L.rows, nrows = N.rows;
-  if (nb1 + lb1 <= room) {
-    while (bs > 1 && side_bytes(N.rows, plane_rows(N), Kr, bs) + side_bytes(L.rows, plane_rows(L), Kr, bs) > room)
-      bs = (bs + 1) / 2;
-  } else {
-    bs = 1;
-    while (nrows > TN && side_bytes(nrows, N.emb ? 2L * nrows : nrows, Kr, 1) > room / 2) nrows = (nrows + 1) / 2;
-    nrows = std::min(N.rows, (nrows + TN - 1) / TN * TN);
-    const size_t left = room - std::min(room, side_bytes(nrows, N.emb ? 2L * nrows : nrows, Kr, 1));
-    while (lrows > TL && side_bytes(lrows, L.emb ? 2L * lrows : lrows, Kr, 1) > left) lrows = (lrows + 1) / 2;
-    lrows = std::min(L.rows, (lrows + TL - 1) / TL * TL);
-    while (lrows > TL && side_bytes(lrows, L.emb ? 2L * lrows : lrows, Kr, 1) > left) lrows -= TL;
-    if (side_bytes(nrows, N.emb ? 2L * nrows : nrows, Kr, 1) + side_bytes(lrows, L.emb ? 2L * lrows : lrows, Kr, 1) > room)
-      return cudaErrorMemoryAllocation;
-  }
+  const int Kr = K * CX;
+  Slabs pl;
+  if (!plan_slabs(L.rows, L.emb, N.rows, N.emb, Kr, batch, room_of(w), pl))
+    return cudaErrorMemoryAllocation;
+  const int bs = pl.bs, lrows = pl.lrows, nrows = pl.nrows;
   for (int b0 = 0; b0 < batch; b0 += bs) {
     const int nb = std::min(bs, batch - b0);
     for (int n0 = 0; n0 < N.rows; n0 += nrows) {
@@ -705,15 +755,35 @@ size_t oz_work_bytes(int M, int N, int K, int batch) {
   return HEAD + side_bytes(small, 2 * small, 2 * K, batch) + side_bytes(big, big, 2 * K, batch);
 }
 
-size_t oz_work_min(int K) { return HEAD + side_bytes(TN, 2 * TN, 2 * K, 1) + side_bytes(TL, 2 * TL, 2 * K, 1); }
+size_t oz_work_min(int K) { return HEAD + side_bytes(TN, TN, 2 * K, 1) + side_bytes(TL, TL, 2 * K, 1); }
+
+bool oz_fits(int M, int N, int K, int batch, bool real, const OzWork& w) {
+  const bool ea = !real && embed_a(M, N);
+  const int Kr = real ? K : 2 * K;
+  Slabs p;
+  return w.buf && Kr <= OZ_MAX_K && plan_slabs(N, !real && !ea, M, ea, Kr, batch, room_of(w), p);
+}
+
+void oz_limit(long long bytes) { g_limit = bytes; }
+
+bool oz_plan(int M, int N, int K, int batch, bool real, size_t bytes, int plan[3]) {
+  const bool ea = !real && embed_a(M, N);
+  Slabs p;
+  const bool ok = plan_slabs(N, !real && !ea, M, ea, real ? K : 2 * K, batch, bytes > HEAD ? bytes - HEAD : 0, p);
+  plan[0] = p.bs;
+  plan[1] = p.nrows;
+  plan[2] = p.lrows;
+  return ok;
+}
 
 cudaError_t oz_alloc(OzWork& w, size_t want, size_t least, cudaStream_t s) {
   cudaError_t e = cudaErrorMemoryAllocation;
-  for (w.bytes = std::max(want, least); w.bytes >= least; w.bytes /= 2) {
+  for (w.bytes = std::max(want, least);; w.bytes = std::max(least, w.bytes / 2)) {
     e = cudaMalloc((void**)&w.buf, w.bytes);
     if (e != cudaErrorMemoryAllocation) break;
     cudaGetLastError();
     w.buf = nullptr;
+    if (w.bytes <= least) break;
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(w.buf, 0, 64, s);
   if (e != cudaSuccess) oz_free(w);
@@ -738,13 +808,7 @@ cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int
                       int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s) {
   Side a{(const double*)A, M, la == A_KM ? 1L : (long)lda, la == A_KM ? (long)lda : 1L, sA, la == A_MK_CONJ, false};
   Side b{(const double*)B, N, lb == B_KN ? 1L : (long)ldb, lb == B_KN ? (long)ldb : 1L, sB, lb == B_NK_CONJ, false};
-  // The embedded operand may be either one.  The time of the two choices, in
-  // units of 1 / 152 of a tile's 114 cycles per real K: the tiles, and the
-  // planes of both operands (22 bytes read and written per real at 6.5 TB/s).
-  auto cost = [](long lanes, long cols) {
-    return (double)((lanes + TL - 1) / TL) * ((cols + TN - 1) / TN) + 0.009 * (lanes + cols);
-  };
-  if (cost(N, 2L * M) <= cost(2L * N, M)) {
+  if (embed_a(M, N)) {
     // embedded A as the columns, lanes along N: out[m][n] one double2 per lane
     a.emb = true;
     return product<2>(b, a, K, batch, (double*)C, ldc, sC, true, 1.0, false, w, s);
@@ -756,11 +820,13 @@ cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int
 
 cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
                         int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s) {
-  if (w.buf && oz_wins(M, N, K, batch) && w.bytes >= oz_work_min(K))
+  if (oz_wins(M, N, K, batch) && oz_fits(M, N, K, batch, false, w))
     return oz_gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, w, s);
   if (w.launches) ++*w.launches;
   return gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, s);
 }
+
+bool oz_lanes_fit(int M, int K, const OzWork& w) { return w.buf && side_bytes(M, 2L * M, 2 * K, 1) <= room_of(w); }
 
 size_t oz_lane_bytes(int N, int K) { return side_bytes(N, N, 2 * K, 1); }
 
@@ -772,7 +838,7 @@ cudaError_t oz_lane_prepare(const double2* B, int ldb, int N, int K, void* lanes
 
 cudaError_t oz_gemm_z_lanes(int la, int M, int N, int K, const double2* A, int lda, const void* lanes, double2* C,
                             int ldc, const OzWork& w, cudaStream_t s) {
-  if (w.bytes < HEAD + side_bytes(M, 2L * M, 2 * K, 1)) return cudaErrorMemoryAllocation;
+  if (!oz_lanes_fit(M, K, w)) return cudaErrorMemoryAllocation;
   const Side a{(const double*)A, M, la == A_KM ? 1L : (long)lda, la == A_KM ? (long)lda : 1L, 0, la == A_MK_CONJ, true};
   const Side b{nullptr, N, 1L, 1L, 0, false, false};
   int* eA = (int*)(w.buf + HEAD);

@@ -11,7 +11,17 @@ constexpr long OZ_MAX_K = 1L << 19;
 size_t oz_work_bytes(int M, int N, int K, int batch);
 size_t oz_work_min(int K);
 
-// Allocates scratch: `want` bytes, or halves of it down to `least` where the
+// Whether w has room for the digits of this product (complex, or real), whole
+// or in slabs.
+bool oz_fits(int M, int N, int K, int batch, bool real, const OzWork& w);
+
+// Test hooks: the most scratch that products on the calling thread use from now
+// on (negative: all they have), and the slabs of a product with `bytes` of it:
+// batch entries, rows of A and rows of B of a slab; false where none fits.
+void oz_limit(long long bytes);
+bool oz_plan(int M, int N, int K, int batch, bool real, size_t bytes, int plan[3]);
+
+// Allocates scratch: `want` bytes, or halves of it and at last `least` where the
 // device has no room for more (cudaErrorMemoryAllocation when it has not even
 // that), and clears its error word on `s`.  oz_free gives it back.
 cudaError_t oz_alloc(OzWork& w, size_t want, size_t least, cudaStream_t s);
@@ -31,6 +41,7 @@ cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int
 // The same product of A (any layout) with a B of N columns stored [k][n] whose
 // digits were prepared once: oz_lane_bytes of device memory at `lanes`.
 size_t oz_lane_bytes(int N, int K);
+bool oz_lanes_fit(int M, int K, const OzWork& w);   // room in w for the digits of A (M rows)
 cudaError_t oz_lane_prepare(const double2* B, int ldb, int N, int K, void* lanes, cudaStream_t s);
 cudaError_t oz_gemm_z_lanes(int la, int M, int N, int K, const double2* A, int lda, const void* lanes, double2* C,
                             int ldc, const OzWork& w, cudaStream_t s);

@@ -412,6 +412,9 @@ struct Blocks {
     const size_t least = std::max(oz_work_bytes(MS, MS, nfunc, 1), oz_work_min(npts));
     if (e == cudaSuccess)
       e = oz_alloc(w, std::max(least, std::min(oz_work_bytes(TP, ncand, (npts + 1) / 2, 1), (size_t)1 << 30)), least, s);
+    if (e == cudaSuccess && !(oz_fits(MS, MS, nfunc, 1, false, w) && oz_fits(MS, MS, npts, 1, true, w) &&
+                              oz_lanes_fit(TP, nfunc, w) && oz_fits(TP, ncand, npts, 1, true, w)))
+      e = cudaErrorMemoryAllocation;
     return e;
   }
   void drop() {

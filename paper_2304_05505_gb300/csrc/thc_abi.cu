@@ -922,6 +922,16 @@ thc_status thc_debug_fail_alloc(int nth) {
   return THC_OK;
 }
 
+thc_status thc_debug_limit_scratch(long long bytes) {
+  oz_limit(bytes);
+  return THC_OK;
+}
+
+thc_status thc_debug_slab_plan(int M, int N, int K, int batch, int real, size_t bytes, int plan[3]) {
+  if (M < 1 || N < 1 || K < 1 || batch < 1 || !plan) return THC_ERR_ARG;
+  return oz_plan(M, N, K, batch, real != 0, bytes, plan) ? THC_OK : THC_ERR_OOM;
+}
+
 thc_status thc_sync(thc_ctx* c) {
   if (!c) return THC_ERR_ARG;
   // the error word comes back with the stream's last work: one wait

@@ -654,7 +654,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     chol_solve<<<blocks(ng), TB, 0, s>>>(L, Lam, np, ng);
     if ((e = cudaMalloc(&Sbar, sizeof(double) * npq)) != cudaSuccess) break;
     // S-bar = -Lam xi^T
-    if (ng <= OZ_MAX_K && oz.bytes >= oz_work_min((int)((ng + 1) / 2))) {
+    if (oz_fits(np, np, (int)ng, 1, true, oz)) {
       if ((e = oz_gemm_d(false, false, np, np, (int)ng, Lam, ng, R, ng, Sbar, np, -1.0, false, oz, s)) != cudaSuccess)
         break;
     } else {

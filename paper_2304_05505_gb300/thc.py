@@ -33,7 +33,7 @@ EXPORTS = ["thc_create", "thc_memory_bytes", "thc_set_collocation", "thc_set_ker
            "thc_select_points", "thc_fit_kernel", "thc_profile_kernels", "thc_mlp_features", "thc_mlp_score",
            "thc_mlp_workspace_bytes", "thc_mlp_train_step", "thc_mlp_candidates", "thc_select_points_among",
            "thc_debug_set_wait_limit", "thc_debug_fail_alloc", "thc_rebuild_kernel", "thc_build_K",
-           "thc_measure_fp64_rate", "thc_vo_gradient"]
+           "thc_measure_fp64_rate", "thc_vo_gradient", "thc_debug_limit_scratch", "thc_debug_slab_plan"]
 
 MLP_NPARAM = 8641
 
@@ -80,6 +80,8 @@ def load(path: str | None = None) -> ctypes.CDLL:
     lib.thc_sync.argtypes = [vp]
     lib.thc_debug_set_wait_limit.argtypes = [vp, ctypes.c_longlong]
     lib.thc_debug_fail_alloc.argtypes = [ip]
+    lib.thc_debug_limit_scratch.argtypes = [ctypes.c_longlong]
+    lib.thc_debug_slab_plan.argtypes = [ip, ip, ip, ip, ip, ctypes.c_size_t, ctypes.POINTER(ip)]
     lib.thc_measure_fp64_rate.argtypes = [vp, ctypes.POINTER(ctypes.c_double)]
     lib.thc_kconv_noalloc.argtypes = [dp, dp, dp, ip, ip, ip, ctypes.c_long, vp]
     lib.thc_select_points.argtypes = [dp, ip, ip, ip, ctypes.c_double, ctypes.POINTER(ctypes.c_int),
@@ -271,6 +273,22 @@ def thc_sync(ctx) -> None:
 def thc_debug_set_wait_limit(ctx, cycles: int) -> None:
     """Test hook: the limit of the context's bounded device waits (see include/thc.h)."""
     _check(load().thc_debug_set_wait_limit(ctx, int(cycles)), "thc_debug_set_wait_limit", ctx)
+
+
+def thc_debug_limit_scratch(nbytes: int) -> None:
+    """Test hook: most scratch of the FP64 products of later calls on this thread (< 0: no limit)."""
+    _check(load().thc_debug_limit_scratch(int(nbytes)), "thc_debug_limit_scratch")
+
+
+def thc_debug_slab_plan(M: int, N: int, K: int, batch: int, real: int, nbytes: int):
+    """(batch entries, rows of A, columns of B) of a slab of a product with `nbytes` of scratch, None where none
+    fits (host only)."""
+    p = (ctypes.c_int * 3)()
+    code = load().thc_debug_slab_plan(int(M), int(N), int(K), int(batch), int(real), int(nbytes), p)
+    if code == 2:
+        return None
+    _check(code, "thc_debug_slab_plan")
+    return tuple(p)
 
 
 def thc_debug_fail_alloc(nth: int) -> None:
