@@ -23,6 +23,18 @@
 // any depth, where the FP64 kernel's running sums leave 4e-16 (K = 60) to
 // 3e-15 (K = 3840).
 //
+// That is an error relative to the largest entries of the two rows.  Where a
+// row's large entries all meet small ones of the other row, as those of a
+// compact basis function far from an orbital, sum |a||b| is far below their
+// product and an FP64 loop would do better.  So every product is checked
+// first: with m = |x| 2^-e of every entry (bf16, of the larger of re and im),
+// S = sum m_a m_b per result, in one product on the tensor cores.  Where S is
+// below 2^-10 (0.06 % of S4b's entries and 0.3 to 0.6 % of THC-AO-K's at
+// benzene-shaped cells) the result is computed in FP64 instead, as is one
+// whose rows hold a NaN or an Inf: single entries by a warp each, tiles with
+// many of them as gemm_z computes them.  At S = 2^-10 the digits leave 5e-17 of
+// sum |a||b| (K = 1200, twice that at most), FP64 sums 3e-16.
+//
 // Complex products run as real ones with K = 2 K: one operand plain
 // (interleaved), the smaller one embedded as rows (re, -im) and (im, re).
 //
@@ -65,13 +77,33 @@ constexpr int EC = TN / 4;                             // columns of an epilogue
 constexpr int NB_ROW = 2047;                           // biased exponent of a row with a NaN or an Inf
 constexpr size_t HEAD = 1024;                          // bytes before the planes: the error block
 
+// The check of a product: stages of 64 K of the magnitudes, 128B swizzle
+constexpr int MK = 64;
+constexpr uint32_t MLB = TL * MK * 2, MCB = TN * MK * 2, MSTAGE = MLB + MCB;   // 16 KB + 10 KB
+constexpr int MSTAGES = 6, MEPI = 8, MNT = 32 * (4 + MEPI);
+constexpr size_t MSMEM = MSTAGES * MSTAGE + 1024 + 256;
+constexpr float CHECK = 0x1p-10f;                      // S below which digits are not enough
+constexpr int MANY = 80;                               // entries of a warp's 32 x 40 from which the tile goes whole
+constexpr int EPU = 64;                                // room for single entries, per tile
+
 static_assert(SMEM <= 232448, "227 KB of shared memory per block");
 
 struct OzMaps {
   CUtensorMap l, n;
 };
 
+// What the check leaves: cnt[0] tiles (flag 1, listed in tiles) and cnt[1]
+// entries (tile, lane row << 8 | column row of it) to be computed in FP64.
+struct OzList {
+  int *cnt, *flag, *tiles;
+  uint2* ents;
+  int cap;
+};
+
 struct OzShape {
+  int lr, nr;        // rows of the two sides, and of a tile (an embedded row counts two)
+  int lt, nt;
+  int mst;           // stages of the check
   int nl, nn;        // valid lanes (rows of the lane operand) and columns
   int nst;           // K stages
   int tl, tn;        // tiles
@@ -83,6 +115,14 @@ struct OzShape {
   double alpha;
   long ldo, sbo;     // doubles (pairs: double2)
 };
+
+// unit -> (batch entry, lane tile, column tile), column tiles fastest: CTAs side by side share the lane tile
+__device__ __forceinline__ void decode(const OzShape& g, long u, int& b, int& li, int& ni) {
+  const unsigned r = (unsigned)u / (unsigned)g.tn;
+  ni = (int)((unsigned)u - r * (unsigned)g.tn);
+  b = (int)(r / (unsigned)g.tl);
+  li = (int)(r - (unsigned)b * (unsigned)g.tl);
+}
 
 __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t accumulate) {
   // kind::f16, D f32 (bit 4), A and B bf16 (bits 7 and 10), K-major, N >> 3 at bit 17, M >> 4 at bit 24
@@ -160,7 +200,7 @@ __device__ __forceinline__ double flip(double x) {
 
 __global__ void __launch_bounds__(NT, 1)
 oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict__ eL, const int* __restrict__ eN,
-          double* __restrict__ out, int* err) {
+          double* __restrict__ out, OzList f, int* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE);
@@ -201,13 +241,8 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const int nchunk = (g.nst + CHUNK_ST - 1) / CHUNK_ST;
-  // unit -> (batch entry, lane tile, column tile), column tiles fastest: CTAs side by side share the lane tile
-  auto decode = [&](long u, int& b, int& li, int& ni) {
-    const unsigned r = (unsigned)u / (unsigned)g.tn;
-    ni = (int)((unsigned)u - r * (unsigned)g.tn);
-    b = (int)(r / (unsigned)g.tl);
-    li = (int)(r - (unsigned)b * (unsigned)g.tl);
-  };
+  // tiles that the check has left to FP64 are passed over by every warp
+  const bool holes = f.cnt && *f.cnt != 0;
 
   // (warps 0 and 1 keep all lanes in their loops and elect one per batch of
   // copies or MMAs: see tc_gemm.cu)
@@ -216,8 +251,9 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
       uint32_t it = 0;
       bool ok = true;
       for (long u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
+        if (holes && f.flag[u]) continue;
         int b, li, ni;
-        decode(u, b, li, ni);
+        decode(g, u, b, li, ni);
         for (int st = 0; st < g.nst; st++, it++) {
           const uint32_t sl = it & 1;
           if (!mbar_wait_uniform(EMPTY(sl), ((it >> 1) & 1) ^ 1, err, 2)) { ok = false; break; }
@@ -240,6 +276,7 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
       uint32_t it = 0, ch = 0;
       bool ok = true;
       for (long u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
+        if (holes && f.flag[u]) continue;
         for (int c = 0; c < nchunk && ok; c++, ch++) {
           const int st1 = min(g.nst, (c + 1) * CHUNK_ST);
           for (int st = c * CHUNK_ST; st < st1; st++, it++) {
@@ -283,8 +320,9 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
     uint32_t ch = 0;
     bool ok = true;
     for (long u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
+      if (holes && f.flag[u]) continue;
       int b, li, ni;
-      decode(u, b, li, ni);
+      decode(g, u, b, li, ni);
       long long acc[EC];
       float rest[EC];
 #pragma unroll
@@ -339,8 +377,10 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
             const bool two = col + 1 < g.nn;
             const int e0 = en[col >> g.nsh], e1 = two ? en[(col + 1) >> g.nsh] : 0;
             double x = round_sum(acc[j], rest[j], es + e0), y = two ? round_sum(acc[j + 1], rest[j + 1], es + e1) : 0.0;
-            if (ei == NB_ROW || e0 == NB_ROW) x = __longlong_as_double(0x7ff8000000000000ll);
-            if (ei == NB_ROW || e1 == NB_ROW) y = __longlong_as_double(0x7ff8000000000000ll);
+            if (!f.cnt) {   // (else rows with a NaN or an Inf are left to FP64)
+              if (ei == NB_ROW || e0 == NB_ROW) x = __longlong_as_double(0x7ff8000000000000ll);
+              if (ei == NB_ROW || e1 == NB_ROW) y = __longlong_as_double(0x7ff8000000000000ll);
+            }
             if (g.alpha < 0) {
               x = flip(x);
               y = flip(y);
@@ -368,6 +408,291 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
   tc_fence_after();
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// the check, and what it leaves to FP64
+// ---------------------------------------------------------------------------
+
+// K-major tile of 64 bf16, 128B swizzle, 8-row groups 1024 B apart.
+__device__ __forceinline__ uint64_t desc128(uint32_t addr) {
+  return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
+         ((uint64_t)2 << 61);
+}
+
+// S of every entry, tiles as in oz_kernel (rows of an embedded side counted
+// once, so its box is half used): warp 0 loads, warp 1 multiplies into one of
+// two accumulators, warps 4-11 compare (32 lanes x 40 columns each).  It reads
+// a fifteenth of the product's planes and multiplies a 68th to a 136th as much.
+__global__ void __launch_bounds__(MNT, 1)
+oz_check_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict__ eL, const int* __restrict__ eN,
+                OzList f, int* err) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = (uint64_t*)(smem + MSTAGES * MSTAGE);
+  uint32_t* tmem_slot = (uint32_t*)(bars + 17);
+  const uint32_t sbase = smem_u32(smem), bar0 = smem_u32(bars);
+  auto FULL = [&](int s) { return bar0 + 8u * s; };
+  auto EMPTY = [&](int s) { return bar0 + 8u * (6 + s); };
+  auto AFULL = [&](int c) { return bar0 + 8u * (12 + c); };
+  auto AEMPTY = [&](int c) { return bar0 + 8u * (14 + c); };
+  const uint32_t DONE = bar0 + 8u * 16;
+  static_assert(MSTAGES == 6, "barrier slots");
+
+  __shared__ int abort_flag;
+  if (threadIdx.x == 0) abort_flag = *(volatile int*)err;
+  __syncthreads();
+  if (abort_flag) return;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < MSTAGES; s++) {
+      mbar_init(FULL(s), 1);
+      mbar_init(EMPTY(s), 1);
+    }
+    for (int c = 0; c < 2; c++) {
+      mbar_init(AFULL(c), 1);
+      mbar_init(AEMPTY(c), MEPI);
+    }
+    mbar_init(DONE, 1);
+    mbar_fence_init();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(256)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+
+  if (warp == 0) {
+    uint32_t it = 0;
+    bool ok = true;
+    for (long u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
+      int b, li, ni;
+      decode(g, u, b, li, ni);
+      for (int st = 0; st < g.mst; st++, it++) {
+        const uint32_t sl = it % MSTAGES;
+        if (!mbar_wait_uniform(EMPTY(sl), ((it / MSTAGES) & 1) ^ 1, err, 2)) { ok = false; break; }
+        if (elect_one()) {
+          mbar_expect_tx(FULL(sl), MSTAGE);
+          tma_load_3d(sbase + sl * MSTAGE, &maps.l, FULL(sl), st * MK, li * g.lt, b);
+          tma_load_3d(sbase + sl * MSTAGE + MLB, &maps.n, FULL(sl), st * MK, ni * g.nt, b);
+        }
+        __syncwarp();
+      }
+    }
+    // the copies still in flight land before the CTA exits
+    const uint32_t n = it < MSTAGES ? it : MSTAGES;
+    for (uint32_t j = it - n; j < it; j++) mbar_drain(FULL(j % MSTAGES), (j / MSTAGES) & 1);
+  } else if (warp == 1) {
+    uint32_t it = 0, local = 0;
+    bool ok = true;
+    for (long u = blockIdx.x; u < g.units && ok; u += gridDim.x, local++) {
+      const uint32_t set = local & 1;
+      if (!mbar_wait_uniform(AEMPTY(set), ((local >> 1) & 1) ^ 1, err, 4)) break;
+      for (int st = 0; st < g.mst; st++, it++) {
+        const uint32_t sl = it % MSTAGES;
+        if (!mbar_wait_uniform(FULL(sl), (it / MSTAGES) & 1, err, 8)) { ok = false; break; }
+        tc_fence_after();
+        const uint64_t al = desc128(sbase + sl * MSTAGE), bn = desc128(sbase + sl * MSTAGE + MLB);
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < MK / 16; kk++) mma_bf16(tmem + 128 * set, al + 2 * kk, bn + 2 * kk, st > 0 || kk > 0);
+          commit(EMPTY(sl));
+          if (st == g.mst - 1) commit(AFULL(set));
+        }
+        __syncwarp();
+      }
+    }
+    // every MMA issued complete before TMEM is released
+    if (elect_one()) commit(DONE);
+    __syncwarp();
+    mbar_drain(DONE, 0);
+  } else if (warp >= 4) {
+    const int q = warp & 3, h = (warp - 4) >> 2;            // lane quadrant, column half
+    constexpr int MC = TN / 2;
+    const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16) + MC * h;
+    uint32_t local = 0;
+    for (long u = blockIdx.x; u < g.units; u += gridDim.x, local++) {
+      int b, li, ni;
+      decode(g, u, b, li, ni);
+      const uint32_t set = local & 1;
+      // rows with a NaN or an Inf: of this lane, and of the columns as bits
+      const int r = 32 * q + lane, c0 = MC * h;
+      const bool row = r < g.lt && li * g.lt + r < g.lr;
+      const bool nb = row && eL[(long)b * g.el + li * g.lt + r] == NB_ROW;
+      auto column = [&](int c) { return c < g.nt && ni * g.nt + c < g.nr; };
+      auto bad = [&](int c) { return column(c) && eN[(long)b * g.en + ni * g.nt + c] == NB_ROW; };
+      const unsigned long long cols = (unsigned long long)__ballot_sync(0xffffffffu, column(c0 + lane)) |
+                                      (unsigned long long)__ballot_sync(0xffffffffu, lane < MC - 32 && column(c0 + 32 + lane)) << 32;
+      unsigned long long m = (unsigned long long)__ballot_sync(0xffffffffu, bad(c0 + lane)) |
+                             (unsigned long long)__ballot_sync(0xffffffffu, lane < MC - 32 && bad(c0 + 32 + lane)) << 32;
+      if (nb) m = ~0ull;
+      if (!__all_sync(0xffffffffu, mbar_wait(AFULL(set), (local >> 1) & 1, err, 16))) break;
+      tc_fence_after();
+#pragma unroll
+      for (int j0 = 0; j0 < MC; j0 += 10) {
+        float v[10];
+        tmem_ld10(tl + 128 * set + j0, v);
+#pragma unroll
+        for (int j = 0; j < 10; j++)
+          if (v[j] > 0.f && v[j] < CHECK) m |= 1ull << (j0 + j);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(AEMPTY(set));
+      m = row ? m & cols : 0ull;
+      const int mine = __popcll(m), all = (int)__reduce_add_sync(0xffffffffu, (unsigned)mine);
+      if (all == 0) continue;
+      bool whole = g.acc || all > MANY;      // (an entry that is added to cannot be overwritten later)
+      if (!whole) {
+        int off = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, off, o);
+          if (lane >= o) off += t;
+        }
+        int base = 0;
+        if (lane == 0) base = atomicAdd(f.cnt + 1, all);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        whole = base < 0 || base > f.cap - all;   // no room: the slots up to cap are left empty
+        for (int i = base + off - mine; m && base >= 0; m &= m - 1, i++)
+          if (i < f.cap)
+            f.ents[i] = whole ? make_uint2(~0u, 0u)
+                              : make_uint2((unsigned)u, (unsigned)(r << 8 | (c0 + __ffsll((long long)m) - 1)));
+      }
+      if (whole && lane == 0 && atomicExch(f.flag + u, 1) == 0) f.tiles[atomicAdd(f.cnt, 1)] = (int)u;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
+}
+
+// A side in memory: element (r, k) of batch entry b at src[b sb + r lr + k lk].
+struct Source {
+  const double* src;
+  long sb, lr, lk;
+  bool conj;
+};
+
+template <int CX>
+struct Num;
+template <>
+struct Num<1> {
+  double x;
+  __device__ __forceinline__ void fma_(const Num& a, const Num& b) { x = fma(a.x, b.x, x); }
+  __device__ __forceinline__ void add(int o) { x += __shfl_xor_sync(0xffffffffu, x, o); }
+};
+template <>
+struct Num<2> {
+  double x, y;
+  // the order of gemm_z
+  __device__ __forceinline__ void fma_(const Num& a, const Num& b) {
+    x = fma(a.x, b.x, x);
+    x = fma(-a.y, b.y, x);
+    y = fma(a.x, b.y, y);
+    y = fma(a.y, b.x, y);
+  }
+  __device__ __forceinline__ void add(int o) {
+    x += __shfl_xor_sync(0xffffffffu, x, o);
+    y += __shfl_xor_sync(0xffffffffu, y, o);
+  }
+};
+
+template <int CX>
+__device__ __forceinline__ Num<CX> element(const Source& s, int b, int r, int k) {
+  const double* p = s.src + (b * s.sb + r * s.lr + k * s.lk) * CX;
+  if constexpr (CX == 2) {
+    const double2 v = *reinterpret_cast<const double2*>(p);
+    return Num<2>{v.x, s.conj ? -v.y : v.y};
+  } else {
+    return Num<1>{*p};
+  }
+}
+
+template <int CX>
+__device__ __forceinline__ void put(double* __restrict__ out, const OzShape& g, int b, int r, int c, Num<CX> v) {
+  const double sg = g.alpha < 0 ? -1.0 : 1.0;
+  if constexpr (CX == 2) {
+    // embedded columns: double2 along the rows; embedded lanes: two doubles a row
+    double* o = out + (g.pairs ? 2 * (b * g.sbo + c * g.ldo + r) : b * g.sbo + c * g.ldo + 2L * r);
+    *reinterpret_cast<double2*>(o) = make_double2(sg * v.x, sg * v.y);
+  } else {
+    double* o = out + b * g.sbo + c * g.ldo + r;
+    *o = g.acc ? *o + sg * v.x : sg * v.x;
+  }
+}
+
+// The listed tiles (32 LI rows x 8 CJ columns, a block each, as gemm_kernel
+// sums them) and entries (a warp each).  Two FP64 multiply-adds a clock and SM
+// bind both.
+template <int CX, int LI, int CJ>
+__global__ void __launch_bounds__(256) oz_exact_kernel(Source l, Source n, int K, OzShape g, OzList f,
+                                                       double* __restrict__ out, const int* err) {
+  typedef Num<CX> T;
+  constexpr int BK = 8, R = 32 * LI, C = 8 * CJ;
+  __shared__ T ls[BK][R + 1], ns[BK][C + 1];
+  const int ntile = f.cnt[0], nent = (int)min((unsigned)f.cnt[1], (unsigned)f.cap);
+  if ((ntile | nent) == 0 || *(volatile const int*)err) return;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int t = blockIdx.x; t < ntile; t += gridDim.x) {
+    int b, li, ni;
+    decode(g, f.tiles[t], b, li, ni);
+    const int r0 = li * R, c0 = ni * C;
+    T acc[LI][CJ];
+#pragma unroll
+    for (int i = 0; i < LI; i++)
+#pragma unroll
+      for (int j = 0; j < CJ; j++) acc[i][j] = T{};
+    for (int k0 = 0; k0 < K; k0 += BK) {
+      for (int e = threadIdx.x; e < R * BK; e += 256) {
+        const int kk = l.lk == 1 ? e % BK : e / R, r = l.lk == 1 ? e / BK : e % R;
+        ls[kk][r] = r0 + r < g.lr && k0 + kk < K ? element<CX>(l, b, r0 + r, k0 + kk) : T{};
+      }
+      for (int e = threadIdx.x; e < C * BK; e += 256) {
+        const int kk = n.lk == 1 ? e % BK : e / C, c = n.lk == 1 ? e / BK : e % C;
+        ns[kk][c] = c0 + c < g.nr && k0 + kk < K ? element<CX>(n, b, c0 + c, k0 + kk) : T{};
+      }
+      __syncthreads();
+#pragma unroll
+      for (int kk = 0; kk < BK; kk++) {
+        T lv[LI];
+#pragma unroll
+        for (int i = 0; i < LI; i++) lv[i] = ls[kk][tx + 32 * i];
+#pragma unroll
+        for (int j = 0; j < CJ; j++) {
+          const T nv = ns[kk][ty + 8 * j];
+#pragma unroll
+          for (int i = 0; i < LI; i++) acc[i][j].fma_(nv, lv[i]);
+        }
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < LI; i++)
+#pragma unroll
+      for (int j = 0; j < CJ; j++) {
+        const int r = r0 + tx + 32 * i, c = c0 + ty + 8 * j;
+        if (r < g.lr && c < g.nr) put<CX>(out, g, b, r, c, acc[i][j]);
+      }
+  }
+  for (int i = blockIdx.x * 8 + ty; i < nent; i += gridDim.x * 8) {
+    const uint2 e = f.ents[i];
+    if (e.x == ~0u || f.flag[e.x]) continue;
+    int b, li, ni;
+    decode(g, e.x, b, li, ni);
+    const int r = li * R + (int)(e.y >> 8), c = ni * C + (int)(e.y & 255);
+    T v{};
+#pragma unroll 4
+    for (int k = tx; k < K; k += 32) v.fma_(element<CX>(n, b, c, k), element<CX>(l, b, r, k));
+    for (int o = 16; o > 0; o >>= 1) v.add(o);
+    if (tx == 0) put<CX>(out, g, b, r, c, v);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -424,6 +749,33 @@ __device__ __forceinline__ long long fixed62(double x, int E) {
   return (long long)u < 0 ? -(long long)m : (long long)m;
 }
 
+// u 2^-e (u: the bits of a nonnegative double of a row of biased exponent E) truncated to bf16; at least 2^-41 for u > 0.
+__device__ __forceinline__ uint32_t mag16(unsigned long long u, int E) {
+  const int ex = (int)(u >> 52), d = E - ex;
+  if (u == 0 || E == NB_ROW) return 0;
+  return ex == 0 || d > 40 ? 86u << 7 : (uint32_t)(126 - d) << 7 | (uint32_t)(u >> 45 & 0x7f);
+}
+
+// The magnitudes of 8 consecutive reals of a row (CX = 2: of 4 complex values).
+template <int CX>
+__device__ __forceinline__ void put_mags(const double* x, int E, uint16_t* dst) {
+  uint32_t w[4 / CX];
+#pragma unroll
+  for (int i = 0; i < 4 / CX; i++) {
+    uint32_t v[2];
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+      const double* y = x + (2 * i + j) * CX;
+      unsigned long long u = (unsigned long long)__double_as_longlong(y[0]) & ~(1ull << 63);
+      if (CX == 2) u = max(u, (unsigned long long)__double_as_longlong(y[CX - 1]) & ~(1ull << 63));
+      v[j] = mag16(u, E);
+    }
+    w[i] = v[0] | v[1] << 16;
+  }
+  if constexpr (CX == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+  else *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // The planes of 8 consecutive reals of a row: digits from the last, each
 // balanced digit taken off with its carry; the plane value 2^(-9 s) d is formed
 // by adding d to the bits of 1.5 2^(23 - 9 s) and subtracting that number.
@@ -470,7 +822,7 @@ __device__ __forceinline__ void put8(const double* x, int E, uint16_t* dst, long
 template <int CX, bool EMB>
 __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ src, long sb, long lr, int rows, int K,
                                                      int conj, const int* __restrict__ e, uint16_t* __restrict__ dst,
-                                                     int ldp) {
+                                                     int ldp, uint16_t* __restrict__ mag, int ldm) {
   const int ng = (K * CX + 7) / 8;
   const long i = (long)blockIdx.x * 256 + threadIdx.x;
   if (i >= (long)rows * ng) return;
@@ -490,7 +842,9 @@ __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ 
     }
   }
   const long plane = (long)rows * (EMB ? 2 : 1) * ldp;
-  put8<EMB>(x, e[b * rows + r], dst + b * ND * plane + (long)r * (EMB ? 2 : 1) * ldp + k0 * CX, plane, ldp);
+  const int E = e[b * rows + r];
+  put8<EMB>(x, E, dst + b * ND * plane + (long)r * (EMB ? 2 : 1) * ldp + k0 * CX, plane, ldp);
+  if (mag) put_mags<CX>(x, E, mag + (b * rows + r) * ldm + k0);
 }
 
 // The same for row-contiguous sources (stride lk along K): a block turns a
@@ -498,7 +852,7 @@ __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ 
 template <int CX, bool EMB>
 __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ src, long sb, long lk, int rows, int K,
                                                      int conj, const int* __restrict__ e, uint16_t* __restrict__ dst,
-                                                     int ldp) {
+                                                     int ldp, uint16_t* __restrict__ mag, int ldm) {
   constexpr int KT = 64 / CX;                       // 64 reals of K
   __shared__ double t[KT][33 * CX];
   const int r0 = blockIdx.x * 32, k0 = blockIdx.y * KT;
@@ -529,8 +883,9 @@ __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ 
     }
   }
   const long plane = (long)rows * (EMB ? 2 : 1) * ldp;
-  put8<EMB>(x, e[b * rows + r0 + r], dst + b * ND * plane + (long)(r0 + r) * (EMB ? 2 : 1) * ldp + k0 * CX + 8 * c,
-            plane, ldp);
+  const int E = e[b * rows + r0 + r];
+  put8<EMB>(x, E, dst + b * ND * plane + (long)(r0 + r) * (EMB ? 2 : 1) * ldp + k0 * CX + 8 * c, plane, ldp);
+  if (mag) put_mags<CX>(x, E, mag + (b * rows + r0 + r) * ldm + k0 + 8 / CX * c);
 }
 
 // One operand of a product: `rows` rows of K elements, element (r, k) at
@@ -546,32 +901,72 @@ int pad8i(int x) { return (x + 7) & ~7; }
 
 long plane_rows(const Side& s) { return s.emb ? 2L * s.rows : s.rows; }
 
+size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Scratch of one operand: exponents, digit planes, magnitudes (null: none are made).
+struct Planes {
+  int* e;
+  uint16_t *pl, *mag;
+};
+
+size_t exp_bytes(long rows, int batch) { return align256(sizeof(int) * (size_t)rows * batch); }
+size_t digit_bytes(long rows, bool emb, int K, int CX, int batch) {
+  return align256(2 * (size_t)ND * (rows << emb) * pad8i(K * CX) * batch);
+}
+size_t side_bytes(long rows, bool emb, int K, int CX, int batch) {
+  return exp_bytes(rows, batch) + digit_bytes(rows, emb, K, CX, batch) + align256(2 * (size_t)rows * pad8i(K) * batch);
+}
+
+Planes planes_at(void* at, long rows, bool emb, int K, int CX, int batch) {
+  unsigned char* p = (unsigned char*)at + exp_bytes(rows, batch);
+  return Planes{(int*)at, (uint16_t*)p, (uint16_t*)(p + digit_bytes(rows, emb, K, CX, batch))};
+}
+
+long tiles_of(long rows, bool emb, int t) { return ((rows << emb) + t - 1) / t; }
+
+// Scratch of the check's list, for `units` tiles.
+size_t list_bytes(long units) { return align256(64 + 2 * sizeof(int) * (size_t)units) + align256(sizeof(uint2) * EPU * (size_t)units); }
+
+OzList list_at(void* at, long units) {
+  OzList f;
+  f.cnt = (int*)at;
+  f.flag = f.cnt + 16;
+  f.tiles = f.flag + units;
+  f.ents = (uint2*)((unsigned char*)at + align256(64 + 2 * sizeof(int) * (size_t)units));
+  f.cap = (int)std::min<long>(EPU * units, 0x7fffff00L);
+  return f;
+}
+
 template <int CX>
-cudaError_t prepare(const Side& a, int K, int batch, int* e, uint16_t* pl, cudaStream_t s) {
-  const int ldp = pad8i(K * CX);
+cudaError_t prepare(const Side& a, int K, int batch, const Planes& p, cudaStream_t s) {
+  const int ldp = pad8i(K * CX), ldm = pad8i(K);
   if (a.lk == 1) {
-    oz_exp_rows<CX><<<dim3((a.rows + 7) / 8, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, e);
+    oz_exp_rows<CX><<<dim3((a.rows + 7) / 8, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, p.e);
     const unsigned nb = (unsigned)(((long)a.rows * (ldp / 8) + 255) / 256);
     if (a.emb)
-      oz_slice_rows<2, true><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, e, pl, ldp);
+      oz_slice_rows<2, true><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag,
+                                                             ldm);
     else
-      oz_slice_rows<CX, false><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, e, pl, ldp);
+      oz_slice_rows<CX, false><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, p.e, p.pl, ldp,
+                                                               p.mag, ldm);
   } else {
-    cudaError_t st = cudaMemsetAsync(e, 0, sizeof(int) * (size_t)batch * a.rows, s);
+    cudaError_t st = cudaMemsetAsync(p.e, 0, sizeof(int) * (size_t)batch * a.rows, s);
     if (st != cudaSuccess) return st;
     oz_exp_cols<CX><<<dim3((a.rows + 127) / 128, (K + KS - 1) / KS, batch), 128, 0, s>>>(a.src, a.sb, a.lk, a.rows, K,
-                                                                                        e);
+                                                                                        p.e);
     const dim3 grid((a.rows + 31) / 32, (K * CX + 63) / 64, batch);
     if (a.emb)
-      oz_slice_cols<2, true><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, e, pl, ldp);
+      oz_slice_cols<2, true><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm);
     else
-      oz_slice_cols<CX, false><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, e, pl, ldp);
+      oz_slice_cols<CX, false><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm);
   }
   return cudaGetLastError();
 }
 
-// [batch x 7 planes][rows][ldp] bf16 read as boxes of 7 planes x `box` rows x 32 K.
-cudaError_t plane_map(CUtensorMap* map, const void* base, int batch, long rows, int Kr, int ldp, int box) {
+// bf16 [n][rows][ldk] with K valid: digit planes (n = 7 per batch entry) in
+// boxes of 7 planes x `box` rows x 32 K, 64B swizzle, or magnitudes (n = batch)
+// in boxes of `box` rows x 64 K, 128B swizzle.
+cudaError_t plane_map(CUtensorMap* map, const void* base, long n, long rows, int K, int ldk, int box, bool digits) {
   static const PFN_cuTensorMapEncodeTiled_v12000 enc = [] {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -581,54 +976,33 @@ cudaError_t plane_map(CUtensorMap* map, const void* base, int batch, long rows, 
     return (PFN_cuTensorMapEncodeTiled_v12000)p;
   }();
   if (!enc) return cudaErrorNotSupported;
-  cuuint64_t dims[3] = {(cuuint64_t)Kr, (cuuint64_t)rows, (cuuint64_t)batch * ND};
-  cuuint64_t strides[2] = {(cuuint64_t)ldp * 2, (cuuint64_t)ldp * 2 * rows};
-  cuuint32_t bx[3] = {TK, (cuuint32_t)box, ND};
+  cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)n};
+  cuuint64_t strides[2] = {(cuuint64_t)ldk * 2, (cuuint64_t)ldk * 2 * rows};
+  cuuint32_t bx[3] = {(cuuint32_t)(digits ? TK : MK), (cuuint32_t)box, (cuuint32_t)(digits ? ND : 1)};
   cuuint32_t estr[3] = {1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)base, dims, strides, bx, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, digits ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
              ? cudaSuccess
              : cudaErrorInvalidValue;
 }
 
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-// Scratch of one operand: exponents, then planes.
-size_t side_bytes(long rows, long prow, int Kr, int batch) {
-  return align256(sizeof(int) * (size_t)rows * batch) + align256(2 * (size_t)ND * prow * pad8i(Kr) * batch);
-}
-
+// One slab: the check (unless list is null), the digits, and what the check left.
 template <int CX>
-cudaError_t launch(const OzMaps& maps, const OzShape& g, const int* eL, const int* eN, double* out, const OzWork& w,
-                   cudaStream_t s) {
-  int dev = 0, nsm = 0;
-  if (g.units >= (1L << 31)) return cudaErrorInvalidValue;   // counted in 32 bits
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
-  if (e != cudaSuccess) return e;
-  oz_kernel<<<(unsigned)std::min<long>(g.units, nsm), NT, SMEM, s>>>(maps, g, eL, eN, out, w.err());
-  if (w.launches) ++*w.launches;
-  return cudaGetLastError();
-}
-
-// One slab: lane planes pL with exponents eL against column planes pN, eN.
-template <int CX>
-cudaError_t slab(const Side& l, const Side& n, int K, int nb, const int* eL, const uint16_t* pL, const int* eN,
-                 const uint16_t* pN, double* out, long ldo, long sbo, bool pairs, double alpha, bool acc, const OzWork& w,
-                 cudaStream_t s) {
+cudaError_t slab(const Side& l, const Side& n, int K, int nb, const Planes& pl, const Planes& pn, void* list, double* out,
+                 long ldo, long sbo, bool pairs, double alpha, bool acc, const OzWork& w, cudaStream_t s) {
   const int Kr = K * CX, ldp = pad8i(Kr);
-  OzMaps maps;
-  cudaError_t e = plane_map(&maps.n, pN, nb, plane_rows(n), Kr, ldp, TN);
-  if (e == cudaSuccess) e = plane_map(&maps.l, pL, nb, plane_rows(l), Kr, ldp, TL);
-  if (e != cudaSuccess) return e;
   OzShape g;
+  g.lr = l.rows;
+  g.nr = n.rows;
+  g.lt = TL >> l.emb;
+  g.nt = TN >> n.emb;
+  g.mst = (K + MK - 1) / MK;
   g.nl = (int)plane_rows(l);
   g.nn = (int)plane_rows(n);
   g.nst = (Kr + TK - 1) / TK;
-  g.tl = (g.nl + TL - 1) / TL;
-  g.tn = (g.nn + TN - 1) / TN;
+  g.tl = (int)tiles_of(l.rows, l.emb, TL);
+  g.tn = (int)tiles_of(n.rows, n.emb, TN);
   g.lsh = l.emb;
   g.nsh = n.emb;
   g.el = l.rows;
@@ -639,7 +1013,41 @@ cudaError_t slab(const Side& l, const Side& n, int K, int nb, const int* eL, con
   g.alpha = alpha;
   g.ldo = ldo;
   g.sbo = sbo;
-  return launch<CX>(maps, g, eL, eN, out, w, s);
+  if (g.units >= (1L << 31)) return cudaErrorInvalidValue;   // counted in 32 bits
+  OzMaps maps, mags;
+  cudaError_t e = plane_map(&maps.n, pn.pl, (long)nb * ND, g.nn, Kr, ldp, TN, true);
+  if (e == cudaSuccess) e = plane_map(&maps.l, pl.pl, (long)nb * ND, g.nl, Kr, ldp, TL, true);
+  if (e == cudaSuccess && list) e = plane_map(&mags.n, pn.mag, nb, n.rows, K, pad8i(K), TN, false);
+  if (e == cudaSuccess && list) e = plane_map(&mags.l, pl.mag, nb, l.rows, K, pad8i(K), TL, false);
+  int dev = 0, nsm = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(oz_check_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSMEM);
+  OzList f{};
+  const unsigned grid = (unsigned)std::min<long>(g.units, nsm);
+  if (!list) {
+    if (e != cudaSuccess) return e;
+    oz_kernel<<<grid, NT, SMEM, s>>>(maps, g, pl.e, pn.e, out, f, w.err());
+    if (w.launches) ++*w.launches;
+    return cudaGetLastError();
+  }
+  f = list_at(list, g.units);
+  if (e == cudaSuccess) e = cudaMemsetAsync(f.cnt, 0, 64 + sizeof(int) * (size_t)g.units, s);
+  if (e != cudaSuccess) return e;
+  oz_check_kernel<<<grid, MNT, MSMEM, s>>>(mags, g, pl.e, pn.e, f, w.err());
+  oz_kernel<<<grid, NT, SMEM, s>>>(maps, g, pl.e, pn.e, out, f, w.err());
+  const Source sl{l.src, l.sb, l.lr, l.lk, l.conj}, sn{n.src, n.sb, n.lr, n.lk, n.conj};
+  const unsigned xg = (unsigned)std::min<long>(2 * g.units, 2L * nsm);
+  if constexpr (CX == 1)
+    oz_exact_kernel<1, 4, 10><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err());
+  else if (pairs)
+    oz_exact_kernel<2, 4, 5><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err());
+  else
+    oz_exact_kernel<2, 2, 10><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err());
+  if (w.launches) *w.launches += 3;
+  return cudaGetLastError();
 }
 
 // Whether a complex product embeds A (as the columns) or B (as the lanes).
@@ -671,9 +1079,11 @@ struct Slabs {
 // one entry: column tiles in up to half the room, lane tiles in what is left.
 // Rows are rounded down to tiles, so that room for one tile of each side is
 // enough and more of it never fails.
-bool plan_slabs(int lrows, bool lemb, int nrows, bool nemb, int Kr, int batch, size_t room, Slabs& p) {
-  auto lane = [&](int nb, int r) { return side_bytes(r, lemb ? 2L * r : r, Kr, nb); };
-  auto col = [&](int nb, int r) { return side_bytes(r, nemb ? 2L * r : r, Kr, nb); };
+bool plan_slabs(int lrows, bool lemb, int nrows, bool nemb, int K, int CX, int batch, size_t room, Slabs& p) {
+  auto need = [&](int nb, int l, int n) {
+    return side_bytes(l, lemb, K, CX, nb) + side_bytes(n, nemb, K, CX, nb) +
+           list_bytes(nb * tiles_of(l, lemb, TL) * tiles_of(n, nemb, TN));
+  };
   // the largest n <= most for which fits(n), 0 where there is none
   auto largest = [](int most, auto fits) {
     int lo = 0, hi = most + 1;
@@ -685,63 +1095,61 @@ bool plan_slabs(int lrows, bool lemb, int nrows, bool nemb, int Kr, int batch, s
     return lo;
   };
   p = Slabs{1, lrows, nrows};
-  const int bs = largest(batch, [&](int nb) { return lane(nb, lrows) + col(nb, nrows) <= room; });
+  const int bs = largest(batch, [&](int nb) { return need(nb, lrows, nrows) <= room; });
   if (bs > 0) {
     const int parts = (batch + bs - 1) / bs;
     p.bs = (batch + parts - 1) / parts;
     return true;
   }
   const int lt = TL >> lemb, nt = TN >> nemb;   // rows of a tile
-  const size_t lane1 = lane(1, std::min(lt, lrows));
-  if (lane1 + col(1, std::min(nt, nrows)) > room) return false;
+  auto lanes = [&](int t) { return (int)std::min<long>(lrows, (long)t * lt); };
+  auto columns = [&](int t) { return (int)std::min<long>(nrows, (long)t * nt); };
+  if (need(1, lanes(1), columns(1)) > room) return false;
   const int ct = std::max(1, largest((nrows + nt - 1) / nt, [&](int t) {
-    const size_t c = col(1, (int)std::min<long>(nrows, (long)t * nt));
-    return c <= room / 2 && c + lane1 <= room;
+    return side_bytes(columns(t), nemb, K, CX, 1) <= room / 2 && need(1, lanes(1), columns(t)) <= room;
   }));
-  p.nrows = (int)std::min<long>(nrows, (long)ct * nt);
-  const size_t left = room - col(1, p.nrows);
-  const int rt = largest((lrows + lt - 1) / lt,
-                         [&](int t) { return lane(1, (int)std::min<long>(lrows, (long)t * lt)) <= left; });
-  p.lrows = (int)std::min<long>(lrows, (long)rt * lt);
+  p.nrows = columns(ct);
+  p.lrows = lanes(largest((lrows + lt - 1) / lt, [&](int t) { return need(1, lanes(t), p.nrows) <= room; }));
   return true;
 }
 
 // out(lane i, column j) over batch entries, in slabs that fit the scratch.
-// pairs: the N side is embedded and out is complex [j / 2][i].
+// pairs: the N side is embedded and out is complex [j / 2][i].  check: see the top.
 template <int CX>
 cudaError_t product(Side L, Side N, int K, int batch, double* out, long ldo, long sbo, bool pairs, double alpha,
-                    bool acc, const OzWork& w, cudaStream_t s) {
+                    bool acc, bool check, const OzWork& w, cudaStream_t s) {
   if (L.rows <= 0 || N.rows <= 0 || batch <= 0) return cudaSuccess;
   if (K <= 0 || (long)K * CX > OZ_MAX_K) return cudaErrorInvalidValue;   // the int64 sums stay below 2^62
-  const int Kr = K * CX;
-  Slabs pl;
-  if (!plan_slabs(L.rows, L.emb, N.rows, N.emb, Kr, batch, room_of(w), pl))
-    return cudaErrorMemoryAllocation;
-  const int bs = pl.bs, lrows = pl.lrows, nrows = pl.nrows;
+  Slabs p;
+  if (!plan_slabs(L.rows, L.emb, N.rows, N.emb, K, CX, batch, room_of(w), p)) return cudaErrorMemoryAllocation;
+  const int bs = p.bs, lrows = p.lrows, nrows = p.nrows;
   for (int b0 = 0; b0 < batch; b0 += bs) {
     const int nb = std::min(bs, batch - b0);
     for (int n0 = 0; n0 < N.rows; n0 += nrows) {
       Side n = N;
       n.src += ((long)b0 * N.sb + (long)n0 * N.lr) * CX;
       n.rows = std::min(nrows, N.rows - n0);
-      int* eN = (int*)(w.buf + HEAD);
-      uint16_t* pN = (uint16_t*)((unsigned char*)eN + align256(sizeof(int) * (size_t)n.rows * nb));
-      cudaError_t e = prepare<CX>(n, K, nb, eN, pN, s);
+      unsigned char* at = w.buf + HEAD;
+      Planes pn = planes_at(at, n.rows, n.emb, K, CX, nb);
+      if (!check) pn.mag = nullptr;
+      cudaError_t e = prepare<CX>(n, K, nb, pn, s);
       if (e != cudaSuccess) return e;
       if (w.launches) *w.launches += 2;
-      unsigned char* lbuf = (unsigned char*)eN + side_bytes(n.rows, plane_rows(n), Kr, nb);
+      at += side_bytes(n.rows, n.emb, K, CX, nb);
       for (int l0 = 0; l0 < L.rows; l0 += lrows) {
         Side l = L;
         l.src += ((long)b0 * L.sb + (long)l0 * L.lr) * CX;
         l.rows = std::min(lrows, L.rows - l0);
-        int* eL = (int*)lbuf;
-        uint16_t* pL = (uint16_t*)(lbuf + align256(sizeof(int) * (size_t)l.rows * nb));
-        if ((e = prepare<CX>(l, K, nb, eL, pL, s)) != cudaSuccess) return e;
+        Planes pl = planes_at(at, l.rows, l.emb, K, CX, nb);
+        if (!check) pl.mag = nullptr;
+        if ((e = prepare<CX>(l, K, nb, pl, s)) != cudaSuccess) return e;
         if (w.launches) *w.launches += 2;
         // pairs: double2 units along rows; embedded lanes: two doubles per complex column
         double* o = out + (pairs ? 2 * ((long)b0 * sbo + (long)n0 * ldo + l0)
                                  : (long)b0 * sbo + (long)n0 * ldo + (L.emb ? 2L : 1L) * l0);
-        if ((e = slab<CX>(l, n, K, nb, eL, pL, eN, pN, o, ldo, sbo, pairs, alpha, acc, w, s)) != cudaSuccess) return e;
+        e = slab<CX>(l, n, K, nb, pl, pn, check ? at + side_bytes(l.rows, l.emb, K, CX, nb) : nullptr, o, ldo, sbo, pairs,
+                     alpha, acc, w, s);
+        if (e != cudaSuccess) return e;
       }
     }
   }
@@ -751,28 +1159,31 @@ cudaError_t product(Side L, Side N, int K, int batch, double* out, long ldo, lon
 }  // namespace
 
 size_t oz_work_bytes(int M, int N, int K, int batch) {
-  const long small = std::min(M, N), big = std::max(M, N);
-  return HEAD + side_bytes(small, 2 * small, 2 * K, batch) + side_bytes(big, big, 2 * K, batch);
+  const bool ea = embed_a(M, N);
+  return HEAD + side_bytes(M, ea, K, 2, batch) + side_bytes(N, !ea, K, 2, batch) +
+         list_bytes(batch * tiles_of(N, !ea, TL) * tiles_of(M, ea, TN));
 }
 
-size_t oz_work_min(int K) { return HEAD + side_bytes(TN, TN, 2 * K, 1) + side_bytes(TL, TL, 2 * K, 1); }
+size_t oz_work_min(int K) { return HEAD + side_bytes(TN, false, K, 2, 1) + side_bytes(TL, false, K, 2, 1) + list_bytes(1); }
+
+static bool plan(int M, int N, int K, int batch, bool real, size_t room, Slabs& p) {
+  const bool ea = !real && embed_a(M, N);
+  return plan_slabs(N, !real && !ea, M, ea, K, real ? 1 : 2, batch, room, p);
+}
 
 bool oz_fits(int M, int N, int K, int batch, bool real, const OzWork& w) {
-  const bool ea = !real && embed_a(M, N);
-  const int Kr = real ? K : 2 * K;
   Slabs p;
-  return w.buf && Kr <= OZ_MAX_K && plan_slabs(N, !real && !ea, M, ea, Kr, batch, room_of(w), p);
+  return w.buf && (real ? K : 2L * K) <= OZ_MAX_K && plan(M, N, K, batch, real, room_of(w), p);
 }
 
 void oz_limit(long long bytes) { g_limit = bytes; }
 
-bool oz_plan(int M, int N, int K, int batch, bool real, size_t bytes, int plan[3]) {
-  const bool ea = !real && embed_a(M, N);
+bool oz_plan(int M, int N, int K, int batch, bool real, size_t bytes, int out[3]) {
   Slabs p;
-  const bool ok = plan_slabs(N, !real && !ea, M, ea, real ? K : 2 * K, batch, bytes > HEAD ? bytes - HEAD : 0, p);
-  plan[0] = p.bs;
-  plan[1] = p.nrows;
-  plan[2] = p.lrows;
+  const bool ok = plan(M, N, K, batch, real, bytes > HEAD ? bytes - HEAD : 0, p);
+  out[0] = p.bs;
+  out[1] = p.nrows;
+  out[2] = p.lrows;
   return ok;
 }
 
@@ -797,62 +1208,67 @@ void oz_free(OzWork& w) {
 
 // The FP64 kernel takes 4.3 us per unit of K and round of its 64 x 64 tiles
 // over the SMs (two multiply-adds a clock on each): 35 us for one tile of
-// K = 8, and 0.3 ms for one of K = 71.  The digit form's five launches are
-// about 35 us in all.
+// K = 8 (70 us measured for a stage of K = 8 to 16), and 0.3 ms for one of
+// K = 71.  The digit form's seven launches are 41 us in all at K = 12, 50 to 60
+// at K = 16 to 40.
 bool oz_wins(int M, int N, int K, int batch) {
   const double tiles = ((M + 63) / 64) * (double)((N + 63) / 64) * batch;
   return ceil(tiles / 152.0) * K >= 10.0 && 2L * K <= OZ_MAX_K;
 }
 
 cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
-                      int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s) {
+                      int ldb, long sB, double2* C, int ldc, long sC, int batch, bool check, const OzWork& w,
+                      cudaStream_t s) {
   Side a{(const double*)A, M, la == A_KM ? 1L : (long)lda, la == A_KM ? (long)lda : 1L, sA, la == A_MK_CONJ, false};
   Side b{(const double*)B, N, lb == B_KN ? 1L : (long)ldb, lb == B_KN ? (long)ldb : 1L, sB, lb == B_NK_CONJ, false};
   if (embed_a(M, N)) {
     // embedded A as the columns, lanes along N: out[m][n] one double2 per lane
     a.emb = true;
-    return product<2>(b, a, K, batch, (double*)C, ldc, sC, true, 1.0, false, w, s);
+    return product<2>(b, a, K, batch, (double*)C, ldc, sC, true, 1.0, false, check, w, s);
   }
   // embedded B as the lanes (real columns of the interleaved C), plain A rows as the columns
   b.emb = true;
-  return product<2>(b, a, K, batch, (double*)C, 2L * ldc, 2 * sC, false, 1.0, false, w, s);
+  return product<2>(b, a, K, batch, (double*)C, 2L * ldc, 2 * sC, false, 1.0, false, check, w, s);
 }
 
 cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
                         int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s) {
   if (oz_wins(M, N, K, batch) && oz_fits(M, N, K, batch, false, w))
-    return oz_gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, w, s);
+    return oz_gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, true, w, s);
   if (w.launches) ++*w.launches;
   return gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, s);
 }
 
-bool oz_lanes_fit(int M, int K, const OzWork& w) { return w.buf && side_bytes(M, 2L * M, 2 * K, 1) <= room_of(w); }
+size_t oz_lane_bytes(int N, int K) { return exp_bytes(N, 1) + digit_bytes(N, false, K, 2, 1); }
+size_t oz_lanes_work(int M, int K) { return HEAD + exp_bytes(M, 1) + digit_bytes(M, true, K, 2, 1); }
+bool oz_lanes_fit(int M, int K, const OzWork& w) { return w.buf && oz_lanes_work(M, K) <= HEAD + room_of(w); }
 
-size_t oz_lane_bytes(int N, int K) { return side_bytes(N, N, 2 * K, 1); }
+static Planes unchecked(void* at, int rows, bool emb, int K) {
+  Planes p = planes_at(at, rows, emb, K, 2, 1);
+  p.mag = nullptr;
+  return p;
+}
 
 cudaError_t oz_lane_prepare(const double2* B, int ldb, int N, int K, void* lanes, cudaStream_t s) {
   if (2L * K > OZ_MAX_K) return cudaErrorInvalidValue;
   const Side b{(const double*)B, N, 1L, (long)ldb, 0, false, false};
-  return prepare<2>(b, K, 1, (int*)lanes, (uint16_t*)((unsigned char*)lanes + align256(sizeof(int) * (size_t)N)), s);
+  return prepare<2>(b, K, 1, unchecked(lanes, N, false, K), s);
 }
 
-cudaError_t oz_gemm_z_lanes(int la, int M, int N, int K, const double2* A, int lda, const void* lanes, double2* C,
-                            int ldc, const OzWork& w, cudaStream_t s) {
+cudaError_t oz_gemm_z_lanes(int la, int M, int N, int K, const double2* A, int lda, void* lanes, double2* C, int ldc,
+                            const OzWork& w, cudaStream_t s) {
   if (!oz_lanes_fit(M, K, w)) return cudaErrorMemoryAllocation;
   const Side a{(const double*)A, M, la == A_KM ? 1L : (long)lda, la == A_KM ? (long)lda : 1L, 0, la == A_MK_CONJ, true};
   const Side b{nullptr, N, 1L, 1L, 0, false, false};
-  int* eA = (int*)(w.buf + HEAD);
-  uint16_t* pA = (uint16_t*)((unsigned char*)eA + align256(sizeof(int) * (size_t)M));
-  const cudaError_t e = prepare<2>(a, K, 1, eA, pA, s);
+  const Planes pa = unchecked(w.buf + HEAD, M, true, K);
+  const cudaError_t e = prepare<2>(a, K, 1, pa, s);
   if (e != cudaSuccess) return e;
-  return slab<2>(b, a, K, 1, (const int*)lanes,
-                 (const uint16_t*)((const unsigned char*)lanes + align256(sizeof(int) * (size_t)N)), eA, pA, (double*)C,
-                 ldc, 0, true, 1.0, false, w, s);
+  return slab<2>(b, a, K, 1, unchecked(lanes, N, false, K), pa, nullptr, (double*)C, ldc, 0, true, 1.0, false, w, s);
 }
 
 cudaError_t oz_gemm_d(bool a_km, bool b_kn, int M, int N, int K, const double* A, long lda, const double* B, long ldb,
-                      double* C, long ldc, double alpha, bool acc, const OzWork& w, cudaStream_t s) {
+                      double* C, long ldc, double alpha, bool acc, bool check, const OzWork& w, cudaStream_t s) {
   Side a{A, M, a_km ? 1L : lda, a_km ? lda : 1L, 0, false, false};
   Side b{B, N, b_kn ? 1L : ldb, b_kn ? ldb : 1L, 0, false, false};
-  return product<1>(b, a, K, 1, C, ldc, 0, false, alpha, acc, w, s);
+  return product<1>(b, a, K, 1, C, ldc, 0, false, alpha, acc, check, w, s);
 }

@@ -34,19 +34,25 @@ bool oz_wins(int M, int N, int K, int batch);
 cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
                         int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s);
 
-// gemm_z's product (operand layouts of GemmA, GemmB) from digits.
+// gemm_z's product (operand layouts of GemmA, GemmB) from digits.  check: to
+// FP64 accuracy of every entry (those that digits relative to the rows' largest
+// entries do not hold to it are computed in FP64); else to 4 K 2^-62 of the
+// product of the largest entries of its two rows.
 cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
-                      int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s);
+                      int ldb, long sB, double2* C, int ldc, long sC, int batch, bool check, const OzWork& w,
+                      cudaStream_t s);
 
-// The same product of A (any layout) with a B of N columns stored [k][n] whose
-// digits were prepared once: oz_lane_bytes of device memory at `lanes`.
+// The unchecked product of A (any layout) with a B of N columns stored [k][n]
+// whose digits were prepared once: oz_lane_bytes of device memory at `lanes`.
 size_t oz_lane_bytes(int N, int K);
-bool oz_lanes_fit(int M, int K, const OzWork& w);   // room in w for the digits of A (M rows)
+size_t oz_lanes_work(int M, int K);                  // scratch for the digits of A (M rows)
+bool oz_lanes_fit(int M, int K, const OzWork& w);    // w has that much
 cudaError_t oz_lane_prepare(const double2* B, int ldb, int N, int K, void* lanes, cudaStream_t s);
-cudaError_t oz_gemm_z_lanes(int la, int M, int N, int K, const double2* A, int lda, const void* lanes, double2* C,
-                            int ldc, const OzWork& w, cudaStream_t s);
+cudaError_t oz_gemm_z_lanes(int la, int M, int N, int K, const double2* A, int lda, void* lanes, double2* C, int ldc,
+                            const OzWork& w, cudaStream_t s);
 
 // Real C[m][n] = alpha sum_k A(m, k) B(n, k) (+ C when acc): A(m, k) = A[m lda + k]
 // or, a_km, A[k lda + m]; B(n, k) = B[n ldb + k] or, b_kn, B[k ldb + n].  alpha is 1 or -1.
+// check as in oz_gemm_z (2 K 2^-62).
 cudaError_t oz_gemm_d(bool a_km, bool b_kn, int M, int N, int K, const double* A, long lda, const double* B, long ldb,
-                      double* C, long ldc, double alpha, bool acc, const OzWork& w, cudaStream_t s);
+                      double* C, long ldc, double alpha, bool acc, bool check, const OzWork& w, cudaStream_t s);

@@ -29,6 +29,15 @@
 //   4. the block's columns for all candidates: one product with the digits of
 //      U, which are made once, one with the earlier rows of L, and a kernel
 //      that finishes the block's own triangle, d and sum d after every pivot
+// The products are not checked entry by entry (oz_gemm.cu); what the selection
+// needs of A(p, c) is its error relative to sqrt(A(p, p) A(c, c)), and digits
+// hold that to 2^-8 of what FP64 sums may leave.  |u| of a candidate is at most
+// A(c, c)^(1/4) and |L[s][c]| at most sqrt(A(c, c)), so B errs by at most 4 K 2^-62
+// (A(p, p) A(c, c))^(1/4), for K functions, and the sum over j earlier rows by
+// 2 j 2^-62 sqrt(A(p, p) A(c, c)).  With d_c <= d_p that reaches the residual of c
+// as 2 l dl <= (8 K + 2 j) 2^-61 sqrt(A(p, p) / d_p) of A(c, c).  (With the check
+// the rows of points far apart, which have no entry in common, ran in FP64: 93
+// ms at 600 points, the residuals as far from 64 bits as without, 4.5e-12.)
 // (767 ms to 49 ms for 600 points.)  Where S comes out empty (more than 800
 // candidates within a bin of the largest) one pivot is taken the first way.
 #include "oz_gemm.cuh"
@@ -409,7 +418,7 @@ struct Blocks {
     get(pk, 1);
     if (e == cudaSuccess) e = cudaMalloc(&lanes, oz_lane_bytes(ncand, nfunc));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&host, sizeof(Picked));
-    const size_t least = std::max(oz_work_bytes(MS, MS, nfunc, 1), oz_work_min(npts));
+    const size_t least = std::max({oz_work_bytes(MS, MS, nfunc, 1), oz_work_min(npts), oz_lanes_work(TP, nfunc)});
     if (e == cudaSuccess)
       e = oz_alloc(w, std::max(least, std::min(oz_work_bytes(TP, ncand, (npts + 1) / 2, 1), (size_t)1 << 30)), least, s);
     if (e == cudaSuccess && !(oz_fits(MS, MS, nfunc, 1, false, w) && oz_fits(MS, MS, npts, 1, true, w) &&
@@ -476,13 +485,13 @@ extern "C" thc_status thc_select_points(const double* U, int nfunc, int ncand, i
       hist_kernel<<<nb, PT, 0, s>>>(d, ncand, selv, bk.hist);
       pick_kernel<<<1, 1024, 0, s>>>(d, ncand, selv, bk.hist, bk.idx, bk.edge);
       gather_u<<<nblk((long)MS * nfunc, PT), PT, 0, s>>>(u, nfunc, ncand, bk.idx, MS, false, bk.Us);
-      if ((e = oz_gemm_z(A_MK_CONJ, B_NK, MS, MS, nfunc, bk.Us, nfunc, 0, bk.Us, nfunc, 0, bk.G2, MS, 0, 1, bk.w, s)) !=
+      if ((e = oz_gemm_z(A_MK_CONJ, B_NK, MS, MS, nfunc, bk.Us, nfunc, 0, bk.Us, nfunc, 0, bk.G2, MS, 0, 1, false, bk.w, s)) !=
           cudaSuccess)
         return 0;
       abs2<<<nblk((long)MS * MS, PT), PT, 0, s>>>(bk.G2, (long)MS * MS, bk.G);
       if (j > 0) {
         gather_l<<<nblk((long)j * MS, PT), PT, 0, s>>>(L, ncand, bk.idx, MS, MS, j, bk.Ls);
-        if ((e = oz_gemm_d(true, true, MS, MS, j, bk.Ls, MS, bk.Ls, MS, bk.G, MS, -1.0, true, bk.w, s)) != cudaSuccess)
+        if ((e = oz_gemm_d(true, true, MS, MS, j, bk.Ls, MS, bk.Ls, MS, bk.G, MS, -1.0, true, false, bk.w, s)) != cudaSuccess)
           return 0;
       }
       pivots_kernel<<<1, 1024, 0, s>>>(bk.G, bk.idx, d, selv, bk.edge, std::min(TP, npts - j), bk.lb, bk.pk);
@@ -496,7 +505,8 @@ extern "C" thc_status thc_select_points(const double* U, int nfunc, int ncand, i
       abs2<<<nblk((long)T * ncand, PT), PT, 0, s>>>(bk.Bc, (long)T * ncand, bk.R);
       if (j > 0) {
         gather_l<<<nblk((long)j * T, PT), PT, 0, s>>>(L, ncand, bk.pk->piv, T, TP, j, bk.Ls);
-        if ((e = oz_gemm_d(true, true, T, ncand, j, bk.Ls, TP, L, ncand, bk.R, ncand, -1.0, true, bk.w, s)) != cudaSuccess)
+        if ((e = oz_gemm_d(true, true, T, ncand, j, bk.Ls, TP, L, ncand, bk.R, ncand, -1.0, true, false, bk.w,
+                           s)) != cudaSuccess)
           return 0;
       }
       if ((e = cudaMemcpyAsync(bk.dold, d, sizeof(double) * ncand, cudaMemcpyDeviceToDevice, s)) != cudaSuccess) return 0;

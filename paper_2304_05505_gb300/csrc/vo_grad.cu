@@ -655,7 +655,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     if ((e = cudaMalloc(&Sbar, sizeof(double) * npq)) != cudaSuccess) break;
     // S-bar = -Lam xi^T
     if (oz_fits(np, np, (int)ng, 1, true, oz)) {
-      if ((e = oz_gemm_d(false, false, np, np, (int)ng, Lam, ng, R, ng, Sbar, np, -1.0, false, oz, s)) != cudaSuccess)
+      if ((e = oz_gemm_d(false, false, np, np, (int)ng, Lam, ng, R, ng, Sbar, np, -1.0, false, true, oz, s)) != cudaSuccess)
         break;
     } else {
       dim3 grid((np + DT - 1) / DT, (np + DT - 1) / DT);
