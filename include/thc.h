@@ -99,10 +99,9 @@ typedef struct thc_ctx thc_ctx;
 thc_status thc_create(thc_ctx** ctx, const thc_dims* dims, int precision, void* stream);
 
 /* Device bytes the context holds (X copy, prepared kernel, workspace).
- * THC_FP64: besides these, thc_set_collocation sets aside up to 2 GB for the
- * digits of its products where the device has them (half as much is tried
- * each time it has not; without any, the products run in FP64 on CUDA
- * cores). */
+ * THC_FP64: the digits of the products go to the workspace of D and M; where
+ * that is below 512 MB, thc_set_collocation also takes up to 512 MB for them if
+ * eight times as much is free (thc_build_K gives it back if it needs the room). */
 thc_status thc_memory_bytes(const thc_dims* dims, int precision, size_t* bytes);
 
 /* X: device, [N_k][nbas][nisdf] complex128.  Copied (and converted for
@@ -148,7 +147,7 @@ thc_status thc_build_host(thc_ctx* ctx, const double* C_host, double* KC_host, d
  * orbitals); the build takes any V.  C: device [N_k][nbas][nocc] complex128;
  * K: device [N_k][nbas][nbas] complex128 (written, must not overlap C); ex:
  * device, 2 doubles as in thc_build.  THC_FP64: every step to FP64 accuracy
- * (products as in thc_build).  THC_MIXED: Z = M X^T and K = conj(X) Z on the
+ * (products as in thc_build; the energy is summed before them).  THC_MIXED: Z = M X^T and K = conj(X) Z on the
  * tensor cores (three fp16 slices, 8 slice products, exact leading sums; the
  * planes of X^T are made once per thc_set_collocation).  THC_MIXED_SIMT:
  * THC_ERR_UNSUPPORTED.  The first call on a context allocates the form's

@@ -308,7 +308,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     {
       int h = 0, ho = 0;
       if (tcerr && (e = cudaMemcpy(&h, tcerr, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
-      if (dig && (e = cudaMemcpy(&ho, oz.err(), sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
+      if (dig && (e = cudaMemcpy(&ho, oz.err, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
       if (h || ho) {
         st = THC_ERR_TIMEOUT;
         set_global_error("thc_rebuild_kernel: a device wait of a tensor-core product timed out");

@@ -75,7 +75,7 @@ constexpr size_t SMEM = STAGES * STAGE + 1024 + 128;
 constexpr int EPI0 = 4, EPI_W = 16, NT = 32 * (EPI0 + EPI_W);
 constexpr int EC = TN / 4;                             // columns of an epilogue warp
 constexpr int NB_ROW = 2047;                           // biased exponent of a row with a NaN or an Inf
-constexpr size_t HEAD = 1024;                          // bytes before the planes: the error block
+constexpr size_t HEAD = 256;                           // bytes before scratch of its own: the error block
 
 // The check of a product: stages of 64 K of the magnitudes, 128B swizzle
 constexpr int MK = 64;
@@ -1029,23 +1029,23 @@ cudaError_t slab(const Side& l, const Side& n, int K, int nb, const Planes& pl, 
   const unsigned grid = (unsigned)std::min<long>(g.units, nsm);
   if (!list) {
     if (e != cudaSuccess) return e;
-    oz_kernel<<<grid, NT, SMEM, s>>>(maps, g, pl.e, pn.e, out, f, w.err());
+    oz_kernel<<<grid, NT, SMEM, s>>>(maps, g, pl.e, pn.e, out, f, w.err);
     if (w.launches) ++*w.launches;
     return cudaGetLastError();
   }
   f = list_at(list, g.units);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.cnt, 0, 64 + sizeof(int) * (size_t)g.units, s);
   if (e != cudaSuccess) return e;
-  oz_check_kernel<<<grid, MNT, MSMEM, s>>>(mags, g, pl.e, pn.e, f, w.err());
-  oz_kernel<<<grid, NT, SMEM, s>>>(maps, g, pl.e, pn.e, out, f, w.err());
+  oz_check_kernel<<<grid, MNT, MSMEM, s>>>(mags, g, pl.e, pn.e, f, w.err);
+  oz_kernel<<<grid, NT, SMEM, s>>>(maps, g, pl.e, pn.e, out, f, w.err);
   const Source sl{l.src, l.sb, l.lr, l.lk, l.conj}, sn{n.src, n.sb, n.lr, n.lk, n.conj};
   const unsigned xg = (unsigned)std::min<long>(2 * g.units, 2L * nsm);
   if constexpr (CX == 1)
-    oz_exact_kernel<1, 4, 10><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err());
+    oz_exact_kernel<1, 4, 10><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err);
   else if (pairs)
-    oz_exact_kernel<2, 4, 5><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err());
+    oz_exact_kernel<2, 4, 5><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err);
   else
-    oz_exact_kernel<2, 2, 10><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err());
+    oz_exact_kernel<2, 2, 10><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err);
   if (w.launches) *w.launches += 3;
   return cudaGetLastError();
 }
@@ -1065,8 +1065,7 @@ thread_local long long g_limit = -1;   // test hook: most scratch of a product
 
 // Scratch for planes and exponents.
 size_t room_of(const OzWork& w) {
-  const size_t b = g_limit < 0 ? w.bytes : std::min(w.bytes, (size_t)g_limit);
-  return b > HEAD ? b - HEAD : 0;
+  return g_limit < 0 ? w.bytes : std::min(w.bytes, (size_t)g_limit);
 }
 
 // Slabs of a product that fit in `room` bytes: batch entries, lane rows and
@@ -1075,8 +1074,8 @@ struct Slabs {
   int bs, lrows, nrows;
 };
 
-// Whole batch entries where one fits, as even as they go; else whole tiles of
-// one entry: column tiles in up to half the room, lane tiles in what is left.
+// Whole batch entries where one fits, as many as take the fewest rounds of the
+// SMs in all; else whole tiles of one entry: column tiles in up to half the room, lane tiles in what is left.
 // Rows are rounded down to tiles, so that room for one tile of each side is
 // enough and more of it never fails.
 bool plan_slabs(int lrows, bool lemb, int nrows, bool nemb, int K, int CX, int batch, size_t room, Slabs& p) {
@@ -1097,19 +1096,29 @@ bool plan_slabs(int lrows, bool lemb, int nrows, bool nemb, int K, int CX, int b
   p = Slabs{1, lrows, nrows};
   const int bs = largest(batch, [&](int nb) { return need(nb, lrows, nrows) <= room; });
   if (bs > 0) {
-    const int parts = (batch + bs - 1) / bs;
-    p.bs = (batch + parts - 1) / parts;
+    const long t = tiles_of(lrows, lemb, TL) * tiles_of(nrows, nemb, TN);
+    auto rounds = [&](long n) { return (n * t + 151) / 152; };
+    long best = -1;
+    for (int n = bs; n > bs / 2; n--) {
+      const long r = batch / n * rounds(n) + rounds(batch % n);
+      if (best < 0 || r < best) {
+        best = r;
+        p.bs = n;
+      }
+    }
     return true;
   }
   const int lt = TL >> lemb, nt = TN >> nemb;   // rows of a tile
   auto lanes = [&](int t) { return (int)std::min<long>(lrows, (long)t * lt); };
   auto columns = [&](int t) { return (int)std::min<long>(nrows, (long)t * nt); };
   if (need(1, lanes(1), columns(1)) > room) return false;
-  const int ct = std::max(1, largest((nrows + nt - 1) / nt, [&](int t) {
+  // (t: tiles in all, m: as many as fit; in as many slabs, but even ones)
+  auto even = [](int t, int m) { const int parts = (t + m - 1) / m; return (t + parts - 1) / parts; };
+  const int ct = (nrows + nt - 1) / nt, rt = (lrows + lt - 1) / lt;
+  p.nrows = columns(even(ct, std::max(1, largest(ct, [&](int t) {
     return side_bytes(columns(t), nemb, K, CX, 1) <= room / 2 && need(1, lanes(1), columns(t)) <= room;
-  }));
-  p.nrows = columns(ct);
-  p.lrows = lanes(largest((lrows + lt - 1) / lt, [&](int t) { return need(1, lanes(t), p.nrows) <= room; }));
+  }))));
+  p.lrows = lanes(even(rt, largest(rt, [&](int t) { return need(1, lanes(t), p.nrows) <= room; })));
   return true;
 }
 
@@ -1129,7 +1138,7 @@ cudaError_t product(Side L, Side N, int K, int batch, double* out, long ldo, lon
       Side n = N;
       n.src += ((long)b0 * N.sb + (long)n0 * N.lr) * CX;
       n.rows = std::min(nrows, N.rows - n0);
-      unsigned char* at = w.buf + HEAD;
+      unsigned char* at = w.buf;
       Planes pn = planes_at(at, n.rows, n.emb, K, CX, nb);
       if (!check) pn.mag = nullptr;
       cudaError_t e = prepare<CX>(n, K, nb, pn, s);
@@ -1160,11 +1169,11 @@ cudaError_t product(Side L, Side N, int K, int batch, double* out, long ldo, lon
 
 size_t oz_work_bytes(int M, int N, int K, int batch) {
   const bool ea = embed_a(M, N);
-  return HEAD + side_bytes(M, ea, K, 2, batch) + side_bytes(N, !ea, K, 2, batch) +
+  return side_bytes(M, ea, K, 2, batch) + side_bytes(N, !ea, K, 2, batch) +
          list_bytes(batch * tiles_of(N, !ea, TL) * tiles_of(M, ea, TN));
 }
 
-size_t oz_work_min(int K) { return HEAD + side_bytes(TN, false, K, 2, 1) + side_bytes(TL, false, K, 2, 1) + list_bytes(1); }
+size_t oz_work_min(int K) { return side_bytes(TN, false, K, 2, 1) + side_bytes(TL, false, K, 2, 1) + list_bytes(1); }
 
 static bool plan(int M, int N, int K, int batch, bool real, size_t room, Slabs& p) {
   const bool ea = !real && embed_a(M, N);
@@ -1180,7 +1189,7 @@ void oz_limit(long long bytes) { g_limit = bytes; }
 
 bool oz_plan(int M, int N, int K, int batch, bool real, size_t bytes, int out[3]) {
   Slabs p;
-  const bool ok = plan(M, N, K, batch, real, bytes > HEAD ? bytes - HEAD : 0, p);
+  const bool ok = plan(M, N, K, batch, real, bytes, p);
   out[0] = p.bs;
   out[1] = p.nrows;
   out[2] = p.lrows;
@@ -1189,20 +1198,26 @@ bool oz_plan(int M, int N, int K, int batch, bool real, size_t bytes, int out[3]
 
 cudaError_t oz_alloc(OzWork& w, size_t want, size_t least, cudaStream_t s) {
   cudaError_t e = cudaErrorMemoryAllocation;
+  unsigned char* p = nullptr;
   for (w.bytes = std::max(want, least);; w.bytes = std::max(least, w.bytes / 2)) {
-    e = cudaMalloc((void**)&w.buf, w.bytes);
+    e = cudaMalloc((void**)&p, HEAD + w.bytes);
     if (e != cudaErrorMemoryAllocation) break;
     cudaGetLastError();
-    w.buf = nullptr;
     if (w.bytes <= least) break;
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.buf, 0, 64, s);
+  if (e != cudaSuccess) {
+    w = OzWork{};
+    return e;
+  }
+  w.err = (int*)p;
+  w.buf = p + HEAD;
+  e = cudaMemsetAsync(p, 0, 64, s);
   if (e != cudaSuccess) oz_free(w);
   return e;
 }
 
 void oz_free(OzWork& w) {
-  if (w.buf) cudaFree(w.buf);
+  if (w.buf) cudaFree(w.buf - HEAD);
   w = OzWork{};
 }
 
@@ -1240,8 +1255,8 @@ cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, i
 }
 
 size_t oz_lane_bytes(int N, int K) { return exp_bytes(N, 1) + digit_bytes(N, false, K, 2, 1); }
-size_t oz_lanes_work(int M, int K) { return HEAD + exp_bytes(M, 1) + digit_bytes(M, true, K, 2, 1); }
-bool oz_lanes_fit(int M, int K, const OzWork& w) { return w.buf && oz_lanes_work(M, K) <= HEAD + room_of(w); }
+size_t oz_lanes_work(int M, int K) { return exp_bytes(M, 1) + digit_bytes(M, true, K, 2, 1); }
+bool oz_lanes_fit(int M, int K, const OzWork& w) { return w.buf && oz_lanes_work(M, K) <= room_of(w); }
 
 static Planes unchecked(void* at, int rows, bool emb, int K) {
   Planes p = planes_at(at, rows, emb, K, 2, 1);
@@ -1260,7 +1275,7 @@ cudaError_t oz_gemm_z_lanes(int la, int M, int N, int K, const double2* A, int l
   if (!oz_lanes_fit(M, K, w)) return cudaErrorMemoryAllocation;
   const Side a{(const double*)A, M, la == A_KM ? 1L : (long)lda, la == A_KM ? (long)lda : 1L, 0, la == A_MK_CONJ, true};
   const Side b{nullptr, N, 1L, 1L, 0, false, false};
-  const Planes pa = unchecked(w.buf + HEAD, M, true, K);
+  const Planes pa = unchecked(w.buf, M, true, K);
   const cudaError_t e = prepare<2>(a, K, 1, pa, s);
   if (e != cudaSuccess) return e;
   return slab<2>(b, a, K, 1, unchecked(lanes, N, false, K), pa, nullptr, (double*)C, ldc, 0, true, 1.0, false, w, s);

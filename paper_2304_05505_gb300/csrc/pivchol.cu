@@ -552,7 +552,7 @@ extern "C" thc_status thc_select_points(const double* U, int nfunc, int ncand, i
     }
     if (e == cudaSuccess && blocks) {
       int h = 0;
-      e = cudaMemcpyAsync(&h, bk.w.err(), sizeof(int), cudaMemcpyDeviceToHost, s);
+      e = cudaMemcpyAsync(&h, bk.w.err, sizeof(int), cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (h) {
         set_global_error("thc_select_points: a device wait of a tensor-core product timed out");

@@ -151,7 +151,19 @@ void free_all(thc_ctx* c) {
   c->cstream = nullptr;
 }
 
+// The error word (and wait limit) of the context's kernels with bounded waits, null for THC_MIXED_SIMT.  THC_FP64:
+// in the flag word's block (where the tensor-core forms keep the caller's addresses).
+int* wait_error(const thc_ctx* c) {
+  return c->precision == THC_FP64 ? (int*)((char*)c->flag + 16) : c->tc_err;
+}
+
 constexpr int kStages = 6;
+
+// Position in time of each slot (S1, S2, S3, S4a or Z, S4b or K, S5).
+const int* stage_order(bool e_first) {
+  static const int plain[kStages] = {0, 1, 2, 3, 4, 5}, early[kStages] = {0, 1, 2, 4, 5, 3};
+  return e_first ? early : plain;
+}
 
 }  // namespace
 
@@ -314,7 +326,7 @@ thc_status thc_create(thc_ctx** out, const thc_dims* d, int precision, void* str
     delete c;
     return THC_ERR_CUDA;
   }
-  if (c->tc_err && (e = cudaMallocHost(&c->tc_err_host, sizeof(int))) != cudaSuccess) {
+  if (wait_error(c) && (e = cudaMallocHost(&c->tc_err_host, sizeof(int))) != cudaSuccess) {
     g_create_error = std::string("cudaMallocHost: ") + cudaGetErrorString(e);
     free_all(c);
     delete c;
@@ -352,26 +364,24 @@ thc_status thc_destroy(thc_ctx* c) {
   return THC_OK;
 }
 
-// Scratch of an FP64 context's digit products: its largest product whole, up
-// to 2 GB, less where the device has no room (the products then go in smaller
-// slabs, and without any on the FP64 pipe).
+// The digits of M take twice the memory of D.  With many k points S4a goes in
+// slabs of whole ones without loss; with few its 15 tiles a k point (n_occ = 60,
+// N_P = 1200) do not fill the SMs even whole, and slabs of rows take their time
+// one after the other (N_P = 1200, 2 x 2 x 1 k: 0.27 ms whole, 0.99 in D; one k
+// point, N_P = 2400: 0.45 and 2.1).  So contexts whose D is below 512 MB get
+// scratch of their own, up to that, where it is less than an eighth of the free
+// memory.
 static void oz_prepare(thc_ctx* c) {
   if (c->precision != THC_FP64 || c->oz_asked) return;
   c->oz_asked = true;
   const int nk = c->nk, N = c->nbas, n = c->nocc, P = c->nisdf;
   if (!oz_wins(P, P, n, nk) && !oz_wins(P, n, P, nk) && !oz_wins(P, n, N, nk)) return;
   const size_t want = std::max({oz_work_bytes(P, n, N, nk), oz_work_bytes(P, P, n, nk), oz_work_bytes(P, n, P, nk),
-                                oz_work_bytes(N, n, P, nk)});
-  if (oz_alloc(c->oz, std::min(want, (size_t)2 << 30), oz_work_min(std::min(N, P)), c->stream) != cudaSuccess) {
-    cudaGetLastError();
-    oz_free(c->oz);
-    return;
-  }
-  if (cudaMallocHost(&c->tc_err_host, sizeof(int)) != cudaSuccess) {
-    cudaGetLastError();
-    c->tc_err_host = nullptr;
-    oz_free(c->oz);
-  }
+                                oz_work_bytes(N, n, P, nk), oz_work_bytes(N, P, P, nk), oz_work_bytes(N, N, P, nk)});
+  const size_t have = sizeof(double2) * (size_t)nk * P * P, take = std::min(want, (size_t)512 << 20);
+  size_t room = 0, total = 0;
+  if (have >= take || cudaMemGetInfo(&room, &total) != cudaSuccess || room / 8 < take) return;
+  if (oz_alloc(c->oz, take, take, c->stream) != cudaSuccess) cudaGetLastError();
 }
 
 static thc_status finite_check(thc_ctx* c, const double2* p, long n) {
@@ -479,6 +489,9 @@ static cudaError_t mark(thc_ctx* c, int i, cudaStream_t s, bool simple) {
 
 // Kao (THC-AO-K): after S3, K^k = conj(X^k) M^k X^{kT} into Kao instead of S4a,
 // S4b, and E_x = -(1/N_k) sum_k sum_PQ conj(D^k_PQ) M^k_PQ (the same energy).
+// The digits of the products go to the buffers that hold nothing at the time:
+// M before S3, D after it (after the energy, which reads D, in THC-AO-K), or to
+// scratch of their own where those are small.
 static thc_status build_fp64(thc_ctx* c, const double2* C, double2* KC, double* ex, double2* Kao = nullptr) {
   const int nk = c->nk, N = c->nbas, n = c->nocc, P = c->nisdf;
   const long PP = (long)P * P;
@@ -488,29 +501,43 @@ static thc_status build_fp64(thc_ctx* c, const double2* C, double2* KC, double* 
   double2* Y = (double2*)c->Y;
   cudaStream_t s = c->stream;
   c->n_launch = 3;   // the convolution and the two kernels of the energy; the products add theirs
-  c->oz.launches = &c->n_launch;
+  auto in = [&](double2* buf) {
+    OzWork w = c->oz;
+    if (!w.buf) {
+      w.buf = (unsigned char*)buf;
+      w.bytes = sizeof(double2) * (size_t)nk * PP;
+    }
+    w.err = wait_error(c);
+    w.launches = &c->n_launch;
+    return w;
+  };
   CKC(c, mark(c, 0, s, true));
   CKC(c, gemm_z_best(A_KM, B_KN, P, n, N, c->X64, P, (long)N * P, C, n, (long)N * n, Psi, n,
-                (long)P * n, nk, c->oz, s));
+                (long)P * n, nk, in(M), s));
   CKC(c, mark(c, 1, s, true));
   CKC(c, gemm_z_best(A_MK, B_NK_CONJ, P, P, n, Psi, n, (long)P * n, Psi, n, (long)P * n, D, P, PP,
-                nk, c->oz, s));
+                nk, in(M), s));
+  c->d_lost = false;
   CKC(c, mark(c, 2, s, true));
   CKC(c, kconv_z(D, c->Vh64, M, PP, c->n1, c->n2, c->n3, s));
   CKC(c, mark(c, 3, s, true));
+  c->e_first = Kao != nullptr;
+  if (profiling(c)) c->prof_e_first[c->prof_n] = c->e_first;
   if (Kao) {
-    CKC(c, gemm_z_best(A_MK_CONJ, B_KN, N, P, P, c->X64, P, (long)N * P, M, P, PP, c->Wao, P, (long)N * P, nk, c->oz, s));
-    CKC(c, mark(c, 4, s, true));
-    CKC(c, gemm_z_best(A_MK, B_NK, N, N, P, c->Wao, P, (long)N * P, c->X64, P, (long)N * P, Kao, N, (long)N * N, nk, c->oz, s));
-    CKC(c, mark(c, 5, s, true));
     CKC(c, ex_reduce_z(D, M, (long)nk * PP, nk, c->partial, c->n_partial, ex, s));
+    CKC(c, mark(c, 4, s, true));
+    c->d_lost = !c->oz.buf;
+    CKC(c, gemm_z_best(A_MK_CONJ, B_KN, N, P, P, c->X64, P, (long)N * P, M, P, PP, c->Wao, P, (long)N * P, nk, in(D), s));
+    CKC(c, mark(c, 5, s, true));
+    CKC(c, gemm_z_best(A_MK, B_NK, N, N, P, c->Wao, P, (long)N * P, c->X64, P, (long)N * P, Kao, N, (long)N * N, nk, in(D), s));
     CKC(c, mark(c, 6, s, true));
     return THC_OK;
   }
-  CKC(c, gemm_z_best(A_MK, B_KN, P, n, P, M, P, PP, Psi, n, (long)P * n, Y, n, (long)P * n, nk, c->oz, s));
+  c->d_lost = !c->oz.buf;
+  CKC(c, gemm_z_best(A_MK, B_KN, P, n, P, M, P, PP, Psi, n, (long)P * n, Y, n, (long)P * n, nk, in(D), s));
   CKC(c, mark(c, 4, s, true));
   CKC(c, gemm_z_best(A_MK_CONJ, B_KN, N, n, P, c->X64, P, (long)N * P, Y, n, (long)P * n, KC, n,
-                (long)N * n, nk, c->oz, s));
+                (long)N * n, nk, in(D), s));
   CKC(c, mark(c, 5, s, true));
   CKC(c, ex_reduce_z(Psi, Y, (long)nk * P * n, nk, c->partial, c->n_partial, ex, s));
   CKC(c, mark(c, 6, s, true));
@@ -810,6 +837,11 @@ static thc_status ao_prepare(thc_ctx* c) {
   }
   for (auto& w : want) {
     cudaError_t e = cudaMalloc(w.p, w.bytes);
+    if (e == cudaErrorMemoryAllocation && c->oz.buf) {   // optional scratch goes first
+      cudaGetLastError();
+      oz_free(c->oz);
+      e = cudaMalloc(w.p, w.bytes);
+    }
     if (e == cudaSuccess) e = cudaMemset(*w.p, 0, w.bytes);   // plane padding stays zero
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -935,7 +967,7 @@ thc_status thc_debug_slab_plan(int M, int N, int K, int batch, int real, size_t 
 thc_status thc_sync(thc_ctx* c) {
   if (!c) return THC_ERR_ARG;
   // the error word comes back with the stream's last work: one wait
-  int* err = c->tc_err ? c->tc_err : c->oz.buf ? c->oz.err() : nullptr;
+  int* err = wait_error(c);
   if (err) CKC(c, cudaMemcpyAsync(c->tc_err_host, err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CKC(c, cudaStreamSynchronize(c->stream));
   if (!err) return THC_OK;
@@ -966,6 +998,12 @@ thc_status thc_get_intermediate(thc_ctx* c, int which, double* out) {
   }
   const long n = (which == 0 || which == 3) ? (long)c->nk * c->nisdf * c->nocc
                                             : (long)c->nk * c->nisdf * c->nisdf;
+  if (which == 1 && c->d_lost) {
+    const long P = c->nisdf, n = c->nocc;
+    CKC(c, gemm_z(A_MK, B_NK_CONJ, (int)P, (int)P, (int)n, (const double2*)c->Psi, (int)n, P * n, (const double2*)c->Psi, (int)n,
+                  P * n, (double2*)c->D, (int)P, P * P, c->nk, c->stream));
+    c->d_lost = false;
+  }
   void* src = which == 0 ? c->Psi : which == 1 ? c->D : which == 2 ? c->M : c->Y;
   if (which == 2 && c->Mlo && c->m_ext)
     CKC(c, mlo_combine_c2z((const float2*)src, c->Mlo, (double2*)out, n, c->stream));
@@ -987,7 +1025,8 @@ thc_status thc_stage_times(thc_ctx* c, float ms[6]) {
   if (!c->built) return THC_OK;
   if (c->prof_max > 0) return THC_ERR_STATE;  // events are going to the profile slots
   CKC(c, cudaEventSynchronize(c->ev[6]));
-  for (int i = 0; i < kStages; i++) CKC(c, cudaEventElapsedTime(&ms[i], c->ev[i], c->ev[i + 1]));
+  const int* at = stage_order(c->e_first);
+  for (int i = 0; i < kStages; i++) CKC(c, cudaEventElapsedTime(&ms[i], c->ev[at[i]], c->ev[at[i] + 1]));
   return THC_OK;
 }
 
@@ -996,6 +1035,7 @@ thc_status thc_profile_begin(thc_ctx* c, int max_builds) {
   for (cudaEvent_t e : c->prof) cudaEventDestroy(e);
   c->prof.assign((size_t)max_builds * kProfEv, nullptr);
   for (auto& e : c->prof) CKC(c, cudaEventCreate(&e));
+  c->prof_e_first.assign((size_t)max_builds, 0);
   c->prof_max = max_builds;
   c->prof_n = 0;
   return THC_OK;
@@ -1010,11 +1050,13 @@ thc_status thc_profile_end(thc_ctx* c, float mean_ms[6], int* nbuilds) {
   for (int b = 0; b < nb; b++) {
     cudaEvent_t* e = &c->prof[(size_t)b * kProfEv];
     CKC(c, cudaEventSynchronize(e[6]));
+    const int* order = stage_order(c->prof_e_first[b]);
     for (int i = 0; i < kStages; i++) {
+      const int at = order[i];
       float t = 0.f;
-      CKC(c, cudaEventElapsedTime(&t, e[i], e[i + 1]));
+      CKC(c, cudaEventElapsedTime(&t, e[at], e[at + 1]));
       mean_ms[i] += t;
-      CKC(c, cudaEventElapsedTime(&t, e[7 + 2 * i], e[8 + 2 * i]));
+      CKC(c, cudaEventElapsedTime(&t, e[7 + 2 * at], e[8 + 2 * at]));
       core[i] += t;
     }
   }

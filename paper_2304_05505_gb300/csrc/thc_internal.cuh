@@ -17,8 +17,8 @@
 struct OzWork {
   unsigned char* buf = nullptr;
   size_t bytes = 0;
+  int* err = nullptr;        // error word and wait limit (16 bytes, cleared) of the kernels' bounded waits
   int* launches = nullptr;   // counts the kernels launched, when set
-  int* err() const { return (int*)buf; }
 };
 
 // ---------------------------------------------------------------------------
@@ -58,10 +58,14 @@ struct thc_ctx {
   int device;
   cudaStream_t stream;
   bool have_x, have_v, built;
-  // THC_FP64: scratch of the digit products of S1, S2, S4a and S4b, taken when
-  // the inputs are first set; without it they run on the FP64 pipe
+  // THC_FP64: scratch of the products where M and D, which serve as it otherwise,
+  // are small (up to 512 MB, taken when X is first set)
   OzWork oz;
   bool oz_asked;
+  // D was scratch of the products after S3 (it is made again from Psi
+  // where it is asked for), and the energy came before them (thc_build_K)
+  bool d_lost, e_first;
+  std::vector<char> prof_e_first;   // the same per profiled build
   int n_launch;     // kernels of the last FP64 build (0: none yet)
   // the tensor-core build replayed as a CUDA graph while not profiled: its
   // executable graph, which finds the caller's buffers through three

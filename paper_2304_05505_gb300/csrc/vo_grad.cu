@@ -737,7 +737,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     {
       int h = 0, ho = 0;
       if (tcerr && (e = cudaMemcpy(&h, tcerr, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
-      if ((e = cudaMemcpy(&ho, oz.err(), sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
+      if ((e = cudaMemcpy(&ho, oz.err, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
       if (h || ho) {
         st = THC_ERR_TIMEOUT;
         set_global_error("thc_vo_gradient: a device wait of a tensor-core product timed out");
