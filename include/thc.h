@@ -199,8 +199,8 @@ thc_status thc_sync(thc_ctx* ctx);
 /* Test hooks for failure detection (no GPU fault is involved in any).
  *
  * thc_debug_set_wait_limit: the limit, in SM clock cycles, of the bounded
- * device-side waits of the context's kernels (THC_MIXED; THC_ERR_UNSUPPORTED
- * for the forms without such waits).  cycles <= 0 restores the default (about
+ * device-side waits of the context's kernels (THC_ERR_UNSUPPORTED for
+ * THC_MIXED_SIMT, which has none).  cycles <= 0 restores the default (about
  * 2 s).  A limit of a few hundred cycles makes the waits of the next build
  * give up before their data arrives: each kernel then lets its copies and
  * MMAs in flight finish (with the default limit), stops, and thc_sync returns

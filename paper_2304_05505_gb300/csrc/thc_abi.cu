@@ -942,9 +942,10 @@ thc_status thc_build_host(thc_ctx* c, const double* C_host, double* KC_host, dou
 
 thc_status thc_debug_set_wait_limit(thc_ctx* c, long long cycles) {
   if (!c) return THC_ERR_ARG;
-  if (!c->tc_err) return THC_ERR_UNSUPPORTED;   // only the tensor-core form has device-side waits
+  int* err = wait_error(c);
+  if (!err) return THC_ERR_UNSUPPORTED;   // the CUDA-core form has no device-side waits
   const long long v = cycles > 0 ? cycles : 0;
-  CKC(c, cudaMemcpyAsync(reinterpret_cast<char*>(c->tc_err) + 8, &v, sizeof v, cudaMemcpyHostToDevice, c->stream));
+  CKC(c, cudaMemcpyAsync(reinterpret_cast<char*>(err) + 8, &v, sizeof v, cudaMemcpyHostToDevice, c->stream));
   CKC(c, cudaStreamSynchronize(c->stream));
   return THC_OK;
 }

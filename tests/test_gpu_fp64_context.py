@@ -80,3 +80,28 @@ def test_intermediates_after_builds(thc, mesh, nbas, nocc, nisdf):
             assert all(t > 0 for t in thc.thc_stage_times(eb.ctx))
     finally:
         eb.close()
+
+
+def test_wait_timeout_of_products_is_reported(thc):
+    """A limit of a few hundred cycles lets the waits of the digit products
+    give up before their data arrive; thc_sync says so, and with the default
+    limit the context builds correctly again."""
+    mesh, nbas, nocc, nisdf = (2, 2, 2), 60, 33, 260
+    r = cells.random_problem(mesh, nbas=nbas, nocc=nocc, nisdf=nisdf, seed=3)
+    ref = O.build(r["X"], r["C"], r["V"], mesh, route="direct")
+    eb = _context(thc, mesh, nbas, nocc, nisdf)
+    try:
+        eb.set_collocation(r["X"])
+        eb.set_kernel(r["V"])
+        thc.thc_debug_set_wait_limit(eb.ctx, 200)
+        eb.build(r["C"])
+        with pytest.raises(thc.ThcError) as e:
+            eb.sync()
+        assert e.value.code == 5                      # THC_ERR_TIMEOUT
+        thc.thc_debug_set_wait_limit(eb.ctx, 0)
+        KC, ex = eb.build(r["C"])
+        eb.sync()
+        assert np.abs(KC.cpu().numpy() - ref["KC"]).max() <= 1e-13 * np.abs(ref["KC"]).max()
+    finally:
+        thc.thc_debug_set_wait_limit(eb.ctx, 0)
+        eb.close()
