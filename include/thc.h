@@ -211,7 +211,9 @@ thc_status thc_sync(thc_ctx* ctx);
  * thc_create makes them) of the next thc_create on the calling thread fails
  * as if the device were out of memory, without calling the allocator; that
  * thc_create then returns THC_ERR_OOM having freed everything it allocated.
- * nth < 0 disables the hook. */
+ * In the next thc_fit_kernel, thc_rebuild_kernel or thc_vo_gradient it does so
+ * the first time: where the call holds scratch for digits it gives that back,
+ * allocates again and goes on without.  nth < 0 disables the hook. */
 thc_status thc_debug_set_wait_limit(thc_ctx* ctx, long long cycles);
 thc_status thc_debug_fail_alloc(int nth);
 

@@ -332,16 +332,51 @@ inline bool fit_geometry(const int* grid_host, const double* lattice_host, const
   return true;
 }
 
-// Scratch of the digit products of a fit and of its adjoint: the whole
-// operands of the metric and of the products of depth kdeep (over the
-// grid or its G set, npts x ndeep; 0: none), up to 1.25 GB (larger slabs
-// measured no faster for the metric).  At least what the metric's least slab
-// needs: a product without room for its own runs on the FP64 pipe.
-inline cudaError_t fit_scratch(OzWork& w, int npts, long ng, int nfunc, int ndeep, int kdeep, cudaStream_t s) {
-  const size_t least = oz_work_min(nfunc);
-  size_t want = std::max(oz_work_bytes(npts, (int)ng, nfunc, 1), oz_work_bytes(npts, (int)ng, npts, 1));
-  if (ndeep > 0) want = std::max(want, std::max(oz_work_min(kdeep), oz_work_bytes(npts, ndeep, kdeep, 1)));
-  return oz_alloc(w, std::max(least, std::min(want, (size_t)5 << 28)), least, s);
-}
+// The device memory of one call.  The scratch of its digit products is
+// optional (without it they run on the FP64 pipe): an allocation that the device
+// has no room for is tried again once the scratch is given back.
+struct DeviceMemory {
+  OzWork oz;
+  int lost = 0;                       // error word of scratch given back
+  int fail_at = take_fail_alloc();    // test hook: index of the allocation that fails the first time
+  int n = 0;
+
+  template <typename T>
+  cudaError_t get(T** p, size_t bytes) {
+    cudaError_t e = n++ == fail_at ? cudaErrorMemoryAllocation : cudaMalloc((void**)p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    *p = nullptr;
+    if (!oz.buf) return e;
+    e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = wait_error(&lost);
+    oz_free(oz);
+    return e == cudaSuccess ? cudaMalloc((void**)p, bytes) : e;
+  }
+
+  // Whether a wait of a digit product gave up (nonzero), of the work complete so far.
+  cudaError_t wait_error(int* h) {
+    *h = lost;
+    if (!oz.buf) return cudaSuccess;
+    int now = 0;
+    const cudaError_t e = cudaMemcpy(&now, oz.err, sizeof(int), cudaMemcpyDeviceToHost);
+    *h |= now;
+    return e;
+  }
+
+  // Scratch of a fit and of its adjoint: the whole operands of the metric and of
+  // the products of depth kdeep (over the grid or its G set, npts x ndeep; 0:
+  // none), up to 1.25 GB (larger slabs measured no faster for the metric), at
+  // least what the metric's least slab needs.
+  cudaError_t scratch(int npts, long ng, int nfunc, int ndeep, int kdeep, cudaStream_t s) {
+    const size_t least = oz_work_min(nfunc);
+    size_t want = std::max(oz_work_bytes(npts, (int)ng, nfunc, 1), oz_work_bytes(npts, (int)ng, npts, 1));
+    if (ndeep > 0) want = std::max(want, std::max(oz_work_min(kdeep), oz_work_bytes(npts, ndeep, kdeep, 1)));
+    const cudaError_t e = oz_alloc(oz, std::max(least, std::min(want, (size_t)5 << 28)), least, s);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    return cudaSuccess;
+  }
+};
 
 }  // namespace

@@ -167,24 +167,25 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
   double* svd = nullptr;
   unsigned* rmax = nullptr;
   double *R = nullptr, *S = nullptr, *L = nullptr, *rPd = nullptr;
-  OzWork oz;
+  DeviceMemory dm;
+  OzWork& oz = dm.oz;
   int *ptsd = nullptr, *gmd = nullptr, *flatd = nullptr, *bad = nullptr;
   cudaError_t e = cudaSuccess;
   thc_status st = THC_OK;
   int hbad = 0;
   do {
-    if ((e = cudaMalloc(&ptsd, sizeof(int) * npts)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&Ugc, sizeof(double2) * (size_t)npts * nfunc)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&Bm, sizeof(double2) * (size_t)npts * ng)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&R, sizeof(double) * (size_t)npts * ng)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&S, sizeof(double) * npq)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&L, sizeof(double) * npq)) != cudaSuccess) break;
-    if (dig && (e = fit_scratch(oz, npts, ng, nfunc, npts, nG, s)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&bad, sizeof(int))) != cudaSuccess) break;
-    if ((e = cudaMalloc(&twd, sizeof(double2) * tw.size())) != cudaSuccess) break;
-    if ((e = cudaMalloc(&gmd, sizeof(int) * gm.size())) != cudaSuccess) break;
-    if ((e = cudaMalloc(&flatd, sizeof(int) * flat.size())) != cudaSuccess) break;
-    if ((e = cudaMalloc(&rPd, sizeof(double) * rP.size())) != cudaSuccess) break;
+    if ((e = dm.get(&ptsd, sizeof(int) * npts)) != cudaSuccess) break;
+    if ((e = dm.get(&Ugc, sizeof(double2) * (size_t)npts * nfunc)) != cudaSuccess) break;
+    if ((e = dm.get(&Bm, sizeof(double2) * (size_t)npts * ng)) != cudaSuccess) break;
+    if ((e = dm.get(&R, sizeof(double) * (size_t)npts * ng)) != cudaSuccess) break;
+    if ((e = dm.get(&S, sizeof(double) * npq)) != cudaSuccess) break;
+    if ((e = dm.get(&L, sizeof(double) * npq)) != cudaSuccess) break;
+    if (dig && (e = dm.scratch(npts, ng, nfunc, npts, nG, s)) != cudaSuccess) break;
+    if ((e = dm.get(&bad, sizeof(int))) != cudaSuccess) break;
+    if ((e = dm.get(&twd, sizeof(double2) * tw.size())) != cudaSuccess) break;
+    if ((e = dm.get(&gmd, sizeof(int) * gm.size())) != cudaSuccess) break;
+    if ((e = dm.get(&flatd, sizeof(int) * flat.size())) != cudaSuccess) break;
+    if ((e = dm.get(&rPd, sizeof(double) * rP.size())) != cudaSuccess) break;
     if ((e = cudaMemcpyAsync(ptsd, points_host, sizeof(int) * npts, cudaMemcpyHostToDevice, s)) != cudaSuccess) break;
     if ((e = cudaMemcpyAsync(twd, tw.data(), sizeof(double2) * tw.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess)
       break;
@@ -223,7 +224,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     // 3. xh = DFT of xi, axis by axis (Bm holds the last two passes' input/output)
     cudaFree(Ugc);
     Ugc = nullptr;
-    if ((e = cudaMalloc(&F, sizeof(double2) * (size_t)npts * ng)) != cudaSuccess) break;
+    if ((e = dm.get(&F, sizeof(double2) * (size_t)npts * ng)) != cudaSuccess) break;
     const long tot = (long)npts * ng;
     if ((e = dft_axis(R, true, F, tot, g3, 1, twd + off[2], s)) != cudaSuccess) break;
     if ((e = dft_axis(F, false, Bm, tot, g2, g3, twd + off[1], s)) != cudaSuccess) break;
@@ -240,24 +241,24 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     long npart = 0;
     if (tc) {
       for (int g0 = 0; g0 < nG; g0 += slab) npart = std::max(npart, tc_partial_elems(npts, 2 * npts, 2 * std::min(slab, nG - g0), 1));
-      if ((e = cudaMalloc(&Xq32, sizeof(float2) * (size_t)npts * ldq)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&Bpl, 3 * 2 * (size_t)plane)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&eX, sizeof(int) * npts)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&tcerr, 64)) != cudaSuccess) break;
+      if ((e = dm.get(&Xq32, sizeof(float2) * (size_t)npts * ldq)) != cudaSuccess) break;
+      if ((e = dm.get(&Bpl, 3 * 2 * (size_t)plane)) != cudaSuccess) break;
+      if ((e = dm.get(&eX, sizeof(int) * npts)) != cudaSuccess) break;
+      if ((e = dm.get(&tcerr, 64)) != cudaSuccess) break;
       if ((e = cudaMemsetAsync(tcerr, 0, 64, s)) != cudaSuccess) break;
       if ((e = cudaMemsetAsync(Xq32, 0, sizeof(float2) * (size_t)npts * ldq, s)) != cudaSuccess) break;
       if ((e = cudaMemsetAsync(Bpl, 0, 3 * 2 * (size_t)plane, s)) != cudaSuccess) break;
       if (npart > 0) {
-        if ((e = cudaMalloc(&ps0, sizeof(int) * npart)) != cudaSuccess) break;
-        if ((e = cudaMalloc(&pbc, sizeof(float) * npart)) != cudaSuccess) break;
+        if ((e = dm.get(&ps0, sizeof(int) * npart)) != cudaSuccess) break;
+        if ((e = dm.get(&pbc, sizeof(float) * npart)) != cudaSuccess) break;
       }
-    } else if ((e = cudaMalloc(&Xq, sizeof(double2) * (size_t)npts * nG)) != cudaSuccess) {
+    } else if ((e = dm.get(&Xq, sizeof(double2) * (size_t)npts * nG)) != cudaSuccess) {
       break;
     }
-    if ((e = cudaMalloc(&W, sizeof(double2) * npq)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&svd, sizeof(double) * nG)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&phd, sizeof(double2) * npts)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&rmax, sizeof(unsigned) * npts)) != cudaSuccess) break;
+    if ((e = dm.get(&W, sizeof(double2) * npq)) != cudaSuccess) break;
+    if ((e = dm.get(&svd, sizeof(double) * nG)) != cudaSuccess) break;
+    if ((e = dm.get(&phd, sizeof(double2) * npts)) != cudaSuccess) break;
+    if ((e = dm.get(&rmax, sizeof(unsigned) * npts)) != cudaSuccess) break;
     const dim3 sgrid((nG + TB * SG - 1) / (TB * SG), npts);
     double2* V = (double2*)V_out;
     if ((e = cudaMemsetAsync(V, 0, sizeof(double2) * nk * npq, s)) != cudaSuccess) break;
@@ -308,7 +309,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     {
       int h = 0, ho = 0;
       if (tcerr && (e = cudaMemcpy(&h, tcerr, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
-      if (dig && (e = cudaMemcpy(&ho, oz.err, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
+      if ((e = dm.wait_error(&ho)) != cudaSuccess) break;
       if (h || ho) {
         st = THC_ERR_TIMEOUT;
         set_global_error("thc_rebuild_kernel: a device wait of a tensor-core product timed out");
@@ -328,7 +329,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
   void* ptrs[] = {Ugc, Bm, F, Xq, W, twd, R, S, L, rPd, phd, svd, rmax, ptsd, gmd, flatd, bad, Xq32, Bpl, eX, ps0, pbc, tcerr};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  oz_free(oz);
+  oz_free(dm.oz);
   for (auto& x : ev)
     if (x) cudaEventDestroy(x);
   return st;

@@ -22,7 +22,7 @@
 namespace {
 
 thread_local std::string g_create_error;
-thread_local int g_fail_alloc = -1;   // test hook: index of the next thc_create allocation to fail
+thread_local int g_fail_alloc = -1;   // test hook: index of the allocation to fail in the next call
 
 #define CKC(ctx, call)                                                       \
   do {                                                                       \
@@ -167,6 +167,12 @@ const int* stage_order(bool e_first) {
 
 }  // namespace
 
+int take_fail_alloc() {
+  const int n = g_fail_alloc;
+  g_fail_alloc = -1;
+  return n;
+}
+
 void set_global_error(const std::string& msg) { g_create_error = msg; }
 
 extern "C" {
@@ -256,8 +262,7 @@ thc_status thc_create(thc_ctx** out, const thc_dims* d, int precision, void* str
   W((void**)&c->exdev, 2 * sizeof(double));
   W((void**)&c->partial, 2 * kPartials * sizeof(double));
   W((void**)&c->flag, 64);
-  const int fail_at = g_fail_alloc;
-  g_fail_alloc = -1;
+  const int fail_at = take_fail_alloc();
   for (int i = 0; i < nw; i++) {
     Want& w = want[i];
     e = i == fail_at ? cudaErrorMemoryAllocation : cudaMalloc(w.p, w.bytes);

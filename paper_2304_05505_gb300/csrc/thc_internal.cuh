@@ -256,6 +256,9 @@ cudaError_t ex_reduce_c(const float2* Psi, const float2* Y, long n, int nk, doub
                         int npartial, double* ex, cudaStream_t s, double* const* ex_at = nullptr);
 
 // Message returned by thc_last_error(NULL) for calls made without a context.
+// Test hook: the index of the allocation that is to fail in the next call of this thread (-1: none); taken once.
+int take_fail_alloc();
+
 void set_global_error(const std::string& msg);
 
 // conversions and checks

@@ -346,7 +346,7 @@ __global__ void gather_conj_t32(const double2* __restrict__ U, int nf, long ng, 
 // slice products, exact K chunks of at most 1024 reals combined in FP64; out
 // complex128 with rows ldo and batches sbo complex apart.  Allocates its planes
 // and partial sums and frees them before returning.
-cudaError_t tc_product(const float2* A, int lda, const int* eA, const double2* src, long sbs, long ldk, long ldj,
+cudaError_t tc_product(DeviceMemory& dm, const float2* A, int lda, const int* eA, const double2* src, long sbs, long ldk, long ldj,
                        const int* eB, int batch, int M, int N, int K, double2* out, long ldo, long sbo, int* err,
                        cudaStream_t s) {
   if (batch > 1 && N > 65536) return cudaErrorInvalidValue;   // the embedding takes one slab of N per batch
@@ -358,11 +358,11 @@ cudaError_t tc_product(const float2* A, int lda, const int* eA, const double2* s
   float* pbc = nullptr;
   cudaError_t e = cudaSuccess;
   do {
-    if ((e = cudaMalloc(&pl, sizeof(uint16_t) * 3 * (size_t)plane)) != cudaSuccess) break;
+    if ((e = dm.get(&pl, sizeof(uint16_t) * 3 * (size_t)plane)) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(pl, 0, sizeof(uint16_t) * 3 * (size_t)plane, s)) != cudaSuccess) break;
     if (npart > 0) {
-      if ((e = cudaMalloc(&ps0, sizeof(int) * npart)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&pbc, sizeof(float) * npart)) != cudaSuccess) break;
+      if ((e = dm.get(&ps0, sizeof(int) * npart)) != cudaSuccess) break;
+      if ((e = dm.get(&pbc, sizeof(float) * npart)) != cudaSuccess) break;
     }
     TcOperand opA, opB;
     if ((e = make_f32_map(opA.map[0], A, batch, M, 2 * K, 2 * lda)) != cudaSuccess) break;
@@ -441,7 +441,8 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
   double2 *Psi = nullptr, *Psivt = nullptr, *D = nullptr, *M = nullptr, *W = nullptr, *Y = nullptr, *Ge = nullptr;
   double2 *Ugc = nullptr, *Bm = nullptr, *F = nullptr, *T = nullptr, *Gam = nullptr, *Aq = nullptr, *Bq = nullptr;
   double2 *Z = nullptr, *T1 = nullptr, *T2 = nullptr, *Uvp = nullptr, *G1 = nullptr, *G2 = nullptr, *twd = nullptr;
-  OzWork oz;
+  DeviceMemory dm;
+  OzWork& oz = dm.oz;
   double *R = nullptr, *S = nullptr, *L = nullptr, *Lam = nullptr, *Sbar = nullptr, *rPd = nullptr, *part = nullptr;
   int *ptsd = nullptr, *gmd = nullptr, *flatd = nullptr, *bad = nullptr, *kqd = nullptr, *qkd = nullptr;
   // tensor-core state of the (q, G) contraction (THC_MIXED)
@@ -459,7 +460,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
   const long ngo = (long)nk * nvir * nocc;
   do {
 #define ALLOC(p, n) \
-  if ((e = cudaMalloc(&p, sizeof(*p) * (size_t)(n))) != cudaSuccess) break
+  if ((e = dm.get(&p, sizeof(*p) * (size_t)(n))) != cudaSuccess) break
     ALLOC(ptsd, np);
     ALLOC(kqd, (long)nk * nk);
     ALLOC(qkd, (long)nk * nk);
@@ -496,7 +497,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
       break;
     if ((e = cudaMemsetAsync(bad, 0, sizeof(int), s)) != cudaSuccess) break;
 
-    if ((e = fit_scratch(oz, np, ng, nf, precision == THC_FP64 ? std::max(nf, nvir) : np, (int)ng, s)) != cudaSuccess) break;
+    if ((e = dm.scratch(np, ng, nf, precision == THC_FP64 ? std::max(nf, nvir) : np, (int)ng, s)) != cudaSuccess) break;
 
     // 1. the kernel held fixed: Psi, Psi_v at the points, D, W, M, Y, E_x, g_e
     mark(0);
@@ -529,11 +530,11 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
 
     // 2. the fit: B = conj(U_P)^T U, R = |B|^2, S = R[:, points], L L^T = S, xi = S^-1 R, F = DFT(xi)
     mark(1);
-    if ((e = cudaMalloc(&Ugc, sizeof(double2) * (size_t)np * nf)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&Bm, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&R, sizeof(double) * (size_t)np * ng)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&S, sizeof(double) * npq)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&L, sizeof(double) * npq)) != cudaSuccess) break;
+    if ((e = dm.get(&Ugc, sizeof(double2) * (size_t)np * nf)) != cudaSuccess) break;
+    if ((e = dm.get(&Bm, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
+    if ((e = dm.get(&R, sizeof(double) * (size_t)np * ng)) != cudaSuccess) break;
+    if ((e = dm.get(&S, sizeof(double) * npq)) != cudaSuccess) break;
+    if ((e = dm.get(&L, sizeof(double) * npq)) != cudaSuccess) break;
     gather_conj<<<blocks((long)np * nf), TB, 0, s>>>(U2, nf, ng, ptsd, np, Ugc);
     if ((e = dig ? gemm_z_best(A_MK, B_KN, np, (int)ng, nf, Ugc, nf, 0, U2, (int)ng, 0, Bm, (int)ng, 0, 1, oz, s)
                  : gemm_z(A_MK, B_KN, np, (int)ng, nf, Ugc, nf, 0, U2, (int)ng, 0, Bm, (int)ng, 0, 1, s)) !=
@@ -550,8 +551,8 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
       break;
     }
     chol_solve<<<blocks(ng), TB, 0, s>>>(L, R, np, ng);   // R now holds xi
-    if ((e = cudaMalloc(&F, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&T, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
+    if ((e = dm.get(&F, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
+    if ((e = dm.get(&T, sizeof(double2) * (size_t)np * ng)) != cudaSuccess) break;
     const long tot = (long)np * ng;
     // (THC_MIXED: the direct sums, as in step 4 below; an FFT's last bits would
     // come out of the solve there at 8e-8 of single entries of g)
@@ -562,14 +563,14 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
 
     // 3. Gam = sum over q and its representatives of (c ph W^q ph^H) (v o conj(xh))
     mark(2);
-    if ((e = cudaMalloc(&Gam, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
-    if (precision == THC_FP64 && (e = cudaMalloc(&Aq, sizeof(double2) * npq)) != cudaSuccess) break;
+    if ((e = dm.get(&Gam, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
+    if (precision == THC_FP64 && (e = dm.get(&Aq, sizeof(double2) * npq)) != cudaSuccess) break;
     if (precision == THC_FP64) {
-      if ((e = cudaMalloc(&Bq, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&Z, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
+      if ((e = dm.get(&Bq, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
+      if ((e = dm.get(&Z, sizeof(double2) * (size_t)np * nG)) != cudaSuccess) break;
     }
-    if ((e = cudaMalloc(&vt, sizeof(double) * nG)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&phd, sizeof(double2) * np)) != cudaSuccess) break;
+    if ((e = dm.get(&vt, sizeof(double) * nG)) != cudaSuccess) break;
+    if ((e = dm.get(&phd, sizeof(double2) * np)) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(Gam, 0, sizeof(double2) * (size_t)np * nG, s)) != cudaSuccess) break;
     // THC_MIXED: Z = A Bq on the tensor cores, A (FP32, sliced in the GEMM with
     // its row exponents) against the embedded Bq (three fp16 slices with the
@@ -582,16 +583,16 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     TcOperand opA, opB;
     if (tc) {
       const long npart = tc_partial_elems(np, 2 * nG, 2 * np, 1);
-      if ((e = cudaMalloc(&Aq32, sizeof(float2) * (size_t)np * lda)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&Bpl, sizeof(uint16_t) * 3 * (size_t)plane)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&eA, sizeof(int) * np)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&eB, sizeof(int) * nG)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&cm, sizeof(double) * nG)) != cudaSuccess) break;
+      if ((e = dm.get(&Aq32, sizeof(float2) * (size_t)np * lda)) != cudaSuccess) break;
+      if ((e = dm.get(&Bpl, sizeof(uint16_t) * 3 * (size_t)plane)) != cudaSuccess) break;
+      if ((e = dm.get(&eA, sizeof(int) * np)) != cudaSuccess) break;
+      if ((e = dm.get(&eB, sizeof(int) * nG)) != cudaSuccess) break;
+      if ((e = dm.get(&cm, sizeof(double) * nG)) != cudaSuccess) break;
       col_max<<<blocks(nG), TB, 0, s>>>(F, ng, flatd, nG, np, cm);
-      if ((e = cudaMalloc(&tcerr, 64)) != cudaSuccess) break;
+      if ((e = dm.get(&tcerr, 64)) != cudaSuccess) break;
       if (npart > 0) {
-        if ((e = cudaMalloc(&ps0, sizeof(int) * npart)) != cudaSuccess) break;
-        if ((e = cudaMalloc(&pbc, sizeof(float) * npart)) != cudaSuccess) break;
+        if ((e = dm.get(&ps0, sizeof(int) * npart)) != cudaSuccess) break;
+        if ((e = dm.get(&pbc, sizeof(float) * npart)) != cudaSuccess) break;
       }
       if ((e = cudaMemsetAsync(tcerr, 0, 64, s)) != cudaSuccess) break;
       if ((e = cudaMemsetAsync(Aq32, 0, sizeof(float2) * (size_t)np * lda, s)) != cudaSuccess) break;
@@ -649,10 +650,10 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     if ((e = dft_axis(F, false, T, tot, g3, 1, twd + geo.off[2], s, dig)) != cudaSuccess) break;
     if ((e = dft_axis(T, false, F, tot, g2, g3, twd + geo.off[1], s, dig)) != cudaSuccess) break;
     if ((e = dft_axis(F, false, T, tot, g1, (long)g2 * g3, twd + geo.off[0], s, dig)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&Lam, sizeof(double) * (size_t)np * ng)) != cudaSuccess) break;
+    if ((e = dm.get(&Lam, sizeof(double) * (size_t)np * ng)) != cudaSuccess) break;
     real_part<<<blocks(tot), TB, 0, s>>>(T, tot, Lam);
     chol_solve<<<blocks(ng), TB, 0, s>>>(L, Lam, np, ng);
-    if ((e = cudaMalloc(&Sbar, sizeof(double) * npq)) != cudaSuccess) break;
+    if ((e = dm.get(&Sbar, sizeof(double) * npq)) != cudaSuccess) break;
     // S-bar = -Lam xi^T
     if (oz_fits(np, np, (int)ng, 1, true, oz)) {
       if ((e = oz_gemm_d(false, false, np, np, (int)ng, Lam, ng, R, ng, Sbar, np, -1.0, false, true, oz, s)) != cudaSuccess)
@@ -672,11 +673,11 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     //    g = g_e + g_r
     mark(4);
     abs2_adjoint<<<blocks(tot), TB, 0, s>>>(Bm, Lam, tot);
-    if ((e = cudaMalloc(&T1, sizeof(double2) * (size_t)nf * np)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&T2, sizeof(double2) * (size_t)nf * ng)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&Uvp, sizeof(double2) * (size_t)nk * nvir * np)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&G1, sizeof(double2) * ngo)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&G2, sizeof(double2) * ngo)) != cudaSuccess) break;
+    if ((e = dm.get(&T1, sizeof(double2) * (size_t)nf * np)) != cudaSuccess) break;
+    if ((e = dm.get(&T2, sizeof(double2) * (size_t)nf * ng)) != cudaSuccess) break;
+    if ((e = dm.get(&Uvp, sizeof(double2) * (size_t)nk * nvir * np)) != cudaSuccess) break;
+    if ((e = dm.get(&G1, sizeof(double2) * ngo)) != cudaSuccess) break;
+    if ((e = dm.get(&G2, sizeof(double2) * ngo)) != cudaSuccess) break;
     // THC_MIXED: T1, T2 and the projection of T2 on the tensor cores when the
     // grid sum fits the exact K chunks of one product (2 N_g reals in at most
     // 126 chunks of 1024); else, and in THC_FP64, FP64 GEMMs
@@ -694,10 +695,10 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
       const int ldy = (int)(ng + (ng & 1));           // FP32 grid rows 16-byte strided
       const int lda2 = np + (np & 1);
       const long nfv = (long)nk * nvir;
-      if ((e = cudaMalloc(&Y32, sizeof(float2) * (size_t)np * ldy)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&A2, sizeof(float2) * (size_t)nf * lda2)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&Uv32, sizeof(float2) * (size_t)nfv * ldy)) != cudaSuccess) break;
-      if ((e = cudaMalloc(&eOrb, sizeof(int) * (size_t)(np + 3L * nf + ng + nfv))) != cudaSuccess) break;
+      if ((e = dm.get(&Y32, sizeof(float2) * (size_t)np * ldy)) != cudaSuccess) break;
+      if ((e = dm.get(&A2, sizeof(float2) * (size_t)nf * lda2)) != cudaSuccess) break;
+      if ((e = dm.get(&Uv32, sizeof(float2) * (size_t)nfv * ldy)) != cudaSuccess) break;
+      if ((e = dm.get(&eOrb, sizeof(int) * (size_t)(np + 3L * nf + ng + nfv))) != cudaSuccess) break;
       int* eY = eOrb;
       int* eU = eY + np;
       int* eA2 = eU + nf;
@@ -708,20 +709,20 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
       to_f32_rows<<<blocks((long)np * ng), TB, 0, s>>>(Bm, np, (int)ng, ng, Y32, ldy);
       if ((e = row_exponents_c(Y32, 0, ldy, 1, np, (int)ng, eY, s)) != cudaSuccess) break;
       if ((e = row_exponents_z(U2, 0, (int)ng, 1, nf, (int)ng, eU, s)) != cudaSuccess) break;
-      if ((e = tc_product(Y32, ldy, eY, U2, 0, 1, ng, eU, 1, np, nf, (int)ng, T1, nf, 0, tcerr, s)) != cudaSuccess)
+      if ((e = tc_product(dm, Y32, ldy, eY, U2, 0, 1, ng, eU, 1, np, nf, (int)ng, T1, nf, 0, tcerr, s)) != cudaSuccess)
         break;
       // T2[f][r] = sum_P conj(U[f][r_P]) Y2[P][r]
       gather_conj_t32<<<blocks((long)nf * np), TB, 0, s>>>(U2, nf, ng, ptsd, np, A2, lda2);
       if ((e = row_exponents_c(A2, 0, lda2, 1, nf, np, eA2, s)) != cudaSuccess) break;
       if ((e = col_exponents_z(Bm, 0, (int)ng, 1, np, (int)ng, eBm, s)) != cudaSuccess) break;
-      if ((e = tc_product(A2, lda2, eA2, Bm, 0, ng, 1, eBm, 1, nf, (int)ng, np, T2, ng, 0, tcerr, s)) !=
+      if ((e = tc_product(dm, A2, lda2, eA2, Bm, 0, ng, 1, eBm, 1, nf, (int)ng, np, T2, ng, 0, tcerr, s)) !=
           cudaSuccess)
         break;
       // G1^k[a][i] = sum_r Uv[(k,a)][r] T2[(k,i)][r]
       to_f32_rows<<<blocks(nfv * ng), TB, 0, s>>>(Uv2, nfv, (int)ng, ng, Uv32, ldy);
       if ((e = row_exponents_c(Uv32, 0, ldy, 1, (int)nfv, (int)ng, eUv, s)) != cudaSuccess) break;
       if ((e = row_exponents_z(T2, 0, (int)ng, 1, nf, (int)ng, eT2, s)) != cudaSuccess) break;
-      if ((e = tc_product(Uv32, ldy, eUv, T2, (long)nocc * ng, 1, ng, eT2, nk, nvir, nocc, (int)ng, G1, nocc,
+      if ((e = tc_product(dm, Uv32, ldy, eUv, T2, (long)nocc * ng, 1, ng, eT2, nk, nvir, nocc, (int)ng, G1, nocc,
                           (long)nvir * nocc, tcerr, s)) != cudaSuccess)
         break;
     }
@@ -737,7 +738,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
     {
       int h = 0, ho = 0;
       if (tcerr && (e = cudaMemcpy(&h, tcerr, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
-      if ((e = cudaMemcpy(&ho, oz.err, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) break;
+      if ((e = dm.wait_error(&ho)) != cudaSuccess) break;
       if (h || ho) {
         st = THC_ERR_TIMEOUT;
         set_global_error("thc_vo_gradient: a device wait of a tensor-core product timed out");
@@ -764,7 +765,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
                   flatd, bad, kqd, qkd, Aq32, Bpl, eA,  eB,  ps0, pbc, tcerr, Y32, A2, Uv32, eOrb, vt, cm, phd};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  oz_free(oz);
+  oz_free(dm.oz);
   for (auto& x : ev)
     if (x) cudaEventDestroy(x);
   return st;
