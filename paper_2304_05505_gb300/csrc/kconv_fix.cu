@@ -19,6 +19,14 @@
 // exchanges with one partner per radix-2 step.  With N1 = 4 the forward
 // transform leaves index m = 2 (t & 1) + (t >> 1) in slot t, Vh is read in
 // that order, and the inverse starts from it.
+//
+// Fixed point is no coarser than FP64 here: an FP64 DFT rounds its sums at
+// 2^-53 of their size, and every output adds the element's largest input, which
+// fixed point rounds at 2^-57 (4 x 4 x 4, rms of the element's largest M: 4e-17
+// to 8e-17 against 9e-17 to 1.2e-16 in FP64, for values within one order of
+// magnitude to spread over 16 between the k points).  Values with a NaN or an Inf, and products that
+// overflow, have no scale: their elements are transformed in FP64.
+#include "kconv_dft.cuh"
 #include "thc_internal.cuh"
 
 #include <math.h>
@@ -154,9 +162,20 @@ __device__ __forceinline__ int group_max(int e, int el) {
   return e;
 }
 
+// One element by the general FP64 transform, in place in its output (the
+// operations of kconv_kernel).
+__device__ __noinline__ void general(const double2* D, const double2* Vh, double2* M, long npq, const Twiddles& tw) {
+  const int nk = tw.n[0] * tw.n[1] * tw.n[2];
+  for (int k = 0; k < nk; k++) M[k * npq] = D[k * npq];
+  dft3<double>(M, npq, tw, -1);
+  for (int k = 0; k < nk; k++) M[k * npq] = cmul(M[k * npq], Vh[k * npq]);
+  dft3<double>(M, npq, tw, +1);
+}
+
 template <int N1, int N2, int N3>
 __global__ void __launch_bounds__(128) kconv_fix_kernel(const double2* __restrict__ D, const double2* __restrict__ Vh,
-                                                        double2* __restrict__ M, long npq) {
+                                                        double2* __restrict__ M, long npq,
+                                                        const __grid_constant__ Twiddles tw) {
   constexpr int L = N2 * N3, EPW = 32 / N1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int sl = lane / EPW, el = lane - sl * EPW;
@@ -196,21 +215,19 @@ __global__ void __launch_bounds__(128) kconv_fix_kernel(const double2* __restric
 #pragma unroll
   for (int j = 0; j < L; j++) x[j] = across<N1>(x[j], slot, el, +1, true);
   if (!ok) return;
-  // a NaN or an Inf among an element's values reaches all of them
-  const bool bad = E == 2047 || F == 2047;
+  if (E == 2047 || F == 2047) {   // (the same for all lanes of an element)
+    if (slot == 0) general(D + e, Vh + e, M + e, npq, tw);
+    return;
+  }
   double2* m = M + (long)slot * L * npq + e;
 #pragma unroll
-  for (int j = 0; j < L; j++) {
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    __stcs(m + (long)j * npq,
-           bad ? make_double2(nan, nan) : make_double2(from_fixed(x[j].x, F), from_fixed(x[j].y, F)));
-  }
+  for (int j = 0; j < L; j++) __stcs(m + (long)j * npq, make_double2(from_fixed(x[j].x, F), from_fixed(x[j].y, F)));
 }
 
 template <int N1, int N2, int N3>
 cudaError_t launch(const double2* D, const double2* Vh, double2* M, long npq, cudaStream_t s) {
   constexpr int EPB = 4 * (32 / N1);
-  kconv_fix_kernel<N1, N2, N3><<<(unsigned)((npq + EPB - 1) / EPB), 128, 0, s>>>(D, Vh, M, npq);
+  kconv_fix_kernel<N1, N2, N3><<<(unsigned)((npq + EPB - 1) / EPB), 128, 0, s>>>(D, Vh, M, npq, make_twiddles(N1, N2, N3));
   return cudaGetLastError();
 }
 

@@ -154,3 +154,57 @@ def test_selection_on_localised_orbitals(thc, decay):
     assert np.array_equal(pts, ref["points"])
     own = (np.abs(Uo) ** 2).sum(0) ** 2
     assert (np.abs(resid.cpu().numpy() - ref["resid"]) <= 1e-10 * own).all()
+
+
+@pytest.mark.parametrize("mesh", [(4, 4, 4), (3, 3, 3), (2, 4, 1), (1, 3, 2), (1, 1, 1)])
+def test_nonfinite_elements_of_the_convolution(thc, mesh):
+    """A NaN, an Inf or a product that overflows in the fixed-point convolution
+    leaves its element what the general FP64 transform makes of it, butterfly by
+    butterfly (numpy below), and touches no other element."""
+    nk, npq = int(np.prod(mesh)), 70
+    rng = np.random.default_rng(nk)
+    D = rng.normal(size=(nk, npq)) + 1j * rng.normal(size=(nk, npq))
+    V = rng.normal(size=(nk, npq)) + 1j * rng.normal(size=(nk, npq))
+    D[nk - 1, 5] = complex(np.inf, 0.0)
+    D[0, 11] = complex(0.5, np.nan)
+    D[:, 23] = complex(1e200, 0.0) * rng.normal(size=nk)
+    V[:, 23] = complex(1e200, 0.0) * rng.normal(size=nk)
+    D[0, 64] = complex(-np.inf, 0.0)
+    D[1 % nk, 64] = complex(np.inf, 1.0)
+
+    def axis(x, sign):       # along the first axis, the butterflies of the library
+        n = x.shape[0]
+        i = lambda z: np.stack([-sign * z[..., 1], sign * z[..., 0]], -1)
+        if n == 2:
+            return np.stack([x[0] + x[1], x[0] - x[1]])
+        if n == 3:
+            t, d = x[1] + x[2], x[1] - x[2]
+            m, s = x[0] - 0.5 * t, i(0.86602540378443864676 * d)
+            return np.stack([x[0] + t, m + s, m - s])
+        if n == 4:
+            a0, a1, b0, b1 = x[0] + x[2], x[0] - x[2], x[1] + x[3], i(x[1] - x[3])
+            return np.stack([a0 + b0, a1 + b1, a0 - b0, a1 - b1])
+        return x
+
+    def dft(x, sign):
+        x = x.reshape(mesh + (npq, 2))
+        for a in range(3):
+            x = np.moveaxis(axis(np.moveaxis(x, a, 0), sign), 0, a)
+        return x.reshape(nk, npq, 2)
+
+    def cmul(a, b):
+        return np.stack([a[..., 0] * b[..., 0] - a[..., 1] * b[..., 1], a[..., 0] * b[..., 1] + a[..., 1] * b[..., 0]], -1)
+
+    with np.errstate(all="ignore"):
+        pair = lambda z: np.stack([z.real, z.imag], -1)
+        vh = dft(pair(V), +1) / nk
+        ref = dft(cmul(dft(pair(D), -1), vh), +1)
+    M = torch.empty((nk, npq), dtype=torch.complex128, device="cuda")
+    thc.thc_kconv_noalloc(torch.from_numpy(D).cuda(), torch.from_numpy(V).cuda(), M, mesh, npq)
+    got = pair(M.cpu().numpy())
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    assert np.array_equal(np.where(np.isinf(got), np.sign(got), 0), np.where(np.isinf(ref), np.sign(ref), 0))
+    fine = np.isfinite(ref).all(axis=(0, 2))
+    assert set(np.nonzero(~fine)[0]) <= {5, 11, 23, 64}
+    scale = np.abs(ref).max(axis=(0, 2), where=np.isfinite(ref), initial=0)
+    assert (np.abs(got[:, fine] - ref[:, fine]) <= 1e-14 * nk * scale[None, fine, None]).all()
