@@ -63,7 +63,7 @@ typedef enum {
    * tensor cores (operand rows rounded to seven digits of 9 bits below their
    * largest entry, sums exact, rounded once), the rest in FP64 on CUDA cores.
    * Every result of such a product is checked: where sum |a||b| is below 2^-10
-   * of the product of the rows' largest entries, so that the digits could lose
+   * (|a|^2 max|b|^2 + |b|^2 max|a|^2)^(1/2), so that the digits could lose
    * accuracy, and where a row holds a NaN or an Inf, it is summed in FP64 */
   THC_FP64 = 0,
   THC_MIXED = 1,           /* S1, S2, S4a, S4b on tensor cores (tcgen05): each

@@ -28,12 +28,18 @@
 // compact basis function far from an orbital, sum |a||b| is far below their
 // product and an FP64 loop would do better.  So every product is checked
 // first: with m = |x| 2^-e of every entry (bf16, of the larger of re and im),
-// S = sum m_a m_b per result, in one product on the tensor cores.  Where S is
-// below 2^-10 (0.06 % of S4b's entries and 0.3 to 0.6 % of THC-AO-K's at
-// benzene-shaped cells) the result is computed in FP64 instead, as is one
-// whose rows hold a NaN or an Inf: single entries by a warp each, tiles with
-// many of them as gemm_z computes them.  At S = 2^-10 the digits leave 5e-17 of
-// sum |a||b| (K = 1200, twice that at most), FP64 sums 3e-16.
+// S = sum m_a m_b per result, in one product on the tensor cores.  The digits'
+// roundings, 2^-62 / sqrt(12) rms each, add up to 2^-63.3 (|m_a|^2 + |m_b|^2)^(1/2)
+// of the product of the largest entries at most.  So where S is below
+// 2^-10 (|m_a|^2 + |m_b|^2)^(1/2), and they would leave more than 2^-53.3 S (half a
+// unit roundoff of sum |a||b|, as FP64 sums do), the result is computed in FP64
+// instead, as is one whose rows hold a NaN or an Inf: single entries by a warp
+// each, tiles with a majority of them as gemm_z computes them.  (A line that
+// knows S alone is not enough: at S = 2^-10 rows with one large entry leave
+// 5e-17 of sum |a||b|, but rows of 1200 small ones beside it 1e-15.)  It is 0.05
+// to 0.15 % of S4b's entries and 0.7 to 3.5 % of THC-AO-K's at benzene-shaped
+// cells; there THC-AO-K pays for them (C1: 3.5 ms without the check, 5.0 ms
+// with it; build at 4 x 4 x 4 k, N_P = 1200: 8.8 ms, 9.3 with it).
 //
 // Complex products run as real ones with K = 2 K: one operand plain
 // (interleaved), the smaller one embedded as rows (re, -im) and (im, re).
@@ -82,9 +88,10 @@ constexpr int MK = 64;
 constexpr uint32_t MLB = TL * MK * 2, MCB = TN * MK * 2, MSTAGE = MLB + MCB;   // 16 KB + 10 KB
 constexpr int MSTAGES = 6, MEPI = 8, MNT = 32 * (4 + MEPI);
 constexpr size_t MSMEM = MSTAGES * MSTAGE + 1024 + 256;
-constexpr float CHECK = 0x1p-10f;                      // S below which digits are not enough
-constexpr int MANY = 80;                               // entries of a warp's 32 x 40 from which the tile goes whole
-constexpr int EPU = 64;                                // room for single entries, per tile
+constexpr float CHECK = 0x1p20f;                       // digits are not enough where S^2 CHECK < |m_a|^2 + |m_b|^2
+constexpr int MANY = 800;                              // entries of a warp's 32 x 40 from which the tile goes whole
+constexpr int EPU = 512;                               // room for single entries, per tile
+constexpr float NORM_UNIT = 4096.f;                    // |m|^2 is counted in units of 2^-12
 
 static_assert(SMEM <= 232448, "227 KB of shared memory per block");
 
@@ -426,7 +433,7 @@ __device__ __forceinline__ uint64_t desc128(uint32_t addr) {
 // a fifteenth of the product's planes and multiplies a 68th to a 136th as much.
 __global__ void __launch_bounds__(MNT, 1)
 oz_check_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict__ eL, const int* __restrict__ eN,
-                OzList f, int* err) {
+                const unsigned* __restrict__ qL, const unsigned* __restrict__ qN, OzList f, int* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(smem + MSTAGES * MSTAGE);
@@ -524,7 +531,10 @@ oz_check_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __res
       const int r = 32 * q + lane, c0 = MC * h;
       const bool row = r < g.lt && li * g.lt + r < g.lr;
       const bool nb = row && eL[(long)b * g.el + li * g.lt + r] == NB_ROW;
+      const float ql = row ? (float)qL[(long)b * g.el + li * g.lt + r] : 0.f;
       auto column = [&](int c) { return c < g.nt && ni * g.nt + c < g.nr; };
+      auto norm = [&](int c) { return column(c) ? (float)qN[(long)b * g.en + ni * g.nt + c] : 0.f; };
+      const float qn0 = norm(c0 + lane), qn1 = lane < MC - 32 ? norm(c0 + 32 + lane) : 0.f;
       auto bad = [&](int c) { return column(c) && eN[(long)b * g.en + ni * g.nt + c] == NB_ROW; };
       const unsigned long long cols = (unsigned long long)__ballot_sync(0xffffffffu, column(c0 + lane)) |
                                       (unsigned long long)__ballot_sync(0xffffffffu, lane < MC - 32 && column(c0 + 32 + lane)) << 32;
@@ -538,8 +548,10 @@ oz_check_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __res
         float v[10];
         tmem_ld10(tl + 128 * set + j0, v);
 #pragma unroll
-        for (int j = 0; j < 10; j++)
-          if (v[j] > 0.f && v[j] < CHECK) m |= 1ull << (j0 + j);
+        for (int j = 0; j < 10; j++) {
+          const float q = ql + __shfl_sync(0xffffffffu, j0 + j < 32 ? qn0 : qn1, (j0 + j) & 31);   // (by every lane)
+          if (v[j] > 0.f && v[j] * v[j] * (CHECK * NORM_UNIT) < q) m |= 1ull << (j0 + j);
+        }
       }
       tc_fence_before();
       __syncwarp();
@@ -630,7 +642,8 @@ __device__ __forceinline__ void put(double* __restrict__ out, const OzShape& g, 
 
 // The listed tiles (32 LI rows x 8 CJ columns, a block each, as gemm_kernel
 // sums them) and entries (a warp each).  Two FP64 multiply-adds a clock and SM
-// bind both.
+// bind both, so entries are listed one by one up to 800 of a warp's 1280 (from
+// 80 on as tiles: up to 16 times the work, on the SMs that get the tiles).
 template <int CX, int LI, int CJ>
 __global__ void __launch_bounds__(256) oz_exact_kernel(Source l, Source n, int K, OzShape g, OzList f,
                                                        double* __restrict__ out, const int* err) {
@@ -702,21 +715,25 @@ __global__ void __launch_bounds__(256) oz_exact_kernel(Source l, Source n, int K
 __device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
 // Largest biased exponent of each row: element (r, k) at src[r lr + k lk], CX
-// doubles each.  Rows with contiguous K: one warp per row.
+// doubles each.  Rows with contiguous K: one warp per row.  (The sums of the
+// magnitudes' squares, sq, are set to zero for the slicing that follows.)
 template <int CX>
 __global__ void __launch_bounds__(256) oz_exp_rows(const double* __restrict__ src, long sb, long lr, int rows, int K,
-                                                   int* __restrict__ e) {
+                                                   int* __restrict__ e, unsigned* __restrict__ sq) {
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= rows) return;
   const double* p = src + ((long)blockIdx.y * sb + (long)r * lr) * CX;
   int m = 0;
   for (int k = lane; k < K * CX; k += 32) m = max(m, expo(p[k]));
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) e[(long)blockIdx.y * rows + r] = m;
+  if (lane == 0) {
+    e[(long)blockIdx.y * rows + r] = m;
+    sq[(long)blockIdx.y * rows + r] = 0u;
+  }
 }
 
 // The same for contiguous rows (stride lk along K): one thread per row, K in
-// slices of KS rows over blockIdx.y, merged by atomicMax (e zeroed before).
+// slices of KS rows over blockIdx.y, merged by atomicMax (e and sq zeroed before).
 constexpr int KS = 64;
 template <int CX>
 __global__ void __launch_bounds__(128) oz_exp_cols(const double* __restrict__ src, long sb, long lk, int rows, int K,
@@ -756,10 +773,11 @@ __device__ __forceinline__ uint32_t mag16(unsigned long long u, int E) {
   return ex == 0 || d > 40 ? 86u << 7 : (uint32_t)(126 - d) << 7 | (uint32_t)(u >> 45 & 0x7f);
 }
 
-// The magnitudes of 8 consecutive reals of a row (CX = 2: of 4 complex values).
+// The magnitudes of 8 consecutive reals of a row (CX = 2: of 4 complex values); the sum of their squares.
 template <int CX>
-__device__ __forceinline__ void put_mags(const double* x, int E, uint16_t* dst) {
+__device__ __forceinline__ unsigned put_mags(const double* x, int E, uint16_t* dst) {
   uint32_t w[4 / CX];
+  float q = 0.f;
 #pragma unroll
   for (int i = 0; i < 4 / CX; i++) {
     uint32_t v[2];
@@ -769,11 +787,14 @@ __device__ __forceinline__ void put_mags(const double* x, int E, uint16_t* dst) 
       unsigned long long u = (unsigned long long)__double_as_longlong(y[0]) & ~(1ull << 63);
       if (CX == 2) u = max(u, (unsigned long long)__double_as_longlong(y[CX - 1]) & ~(1ull << 63));
       v[j] = mag16(u, E);
+      const float m = __uint_as_float(v[j] << 16);
+      q = fmaf(m, m, q);
     }
     w[i] = v[0] | v[1] << 16;
   }
   if constexpr (CX == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
   else *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+  return __float2uint_rn(q * NORM_UNIT);
 }
 
 // The planes of 8 consecutive reals of a row: digits from the last, each
@@ -822,9 +843,11 @@ __device__ __forceinline__ void put8(const double* x, int E, uint16_t* dst, long
 template <int CX, bool EMB>
 __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ src, long sb, long lr, int rows, int K,
                                                      int conj, const int* __restrict__ e, uint16_t* __restrict__ dst,
-                                                     int ldp, uint16_t* __restrict__ mag, int ldm) {
+                                                     int ldp, uint16_t* __restrict__ mag, int ldm,
+                                                     unsigned* __restrict__ sq) {
   const int ng = (K * CX + 7) / 8;
   const long i = (long)blockIdx.x * 256 + threadIdx.x;
+  const unsigned act = __ballot_sync(0xffffffffu, i < (long)rows * ng);
   if (i >= (long)rows * ng) return;
   const int r = (int)(i / ng), k0 = (int)(i % ng) * (8 / CX);
   const long b = blockIdx.y;
@@ -844,7 +867,18 @@ __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ 
   const long plane = (long)rows * (EMB ? 2 : 1) * ldp;
   const int E = e[b * rows + r];
   put8<EMB>(x, E, dst + b * ND * plane + (long)r * (EMB ? 2 : 1) * ldp + k0 * CX, plane, ldp);
-  if (mag) put_mags<CX>(x, E, mag + (b * rows + r) * ldm + k0);
+  if (mag) {
+    // (integer sums: the same whatever their order)
+    const unsigned q = put_mags<CX>(x, E, mag + (b * rows + r) * ldm + k0);
+    int one;
+    __match_all_sync(act, r, &one);
+    if (one) {                     // (the same for every lane: a row of its own)
+      const unsigned w = __reduce_add_sync(act, q);
+      if ((threadIdx.x & 31) == 0) atomicAdd(sq + b * rows + r, w);   // (lane 0 is the first to have work)
+    } else {
+      atomicAdd(sq + b * rows + r, q);
+    }
+  }
 }
 
 // The same for row-contiguous sources (stride lk along K): a block turns a
@@ -852,9 +886,12 @@ __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ 
 template <int CX, bool EMB>
 __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ src, long sb, long lk, int rows, int K,
                                                      int conj, const int* __restrict__ e, uint16_t* __restrict__ dst,
-                                                     int ldp, uint16_t* __restrict__ mag, int ldm) {
+                                                     int ldp, uint16_t* __restrict__ mag, int ldm,
+                                                     unsigned* __restrict__ sq) {
   constexpr int KT = 64 / CX;                       // 64 reals of K
   __shared__ double t[KT][33 * CX];
+  __shared__ unsigned part[32];
+  if (threadIdx.x < 32) part[threadIdx.x] = 0u;
   const int r0 = blockIdx.x * 32, k0 = blockIdx.y * KT;
   const long b = blockIdx.z;
   for (int i = threadIdx.x; i < KT * 32; i += 256) {
@@ -871,7 +908,7 @@ __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ 
   }
   __syncthreads();
   const int r = threadIdx.x / 8, c = threadIdx.x % 8;  // 8 reals of K each
-  if (r0 + r >= rows || k0 * CX + 8 * c >= ldp) return;
+  const bool in = r0 + r < rows && k0 * CX + 8 * c < ldp;
   double x[8];
 #pragma unroll
   for (int j = 0; j < 8 / CX; j++) {
@@ -883,9 +920,14 @@ __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ 
     }
   }
   const long plane = (long)rows * (EMB ? 2 : 1) * ldp;
-  const int E = e[b * rows + r0 + r];
-  put8<EMB>(x, E, dst + b * ND * plane + (long)(r0 + r) * (EMB ? 2 : 1) * ldp + k0 * CX + 8 * c, plane, ldp);
-  if (mag) put_mags<CX>(x, E, mag + (b * rows + r0 + r) * ldm + k0 + 8 / CX * c);
+  if (in) {
+    const int E = e[b * rows + r0 + r];
+    put8<EMB>(x, E, dst + b * ND * plane + (long)(r0 + r) * (EMB ? 2 : 1) * ldp + k0 * CX + 8 * c, plane, ldp);
+    if (mag) atomicAdd(part + r, put_mags<CX>(x, E, mag + (b * rows + r0 + r) * ldm + k0 + 8 / CX * c));
+  }
+  if (!mag) return;
+  __syncthreads();
+  if (threadIdx.x < 32 && r0 + (int)threadIdx.x < rows) atomicAdd(sq + b * rows + r0 + threadIdx.x, part[threadIdx.x]);
 }
 
 // One operand of a product: `rows` rows of K elements, element (r, k) at
@@ -903,13 +945,15 @@ long plane_rows(const Side& s) { return s.emb ? 2L * s.rows : s.rows; }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Scratch of one operand: exponents, digit planes, magnitudes (null: none are made).
+// Scratch of one operand: exponents, sums of the magnitudes' squares, digit
+// planes, magnitudes (null: none are made).
 struct Planes {
   int* e;
+  unsigned* sq;
   uint16_t *pl, *mag;
 };
 
-size_t exp_bytes(long rows, int batch) { return align256(sizeof(int) * (size_t)rows * batch); }
+size_t exp_bytes(long rows, int batch) { return align256(2 * sizeof(int) * (size_t)rows * batch); }
 size_t digit_bytes(long rows, bool emb, int K, int CX, int batch) {
   return align256(2 * (size_t)ND * (rows << emb) * pad8i(K * CX) * batch);
 }
@@ -919,7 +963,7 @@ size_t side_bytes(long rows, bool emb, int K, int CX, int batch) {
 
 Planes planes_at(void* at, long rows, bool emb, int K, int CX, int batch) {
   unsigned char* p = (unsigned char*)at + exp_bytes(rows, batch);
-  return Planes{(int*)at, (uint16_t*)p, (uint16_t*)(p + digit_bytes(rows, emb, K, CX, batch))};
+  return Planes{(int*)at, (unsigned*)at + rows * batch, (uint16_t*)p, (uint16_t*)(p + digit_bytes(rows, emb, K, CX, batch))};
 }
 
 long tiles_of(long rows, bool emb, int t) { return ((rows << emb) + t - 1) / t; }
@@ -941,24 +985,24 @@ template <int CX>
 cudaError_t prepare(const Side& a, int K, int batch, const Planes& p, cudaStream_t s) {
   const int ldp = pad8i(K * CX), ldm = pad8i(K);
   if (a.lk == 1) {
-    oz_exp_rows<CX><<<dim3((a.rows + 7) / 8, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, p.e);
+    oz_exp_rows<CX><<<dim3((a.rows + 7) / 8, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, p.e, p.sq);
     const unsigned nb = (unsigned)(((long)a.rows * (ldp / 8) + 255) / 256);
     if (a.emb)
       oz_slice_rows<2, true><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag,
-                                                             ldm);
+                                                             ldm, p.sq);
     else
       oz_slice_rows<CX, false><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, p.e, p.pl, ldp,
-                                                               p.mag, ldm);
+                                                               p.mag, ldm, p.sq);
   } else {
-    cudaError_t st = cudaMemsetAsync(p.e, 0, sizeof(int) * (size_t)batch * a.rows, s);
+    cudaError_t st = cudaMemsetAsync(p.e, 0, 2 * sizeof(int) * (size_t)batch * a.rows, s);   // p.sq too
     if (st != cudaSuccess) return st;
     oz_exp_cols<CX><<<dim3((a.rows + 127) / 128, (K + KS - 1) / KS, batch), 128, 0, s>>>(a.src, a.sb, a.lk, a.rows, K,
                                                                                         p.e);
     const dim3 grid((a.rows + 31) / 32, (K * CX + 63) / 64, batch);
     if (a.emb)
-      oz_slice_cols<2, true><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm);
+      oz_slice_cols<2, true><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm, p.sq);
     else
-      oz_slice_cols<CX, false><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm);
+      oz_slice_cols<CX, false><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm, p.sq);
   }
   return cudaGetLastError();
 }
@@ -1036,7 +1080,7 @@ cudaError_t slab(const Side& l, const Side& n, int K, int nb, const Planes& pl, 
   f = list_at(list, g.units);
   if (e == cudaSuccess) e = cudaMemsetAsync(f.cnt, 0, 64 + sizeof(int) * (size_t)g.units, s);
   if (e != cudaSuccess) return e;
-  oz_check_kernel<<<grid, MNT, MSMEM, s>>>(mags, g, pl.e, pn.e, f, w.err);
+  oz_check_kernel<<<grid, MNT, MSMEM, s>>>(mags, g, pl.e, pn.e, pl.sq, pn.sq, f, w.err);
   oz_kernel<<<grid, NT, SMEM, s>>>(maps, g, pl.e, pn.e, out, f, w.err);
   const Source sl{l.src, l.sb, l.lr, l.lk, l.conj}, sn{n.src, n.sb, n.lr, n.lk, n.conj};
   const unsigned xg = (unsigned)std::min<long>(2 * g.units, 2L * nsm);

@@ -110,6 +110,36 @@ def test_build_products_entry_by_entry(thc, mesh, nbas, nocc, nisdf, decay):
             assert err <= (4 * A.shape[1] + 2) * U, (what, err)
 
 
+@pytest.mark.parametrize("nbas", [33, 432, 1500])
+def test_many_small_entries_beside_a_large_one(thc, nbas):
+    """Rows of X^T with one large entry, where C is zero, and small ones, so
+    that S = sum |a||b| 2^-(ea+eb) is 2^-10 to 2^-4: it falls only as far as the
+    small entries do, and each of their roundings counts.
+
+    Bound: 6 u sum |a||b| (u = 2^-53).  Digits are kept where their roundings'
+    rms is at most 2^-53.3 sum |a||b| = 0.81 u; 6 sigma over 2^17 entries and
+    the final rounding make 5.4 u.  FP64 sums of random signs leave u
+    sum |a||b| times about 0.5 rms, 3 u at 6 sigma."""
+    rng = np.random.default_rng(nbas)
+    nocc, nisdf = 31, 260
+    X = rng.normal(size=(1, nbas, nisdf)) + 1j * rng.normal(size=(1, nbas, nisdf))
+    # (C's columns have entries of about 0.28 of their scale, so S = 0.31 nbas 2^-s)
+    X *= 2.0 ** -(np.log2(0.31 * nbas) + rng.uniform(4, 9.8, size=(1, 1, nisdf)))
+    X[0, 0] = 0.9
+    C = rng.normal(size=(1, nbas, nocc)) + 1j * rng.normal(size=(1, nbas, nocc))
+    C[0, 0] = 0.0
+    eb = thc.ExchangeBuild(dict(n1=1, n2=1, n3=1, nbas=nbas, nocc=nocc, nisdf=nisdf), "fp64")
+    try:
+        eb.set_collocation(X)
+        eb.set_kernel(cells.random_problem((1, 1, 1), nbas=8, nocc=3, nisdf=nisdf, seed=3)["V"])
+        eb.build(C)
+        eb.sync()
+        Psi = eb.intermediate(0).cpu().numpy()
+    finally:
+        eb.close()
+    assert _product_errors(X[0].T, C[0].T, Psi[0]).max() <= 6 * U
+
+
 @pytest.mark.parametrize("where", ["inf", "nan", "both"])
 def test_nonfinite_coefficients_spread_as_in_fp64_sums(thc, where):
     """An Inf or a NaN in C reaches the entries that it reaches on the FP64
