@@ -126,8 +126,9 @@ thc_status thc_set_kernel(thc_ctx* ctx, const double* V);
  * that is not being profiled runs as one CUDA graph launch: its kernels are
  * captured from the stream on the first build after thc_set_collocation or
  * thc_set_kernel and replayed on later ones, with any buffers (their addresses
- * are written on the stream when they change).  A capture the driver refuses, a
- * KC that is not 32-byte aligned, or a stream that is itself being captured
+ * are written on the stream when they change).  A KC that is not
+ * 32-byte aligned has a capture of its own; where nbas is above 6399, so has
+ * every set of buffers.  A capture the driver refuses, or a stream that is itself being captured,
  * gets the kernels directly. */
 thc_status thc_build(thc_ctx* ctx, const double* C, double* KC, double* ex);
 

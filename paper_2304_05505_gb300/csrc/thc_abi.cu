@@ -352,8 +352,10 @@ thc_status thc_create(thc_ctx** out, const thc_dims* d, int precision, void* str
 
 // Drops the captured build (the inputs or the kernel form changed).
 static void drop_graph(thc_ctx* c) {
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  c->gexec = nullptr;
+  for (cudaGraphExec_t& g : c->gexec) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  }
   c->g_C = c->g_KC = c->g_ex = nullptr;
   if (c->gexec_h) cudaGraphExecDestroy(c->gexec_h);
   c->gexec_h = nullptr;
@@ -760,19 +762,27 @@ __global__ void set_buffers(void** at, const void* C, void* KC, void* ex) {
 // from the stream once per collocation and kernel, and find the caller's
 // buffers through three addresses in device memory, which one small kernel
 // writes on the stream when they are others than the last build's (a capture
-// per set of buffers cost 0.2 ms, twice a small cell's build).  If the capture
-// fails the build runs directly.
+// per set of buffers cost 0.2 ms, twice a small cell's build).  The GEMM's stores
+// are chosen by the alignment of KC: there is a graph for KCs that are 32-byte
+// aligned and one for others (toy cell: 43 us, 70 without a graph).  Basis sets
+// too long for the embedding's shared memory have their C read at its own address
+// and are captured anew for other buffers (86 and 114 us at 6400 functions).  If
+// the capture fails the build runs directly.
 static thc_status build_tc_graph(thc_ctx* c, const double2* C, double2* KC, double* ex) {
-  // (the GEMM's stores are chosen by the alignment of KC; basis sets too long
-  // for the embedding's shared memory take their C directly)
   // (a stream that the caller is capturing takes the kernels themselves: the
   // addresses noted as written would otherwise only be written at a replay)
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
-  if (cap != cudaStreamCaptureStatusNone || !col_embed_fits(c->nbas) || ((uintptr_t)KC & 31))
-    return build_tc(c, C, KC, ex);
-  void** at = (void**)((char*)c->flag + 16);
-  if (!c->gexec) {
+  if (cap != cudaStreamCaptureStatusNone) return build_tc(c, C, KC, ex);
+  const bool any = col_embed_fits(c->nbas);   // the graph serves any buffers
+  void** at = any ? (void**)((char*)c->flag + 16) : nullptr;
+  const bool same = c->g_C == C && c->g_KC == KC && c->g_ex == ex;
+  cudaGraphExec_t& gexec = c->gexec[any && ((uintptr_t)KC & 31)];
+  if (gexec && !any && !same) {
+    cudaGraphExecDestroy(gexec);
+    gexec = nullptr;
+  }
+  if (!gexec) {
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
       cudaGetLastError();
@@ -781,19 +791,24 @@ static thc_status build_tc_graph(thc_ctx* c, const double2* C, double2* KC, doub
     const thc_status st = build_tc(c, C, KC, ex, nullptr, nullptr, at);
     const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
     cudaGraphExec_t x = nullptr;
-    if (st == THC_OK && e == cudaSuccess && g && cudaGraphInstantiate(&x, g, 0) == cudaSuccess) c->gexec = x;
+    if (st == THC_OK && e == cudaSuccess && g && cudaGraphInstantiate(&x, g, 0) == cudaSuccess) gexec = x;
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();   // a failed capture leaves no sticky error: run the build directly
-    if (!c->gexec) return build_tc(c, C, KC, ex);
+    if (!gexec) return build_tc(c, C, KC, ex);
+    c->g_upper = c->d_upper;
+    c->g_mext = c->m_ext;
   }
-  if (c->g_C != C || c->g_KC != KC || c->g_ex != ex) {
-    set_buffers<<<1, 1, 0, c->stream>>>(at, C, KC, ex);
+  // (what a build of another form has left behind is no longer there)
+  c->d_upper = c->g_upper;
+  c->m_ext = c->g_mext;
+  if (!same) {
+    if (any) set_buffers<<<1, 1, 0, c->stream>>>(at, C, KC, ex);
     CKC(c, cudaGetLastError());
     c->g_C = C;
     c->g_KC = KC;
     c->g_ex = ex;
   }
-  CKC(c, cudaGraphLaunch(c->gexec, c->stream));
+  CKC(c, cudaGraphLaunch(gexec, c->stream));
   return THC_OK;
 }
 
@@ -917,11 +932,15 @@ static thc_status build_host_overlapped(thc_ctx* c, const double2* C_host, doubl
       c->gexec_h = x;
       c->gh_C = C_host;
       c->gh_KC = KC_host;
+      c->g_upper = c->d_upper;
+      c->g_mext = c->m_ext;
     }
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
     if (!c->gexec_h) return build_tc(c, C, KC, c->exdev, nullptr, &io);
   }
+  c->d_upper = c->g_upper;
+  c->m_ext = c->g_mext;
   CKC(c, cudaGraphLaunch(c->gexec_h, c->stream));
   return THC_OK;
 }

@@ -68,11 +68,12 @@ struct thc_ctx {
   std::vector<char> prof_e_first;   // the same per profiled build
   int n_launch;     // kernels of the last FP64 build (0: none yet)
   // the tensor-core build replayed as a CUDA graph while not profiled: its
-  // executable graph, which finds the caller's buffers through three
-  // addresses in device memory (in the flag word's block), and the addresses
-  // last put there on the stream
-  cudaGraphExec_t gexec;
+  // executable graphs (KC 32-byte aligned, or not), which find the caller's
+  // buffers through three addresses in device memory (in the flag word's
+  // block), and the addresses last put there on the stream
+  cudaGraphExec_t gexec[2];
   const void *g_C, *g_KC, *g_ex;
+  bool g_upper, g_mext;   // d_upper and m_ext of the captured builds
   // thc_build_host: a copy stream that moves C in and KC out in halves beside
   // the build (events: fork, the two halves in, the two halves out, join),
   // and the captured host-buffer build with its host buffers
