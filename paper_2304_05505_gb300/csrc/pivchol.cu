@@ -39,7 +39,10 @@
 // the rows of points far apart, which have no entry in common, ran in FP64: 93
 // ms at 600 points, the residuals as far from 64 bits as without, 4.5e-12.)
 // (767 ms to 49 ms for 600 points.)  Where S comes out empty (more than 800
-// candidates within a bin of the largest) one pivot is taken the first way.
+// candidates within a bin of the largest), or a block ends after so few pivots
+// that they are cheaper one by one, pivots are taken the first way: 8 of them
+// before the next block, twice as many each time until a block pays again (200
+// points of equal density among 2400 at 420 functions: 48 to 12 ms).
 #include "oz_gemm.cuh"
 #include "thc_internal.cuh"
 
@@ -196,8 +199,8 @@ __global__ void __launch_bounds__(PT) hist_kernel(const double* __restrict__ d, 
   }
 }
 
-// The set: edge = the lowest bin with at most MS candidates in it and above;
-// idx = those candidates, ascending, then -1.  One block of 1024.
+// The set: edge[0] = the lowest bin with at most MS candidates in it and above;
+// idx = those candidates, ascending, then -1; edge[1] their count.  One block of 1024.
 __global__ void __launch_bounds__(1024) pick_kernel(const double* __restrict__ d, int n,
                                                     const double* __restrict__ selv, const int* __restrict__ hist,
                                                     int* __restrict__ idx, int* __restrict__ edge) {
@@ -243,6 +246,7 @@ __global__ void __launch_bounds__(1024) pick_kernel(const double* __restrict__ d
     base += all;
   }
   for (int i = base + t; i < MS; i += 1024) idx[i] = -1;
+  if (t == 0) edge[1] = base;
 }
 
 // Us[i][f] = U[f][idx[i]] (0 past the set); conj negates the imaginary part.
@@ -403,7 +407,7 @@ struct Blocks {
       if (e == cudaSuccess) e = cudaMalloc((void**)&p, n * sizeof(*p));
     };
     get(idx, MS);
-    get(edge, 1);
+    get(edge, 2);
     get(hist, NBIN);
     get(Us, (size_t)MS * nfunc);
     get(G2, (size_t)MS * MS);
@@ -479,11 +483,8 @@ extern "C" thc_status thc_select_points(const double* U, int nfunc, int ncand, i
     if (blocks && (e = oz_lane_prepare(u, ncand, ncand, nfunc, bk.lanes, s)) != cudaSuccess) break;
     double tr0 = -1.0;
     int count = 0;
-    // the pivots of one block; 0: none, one is taken by itself
+    // the pivots of one block, from a set that is not empty
     auto block = [&](int j) -> int {
-      if ((e = cudaMemsetAsync(bk.hist, 0, sizeof(int) * NBIN, s)) != cudaSuccess) return 0;
-      hist_kernel<<<nb, PT, 0, s>>>(d, ncand, selv, bk.hist);
-      pick_kernel<<<1, 1024, 0, s>>>(d, ncand, selv, bk.hist, bk.idx, bk.edge);
       gather_u<<<nblk((long)MS * nfunc, PT), PT, 0, s>>>(u, nfunc, ncand, bk.idx, MS, false, bk.Us);
       if ((e = oz_gemm_z(A_MK_CONJ, B_NK, MS, MS, nfunc, bk.Us, nfunc, 0, bk.Us, nfunc, 0, bk.G2, MS, 0, 1, false, bk.w, s)) !=
           cudaSuccess)
@@ -525,9 +526,21 @@ extern "C" thc_status thc_select_points(const double* U, int nfunc, int ncand, i
         }
       return T;
     };
+    // single pivots to take before the next block, and after the next one that does not pay: one of fewer pivots
+    // than its 0.5 ms of launches take one by one (17 at nfunc ncand = 1e6, 2 at 1e8)
+    int skip = 0, back = 8;
+    const int pays = 2 + (int)(0.5e-3 / (25e-6 + (double)nfunc * ncand / 1.3e11));
     for (int j = 0; j < npts;) {
       argmax_partial<<<nb, PT, 0, s>>>(d, ncand, pv, pi, ps);
       argmax_final<<<1, PT, 0, s>>>(pv, pi, ps, nb, sel, selv);
+      const bool try_block = blocks && skip == 0;
+      if (try_block) {
+        if ((e = cudaMemsetAsync(bk.hist, 0, sizeof(int) * NBIN, s)) != cudaSuccess) break;
+        hist_kernel<<<nb, PT, 0, s>>>(d, ncand, selv, bk.hist);
+        pick_kernel<<<1, 1024, 0, s>>>(d, ncand, selv, bk.hist, bk.idx, bk.edge);
+        if ((e = cudaMemcpyAsync((int*)(host + 3), bk.edge + 1, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+          break;
+      }
       if ((e = cudaMemcpyAsync(host, selv, 2 * sizeof(double), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
       if ((e = cudaMemcpyAsync((int*)(host + 2), sel, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         break;
@@ -535,9 +548,16 @@ extern "C" thc_status thc_select_points(const double* U, int nfunc, int ncand, i
       const double trace = host[1];
       if (j == 0) tr0 = trace;
       if (!(trace > rel_tol * tr0) || !(host[0] > 0.0)) break;   // rank reached
-      if (blocks) {
-        const int T = block(j);
+      if (skip > 0) skip--;
+      if (try_block) {
+        const int T = *(int*)(host + 3) > 0 ? block(j) : 0;
         if (e != cudaSuccess) break;
+        if (T < pays && j + T < npts) {
+          skip = back;
+          back = std::min(2 * back, 1024);
+        } else {
+          back = 8;
+        }
         if (T > 0) {
           for (int t = 0; t < T; t++) points_host[j + t] = bk.host->piv[t];
           j += T;
