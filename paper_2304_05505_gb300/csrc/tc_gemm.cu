@@ -375,6 +375,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   static_assert(NP == 6 || NP == 8, "slice products");
+  static_assert(CV || (OUT == 0 && NP == 6), "the plane-fed forms: FP32 output, one chunk, 6 products");
   static_assert(!(AR && CV), "A is resident planes or converted, not both");
   constexpr int AKB = 4;                                           // K blocks the resident A tile holds
   constexpr int CONV_WARPS = Roles<CV>::CONV_WARPS;
@@ -665,13 +666,7 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
               const uint32_t acc = (kb == kb0 && kk == 0) ? 0u : 1u;
               mma_f16(accA, a, b2, idesc, acc);                           // exact leading class (0,0)
               // the other classes, smallest first, into the second accumulator
-              if constexpr (NP == 8) {
-                mma_f16(accBC, a + PL, b2 + 2 * PL, idesc, acc);          // (1,2)
-                mma_f16(accBC, a + 2 * PL, b2 + PL, idesc, 1u);           // (2,1)
-                mma_f16(accBC, a, b2 + 2 * PL, idesc, 1u);                // (0,2)
-              } else {
-                mma_f16(accBC, a, b2 + 2 * PL, idesc, acc);               // (0,2)
-              }
+              mma_f16(accBC, a, b2 + 2 * PL, idesc, acc);                 // (0,2)
               mma_f16(accBC, a + 2 * PL, b2, idesc, 1u);                  // (2,0)
               mma_f16(accBC, a + PL, b2 + PL, idesc, 1u);                 // (1,1)
               mma_f16(accBC, a, b2 + PL, idesc, 1u);                      // (0,1)
@@ -893,43 +888,31 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
           }
         } else {
           // values of this lane's row into the staging tile
-          if constexpr (OUT == 2) {
-            // the exact leading sum as an int32 (va / 2^16 is an integer below
-            // 2^24) and the remainder, both in units of 2^16
+          float y[16];
 #pragma unroll
-            for (int j = 0; j < 16; j += 4)
-              *reinterpret_cast<float4*>(stg + stage_off(lane, j >> 2)) =
-                  make_float4(__int_as_float(__float2int_rn(va[j] * 0x1p-16f)),
-                              __int_as_float(__float2int_rn(va[j + 1] * 0x1p-16f)),
-                              __int_as_float(__float2int_rn(va[j + 2] * 0x1p-16f)),
-                              __int_as_float(__float2int_rn(va[j + 3] * 0x1p-16f)));
-          } else {
-            float y[16];
+          for (int j = 0; j < 16; j += 4) {
+            const int e0 = ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1)) - 30;
+            const int e1 = ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1) + 1) - 30;
+            const float s0 = plain ? __int_as_float((e0 + 127) << 23) : pow2f(e0);
+            const float s1 = plain ? __int_as_float((e1 + 127) << 23) : pow2f(e1);
+            // va is exact: one rounding in the add (CV: added when vb was read)
+            y[j] = (CV ? va[j] : va[j] + vb[j]) * s0;
+            y[j + 1] = (CV ? va[j + 1] : va[j + 1] + vb[j + 1]) * s0;
+            y[j + 2] = (CV ? va[j + 2] : va[j + 2] + vb[j + 2]) * s1;
+            y[j + 3] = (CV ? va[j + 3] : va[j + 3] + vb[j + 3]) * s1;
+            *reinterpret_cast<float4*>(stg + stage_off(lane, j >> 2)) = make_float4(y[j], y[j + 1], y[j + 2], y[j + 3]);
+          }
+          if (g.herm == 1) {
+            // the mirror image below the diagonal: out[Q][P] = conj(out[P][Q]) for Q > P,
+            // lanes = consecutive P, so each store instruction writes 256 contiguous bytes
+            const int P = row0 + lane;
+            if (P < g.M) {
+              float* ob = (float*)out + (long)b * sbo + 2L * P;
 #pragma unroll
-            for (int j = 0; j < 16; j += 4) {
-              const int e0 = ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1)) - 30;
-              const int e1 = ea + __shfl_sync(0xffffffffu, ebl, 8 * qq + (j >> 1) + 1) - 30;
-              const float s0 = plain ? __int_as_float((e0 + 127) << 23) : pow2f(e0);
-              const float s1 = plain ? __int_as_float((e1 + 127) << 23) : pow2f(e1);
-              // va is exact: one rounding in the add (CV: added when vb was read)
-              y[j] = (CV ? va[j] : va[j] + vb[j]) * s0;
-              y[j + 1] = (CV ? va[j + 1] : va[j + 1] + vb[j + 1]) * s0;
-              y[j + 2] = (CV ? va[j + 2] : va[j + 2] + vb[j + 2]) * s1;
-              y[j + 3] = (CV ? va[j + 3] : va[j + 3] + vb[j + 3]) * s1;
-              *reinterpret_cast<float4*>(stg + stage_off(lane, j >> 2)) = make_float4(y[j], y[j + 1], y[j + 2], y[j + 3]);
-            }
-            if (g.herm == 1) {
-              // the mirror image below the diagonal: out[Q][P] = conj(out[P][Q]) for Q > P,
-              // lanes = consecutive P, so each store instruction writes 256 contiguous bytes
-              const int P = row0 + lane;
-              if (P < g.M) {
-                float* ob = (float*)out + (long)b * sbo + 2L * P;
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                  const int Q = (col0 >> 1) + j;
-                  if (Q > P && 2 * Q < g.Nr)
-                    *reinterpret_cast<float2*>(ob + (long)Q * ldo) = make_float2(y[2 * j], -y[2 * j + 1]);
-                }
+              for (int j = 0; j < 8; j++) {
+                const int Q = (col0 >> 1) + j;
+                if (Q > P && 2 * Q < g.Nr)
+                  *reinterpret_cast<float2*>(ob + (long)Q * ldo) = make_float2(y[2 * j], -y[2 * j + 1]);
               }
             }
           }
@@ -937,8 +920,8 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
           // write out: lane -> (row rr, 4 columns f); 8 rows x 64 B per instruction
           const int f = lane >> 3;
           const int col = col0 + 4 * f;
-          const bool vec = (OUT == 2) ? (g.Nr % 4 == 0) : ((ldo % 4) == 0 && (sbo % 4) == 0);
-          if (OUT == 0 && vec && row0 + 32 <= g.M && col0 + 16 <= g.Nr && (!g.herm || (col0 >> 1) > row0 + 31)) {
+          const bool vec = (ldo % 4) == 0 && (sbo % 4) == 0;
+          if (vec && row0 + 32 <= g.M && col0 + 16 <= g.Nr && (!g.herm || (col0 >> 1) > row0 + 31)) {
             // a block inside the result, above the diagonal: no element to leave out
             float* o = (float*)out + (long)b * sbo + (long)(row0 + (lane & 7)) * ldo + col;
 #pragma unroll
@@ -948,40 +931,23 @@ tc_gemm_kernel(const __grid_constant__ Maps maps, Geometry g, const int* __restr
             continue;
           }
 #pragma unroll
-          for (int pass = 0; pass < (OUT == 2 ? 2 : 1); pass++) {
-            if (pass == 1) {   // FP32 remainders of the chunk through the same tile
-              __syncwarp();
-#pragma unroll
-              for (int j = 0; j < 16; j += 4)
-                *reinterpret_cast<float4*>(stg + stage_off(lane, j >> 2)) =
-                    make_float4(vb[j] * 0x1p-16f, vb[j + 1] * 0x1p-16f, vb[j + 2] * 0x1p-16f, vb[j + 3] * 0x1p-16f);
-              __syncwarp();
+          for (int it = 0; it < 4; it++) {
+            const int rr = (lane & 7) + 8 * it;
+            const int row = row0 + rr;
+            if (row >= g.M || col >= g.Nr) continue;
+            const float4 v = *reinterpret_cast<const float4*>(stg + stage_off(rr, f));
+            float* o = (float*)out + (long)b * sbo + (long)row * ldo;
+            if (g.herm && (col >> 1) + 1 <= row) {   // on or below the diagonal
+              if ((col >> 1) + 1 == row) *reinterpret_cast<float2*>(o + col + 2) = make_float2(v.z, v.w);
+              continue;
             }
+            if (vec && col + 4 <= g.Nr) {
+              *reinterpret_cast<float4*>(o + col) = v;
+            } else {
+              const float w4[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (int it = 0; it < 4; it++) {
-              const int rr = (lane & 7) + 8 * it;
-              const int row = row0 + rr;
-              if (row >= g.M || col >= g.Nr) continue;
-              const float4 v = *reinterpret_cast<const float4*>(stg + stage_off(rr, f));
-              float* o;
-              if constexpr (OUT == 2) {
-                const long base = (((long)kc * g.batch + b) * g.M + row) * g.Nr;
-                o = pass == 0 ? reinterpret_cast<float*>(ps0 + base) : pbc + base;
-              } else {
-                o = (float*)out + (long)b * sbo + (long)row * ldo;
-              }
-              if (OUT == 0 && g.herm && (col >> 1) + 1 <= row) {   // on or below the diagonal
-                if ((col >> 1) + 1 == row) *reinterpret_cast<float2*>(o + col + 2) = make_float2(v.z, v.w);
-                continue;
-              }
-              if (vec && col + 4 <= g.Nr) {
-                *reinterpret_cast<float4*>(o + col) = v;
-              } else {
-                const float w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int i = 0; i < 4; i++)
-                  if (col + i < g.Nr) o[col + i] = w4[i];
-              }
+              for (int i = 0; i < 4; i++)
+                if (col + i < g.Nr) o[col + i] = w4[i];
             }
           }
           __syncwarp();   // the tile is rewritten by the next block
@@ -1321,22 +1287,23 @@ cudaError_t tc_gemm(const TcOperand& A, const TcOperand& B, int M, int Nr, int K
     launch_pdl(tc_gemm_kernel<OUTK, NPK, ARK, CVK>, grid, Roles<CVK>::NT, Smem<CVK>::BYTES, s, maps, g, eA, seA, eB, seB, \
                                                                            out, out_at, ldo, sbo, ps0, pbc, err); \
   }
-#define BY_OUT(NPK, ARK, CVK) \
-  { if (split) LAUNCH(2, NPK, ARK, CVK) else if (out_f64) LAUNCH(1, NPK, ARK, CVK) else LAUNCH(0, NPK, ARK, CVK) }
-  // A resident when all K fits the resident tile (one chunk of at most 4 K blocks)
-  const bool ar = !a_conv && !split && g.nkb <= 4 && products == 6;
+  // (the forms that the builds and the set-up calls take, see tc_gemm.cuh)
   if (a_conv == 1) {
-    if (products == 6) BY_OUT(6, false, 1) else BY_OUT(8, false, 1)
+    if (products != 8) return cudaErrorInvalidValue;
+    if (split) LAUNCH(2, 8, false, 1) else if (out_f64) LAUNCH(1, 8, false, 1) else LAUNCH(0, 8, false, 1)
+  } else if (out_f64) {
+    return cudaErrorInvalidValue;
   } else if (a_conv == 2) {
-    if (products == 6) BY_OUT(6, false, 2) else BY_OUT(8, false, 2)
+    if (products == 6) { if (split) LAUNCH(2, 6, false, 2) else LAUNCH(0, 6, false, 2) }
+    else { if (split) LAUNCH(2, 8, false, 2) else LAUNCH(0, 8, false, 2) }
   } else if (a_conv == 3) {
-    if (products == 6) BY_OUT(6, false, 3) else BY_OUT(8, false, 3)
-  } else if (ar) {
-    if (out_f64) LAUNCH(1, 6, true, 0) else LAUNCH(0, 6, true, 0)
+    if (products != 8) return cudaErrorInvalidValue;
+    if (split) LAUNCH(2, 8, false, 3) else LAUNCH(0, 8, false, 3)
   } else {
-    if (products == 6) BY_OUT(6, false, 0) else BY_OUT(8, false, 0)
+    if (split || products != 6) return cudaErrorInvalidValue;
+    // A resident when all K fits the resident tile (at most 4 K blocks)
+    if (g.nkb <= 4) LAUNCH(0, 6, true, 0) else LAUNCH(0, 6, false, 0)
   }
-#undef BY_OUT
 #undef LAUNCH
   e = cudaGetLastError();
   if (e == cudaSuccess && gemm_done) e = cudaEventRecord(gemm_done, s);

@@ -25,13 +25,14 @@ cudaError_t make_plane_map(void* map_out, const void* base, int batch, int rows,
 // is recorded on `s` right after the GEMM kernel, before any combine kernel,
 // so that the GEMM alone can be timed.  products: 6 or 8 slice products per
 // real product (about 2^-27 or 2^-30 of the row scales dropped).  a_conv: 0 =
-// A is three planes; 1 = A.map[0] is an FP32 map (make_f32_map) of the
+// A is three planes (6 products, one chunk, FP32 output); 1 = A.map[0] is an FP32 map (make_f32_map) of the
 // interleaved complex A [rows][K], cut into its slices inside the kernel with
 // the row exponents eA; 2 = A.map[0] is an FP32 map (make_f32_map_t) of the
 // stored transpose [K][rows] of A; 3 = as 1, and A.map[1] an fp16 plane map
 // (make_plane_map) of A's remainders below its FP32 values, each an fp16
 // multiple q of its value's unit in the last place (q 2^(e - 24) for a value
-// m 2^e, 1/2 <= m < 1), sliced with them.  herm (1 or 2): the product is Hermitian
+// m 2^e, 1/2 <= m < 1), sliced with them.  (1: 8 products, any output; 2: FP32
+// output; 3: 8 products, FP32 output.)  herm (1 or 2): the product is Hermitian
 // (B built from conj(A), Nr = 2 M, one K chunk, FP32 output): only the tiles
 // that reach the diagonal are computed, and each writes its values on or
 // above the diagonal, and with herm = 1 also their conjugates at the mirrored
@@ -101,11 +102,11 @@ cudaError_t col_exponents_c(const float2* src, long sbs, int lds, int batch, int
 
 // The three fp16 slices of the contiguous rows src[row][0..np) (rows = batch
 // x rows per batch) with each row's exact exponent, found by the same kernel;
-// writes the exponents to e[row].  bplanes (optional, same ldp): also the
+// writes the exponents to e[row].  bplanes (same ldp): the
 // embedded B operand of src^H that embed_b writes for (src, conj_src,
 // conj_a = 0) with these exponents (rows 2 row, 2 row + 1).
 cudaError_t slice_rows_exact(const float2* src, int np, long rows, int* e, uint16_t* planes, long plane, int ldp,
-                             cudaStream_t s, uint16_t* bplanes = nullptr, long bplane = 0);
+                             cudaStream_t s, uint16_t* bplanes, long bplane);
 // Exponents alone of the contiguous rows src[row][0..np): one warp per row,
 // 16-byte loads when np is even.
 cudaError_t row_exponents_rows(const float2* src, int np, long rows, int* e, cudaStream_t s);
