@@ -44,12 +44,27 @@ SAMPLE_FRACTION = 8      # the CPU oracle sample is 1/8 of a build
 SLICE_PRODUCTS = {"S1_collocate": 6, "S2_density": 6, "S4a_apply_M": 8, "S4b_backproject": 8}
 
 
-def kernel_names(hermitian: bool) -> dict:
-    """The main kernel of each stage of the tensor-core build."""
+def hermitian_tiles(d: dict) -> bool:
+    """Whether the mixed build convolves a Hermitian V in tiles (csrc/kconv.cu,
+    kconv_c_tile_herm) on a mesh without the 2^3, 3^3 and 4^3 form: axes of 1, 2,
+    3, 4 and 6 points, N_P even, the keys within the planes of the B operands of
+    S2 and S4a.  S2 and S3 then do the work of the Hermitian form."""
+    n, P = (d["n1"], d["n2"], d["n3"]), d["nisdf"]
+    nk = n[0] * n[1] * n[2]
+    pad8 = lambda x: (x + 7) // 8 * 8
+    words = n[0] * ((n[1] * n[2] + 1) // 2) * P
+    return (P % 2 == 0 and P * P < 1 << 29 and all(m in (1, 2, 3, 4, 6) for m in n) and
+            4 * words * ((P + 7) // 8) <= 6 * nk * 2 * P * pad8(2 * d["nocc"]) and
+            4 * words * ((P + 3) // 4) <= 6 * nk * 2 * d["nocc"] * pad8(2 * P))
+
+
+def kernel_names(hermitian: bool, tiled: bool = False) -> dict:
+    """The main kernel of each stage of the tensor-core build (tiled: hermitian_tiles)."""
     return {"S1_collocate": "tc_gemm_kernel<0, 6, 0, 2> (S1, X^T read from FP32 X and sliced in the GEMM)",
-            "S2_density": ("tc_gemm_kernel<0, 6, 1, 0> (S2, A resident, Hermitian tiles)" if hermitian else
+            "S2_density": ("tc_gemm_kernel<0, 6, 1, 0> (S2, A resident, Hermitian tiles)" if hermitian or tiled else
                            "tc_gemm_kernel<0, 6, 1, 0> (S2, A resident, Hermitian tiles mirrored)"),
-            "S3_kconv": ("kconv_herm_kernel<4, 4, 4> (S3, Hermitian tiles)" if hermitian else
+            "S3_kconv": ("kconv_tile_herm_kernel (S3, Hermitian tiles)" if tiled else
+                         "kconv_herm_kernel<4, 4, 4> (S3, Hermitian tiles)" if hermitian else
                          "kconv_tile_kernel (S3, TMA-fed shared-memory DFTs)"),
             "S4a_apply_M": "tc_gemm_kernel<2, 8, 0, 1> (S4a, split-K, M sliced in the GEMM)",
             "S4b_backproject": "tc_gemm_kernel<2, 8, 0, 1> (S4b, split-K, X sliced in the GEMM)",
@@ -218,19 +233,27 @@ def stage_work(d: dict, hermitian: bool = False) -> dict:
     }
 
 
+DIGIT_PRODUCTS = 34     # bf16 products of a real product from digits (csrc/oz_gemm.cu)
+
+
 def fp64_roofline(d: dict, stages_ms: dict, fp64_tflops: float, pk: dict) -> dict:
-    """The FP64 build against its own peaks: its four GEMMs (full D in S2) run
-    on the FP64 pipe of the CUDA cores, reported against the measured FP64
-    FMA rate; its k-convolution (complex128 D, Vh and M) against the copy
-    bandwidth."""
+    """The FP64 build against its own peaks.  Its four GEMMs (full D in S2) are
+    formed from digits on the tensor cores, DIGIT_PRODUCTS bf16 products per real
+    product: issued_tensor_frac is their rate against the sustained bf16 peak;
+    frac is the FP64 rate they come to over the measured FMA rate of the FP64
+    pipe, which they pass.  The k-convolution (complex128 D, Vh and M) stands
+    against the copy bandwidth."""
     nk = d["n1"] * d["n2"] * d["n3"]
     N, n, P = d["nbas"], d["nocc"], d["nisdf"]
     flops = {"S1_collocate": 8.0 * nk * P * n * N, "S2_density": 8.0 * nk * P * P * n,
              "S4a_apply_M": 8.0 * nk * P * P * n, "S4b_backproject": 8.0 * nk * N * n * P}
-    out = {"fp64_peak_tflops": fp64_tflops, "peak_source": "measured FP64 FMA rate (thc_measure_fp64_rate)"}
+    out = {"fp64_peak_tflops": fp64_tflops, "peak_source": "measured FP64 FMA rate (thc_measure_fp64_rate); products "
+           "from digits run on the tensor cores, so their frac can pass 1", "digit_products": DIGIT_PRODUCTS}
     for st, f in flops.items():
         a = f / (stages_ms[st] * 1e-3) / 1e12
-        out[st] = {"bound": "fp64", "achieved_tflops": a, "frac": a / fp64_tflops}
+        out[st] = {"bound": "tensor", "achieved_tflops": a, "frac": a / fp64_tflops}
+        if "bf16_tflops_sustained" in pk:
+            out[st]["issued_tensor_frac"] = DIGIT_PRODUCTS * a / pk["bf16_tflops_sustained"]
     b = 16.0 * nk * 3 * P * P
     a = b / (stages_ms["S3_kconv"] * 1e-3) / 1e9
     out["S3_kconv"] = {"bound": "hbm", "achieved_gbs": a, "frac": a / pk["hbm_gbs"]}
@@ -617,6 +640,8 @@ def run_ours(args, world, rank, local):
     eb.set_collocation(p.X)
     eb.set_kernel(p.V)
     hermitian = thc.thc_hermitian_kernel(eb.ctx)
+    tiled = not hermitian and hermitian_tiles(d) and all(
+        np.abs(v - v.conj().T).max() <= 1e-12 * np.abs(v).max() for v in p.V)
     C = torch.from_numpy(p.C).to(dev)
     KC = torch.empty(eb.kc_shape, dtype=torch.complex128, device=dev)
     ex = torch.empty(2, dtype=torch.float64, device=dev)
@@ -722,13 +747,13 @@ def run_ours(args, world, rank, local):
     if rank != 0:
         return
     pk = peaks()
-    work = stage_work(d, hermitian)
+    work = stage_work(d, hermitian or tiled)
     names = thc.STAGES
     stages = {nm: ms for nm, ms in zip(names, stage_ms)}
     kernels = {nm: ms for nm, ms in zip(names, kernel_ms)}
     dominant = max(kernels, key=kernels.get)
     roof = kernel_roofline(dominant, kernels[dominant], work, pk, args.config)
-    roof["name"] = kernel_names(hermitian)[dominant]
+    roof["name"] = kernel_names(hermitian, tiled)[dominant]
     # (S5 fused into S4a's combine moves only its partial sums: no roofline of its own)
     per_kernel = {nm: kernel_roofline(nm, kernels[nm], work, pk, args.config) for nm in names
                   if not (nm == "S5_energy" and s4a_split(d))}
