@@ -64,7 +64,8 @@ typedef enum {
    * largest entry, sums exact, rounded once), the rest in FP64 on CUDA cores.
    * Every result of such a product is checked: where sum |a||b| is below 2^-10
    * (|a|^2 max|b|^2 + |b|^2 max|a|^2)^(1/2), so that the digits could lose
-   * accuracy, and where a row holds a NaN or an Inf, it is summed in FP64 */
+   * accuracy, it is formed from eight digits or, below 2^-18 of that and where a row
+   * holds a NaN or an Inf, summed in FP64 */
   THC_FP64 = 0,
   THC_MIXED = 1,           /* S1, S2, S4a, S4b on tensor cores (tcgen05): each
                               operand row scaled by a power of two and cut into

@@ -31,15 +31,22 @@
 // S = sum m_a m_b per result, in one product on the tensor cores.  The digits'
 // roundings, 2^-62 / sqrt(12) rms each, add up to 2^-63.3 (|m_a|^2 + |m_b|^2)^(1/2)
 // of the product of the largest entries at most.  So where S is below
-// 2^-10 (|m_a|^2 + |m_b|^2)^(1/2), and they would leave more than 2^-53.3 S (half a
-// unit roundoff of sum |a||b|, as FP64 sums do), the result is computed in FP64
-// instead, as is one whose rows hold a NaN or an Inf: single entries by a warp
-// each, tiles with a majority of them as gemm_z computes them.  (A line that
-// knows S alone is not enough: at S = 2^-10 rows with one large entry leave
-// 5e-17 of sum |a||b|, but rows of 1200 small ones beside it 1e-15.)  It is 0.05
-// to 0.15 % of S4b's entries and 0.7 to 3.5 % of THC-AO-K's at benzene-shaped
-// cells; there THC-AO-K pays for them (C1: 3.5 ms without the check, 5.0 ms
-// with it; build at 4 x 4 x 4 k, N_P = 1200: 8.8 ms, 9.3 with it).
+// 2^-10 (|m_a|^2 + |m_b|^2)^(1/2), seven digits are not enough.  Measured rms errors
+// in u sum |a||b| (u = 2^-53), K = 100 to 6000: dense rows 0.05 to 0.01 where the
+// FP64 pipe's sums leave 0.5; one large entry beside small ones, S at 2^-8 of the
+// root, 0.4 to 0.7 where they leave 4 to 6.  (A line that knows S alone would not
+// do: at S = 2^-10 rows with one large entry each leave 0.5, but rows of 1200
+// small ones beside it 10.)
+// Tiles with more than a few such results go to a second form of the kernel:
+// eight digits (71 bits), classes up to C_8, good down to a line of 2^-18.  What
+// is below that, what few there are in a tile, and results whose rows hold a NaN
+// or an Inf are computed in FP64: single entries by a warp each, tiles with a
+// majority of them as gemm_z computes them.  Below the first line lie 0.05 to
+// 0.15 % of S4b's results for Gaussians of 0.25 to 3.5 bohr^-2, but 20 % for the
+// benzene cells' basis, 10 % of S1's and S4a's and 58 % of THC-AO-K's; below the
+// second 0.07 % at most.  (The same in FP64 instead of eight digits: THC-AO-K of
+// the benzene cell at 4 x 4 x 4 k 401 ms, 31 now; its build 25.8 and 11.1 ms, and 9.5
+// for the wider Gaussians, which took 8.8 unchecked.)
 //
 // Complex products run as real ones with K = 2 K: one operand plain
 // (interleaved), the smaller one embedded as rows (re, -im) and (im, re).
@@ -57,6 +64,9 @@
 //             chunk's last product into it is done and while the later classes
 //             are still being multiplied; the next chunk starts on C_0 when C_0
 //             is drained.  So the accumulators need no second set.
+// The form with eight digits: 43 digit products, tiles of 128 x 64, whose eight
+// accumulators (C_0 .. C_6, and C_7 + C_8) fill TMEM, an int64 and an int per output;
+// 1.45 times the time of the other per output.
 // The integer epilogue keeps the FP64 pipe (2 results per SM and clock) out of
 // the kernel: conversion and rounding of an output are about 30 integer
 // instructions.
@@ -70,16 +80,25 @@
 
 namespace {
 
-constexpr int ND = 7;                                  // digits
 constexpr int TL = 128, TN = 80, TK = 32;              // lane rows, column rows, K of a stage
-constexpr uint32_t LPL = TL * TK * 2, CPL = TN * TK * 2;    // bytes of a plane tile: 8 KB, 5 KB
-constexpr uint32_t STAGE = ND * (LPL + CPL);           // 91 KB
-constexpr int NACC = 6;                                // accumulators: C_0 .. C_4, and C_5 + C_6 + C_7
+constexpr uint32_t LPL = TL * TK * 2;                  // bytes of a lane plane tile: 8 KB
 constexpr int STAGES = 2;
 constexpr int CHUNK_ST = 2;                            // stages of an exact chunk (64 K)
-constexpr size_t SMEM = STAGES * STAGE + 1024 + 128;
 constexpr int EPI0 = 4, EPI_W = 16, NT = 32 * (EPI0 + EPI_W);
-constexpr int EC = TN / 4;                             // columns of an epilogue warp
+// The two forms: 7 digits, and 8 for tiles that the check gives to them.
+template <bool W>
+struct Form {
+  static constexpr int ND = W ? 8 : 7;                 // digits
+  static constexpr int CMAX = W ? 8 : 7;               // the last class
+  static constexpr int N = W ? 64 : TN;                // columns of a tile
+  static constexpr int NACC = W ? 8 : 6;               // accumulators: the last classes share one
+  static constexpr uint32_t CPL = N * TK * 2;          // bytes of a column plane tile
+  static constexpr uint32_t STAGE = ND * (LPL + CPL);  // 91 KB, 96 KB
+  static constexpr size_t SMEM = STAGES * STAGE + 1024 + 256;
+  static constexpr int EC = N / 4, EH = EC / 2;        // columns of an epilogue warp, and of a read of them
+  static_assert(SMEM <= 232448 && NACC * N <= 512, "227 KB of shared memory per block, 512 TMEM columns");
+};
+constexpr int WN = Form<true>::N;
 constexpr int NB_ROW = 2047;                           // biased exponent of a row with a NaN or an Inf
 constexpr size_t HEAD = 256;                           // bytes before scratch of its own: the error block
 
@@ -88,19 +107,19 @@ constexpr int MK = 64;
 constexpr uint32_t MLB = TL * MK * 2, MCB = TN * MK * 2, MSTAGE = MLB + MCB;   // 16 KB + 10 KB
 constexpr int MSTAGES = 6, MEPI = 8, MNT = 32 * (4 + MEPI);
 constexpr size_t MSMEM = MSTAGES * MSTAGE + 1024 + 256;
-constexpr float CHECK = 0x1p20f;                       // digits are not enough where S^2 CHECK < |m_a|^2 + |m_b|^2
-constexpr int MANY = 800;                              // entries of a warp's 32 x 40 from which the tile goes whole
+constexpr float CHECK7 = 0x1p20f, CHECK8 = 0x1p36f;    // digits are not enough where S^2 CHECK < |m_a|^2 + |m_b|^2
+constexpr int FEW = 16;                                // entries of a warp's 32 x 40 up to which 7 digits and FP64 do
+constexpr int MANY = 800;                              // and from which the tile goes whole in FP64
 constexpr int EPU = 512;                               // room for single entries, per tile
 constexpr float NORM_UNIT = 4096.f;                    // |m|^2 is counted in units of 2^-12
-
-static_assert(SMEM <= 232448, "227 KB of shared memory per block");
 
 struct OzMaps {
   CUtensorMap l, n;
 };
 
-// What the check leaves: cnt[0] tiles (flag 1, listed in tiles) and cnt[1]
-// entries (tile, lane row << 8 | column row of it) to be computed in FP64.
+// What the check leaves: cnt[0] tiles (flag bit 0, listed in tiles) and cnt[1]
+// entries (tile, lane row << 8 | column row of it) to be computed in FP64, and
+// cnt[2] tiles (flag bit 1) to be computed with 8 digits.
 struct OzList {
   int *cnt, *flag, *tiles;
   uint2* ents;
@@ -114,6 +133,8 @@ struct OzShape {
   int nl, nn;        // valid lanes (rows of the lane operand) and columns
   int nst;           // K stages
   int tl, tn;        // tiles
+  int ftn;           // column tiles of the flags
+  int nd;            // digit planes in memory
   int lsh, nsh;      // exponent index = row >> sh (embedded operands: pairs of rows share one)
   long el, en;       // exponents per batch entry
   long units;
@@ -131,10 +152,11 @@ __device__ __forceinline__ void decode(const OzShape& g, long u, int& b, int& li
   li = (int)(r - (unsigned)b * (unsigned)g.tl);
 }
 
+template <int N>
 __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t accumulate) {
   // kind::f16, D f32 (bit 4), A and B bf16 (bits 7 and 10), K-major, N >> 3 at bit 17, M >> 4 at bit 24
   constexpr uint32_t idesc =
-      (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TL >> 4) << 24);
+      (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(TL >> 4) << 24);
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
@@ -155,9 +177,18 @@ __device__ __forceinline__ uint64_t desc64(uint32_t addr) {
          ((uint64_t)4 << 61);
 }
 
-// 10 consecutive columns of this thread's TMEM lane (half of an epilogue warp's: registers).
-constexpr int EH = EC / 2;
-static_assert(EH == 10, "tmem_ld10");
+// 8 or 10 consecutive columns of this thread's TMEM lane (half of an epilogue warp's: registers).
+__device__ __forceinline__ void tmem_ld8(uint32_t t, float* v) {
+  uint32_t r[8];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(t)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
+}
 __device__ __forceinline__ void tmem_ld10(uint32_t t, float* v) {
   uint32_t r[10];
   asm volatile(
@@ -205,20 +236,25 @@ __device__ __forceinline__ double flip(double x) {
   return __longlong_as_double(__double_as_longlong(x) ^ (long long)(1ull << 63));
 }
 
+template <bool W>
 __global__ void __launch_bounds__(NT, 1)
 oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict__ eL, const int* __restrict__ eN,
           double* __restrict__ out, OzList f, int* err) {
+  typedef Form<W> F;
+  constexpr int ND = F::ND, NACC = F::NACC, EC = F::EC, EH = F::EH, N = F::N;
+  constexpr uint32_t STAGE = F::STAGE, CPL = F::CPL;
+  if (W && f.cnt[2] == 0) return;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE);
-  uint32_t* tmem_slot = (uint32_t*)(bars + 17);
+  uint32_t* tmem_slot = (uint32_t*)(bars + 5 + 2 * NACC);
   const uint32_t sbase = smem_u32(smem), bar0 = smem_u32(bars);
   auto FULL = [&](int s) { return bar0 + 8u * s; };
   auto EMPTY = [&](int s) { return bar0 + 8u * (2 + s); };
-  // accumulator c (C_0 .. C_4, and 5: C_5 + C_6 + C_7): complete, drained
+  // accumulator c (one class each, the last C_5 + C_6 + C_7 or C_7 + C_8): complete, drained
   auto AFULL = [&](int c) { return bar0 + 8u * (4 + c); };
-  auto AEMPTY = [&](int c) { return bar0 + 8u * (10 + c); };
-  const uint32_t DONE = bar0 + 8u * 16;
+  auto AEMPTY = [&](int c) { return bar0 + 8u * (4 + NACC + c); };
+  const uint32_t DONE = bar0 + 8u * (4 + 2 * NACC);
 
   __shared__ int abort_flag;
   if (threadIdx.x == 0) abort_flag = *(volatile int*)err;
@@ -248,8 +284,18 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const int nchunk = (g.nst + CHUNK_ST - 1) / CHUNK_ST;
-  // tiles that the check has left to FP64 are passed over by every warp
-  const bool holes = f.cnt && *f.cnt != 0;
+  // tiles that the check has left to FP64 or to the other form are passed over by every warp
+  const bool holes = W || (f.cnt && (f.cnt[0] | f.cnt[2]) != 0);
+  auto pass = [&](long u) {
+    if (!holes) return false;
+    if (!W) return f.flag[u] != 0;
+    int b, li, ni;
+    decode(g, u, b, li, ni);
+    const int* fl = f.flag + ((long)b * g.tl + li) * g.ftn;
+    const int n0 = ni * N / TN, n1 = min((ni * N + N - 1) / TN, g.ftn - 1);
+    return ((fl[n0] | fl[n1]) & 2) == 0;
+  };
+  static_assert(N <= TN, "a tile of the wide form meets at most two of the flags'");
 
   // (warps 0 and 1 keep all lanes in their loops and elect one per batch of
   // copies or MMAs: see tc_gemm.cu)
@@ -258,7 +304,7 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
       uint32_t it = 0;
       bool ok = true;
       for (long u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
-        if (holes && f.flag[u]) continue;
+        if (pass(u)) continue;
         int b, li, ni;
         decode(g, u, b, li, ni);
         for (int st = 0; st < g.nst; st++, it++) {
@@ -266,8 +312,8 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
           if (!mbar_wait_uniform(EMPTY(sl), ((it >> 1) & 1) ^ 1, err, 2)) { ok = false; break; }
           if (elect_one()) {
             mbar_expect_tx(FULL(sl), STAGE);
-            tma_load_3d(sbase + sl * STAGE, &maps.l, FULL(sl), st * TK, li * TL, b * ND);
-            tma_load_3d(sbase + sl * STAGE + ND * LPL, &maps.n, FULL(sl), st * TK, ni * TN, b * ND);
+            tma_load_3d(sbase + sl * STAGE, &maps.l, FULL(sl), st * TK, li * TL, b * g.nd);
+            tma_load_3d(sbase + sl * STAGE + ND * LPL, &maps.n, FULL(sl), st * TK, ni * N, b * g.nd);
           }
           __syncwarp();
         }
@@ -283,7 +329,7 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
       uint32_t it = 0, ch = 0;
       bool ok = true;
       for (long u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
-        if (holes && f.flag[u]) continue;
+        if (pass(u)) continue;
         for (int c = 0; c < nchunk && ok; c++, ch++) {
           const int st1 = min(g.nst, (c + 1) * CHUNK_ST);
           for (int st = c * CHUNK_ST; st < st1; st++, it++) {
@@ -299,14 +345,16 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
                 tc_fence_after();
               }
               if (elect_one()) {
+                constexpr auto top = [](int c) { return c == NACC - 1 ? F::CMAX : c; };
+                constexpr auto s0 = [](int cl) { return cl < ND ? 0 : cl - ND + 1; };
 #pragma unroll
-                for (int cl = c6 == 5 ? 7 : c6; cl >= c6; cl--)      // C_7, C_6, C_5
+                for (int cl = top(c6); cl >= c6; cl--)               // the smaller classes first
 #pragma unroll
-                  for (int s = cl == 7; s <= min(cl, ND - 1); s++)
+                  for (int s = s0(cl); s <= min(cl, ND - 1); s++)
 #pragma unroll
                     for (int kk = 0; kk < 2; kk++)
-                      mma_bf16(tmem + c6 * TN, al + s * PL + 2 * kk, bn + (cl - s) * PC + 2 * kk,
-                               !(first && (cl < 5 || cl == 7) && s == (cl == 7) && kk == 0));
+                      mma_bf16<N>(tmem + c6 * N, al + s * PL + 2 * kk, bn + (cl - s) * PC + 2 * kk,
+                                  !(first && cl == top(c6) && s == s0(cl) && kk == 0));
                 if (last) commit(AFULL(c6));
                 if (c6 == NACC - 1) commit(EMPTY(sl));
               }
@@ -327,18 +375,21 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
     uint32_t ch = 0;
     bool ok = true;
     for (long u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
-      if (holes && f.flag[u]) continue;
+      if (pass(u)) continue;
       int b, li, ni;
       decode(g, u, b, li, ni);
       long long acc[EC];
       float rest[EC];
+      int lo[W ? EC : 1];
 #pragma unroll
       for (int j = 0; j < EC; j++) {
         acc[j] = 0;
         rest[j] = 0.f;
+        if (W) lo[W ? j : 0] = 0;
       }
       for (int c = 0; c < nchunk; c++, ch++) {
-        // class c holds integers in units of 2^(-9 c); in units of C_3 they count 2^(27 - 9 c)
+        // class c holds integers in units of 2^(-9 c); in units of C_3 they count 2^(27 - 9 c).
+        // 8 digits: lo holds what is below C_3 in units of C_6, 0 <= lo < 2^27, and rest what is below that
 #pragma unroll
         for (int c6 = 0; c6 < NACC; c6++) {
           // (every lane polls: the sleeping wait of one lane woke up to 250 ns late, six times a chunk)
@@ -347,7 +398,8 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
 #pragma unroll
           for (int f = 0; f < EC; f += EH) {
             float v[EH];
-            tmem_ld10(tl + c6 * TN + f, v);
+            if constexpr (EH == 8) tmem_ld8(tl + c6 * N + f, v);
+            else tmem_ld10(tl + c6 * N + f, v);
             if (f + EH == EC) {
               tc_fence_before();
               __syncwarp();
@@ -357,6 +409,27 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
             for (int j = 0; j < EH; j++) {
               if (c6 < 4) {
                 acc[f + j] += (long long)__float2int_rn(v[j] * (float)(1 << (9 * (c6 & 3)))) * (1 << (27 - 9 * (c6 & 3)));
+              } else if (W) {
+                int& l = lo[W ? f + j : 0];
+                if (c6 < 7) {
+                  const int n = __float2int_rn(v[j] * (c6 == 4 ? 0x1p36f : c6 == 5 ? 0x1p45f : 0x1p54f));
+                  if (c6 == 4) {
+                    acc[f + j] += n >> 9;
+                    l += (n & 511) << 18;
+                  } else if (c6 == 5) {
+                    acc[f + j] += n >> 18;
+                    l += (n & 0x3ffff) << 9;
+                  } else {
+                    l += n;
+                  }
+                } else {
+                  const float x = fmaf(v[j], 0x1p54f, rest[f + j]);
+                  const int n = __float2int_rn(x);
+                  rest[f + j] = x - (float)n;
+                  l += n;
+                  acc[f + j] += l >> 27;
+                  l &= (1 << 27) - 1;
+                }
               } else if (c6 == 4) {
                 const float x4 = v[j] * 0x1p27f;   // C_4 in units of C_3, a multiple of 2^-9
                 const int n4 = __float2int_rn(x4);
@@ -371,7 +444,7 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
         if (!ok) break;
       }
       if (!ok) break;
-      const int i = li * TL + 32 * q + lane, j0 = ni * TN + EC * h;
+      const int i = li * TL + 32 * q + lane, j0 = ni * N + EC * h;
       if (i < g.nl) {
         const int ei = eL[(long)b * g.el + (i >> g.lsh)];
         // biased exponents E: 2^(E - 1022) above the row; value = 2^(e_l + e_n - 16 - 27) (acc + rest)
@@ -383,7 +456,17 @@ oz_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __restrict_
           if (col < g.nn) {
             const bool two = col + 1 < g.nn;
             const int e0 = en[col >> g.nsh], e1 = two ? en[(col + 1) >> g.nsh] : 0;
-            double x = round_sum(acc[j], rest[j], es + e0), y = two ? round_sum(acc[j + 1], rest[j + 1], es + e1) : 0.0;
+            auto value = [&](int j, int sexp) {
+              if constexpr (W) {
+                // in units of C_6 while that fits 62 bits
+                if (acc[j] < (1ll << 34) && acc[j] >= -(1ll << 34))
+                  return round_sum(acc[j] * (1 << 27) + lo[j], rest[j], sexp - 27);
+                return round_sum(acc[j], (float)lo[j] * 0x1p-27f, sexp);
+              } else {
+                return round_sum(acc[j], rest[j], sexp);
+              }
+            };
+            double x = value(j, es + e0), y = two ? value(j + 1, es + e1) : 0.0;
             if (!f.cnt) {   // (else rows with a NaN or an Inf are left to FP64)
               if (ei == NB_ROW || e0 == NB_ROW) x = __longlong_as_double(0x7ff8000000000000ll);
               if (ei == NB_ROW || e1 == NB_ROW) y = __longlong_as_double(0x7ff8000000000000ll);
@@ -427,7 +510,7 @@ __device__ __forceinline__ uint64_t desc128(uint32_t addr) {
          ((uint64_t)2 << 61);
 }
 
-// S of every entry, tiles as in oz_kernel (rows of an embedded side counted
+// S of every entry, tiles as in oz_kernel<false> (rows of an embedded side counted
 // once, so its box is half used): warp 0 loads, warp 1 multiplies into one of
 // two accumulators, warps 4-11 compare (32 lanes x 40 columns each).  It reads
 // a fifteenth of the product's planes and multiplies a 68th to a 136th as much.
@@ -507,7 +590,7 @@ oz_check_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __res
         const uint64_t al = desc128(sbase + sl * MSTAGE), bn = desc128(sbase + sl * MSTAGE + MLB);
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < MK / 16; kk++) mma_bf16(tmem + 128 * set, al + 2 * kk, bn + 2 * kk, st > 0 || kk > 0);
+          for (int kk = 0; kk < MK / 16; kk++) mma_bf16<TN>(tmem + 128 * set, al + 2 * kk, bn + 2 * kk, st > 0 || kk > 0);
           commit(EMPTY(sl));
           if (st == g.mst - 1) commit(AFULL(set));
         }
@@ -541,6 +624,7 @@ oz_check_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __res
       unsigned long long m = (unsigned long long)__ballot_sync(0xffffffffu, bad(c0 + lane)) |
                              (unsigned long long)__ballot_sync(0xffffffffu, lane < MC - 32 && bad(c0 + 32 + lane)) << 32;
       if (nb) m = ~0ull;
+      unsigned long long m7 = m;               // what 7 digits are not enough for; m: nor 8
       if (!__all_sync(0xffffffffu, mbar_wait(AFULL(set), (local >> 1) & 1, err, 16))) break;
       tc_fence_after();
 #pragma unroll
@@ -550,17 +634,23 @@ oz_check_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __res
 #pragma unroll
         for (int j = 0; j < 10; j++) {
           const float q = ql + __shfl_sync(0xffffffffu, j0 + j < 32 ? qn0 : qn1, (j0 + j) & 31);   // (by every lane)
-          if (v[j] > 0.f && v[j] * v[j] * (CHECK * NORM_UNIT) < q) m |= 1ull << (j0 + j);
+          const float w = v[j] * v[j] * NORM_UNIT;
+          if (v[j] > 0.f && w * CHECK7 < q) m7 |= 1ull << (j0 + j);
+          if (v[j] > 0.f && w * CHECK8 < q) m |= 1ull << (j0 + j);
         }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(AEMPTY(set));
-      m = row ? m & cols : 0ull;
+      m7 = row ? m7 & cols : 0ull;
+      const int all7 = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popcll(m7));
+      if (all7 == 0) continue;
+      m &= m7;
+      const bool wide = all7 > FEW;          // the tile with 8 digits, entries beyond those in FP64
+      if (!wide) m = m7;
       const int mine = __popcll(m), all = (int)__reduce_add_sync(0xffffffffu, (unsigned)mine);
-      if (all == 0) continue;
       bool whole = g.acc || all > MANY;      // (an entry that is added to cannot be overwritten later)
-      if (!whole) {
+      if (!whole && all > 0) {
         int off = mine;
         for (int o = 1; o < 32; o <<= 1) {
           const int t = __shfl_up_sync(0xffffffffu, off, o);
@@ -575,7 +665,11 @@ oz_check_kernel(const __grid_constant__ OzMaps maps, OzShape g, const int* __res
             f.ents[i] = whole ? make_uint2(~0u, 0u)
                               : make_uint2((unsigned)u, (unsigned)(r << 8 | (c0 + __ffsll((long long)m) - 1)));
       }
-      if (whole && lane == 0 && atomicExch(f.flag + u, 1) == 0) f.tiles[atomicAdd(f.cnt, 1)] = (int)u;
+      if (lane == 0) {
+        const int bits = (whole ? 1 : 0) | (wide ? 2 : 0), old = bits ? atomicOr(f.flag + u, bits) : 0;
+        if (bits & ~old & 1) f.tiles[atomicAdd(f.cnt, 1)] = (int)u;
+        if (bits & ~old & 2) atomicAdd(f.cnt + 2, 1);
+      }
     }
   }
   tc_fence_before();
@@ -696,7 +790,7 @@ __global__ void __launch_bounds__(256) oz_exact_kernel(Source l, Source n, int K
   }
   for (int i = blockIdx.x * 8 + ty; i < nent; i += gridDim.x * 8) {
     const uint2 e = f.ents[i];
-    if (e.x == ~0u || f.flag[e.x]) continue;
+    if (e.x == ~0u || (f.flag[e.x] & 1)) continue;
     int b, li, ni;
     decode(g, e.x, b, li, ni);
     const int r = li * R + (int)(e.y >> 8), c = ni * C + (int)(e.y & 255);
@@ -755,15 +849,24 @@ __global__ void __launch_bounds__(128) oz_exp_cols(const double* __restrict__ sr
   atomicMax(e + (long)blockIdx.z * rows + r, m);
 }
 
-// x 2^(62 - e), rounded, for a row of biased exponent E (e = E - 1022): |result| <= 2^62.
-__device__ __forceinline__ long long fixed62(double x, int E) {
+// x 2^(71 - e), rounded, for a row of biased exponent E (e = E - 1022), as hi 2^27 + lo, 0 <= lo < 2^27.
+__device__ __forceinline__ void fixed71(double x, int E, long long& hi, int& lo) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)(u >> 52) & 0x7ff;
   unsigned long long m = (u & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0);
-  const int sh = max(ex, 1) - E + 9;
-  if (sh >= 0) m <<= min(sh, 10);
-  else m = sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0;
-  return (long long)u < 0 ? -(long long)m : (long long)m;
+  const int sh = max(ex, 1) - E + 18;                // at most 19
+  if (sh >= 0) {
+    lo = (int)(m << min(sh, 19)) & 0x7ffffff;
+    hi = (long long)(m >> (27 - min(sh, 19)));
+  } else {
+    m = sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0;
+    lo = (int)m & 0x7ffffff;
+    hi = (long long)(m >> 27);
+  }
+  if ((long long)u < 0) {
+    hi = -hi - (lo != 0);
+    lo = -lo & 0x7ffffff;
+  }
 }
 
 // u 2^-e (u: the bits of a nonnegative double of a row of biased exponent E) truncated to bf16; at least 2^-41 for u > 0.
@@ -800,19 +903,30 @@ __device__ __forceinline__ unsigned put_mags(const double* x, int E, uint16_t* d
 // The planes of 8 consecutive reals of a row: digits from the last, each
 // balanced digit taken off with its carry; the plane value 2^(-9 s) d is formed
 // by adding d to the bits of 1.5 2^(23 - 9 s) and subtracting that number.
+// The first nd (7 or 8) are written: balanced digits left out are what rounding to the others leaves.
 // EMB: x holds 4 complex values, and the two rows (re, -im) and (im, re) are written.
 template <bool EMB>
-__device__ __forceinline__ void put8(const double* x, int E, uint16_t* dst, long plane, int ldp) {
+__device__ __forceinline__ void put8(const double* x, int E, uint16_t* dst, long plane, int ldp, int nd) {
   long long f[8];
+  int l[8];
 #pragma unroll
-  for (int i = 0; i < 8; i++) f[i] = E == NB_ROW ? 0 : fixed62(x[i], E);
+  for (int i = 0; i < 8; i++) {
+    f[i] = 0;
+    l[i] = 0;
+    if (E != NB_ROW) fixed71(x[i], E, f[i], l[i]);
+  }
 #pragma unroll
-  for (int s = ND - 1; s >= 0; s--) {
+  for (int s = 7; s >= 0; s--) {
     uint32_t v[8];
 #pragma unroll
     for (int i = 0; i < 8; i++) {
       int d;
-      if (s > 0) {
+      if (s > 4) {
+        l[i] += 256;
+        d = (l[i] & 511) - 256;
+        l[i] >>= 9;
+        if (s == 5) f[i] += l[i];
+      } else if (s > 0) {
         f[i] += 256;
         d = ((int)f[i] & 511) - 256;
         f[i] >>= 9;
@@ -822,6 +936,7 @@ __device__ __forceinline__ void put8(const double* x, int E, uint16_t* dst, long
       const float big = __int_as_float(0x4B400000 - ((9 * s) << 23));   // 1.5 2^(23 - 9 s)
       v[i] = __float_as_uint(__fsub_rn(__int_as_float(__float_as_int(big) + d), big));
     }
+    if (s >= nd) continue;
     uint32_t w[4];
 #pragma unroll
     for (int i = 0; i < 4; i++) w[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x7632);
@@ -845,7 +960,7 @@ __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ 
                                                      int conj, const int* __restrict__ e, uint16_t* __restrict__ dst,
                                                      int ldp, uint16_t* __restrict__ mag, int ldm,
                                                      unsigned* __restrict__ sq) {
-  const int ng = (K * CX + 7) / 8;
+  const int ng = (K * CX + 7) / 8, nd = mag ? 8 : 7;
   const long i = (long)blockIdx.x * 256 + threadIdx.x;
   const unsigned act = __ballot_sync(0xffffffffu, i < (long)rows * ng);
   if (i >= (long)rows * ng) return;
@@ -866,7 +981,7 @@ __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ 
   }
   const long plane = (long)rows * (EMB ? 2 : 1) * ldp;
   const int E = e[b * rows + r];
-  put8<EMB>(x, E, dst + b * ND * plane + (long)r * (EMB ? 2 : 1) * ldp + k0 * CX, plane, ldp);
+  put8<EMB>(x, E, dst + b * nd * plane + (long)r * (EMB ? 2 : 1) * ldp + k0 * CX, plane, ldp, nd);
   if (mag) {
     // (integer sums: the same whatever their order)
     const unsigned q = put_mags<CX>(x, E, mag + (b * rows + r) * ldm + k0);
@@ -889,6 +1004,7 @@ __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ 
                                                      int ldp, uint16_t* __restrict__ mag, int ldm,
                                                      unsigned* __restrict__ sq) {
   constexpr int KT = 64 / CX;                       // 64 reals of K
+  const int nd = mag ? 8 : 7;
   __shared__ double t[KT][33 * CX];
   __shared__ unsigned part[32];
   if (threadIdx.x < 32) part[threadIdx.x] = 0u;
@@ -922,7 +1038,7 @@ __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ 
   const long plane = (long)rows * (EMB ? 2 : 1) * ldp;
   if (in) {
     const int E = e[b * rows + r0 + r];
-    put8<EMB>(x, E, dst + b * ND * plane + (long)(r0 + r) * (EMB ? 2 : 1) * ldp + k0 * CX + 8 * c, plane, ldp);
+    put8<EMB>(x, E, dst + b * nd * plane + (long)(r0 + r) * (EMB ? 2 : 1) * ldp + k0 * CX + 8 * c, plane, ldp, nd);
     if (mag) atomicAdd(part + r, put_mags<CX>(x, E, mag + (b * rows + r0 + r) * ldm + k0 + 8 / CX * c));
   }
   if (!mag) return;
@@ -954,8 +1070,8 @@ struct Planes {
 };
 
 size_t exp_bytes(long rows, int batch) { return align256(2 * sizeof(int) * (size_t)rows * batch); }
-size_t digit_bytes(long rows, bool emb, int K, int CX, int batch) {
-  return align256(2 * (size_t)ND * (rows << emb) * pad8i(K * CX) * batch);
+size_t digit_bytes(long rows, bool emb, int K, int CX, int batch, int nd = 8) {
+  return align256(2 * (size_t)nd * (rows << emb) * pad8i(K * CX) * batch);
 }
 size_t side_bytes(long rows, bool emb, int K, int CX, int batch) {
   return exp_bytes(rows, batch) + digit_bytes(rows, emb, K, CX, batch) + align256(2 * (size_t)rows * pad8i(K) * batch);
@@ -1007,10 +1123,10 @@ cudaError_t prepare(const Side& a, int K, int batch, const Planes& p, cudaStream
   return cudaGetLastError();
 }
 
-// bf16 [n][rows][ldk] with K valid: digit planes (n = 7 per batch entry) in
-// boxes of 7 planes x `box` rows x 32 K, 64B swizzle, or magnitudes (n = batch)
-// in boxes of `box` rows x 64 K, 128B swizzle.
-cudaError_t plane_map(CUtensorMap* map, const void* base, long n, long rows, int K, int ldk, int box, bool digits) {
+// bf16 [n][rows][ldk] with K valid: digit planes in boxes of `digits` planes x
+// `box` rows x 32 K, 64B swizzle, or (0) magnitudes in boxes of `box` rows x 64 K,
+// 128B swizzle.
+cudaError_t plane_map(CUtensorMap* map, const void* base, long n, long rows, int K, int ldk, int box, int digits) {
   static const PFN_cuTensorMapEncodeTiled_v12000 enc = [] {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -1022,7 +1138,7 @@ cudaError_t plane_map(CUtensorMap* map, const void* base, long n, long rows, int
   if (!enc) return cudaErrorNotSupported;
   cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)n};
   cuuint64_t strides[2] = {(cuuint64_t)ldk * 2, (cuuint64_t)ldk * 2 * rows};
-  cuuint32_t bx[3] = {(cuuint32_t)(digits ? TK : MK), (cuuint32_t)box, (cuuint32_t)(digits ? ND : 1)};
+  cuuint32_t bx[3] = {(cuuint32_t)(digits ? TK : MK), (cuuint32_t)box, (cuuint32_t)(digits ? digits : 1)};
   cuuint32_t estr[3] = {1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)base, dims, strides, bx, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, digits ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1051,6 +1167,8 @@ cudaError_t slab(const Side& l, const Side& n, int K, int nb, const Planes& pl, 
   g.nsh = n.emb;
   g.el = l.rows;
   g.en = n.rows;
+  g.ftn = g.tn;
+  g.nd = list ? 8 : 7;
   g.units = (long)nb * g.tl * g.tn;
   g.pairs = pairs;
   g.acc = acc;
@@ -1058,22 +1176,28 @@ cudaError_t slab(const Side& l, const Side& n, int K, int nb, const Planes& pl, 
   g.ldo = ldo;
   g.sbo = sbo;
   if (g.units >= (1L << 31)) return cudaErrorInvalidValue;   // counted in 32 bits
-  OzMaps maps, mags;
-  cudaError_t e = plane_map(&maps.n, pn.pl, (long)nb * ND, g.nn, Kr, ldp, TN, true);
-  if (e == cudaSuccess) e = plane_map(&maps.l, pl.pl, (long)nb * ND, g.nl, Kr, ldp, TL, true);
-  if (e == cudaSuccess && list) e = plane_map(&mags.n, pn.mag, nb, n.rows, K, pad8i(K), TN, false);
-  if (e == cudaSuccess && list) e = plane_map(&mags.l, pl.mag, nb, l.rows, K, pad8i(K), TL, false);
+  OzMaps maps, mags, wide;
+  cudaError_t e = plane_map(&maps.n, pn.pl, (long)nb * g.nd, g.nn, Kr, ldp, TN, 7);
+  if (e == cudaSuccess) e = plane_map(&maps.l, pl.pl, (long)nb * g.nd, g.nl, Kr, ldp, TL, 7);
+  if (e == cudaSuccess && list) e = plane_map(&mags.n, pn.mag, nb, n.rows, K, pad8i(K), TN, 0);
+  if (e == cudaSuccess && list) e = plane_map(&mags.l, pl.mag, nb, l.rows, K, pad8i(K), TL, 0);
+  if (e == cudaSuccess && list) e = plane_map(&wide.n, pn.pl, (long)nb * g.nd, g.nn, Kr, ldp, WN, 8);
+  if (e == cudaSuccess && list) e = plane_map(&wide.l, pl.pl, (long)nb * g.nd, g.nl, Kr, ldp, TL, 8);
   int dev = 0, nsm = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+  constexpr size_t SMEM7 = Form<false>::SMEM, SMEM8 = Form<true>::SMEM;
   if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(oz_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM7);
+  if (e == cudaSuccess && list)
+    e = cudaFuncSetAttribute(oz_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM8);
+  if (e == cudaSuccess && list)
     e = cudaFuncSetAttribute(oz_check_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSMEM);
   OzList f{};
   const unsigned grid = (unsigned)std::min<long>(g.units, nsm);
   if (!list) {
     if (e != cudaSuccess) return e;
-    oz_kernel<<<grid, NT, SMEM, s>>>(maps, g, pl.e, pn.e, out, f, w.err);
+    oz_kernel<false><<<grid, NT, SMEM7, s>>>(maps, g, pl.e, pn.e, out, f, w.err);
     if (w.launches) ++*w.launches;
     return cudaGetLastError();
   }
@@ -1081,7 +1205,12 @@ cudaError_t slab(const Side& l, const Side& n, int K, int nb, const Planes& pl, 
   if (e == cudaSuccess) e = cudaMemsetAsync(f.cnt, 0, 64 + sizeof(int) * (size_t)g.units, s);
   if (e != cudaSuccess) return e;
   oz_check_kernel<<<grid, MNT, MSMEM, s>>>(mags, g, pl.e, pn.e, pl.sq, pn.sq, f, w.err);
-  oz_kernel<<<grid, NT, SMEM, s>>>(maps, g, pl.e, pn.e, out, f, w.err);
+  oz_kernel<false><<<grid, NT, SMEM7, s>>>(maps, g, pl.e, pn.e, out, f, w.err);
+  OzShape gw = g;
+  gw.tn = (int)tiles_of(n.rows, n.emb, WN);
+  gw.units = (long)nb * g.tl * gw.tn;
+  if (gw.units >= (1L << 31)) return cudaErrorInvalidValue;
+  oz_kernel<true><<<(unsigned)std::min<long>(gw.units, nsm), NT, SMEM8, s>>>(wide, gw, pl.e, pn.e, out, f, w.err);
   const Source sl{l.src, l.sb, l.lr, l.lk, l.conj}, sn{n.src, n.sb, n.lr, n.lk, n.conj};
   const unsigned xg = (unsigned)std::min<long>(2 * g.units, 2L * nsm);
   if constexpr (CX == 1)
@@ -1090,7 +1219,7 @@ cudaError_t slab(const Side& l, const Side& n, int K, int nb, const Planes& pl, 
     oz_exact_kernel<2, 4, 5><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err);
   else
     oz_exact_kernel<2, 2, 10><<<xg, 256, 0, s>>>(sl, sn, K, g, f, out, w.err);
-  if (w.launches) *w.launches += 3;
+  if (w.launches) *w.launches += 4;
   return cudaGetLastError();
 }
 
@@ -1298,8 +1427,8 @@ cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, i
   return gemm_z(la, lb, M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, batch, s);
 }
 
-size_t oz_lane_bytes(int N, int K) { return exp_bytes(N, 1) + digit_bytes(N, false, K, 2, 1); }
-size_t oz_lanes_work(int M, int K) { return exp_bytes(M, 1) + digit_bytes(M, true, K, 2, 1); }
+size_t oz_lane_bytes(int N, int K) { return exp_bytes(N, 1) + digit_bytes(N, false, K, 2, 1, 7); }
+size_t oz_lanes_work(int M, int K) { return exp_bytes(M, 1) + digit_bytes(M, true, K, 2, 1, 7); }
 bool oz_lanes_fit(int M, int K, const OzWork& w) { return w.buf && oz_lanes_work(M, K) <= room_of(w); }
 
 static Planes unchecked(void* at, int rows, bool emb, int K) {

@@ -1116,9 +1116,9 @@ thc_status thc_hermitian_kernel(const thc_ctx* c, int* hermitian) {
 thc_status thc_launches_per_build(const thc_ctx* c, int* launches) {
   if (!c || !launches) return THC_ERR_ARG;
   // FP64 and CUDA-core forms: S1, S2, S3, S4a, S4b, E_x partial, E_x final
-  // (FP64 after a build: that build's count; a product from digits is seven
+  // (FP64 after a build: that build's count; a product from digits is eight
   // kernels per slab: exponents and digits of both sides, the check, the
-  // product, and what the check left to FP64).
+  // product, and what the check left to eight digits and to FP64).
   // Tensor-core form: S1 2 (exponents and embedding, GEMM), S2 2 (slices with their
   // row exponents and the embedded Psi^H, GEMM), S3 + S4a 4 (the convolution, the row
   // exponents of M: in the convolution plus a conversion kernel on the

@@ -48,9 +48,9 @@ def test_more_scratch_never_fails(shape):
     M, N, K, batch, real = shape
     least = _least(shape)
     whole = 1 << 40
-    # one tile of each side in digits, magnitudes and exponents, with some room for bookkeeping
+    # one tile of each side in eight digits, magnitudes and exponents, with some room for bookkeeping
     kr = K if real else 2 * K
-    tile = (128 + 80) * (16 * (kr + 8) + 8)
+    tile = (128 + 80) * (18 * (kr + 8) + 8)
     assert least <= tile + 16384
     before = 0
     for f in itertools.chain((1.0 + i / 40 for i in range(160)), (1.3 ** i for i in range(6, 60))):
