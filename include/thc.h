@@ -293,8 +293,8 @@ thc_status thc_select_points(const double* U, int nfunc, int ncand, int npts, do
  * points_host: npts distinct grid indices (host).  V_out: device,
  * [N_k][npts][npts] complex128 (q on the mesh index).  xi_out: device,
  * [npts][N_g] doubles, or NULL.  Allocates its own scratch (about
- * 40 npts N_g bytes, and up to 1.25 GB for the digits of its products, less
- * where the device has less) and waits for `stream`.  THC_ERR_ARG for bad sizes,
+ * 40 npts N_g bytes, and for the digits of its products up to 1.25 GB, less where
+ * the device has less, or up to 8 GB where eight times as much is free) and waits for `stream`.  THC_ERR_ARG for bad sizes,
  * repeated or out-of-range points, or points whose metric S is numerically
  * singular (a Cholesky pivot below 1e-12 of its diagonal entry; message in
  * thc_last_error(NULL)). */
@@ -363,8 +363,8 @@ thc_status thc_rebuild_kernel(const double* U, int nfunc, const int* grid_host, 
  * DFT with the solve, and the orbital contractions.  Outputs must not overlap
  * inputs.  Allocates its own scratch, at most about the largest of
  * 48 N_k npts^2, 16 npts (N_k npts + 7 N_g) and 16 N_k n_occ N_g + 32 npts N_g
- * bytes, and up to 1.25 GB for the digits of its products, and waits for `stream`.  THC_ERR_ARG for
- * bad sizes, null or misaligned pointers, repeated or out-of-range points, or
+ * bytes, and for the digits of its products up to 1.25 GB (THC_FP64: or up to 8 GB
+ * where eight times as much is free), and waits for `stream`.  THC_ERR_ARG for bad sizes, null or misaligned pointers, repeated or out-of-range points, or
  * points whose metric S is numerically singular (as thc_fit_kernel);
  * THC_ERR_TIMEOUT if a device wait of the tensor-core contraction gave up. */
 thc_status thc_vo_gradient(const double* U, int nocc, const double* Uv, int nvir, const int* grid_host,

@@ -367,12 +367,17 @@ struct DeviceMemory {
   // Scratch of a fit and of its adjoint: the whole operands of the metric and of
   // the products of depth kdeep (over the grid or its G set, npts x ndeep; 0:
   // none), up to 1.25 GB (larger slabs measured no faster for the metric), at
-  // least what the metric's least slab needs.
-  cudaError_t scratch(int npts, long ng, int nfunc, int ndeep, int kdeep, cudaStream_t s) {
+  // least what the metric's least slab needs.  deep: the deep products are to be
+  // whole where eight times as much is free, up to 8 GB (their slabs hold a few
+  // tiles each and take the time of a whole product one after the other: FP64
+  // contraction at 3 x 3 x 3 k, N_P = 600, 40^3 grid, 2939 ms in 1.25 GB, 280 whole).
+  cudaError_t scratch(int npts, long ng, int nfunc, int ndeep, int kdeep, bool deep, cudaStream_t s) {
     const size_t least = oz_work_min(nfunc);
     size_t want = std::max(oz_work_bytes(npts, (int)ng, nfunc, 1), oz_work_bytes(npts, (int)ng, npts, 1));
     if (ndeep > 0) want = std::max(want, std::max(oz_work_min(kdeep), oz_work_bytes(npts, ndeep, kdeep, 1)));
-    const cudaError_t e = oz_alloc(oz, std::max(least, std::min(want, (size_t)5 << 28)), least, s);
+    size_t most = (size_t)5 << 28, room = 0, total = 0;
+    if (deep && cudaMemGetInfo(&room, &total) == cudaSuccess) most = std::max(most, std::min(room / 8, (size_t)8 << 30));
+    const cudaError_t e = oz_alloc(oz, std::max(least, std::min(want, most)), least, s);
     if (e != cudaErrorMemoryAllocation) return e;
     cudaGetLastError();
     return cudaSuccess;

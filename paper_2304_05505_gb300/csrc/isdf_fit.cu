@@ -180,7 +180,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
     if ((e = dm.get(&R, sizeof(double) * (size_t)npts * ng)) != cudaSuccess) break;
     if ((e = dm.get(&S, sizeof(double) * npq)) != cudaSuccess) break;
     if ((e = dm.get(&L, sizeof(double) * npq)) != cudaSuccess) break;
-    if (dig && (e = dm.scratch(npts, ng, nfunc, npts, nG, s)) != cudaSuccess) break;
+    if (dig && (e = dm.scratch(npts, ng, nfunc, npts, nG, true, s)) != cudaSuccess) break;
     if ((e = dm.get(&bad, sizeof(int))) != cudaSuccess) break;
     if ((e = dm.get(&twd, sizeof(double2) * tw.size())) != cudaSuccess) break;
     if ((e = dm.get(&gmd, sizeof(int) * gm.size())) != cudaSuccess) break;

@@ -497,7 +497,7 @@ extern "C" thc_status thc_vo_gradient(const double* U, int nocc, const double* U
       break;
     if ((e = cudaMemsetAsync(bad, 0, sizeof(int), s)) != cudaSuccess) break;
 
-    if ((e = dm.scratch(np, ng, nf, precision == THC_FP64 ? std::max(nf, nvir) : np, (int)ng, s)) != cudaSuccess) break;
+    if ((e = dm.scratch(np, ng, nf, dig ? std::max(nf, nvir) : np, (int)ng, dig, s)) != cudaSuccess) break;
 
     // 1. the kernel held fixed: Psi, Psi_v at the points, D, W, M, Y, E_x, g_e
     mark(0);
