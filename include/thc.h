@@ -188,9 +188,9 @@ thc_status thc_profile_end(thc_ctx* ctx, float mean_ms[6], int* nbuilds);
  * last completed profile: the GEMM of S1, S2, S4a and S4b (without operand
  * preparation or the combine of split-K partials), the convolution of S3, the
  * reduction of S5 (its final sum when S4a's split-K combine formed the partial
- * sums, else both of its kernels).  In the FP64 and CUDA-core forms each stage is
- * one kernel and this equals the stage time.  THC_ERR_STATE before a profile
- * has completed. */
+ * sums, else both of its kernels).  In the FP64 and CUDA-core forms this equals
+ * the stage time (a stage of the latter is one kernel, a product of the former
+ * one or, from digits, eight).  THC_ERR_STATE before a profile has completed. */
 thc_status thc_profile_kernels(const thc_ctx* ctx, float core_ms[6]);
 
 /* Wait for the context's stream.  Returns THC_ERR_TIMEOUT if a device-side
@@ -269,8 +269,10 @@ thc_status thc_destroy(thc_ctx* ctx);
  * trace(A).  points_host (host, npts ints) receives the candidate indices in
  * selection order, -1 past the end; npoints_host the number chosen.
  * resid_diag (device, ncand doubles, may be NULL) receives the residual
- * diagonal.  Allocates its own scratch (npts * ncand doubles) and waits for
- * `stream`. */
+ * diagonal.  Allocates its own scratch (npts * ncand doubles; for selections that
+ * go in blocks of pivots, nfunc ncand >= 1e6, also 28 bytes per value of U for its
+ * digits, 1 KB per candidate and up to 1 GB for products, without which the pivots
+ * are taken one by one) and waits for `stream`. */
 thc_status thc_select_points(const double* U, int nfunc, int ncand, int npts, double rel_tol,
                              int* points_host, int* npoints_host, double* resid_diag, void* stream);
 

@@ -1,4 +1,4 @@
-// ISDF kernel fit (setup, not part of the timed build), FP64 throughout.
+// ISDF kernel fit (setup, not part of the timed build).
 //
 // Given the occupied orbitals' periodic parts on the grid, U[f][r] = u^k_i(r)
 // with f = (k, i), and the interpolation points r_P:
@@ -16,10 +16,11 @@
 //                   sum_G v(G + q_r) (xh_P(G) e^{-i q_r.r_P}) conj(xh_Q(G) e^{-i q_r.r_Q})
 //      one Hermitian product per representative (v(K) = 4 pi / |K|^2, K = 0
 //      left out).
-// Steps 1-3 and the Cholesky factor run in FP64 (the ill-conditioned
+// Steps 1-3 and the Cholesky factor have FP64 accuracy (the ill-conditioned
 // least-squares metric).  Step 4, the O(N_k N_P^2 N_G) contraction that
-// dominates the per-iteration rebuild of Algorithm 2, runs in FP64 on CUDA
-// cores (THC_FP64) or on the tcgen05 tensor cores (THC_MIXED): each scaled
+// dominates the per-iteration rebuild of Algorithm 2, runs to FP64 accuracy from
+// digits (THC_FP64, as B does; oz_gemm.cu) or in less on the tcgen05 tensor cores
+// (THC_MIXED): each scaled
 // vector set Xq is rounded to FP32 and sliced inside the GEMM, three fp16
 // slices, 8 slice products, the leading products summed exactly in K chunks of
 // at most 1024 reals; chunks are combined in FP64.
@@ -142,7 +143,7 @@ thc_status fit_impl(const double* U, int nfunc, const int* grid_host, const doub
 
   cudaStream_t s = (cudaStream_t)stream;
   // The all-FP64 form takes its products from exact digits on the tensor cores
-  // (metric 397 -> 15 ms at 3x3x3 k, N_P = 600, 40^3 grid).
+  // (metric 397 -> 16 ms at 3x3x3 k, N_P = 600, 40^3 grid).
   // THC_MIXED keeps the FP64 pipe's sums: the solve passes a change of 1e-15 in
   // the metric on as 1e-12 (cond(S) 1e4), which changes FP32 roundings of the
   // contraction's operands, so that V would move by 1e-10 to 1e-7 per element.

@@ -126,9 +126,9 @@ __global__ void embed_kernel(const CT* __restrict__ src, long sbs, long ldk, lon
 }
 
 // The column exponents and the embedded planes of src[b][k][j] (rows lds
-// apart) in one pass: a block holds 8 columns of all K in shared memory (FP32,
-// read 64 bytes of a row at a time), finds each column's maximum on the way
-// and writes the planes along K.  The two kernels it replaces read the columns
+// apart) in one pass: a block holds EJ = 4 columns of all K in shared memory (as
+// FP32, read 64 bytes of a row at a time, 32 from an FP32 source), finds each
+// column's maximum on the way and writes the planes along K.  The two kernels it replaces read the columns
 // one value per 32-byte sector the second time (0.040 ms for Psi at 4 x 4 x 4
 // k, N_P = 1200, n = 60).
 constexpr int EJ = 4;

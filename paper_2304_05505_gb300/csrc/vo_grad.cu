@@ -25,11 +25,12 @@
 //     (B = conj(U_P)^T U, so dE/dconj(U) = conj(T2) plus T1 at the point columns).
 // The fit (B, R, S, its Cholesky factor, xi and xh) is recomputed here from the
 // orbitals with the same kernels as thc_fit_kernel; V is the caller's (the fit
-// of the same orbitals at the same points).  Every contraction is an FP64
-// complex GEMM on CUDA cores, except that with THC_MIXED the O(N_k N_P^2 N_G)
-// one over (q, G), which dominates as the fit's own V contraction does, and
-// the grid contractions T1, T2 and the projection of T2 run on the tcgen05
-// tensor cores in the form of the rebuild's contraction.
+// of the same orbitals at the same points).  Every contraction has FP64
+// accuracy: from digits on the tensor cores where that is the faster form
+// (oz_gemm.cu; not the fit's B with THC_MIXED), else on CUDA cores.  Except that
+// with THC_MIXED the O(N_k N_P^2 N_G) one over (q, G), which dominates as the fit's
+// own V contraction does, and the grid contractions T1, T2 and the projection
+// of T2 run on the tcgen05 tensor cores in the form of the rebuild's contraction.
 #include "isdf_common.cuh"
 #include "tc_gemm.cuh"
 #include "slices.cuh"
