@@ -233,13 +233,13 @@ def stage_work(d: dict, hermitian: bool = False) -> dict:
     }
 
 
-DIGIT_PRODUCTS = 34     # bf16 products of a real product from digits (csrc/oz_gemm.cu)
+DIGIT_PRODUCTS = 34     # bf16 products of a real product from seven digits (csrc/oz_gemm.cu; 43 from eight)
 
 
 def fp64_roofline(d: dict, stages_ms: dict, fp64_tflops: float, pk: dict) -> dict:
     """The FP64 build against its own peaks.  Its four GEMMs (full D in S2) are
     formed from digits on the tensor cores, DIGIT_PRODUCTS bf16 products per real
-    product: issued_tensor_frac is their rate against the sustained bf16 peak;
+    product (more in the tiles that take eight digits): issued_tensor_frac is their rate against the sustained bf16 peak;
     frac is the FP64 rate they come to over the measured FMA rate of the FP64
     pipe, which they pass.  The k-convolution (complex128 D, Vh and M) stands
     against the copy bandwidth."""
@@ -544,10 +544,12 @@ def time_vo_gradient(p, thc, fp64_rate: float) -> dict:
         achieved = flops / (mean[2] * 1e-3) / 1e12
         out[prec] = {"ms": sum(mean), "steps_ms": dict(zip(names, mean)), "ratio_to_rebuild": sum(mean) / sum(reb),
                      "contraction_achieved_tflops": achieved}
+    pk = peaks()
+    issued = DIGIT_PRODUCTS * out["fp64"]["contraction_achieved_tflops"]
     out["fp64"]["contraction_roofline"] = {
-        "bound": "fp64", "achieved": out["fp64"]["contraction_achieved_tflops"], "peak": fp64_rate,
-        "unit": "TFLOP/s", "frac": out["fp64"]["contraction_achieved_tflops"] / fp64_rate if fp64_rate else None,
-        "peak_source": "measured FP64 FMA rate (thc_measure_fp64_rate)"}
+        "bound": "tensor", "achieved": issued, "peak": pk["bf16_tflops_sustained"], "unit": "TFLOP/s of digit products",
+        "frac": issued / pk["bf16_tflops_sustained"], "peak_source": f"{pk['source']} bf16 sustained (cuBLAS)",
+        "of_fp64_fma_rate": out["fp64"]["contraction_achieved_tflops"] / fp64_rate if fp64_rate else None}
     out["mixed"]["form"] = ("(q, G) contraction on tcgen05 (FP32 operands sliced into 3 fp16 slices, 8 products, "
                             "exact K chunks); the other steps FP64")
     out["mixed"]["max_abs_dg_vs_fp64_rel"] = float((grads["mixed"] - grads["fp64"]).abs().max()
