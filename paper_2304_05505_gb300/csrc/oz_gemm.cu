@@ -869,6 +869,17 @@ __device__ __forceinline__ void fixed71(double x, int E, long long& hi, int& lo)
   }
 }
 
+// x 2^(62 - e), rounded.
+__device__ __forceinline__ long long fixed62(double x, int E) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(u >> 52) & 0x7ff;
+  unsigned long long m = (u & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0);
+  const int sh = max(ex, 1) - E + 9;
+  if (sh >= 0) m <<= min(sh, 10);
+  else m = sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0;
+  return (long long)u < 0 ? -(long long)m : (long long)m;
+}
+
 // u 2^-e (u: the bits of a nonnegative double of a row of biased exponent E) truncated to bf16; at least 2^-41 for u > 0.
 __device__ __forceinline__ uint32_t mag16(unsigned long long u, int E) {
   const int ex = (int)(u >> 52), d = E - ex;
@@ -903,25 +914,28 @@ __device__ __forceinline__ unsigned put_mags(const double* x, int E, uint16_t* d
 // The planes of 8 consecutive reals of a row: digits from the last, each
 // balanced digit taken off with its carry; the plane value 2^(-9 s) d is formed
 // by adding d to the bits of 1.5 2^(23 - 9 s) and subtracting that number.
-// The first nd (7 or 8) are written: balanced digits left out are what rounding to the others leaves.
+// ND: 7, or 8 digits (whose first seven are the value rounded to 62 bits: balanced digits).
 // EMB: x holds 4 complex values, and the two rows (re, -im) and (im, re) are written.
-template <bool EMB>
-__device__ __forceinline__ void put8(const double* x, int E, uint16_t* dst, long plane, int ldp, int nd) {
+template <bool EMB, int ND>
+__device__ __forceinline__ void put8(const double* x, int E, uint16_t* dst, long plane, int ldp) {
   long long f[8];
   int l[8];
 #pragma unroll
   for (int i = 0; i < 8; i++) {
     f[i] = 0;
     l[i] = 0;
-    if (E != NB_ROW) fixed71(x[i], E, f[i], l[i]);
+    if (E != NB_ROW) {
+      if constexpr (ND == 8) fixed71(x[i], E, f[i], l[i]);
+      else f[i] = fixed62(x[i], E);
+    }
   }
 #pragma unroll
-  for (int s = 7; s >= 0; s--) {
+  for (int s = ND - 1; s >= 0; s--) {
     uint32_t v[8];
 #pragma unroll
     for (int i = 0; i < 8; i++) {
       int d;
-      if (s > 4) {
+      if (ND == 8 && s > 4) {
         l[i] += 256;
         d = (l[i] & 511) - 256;
         l[i] >>= 9;
@@ -936,7 +950,6 @@ __device__ __forceinline__ void put8(const double* x, int E, uint16_t* dst, long
       const float big = __int_as_float(0x4B400000 - ((9 * s) << 23));   // 1.5 2^(23 - 9 s)
       v[i] = __float_as_uint(__fsub_rn(__int_as_float(__float_as_int(big) + d), big));
     }
-    if (s >= nd) continue;
     uint32_t w[4];
 #pragma unroll
     for (int i = 0; i < 4; i++) w[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x7632);
@@ -954,13 +967,13 @@ __device__ __forceinline__ void put8(const double* x, int E, uint16_t* dst, long
 }
 
 // Digit planes dst[b][s][row][ldp] of an operand (K-contiguous rows): one
-// thread per 8 reals.  conj negates imaginary parts.
-template <int CX, bool EMB>
+// thread per 8 reals.  conj negates imaginary parts.  ND = 8: also the magnitudes.
+template <int CX, bool EMB, int ND>
 __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ src, long sb, long lr, int rows, int K,
                                                      int conj, const int* __restrict__ e, uint16_t* __restrict__ dst,
                                                      int ldp, uint16_t* __restrict__ mag, int ldm,
                                                      unsigned* __restrict__ sq) {
-  const int ng = (K * CX + 7) / 8, nd = mag ? 8 : 7;
+  const int ng = (K * CX + 7) / 8;
   const long i = (long)blockIdx.x * 256 + threadIdx.x;
   const unsigned act = __ballot_sync(0xffffffffu, i < (long)rows * ng);
   if (i >= (long)rows * ng) return;
@@ -981,8 +994,8 @@ __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ 
   }
   const long plane = (long)rows * (EMB ? 2 : 1) * ldp;
   const int E = e[b * rows + r];
-  put8<EMB>(x, E, dst + b * nd * plane + (long)r * (EMB ? 2 : 1) * ldp + k0 * CX, plane, ldp, nd);
-  if (mag) {
+  put8<EMB, ND>(x, E, dst + b * ND * plane + (long)r * (EMB ? 2 : 1) * ldp + k0 * CX, plane, ldp);
+  if (ND == 8) {
     // (integer sums: the same whatever their order)
     const unsigned q = put_mags<CX>(x, E, mag + (b * rows + r) * ldm + k0);
     int one;
@@ -998,13 +1011,12 @@ __global__ void __launch_bounds__(256) oz_slice_rows(const double* __restrict__ 
 
 // The same for row-contiguous sources (stride lk along K): a block turns a
 // tile of 32 rows by 8 / CX x 8 K values around in shared memory.
-template <int CX, bool EMB>
+template <int CX, bool EMB, int ND>
 __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ src, long sb, long lk, int rows, int K,
                                                      int conj, const int* __restrict__ e, uint16_t* __restrict__ dst,
                                                      int ldp, uint16_t* __restrict__ mag, int ldm,
                                                      unsigned* __restrict__ sq) {
   constexpr int KT = 64 / CX;                       // 64 reals of K
-  const int nd = mag ? 8 : 7;
   __shared__ double t[KT][33 * CX];
   __shared__ unsigned part[32];
   if (threadIdx.x < 32) part[threadIdx.x] = 0u;
@@ -1038,10 +1050,10 @@ __global__ void __launch_bounds__(256) oz_slice_cols(const double* __restrict__ 
   const long plane = (long)rows * (EMB ? 2 : 1) * ldp;
   if (in) {
     const int E = e[b * rows + r0 + r];
-    put8<EMB>(x, E, dst + b * nd * plane + (long)(r0 + r) * (EMB ? 2 : 1) * ldp + k0 * CX + 8 * c, plane, ldp, nd);
-    if (mag) atomicAdd(part + r, put_mags<CX>(x, E, mag + (b * rows + r0 + r) * ldm + k0 + 8 / CX * c));
+    put8<EMB, ND>(x, E, dst + b * ND * plane + (long)(r0 + r) * (EMB ? 2 : 1) * ldp + k0 * CX + 8 * c, plane, ldp);
+    if (ND == 8) atomicAdd(part + r, put_mags<CX>(x, E, mag + (b * rows + r0 + r) * ldm + k0 + 8 / CX * c));
   }
-  if (!mag) return;
+  if (ND == 7) return;
   __syncthreads();
   if (threadIdx.x < 32 && r0 + (int)threadIdx.x < rows) atomicAdd(sq + b * rows + r0 + threadIdx.x, part[threadIdx.x]);
 }
@@ -1097,17 +1109,17 @@ OzList list_at(void* at, long units) {
   return f;
 }
 
-template <int CX>
-cudaError_t prepare(const Side& a, int K, int batch, const Planes& p, cudaStream_t s) {
+template <int CX, int ND>
+cudaError_t prepare_digits(const Side& a, int K, int batch, const Planes& p, cudaStream_t s) {
   const int ldp = pad8i(K * CX), ldm = pad8i(K);
   if (a.lk == 1) {
     oz_exp_rows<CX><<<dim3((a.rows + 7) / 8, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, p.e, p.sq);
     const unsigned nb = (unsigned)(((long)a.rows * (ldp / 8) + 255) / 256);
     if (a.emb)
-      oz_slice_rows<2, true><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag,
+      oz_slice_rows<2, true, ND><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag,
                                                              ldm, p.sq);
     else
-      oz_slice_rows<CX, false><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, p.e, p.pl, ldp,
+      oz_slice_rows<CX, false, ND><<<dim3(nb, batch), 256, 0, s>>>(a.src, a.sb, a.lr, a.rows, K, a.conj, p.e, p.pl, ldp,
                                                                p.mag, ldm, p.sq);
   } else {
     cudaError_t st = cudaMemsetAsync(p.e, 0, 2 * sizeof(int) * (size_t)batch * a.rows, s);   // p.sq too
@@ -1116,11 +1128,16 @@ cudaError_t prepare(const Side& a, int K, int batch, const Planes& p, cudaStream
                                                                                         p.e);
     const dim3 grid((a.rows + 31) / 32, (K * CX + 63) / 64, batch);
     if (a.emb)
-      oz_slice_cols<2, true><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm, p.sq);
+      oz_slice_cols<2, true, ND><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm, p.sq);
     else
-      oz_slice_cols<CX, false><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm, p.sq);
+      oz_slice_cols<CX, false, ND><<<grid, 256, 0, s>>>(a.src, a.sb, a.lk, a.rows, K, a.conj, p.e, p.pl, ldp, p.mag, ldm, p.sq);
   }
   return cudaGetLastError();
+}
+
+template <int CX>
+cudaError_t prepare(const Side& a, int K, int batch, const Planes& p, cudaStream_t s) {
+  return p.mag ? prepare_digits<CX, 8>(a, K, batch, p, s) : prepare_digits<CX, 7>(a, K, batch, p, s);
 }
 
 // bf16 [n][rows][ldk] with K valid: digit planes in boxes of `digits` planes x
@@ -1397,7 +1414,7 @@ void oz_free(OzWork& w) {
 // The FP64 kernel takes 4.3 us per unit of K and round of its 64 x 64 tiles
 // over the SMs (two multiply-adds a clock on each): 35 us for one tile of
 // K = 8 (70 us measured for a stage of K = 8 to 16), and 0.3 ms for one of
-// K = 71.  The digit form's seven launches are 41 us in all at K = 12, 50 to 60
+// K = 71.  The digit form's eight launches are 45 us in all at K = 12, 55 to 65
 // at K = 16 to 40.
 bool oz_wins(int M, int N, int K, int batch) {
   const double tiles = ((M + 63) / 64) * (double)((N + 63) / 64) * batch;

@@ -35,8 +35,8 @@ cudaError_t gemm_z_best(int la, int lb, int M, int N, int K, const double2* A, i
                         int ldb, long sB, double2* C, int ldc, long sC, int batch, const OzWork& w, cudaStream_t s);
 
 // gemm_z's product (operand layouts of GemmA, GemmB) from digits.  check: to
-// FP64 accuracy of every entry (those that digits relative to the rows' largest
-// entries do not hold to it are computed in FP64); else to 4 K 2^-62 of the
+// FP64 accuracy of every entry (those that seven digits relative to the rows'
+// largest entries do not hold to it are computed with eight or in FP64); else to 4 K 2^-62 of the
 // product of the largest entries of its two rows.
 cudaError_t oz_gemm_z(int la, int lb, int M, int N, int K, const double2* A, int lda, long sA, const double2* B,
                       int ldb, long sB, double2* C, int ldc, long sC, int batch, bool check, const OzWork& w,
